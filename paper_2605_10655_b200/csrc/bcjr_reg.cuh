@@ -75,7 +75,14 @@ struct RegBlock {
         if (C::NWARP == 1) __syncwarp();
         else __syncthreads();
     }
-    __device__ __forceinline__ int cta_or(int v) const { return C::NWARP == 1 ? __any_sync(0xffffffffu, v) : __syncthreads_or(v); }
+    // a vote that also orders shared memory: what the threads wrote before it, they all read after it (a warp's vote alone does not)
+    __device__ __forceinline__ int cta_or(int v) const
+    {
+        if (C::NWARP > 1) return __syncthreads_or(v);
+        v = __any_sync(0xffffffffu, v);
+        __syncwarp();
+        return v;
+    }
     __device__ __forceinline__ void block_sync() const         // all CTAs of the block
     {
         if (C::CL > 1) cluster_sync();
