@@ -50,7 +50,7 @@ struct bcjr_ctx {
     int device = 0;
     int num_sms = 0;
     int max_smem_optin = 0;
-    Buffer hist, stepO, msg, gc_part, soft_copy, bp, path_ws, cb_beta, grad_w, grad_c, blk_defect, gauss_cb, lin_flag, lin_list, vit_flag, vit_list, staging[6];
+    Buffer hist, stepO, msg, gc_part, soft_copy, bp, path_ws, cb_beta, grad_w, grad_c, blk_defect, gauss_cb, lin_flag, lin_list, grad_bits, vit_flag, vit_list, staging[6];
     DeviceDiag *diag = nullptr;
     // saved by bcjr_soft_quantize for bcjr_backward
     bool have_fwd = false;
@@ -514,6 +514,23 @@ bcjr_status lin_make_list(bcjr_ctx *ctx, int64_t B, cudaStream_t st, const int *
     return BCJR_OK;
 }
 
+// Sizes of the upstream gradient, for the chunked linear kernels (bcjr_lin_bwd.cuh).
+bcjr_status grad_sizes(bcjr_ctx *ctx, BwdParams &p, cudaStream_t st)
+{
+    bcjr_status rc = ensure(ctx, ctx->grad_bits, ((size_t)p.B + 1) * 4);
+    if (rc) return rc;
+    uint32_t *bits = (uint32_t *)ctx->grad_bits.ptr;
+    CU(cudaMemsetAsync(bits, 0, 4, st));
+    int64_t grid = (p.B + 7) / 8;
+    if (grid > (int64_t)ctx->num_sms * 8) grid = (int64_t)ctx->num_sms * 8;
+    grad_bits_kernel<<<(int)grid, 256, 0, st>>>(p.g, p.B, p.n, bits + 1, bits);
+    ctx->launches += 1;
+    CU(cudaGetLastError());
+    p.g_top = bits;
+    p.g_bits = bits + 1;
+    return BCJR_OK;
+}
+
 // Forward call of the vector trellis on clusters of two CTAs (the table alone fits two tensor memories): the default.
 bcjr_status launch_fwd_vec2(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
 {
@@ -597,6 +614,8 @@ bcjr_status launch_bwd_vec4(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     if (lin) {
         CU(cudaMemsetAsync(ctx->gc_part.ptr, 0, (size_t)parts * S * V * 4, st));      // every launch adds into it
         BwdParams q = p;
+        if ((rc = grad_sizes(ctx, q, st))) return rc;
+        const uint32_t *g_bits = q.g_bits;
         q.stepO = (int *)ctx->stepO.ptr;
         q.lin_x = lin_exponent(p.lam2);
         for (int64_t b0 = 0; b0 < p.B; b0 += chunk) {
@@ -604,6 +623,7 @@ bcjr_status launch_bwd_vec4(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
             q.B = nb;
             q.W = p.W + b0 * p.n; q.g = p.g + b0 * p.n; q.soft = p.soft + b0 * p.n; q.gW = p.gW + b0 * p.n;
             q.lin_flag = (const uint8_t *)ctx->lin_flag.ptr + b0;
+            q.g_bits = g_bits + b0;
             acfg.gridDim = dim3((unsigned)(2 * (nb < acl ? nb : acl)), 1, 1);
             bcfg.gridDim = dim3((unsigned)(Bt::CL * (nb < bcl ? nb : bcl)), 1, 1);
             CU(cudaLaunchKernelEx(&acfg, bwd_vec_alpha_lin_kernel<VEC_ALPHA_NBLK>, q));
@@ -706,12 +726,14 @@ bcjr_status launch_bwd_lin(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     p.stepO = (int *)ctx->stepO.ptr;
     p.gc_part = ACC ? (float *)ctx->gc_part.ptr : nullptr;
     p.lin_x = lin_exponent(p.lam2);
+    if ((rc = grad_sizes(ctx, p, st))) return rc;
     BwdParams q = p;
     for (int64_t b0 = 0; b0 < p.B; b0 += chunk) {
         const int64_t nb = p.B - b0 < chunk ? p.B - b0 : chunk;
         q.B = nb;
         q.W = p.W + b0 * p.n; q.g = p.g + b0 * p.n; q.soft = p.soft + b0 * p.n; q.gW = p.gW + b0 * p.n;
         q.lin_flag = (const uint8_t *)ctx->lin_flag.ptr + b0;
+        q.g_bits = p.g_bits + b0;
         bwd_alpha_lin_kernel<2><<<(int)nb, A::THREADS, AlphaLinCfg<2>::SMEM_BYTES, st>>>(q);
         CU(cudaGetLastError());
         cfg.gridDim = dim3((unsigned)(C::CL * (nb < ncl ? nb : ncl)), 1, 1);
@@ -1220,7 +1242,7 @@ bcjr_status bcjr_destroy(bcjr_ctx *ctx)
     DeviceGuard guard(ctx->device);
     cudaDeviceSynchronize();
     Buffer *all[] = {&ctx->hist, &ctx->stepO, &ctx->msg, &ctx->gc_part, &ctx->soft_copy, &ctx->bp, &ctx->path_ws,
-                     &ctx->cb_beta, &ctx->grad_w, &ctx->grad_c, &ctx->blk_defect, &ctx->gauss_cb, &ctx->lin_flag, &ctx->lin_list, &ctx->vit_flag, &ctx->vit_list, &ctx->staging[0], &ctx->staging[1], &ctx->staging[2], &ctx->staging[3], &ctx->staging[4],
+                     &ctx->cb_beta, &ctx->grad_w, &ctx->grad_c, &ctx->blk_defect, &ctx->gauss_cb, &ctx->lin_flag, &ctx->lin_list, &ctx->grad_bits, &ctx->vit_flag, &ctx->vit_list, &ctx->staging[0], &ctx->staging[1], &ctx->staging[2], &ctx->staging[3], &ctx->staging[4],
                      &ctx->staging[5]};
     for (Buffer *b : all)
         if (b->ptr) cudaFree(b->ptr);
@@ -1778,7 +1800,7 @@ int64_t bcjr_workspace_bytes(const bcjr_ctx *ctx)
 {
     if (!ctx) return 0;
     const Buffer *all[] = {&ctx->hist, &ctx->stepO, &ctx->msg, &ctx->gc_part, &ctx->soft_copy, &ctx->bp,
-                           &ctx->path_ws, &ctx->cb_beta, &ctx->grad_w, &ctx->grad_c, &ctx->blk_defect, &ctx->gauss_cb, &ctx->lin_flag, &ctx->lin_list, &ctx->vit_flag, &ctx->vit_list, &ctx->staging[0], &ctx->staging[1], &ctx->staging[2], &ctx->staging[3],
+                           &ctx->path_ws, &ctx->cb_beta, &ctx->grad_w, &ctx->grad_c, &ctx->blk_defect, &ctx->gauss_cb, &ctx->lin_flag, &ctx->lin_list, &ctx->grad_bits, &ctx->vit_flag, &ctx->vit_list, &ctx->staging[0], &ctx->staging[1], &ctx->staging[2], &ctx->staging[3],
                            &ctx->staging[4], &ctx->staging[5]};
     int64_t tot = 0;
     for (const Buffer *b : all) tot += (int64_t)b->bytes;

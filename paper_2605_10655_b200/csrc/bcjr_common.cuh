@@ -187,6 +187,8 @@ struct BwdParams {
     float invT;              // 1/T
     int lin_x;               // linear-message kernels: exponent the largest forward message is scaled to
     const uint8_t *lin_flag; // linear-message kernels: [B] 1 = not certified, left to the log-domain kernel
+    const uint32_t *g_bits;  // chunked linear-message kernels: [B] bit pattern of the block's largest |g| (grad_bits_kernel)
+    const uint32_t *g_top;   // the largest of them all
     const int *list;         // log-domain kernels behind them: list[0] blocks to run, list[1 ...] their indices; null = all B blocks
     int list_max;            // listed blocks up to this number belong to bwd_reg_kernel, more to the chunked two-kernel form
     int list_base;           // chunked form: first listed block of the chunk (B = blocks in a chunk)

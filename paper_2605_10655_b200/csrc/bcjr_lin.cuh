@@ -73,6 +73,39 @@ __device__ __forceinline__ float2 ex2n_poly2(float2 a)
     return p;
 }
 
+// Backward kernels (see bcjr_lin_bwd.cuh): exponent of a gradient from the bit pattern of its largest |g| (NaN sorts above infinity);
+// GRAD_NONE: all zero.  The bounds keep both factors normal numbers.
+constexpr int GRAD_LEVEL = 2, GRAD_SPAN = 8, GRAD_ROOM = 2, GRAD_NONE = -1000;
+__device__ __forceinline__ uint32_t grad_bits(float g) { return __float_as_uint(fabsf(g)); }
+__device__ __forceinline__ int grad_exponent(uint32_t bits)
+{
+    const int e = (int)(bits >> 23) - 127;
+    return bits == 0u ? GRAD_NONE : e < -100 ? -100 : e > 112 ? 112 : e;
+}
+__device__ __forceinline__ float grad_down(int e) { return e == GRAD_NONE ? 1.f : pow2i(-(e + GRAD_LEVEL)); }
+__device__ __forceinline__ float grad_up(int e) { return e == GRAD_NONE ? 1.f : pow2i(e + GRAD_LEVEL); }
+// scale of a block in a call: the call's, GRAD_SPAN bits less, twice as many ...; the call's where the block has no gradient
+__device__ __forceinline__ int grad_scale(uint32_t bits, uint32_t top_bits)
+{
+    const int e = grad_exponent(bits), top = grad_exponent(top_bits);
+    return e == GRAD_NONE ? top : top - (top - e) / GRAD_SPAN * GRAD_SPAN;
+}
+// bits[b] of every block, *top (zero before the call) of all: a warp per block
+static __global__ void __launch_bounds__(256) grad_bits_kernel(const float *__restrict__ g, int64_t B, int n, uint32_t *__restrict__ bits, uint32_t *__restrict__ top)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t all = 0;
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < B; b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        uint32_t m = 0;
+#pragma unroll 4
+        for (int t = lane; t < n; t += 32) m = max(m, grad_bits(__ldg(g + b * n + t)));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) bits[b] = m;
+        all = max(all, m);
+    }
+    if (lane == 0 && all) atomicMax(top, all);
+}
+
 // Indices of the flagged blocks, ascending, behind their number: list[0] = count, list[1 + i].
 static __global__ void __launch_bounds__(1024) lin_list_kernel(const uint8_t *__restrict__ flag, int64_t B, int *__restrict__ list)
 {

@@ -12,6 +12,14 @@
 // is one product P z, P = E M_b, z = A g + (w - c)/T (A y + AA), where the un-normalised form would need three more
 // packed instructions per pair; its price is one reciprocal per group.
 //
+// Scale of the gradient.  The forward certificate covers A, M and the energies.  What the backward sweeps add to them -- AA, y, z --
+// is linear in g: with A at 2^103 a gradient of 2^16 overflows z where the exponential is zero (0 inf in grad_codebook), one of
+// 2^-34 loses AA's bits to subnormals.  So a block runs on g 2^-(e + 2), its largest |g| between 2^(e-7) and 2^(e+1): AA stays below
+// 2^115, z below 2^126 for weights of twenty units at T = 0.01, and a message of 2^-111 still has a normal AA.  The powers of two are
+// exact, so the results are those of any other scale bit for bit.  The accumulators of grad_codebook are at the block's scale; where
+// the next block's is another, they are written out first.  e is the exponent of the call's largest |g| for every block within
+// eight bits of it (grad_bits_kernel: 3 us for 4 million weights), so that this happens only where blocks differ by more.
+//
 // 592 blocks of 256 weights, T = 0.1: 11.85 -> 10.1 ms with grad_codebook, 11.2 (bwd_solo_kernel) -> 10.0 without
 // (alpha 8.4 k -> 6.1 k, beta 11.6 k clocks per step and block; ncu: alpha XU 67 %, FMA 47 %; beta XU 44 %, FMA 56 %, issue
 // 55 % with packed instructions counted once).
@@ -76,10 +84,12 @@ __global__ void __launch_bounds__(AlphaCfg<KB>::THREADS, 1) bwd_alpha_lin_kernel
     int *aux = p.stepO + (size_t)blk * C::AUX_INTS;
     float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);       // entry t - 1 belongs to step t
     const double isl_d = 1.0 / (double)sl;
+    const int e_g = grad_scale(p.g_bits[blk], *p.g_top);
+    const float down = grad_down(e_g);
     int outside = 0;
     for (int t = tid; t < n; t += CT) {
         const StepEnergy se = step_energy(__ldg(w_s + t), c_lo, c_hi, p.lam2);
-        const float g = __ldg(g_s + t), ws = se.wc * sl;
+        const float g = __ldg(g_s + t) * down, ws = se.wc * sl;
         step[t] = make_float4(ws, (se.wc + 2.f * se.delta) * sl, g * isl, lin_gs(g, ws, isl_d, __ldg(sf_s + t)));
         outside |= se.delta != 0.f;
     }
@@ -189,6 +199,7 @@ struct BetaLinCfg : SkewCfg {
     static constexpr int OFF_MBAR = OFF_PART + 256;
     static constexpr int OFF_TMEM = OFF_MBAR + 8;
     static constexpr int OFF_FLAG = OFF_TMEM + 2;
+    static constexpr int OFF_SCALE = OFF_FLAG + 1;              // scale of the accumulators (kept here: the sweep has no register for it)
     static constexpr int OFF_PUSH = OFF_FLAG + 2;
     static constexpr int SMEM_FLOATS = OFF_PUSH + 2 * BPT * THREADS;
     static constexpr size_t SMEM_BYTES = (size_t)SMEM_FLOATS * 4;
@@ -229,6 +240,7 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
     if (tid == 0) {
         for (int s = 0; s < 2; ++s) { mbar_init(mb_early + 8u * s, 1 + NWARP); mbar_init(mb_late + 8u * s, 1 + SLOTS); }
         *abort_flag = 0;
+        *reinterpret_cast<int *>(smem + C::OFF_SCALE) = GRAD_NONE;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc_512(smem_u32(const_cast<uint32_t *>(tmem_slot)));
@@ -256,14 +268,15 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
     }
     constexpr uint32_t BL_STEP = CT * 16u, BR_STEP = 256u * 16u;     // j0 = 1: next slot (own CTA) / upper half of the threads (peer)
     const uint32_t part_dst = mapa_u32(part_u32 + (uint32_t)((int)rank * NWARP + warp) * 16u, 0u);
-    if (ACC) {                                                   // zero the accumulators (laid out like the beta-paired codebook)
+    auto zero_acc = [&]() {                                     // the accumulators (laid out like the beta-paired codebook)
         float2 z[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) z[e] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int g = 0; g < BPT; ++g) tmem_st16(tm_acc + 16u * g, z);
         tmem_wait_st();
-    }
+    };
+    if (ACC) zero_acc();
 #pragma unroll
     for (int i = 0; i < BPT; ++i)                             // codebook -> TMEM, beta pairing: once per launch
         stage_codebook_scaled<C>(p.cb, C::x_of((int)rank, tid, i), tm_cb + (uint32_t)(16 * i), true, sl);
@@ -271,6 +284,27 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
     // test hook for the waits' abort path: one warp of CTA 0 withholds an arrival of its first block
     const bool drop_hook = blockIdx.x == 0 && warp == 1 && p.diag->drop_history_load != 0;
     float defect = 0.f;
+    int *e_acc = reinterpret_cast<int *>(smem + C::OFF_SCALE);  // scale of the accumulators; the first block sets it
+    // this cluster's partial of grad_codebook, added to what earlier launches left
+    auto write_acc = [&]() {
+        float *gc = p.gc_part + (size_t)cid * C::S;
+        const float up = grad_up(*e_acc);
+        tmem_wait_st();
+#pragma unroll
+        for (int i = 0; i < BPT; ++i) {
+            const int x = C::x_of((int)rank, tid, i);
+            float2 acc[8];
+            tmem_ld16(tm_acc + 16u * i, acc);
+            tmem_wait_ld(acc);
+#pragma unroll
+            for (int jh = 0; jh < K / 2; ++jh)
+#pragma unroll
+                for (int b = 0; b < K; ++b) {
+                    gc[(size_t)(2 * jh) * C::Q + (size_t)x * K + b] += up * acc[C::b_idx(jh, b)].x;
+                    gc[(size_t)(2 * jh + 1) * C::Q + (size_t)x * K + b] += up * acc[C::b_idx(jh, b)].y;
+                }
+        }
+    };
 
     for (int64_t blk = cid; blk < p.B; blk += ncl) {
         if (p.lin_flag[blk]) continue;                        // both CTAs alike
@@ -279,14 +313,19 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
         const float *w_s = p.W + blk * n, *g_s = p.g + blk * n, *sf_s = p.soft + blk * n;
         const float4 *hist4 = reinterpret_cast<const float4 *>(p.hist + (size_t)blk * n * 2 * C::Q) + tid;
         const int *aux = p.stepO + (size_t)blk * (C::MAX_N + 4);
+        const int e_g = grad_scale(p.g_bits[blk], *p.g_top);
+        const bool other = e_g != *e_acc;
+        if (ACC && other && *e_acc != GRAD_NONE) { write_acc(); zero_acc(); }
+        const float down = grad_down(e_g);
         int outside = 0;
         for (int t = tid; t < n; t += CT) {
             const StepEnergy se = step_energy(__ldg(w_s + t), c_lo, c_hi, p.lam2);
-            const float g = __ldg(g_s + t), ws = se.wc * sl;
+            const float g = __ldg(g_s + t) * down, ws = se.wc * sl;
             step[t] = make_float4(ws, g, lin_gs(g, ws, isl_d, __ldg(sf_s + t)), (float)(aux[t + 2] - aux[t + 1]));
             outside |= se.delta != 0.f;
         }
         const bool recentre = __syncthreads_or(outside) != 0;
+        if (other && tid == 0) *e_acc = e_g;
         {
             const float m1 = __int_as_float(aux[n + 2]);         // M_n = 1 / Z, Bt_n = 0
             for (int f = tid; f < C::BUF; f += CT) msg[ib * C::BUF + f] = (f & 1) ? 0.f : m1;
@@ -310,7 +349,7 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
                 float a0 = lane < SLOTS ? pp[0] : 0.f, a2 = lane < SLOTS ? pp[1] : 0.f, az = lane < SLOTS ? pp[2] : 0.f;
                 a0 = warp_sum(a0); a2 = warp_sum(a2); az = warp_sum(az);
                 if (lane == 0) {
-                    const float i0 = 1.f / a0;
+                    const float i0 = grad_up(*e_acc) / a0;
                     p.gW[blk * n + t - 1] = (__ldg(g_s + t - 1) - az * i0) + (a2 * i0) * (__ldg(w_s + t - 1) - __ldg(sf_s + t - 1)) * invT;
                     defect = fmaxf(defect, fabsf(a0 - 1.f));
                 }
@@ -437,25 +476,7 @@ __global__ void __launch_bounds__(SkewCfg::THREADS, 1) bwd_beta_lin_kernel(BwdPa
         }
         cluster_sync();                                          // block end
     }
-    // this cluster's partial of grad_codebook, added to what earlier launches left
-    if (ACC) {
-        float *gc = p.gc_part + (size_t)cid * C::S;
-        tmem_wait_st();
-#pragma unroll
-        for (int i = 0; i < BPT; ++i) {
-            const int x = C::x_of((int)rank, tid, i);
-            float2 acc[8];
-            tmem_ld16(tm_acc + 16u * i, acc);
-            tmem_wait_ld(acc);
-#pragma unroll
-            for (int jh = 0; jh < K / 2; ++jh)
-#pragma unroll
-                for (int b = 0; b < K; ++b) {
-                    gc[(size_t)(2 * jh) * C::Q + (size_t)x * K + b] += acc[C::b_idx(jh, b)].x;
-                    gc[(size_t)(2 * jh + 1) * C::Q + (size_t)x * K + b] += acc[C::b_idx(jh, b)].y;
-                }
-        }
-    }
+    if (ACC && *e_acc != GRAD_NONE) write_acc();
     if (tid == CT - 32 && rank == 0) diag_max(&p.diag->max_defect, defect);
     asm volatile("cp.async.wait_all;" ::: "memory");           // no copy may be in flight at exit (a warp may have left the loop early)
     tmem_wait_st();

@@ -590,8 +590,26 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
     const uint32_t ring = smem_u32(smem + C::OFF_RING) + (uint32_t)tid * 16u;
     const float4 *ring4 = reinterpret_cast<const float4 *>(smem + C::OFF_RING) + tid;
     constexpr uint32_t TX_MSG = (uint32_t)C::BUF * 4u, TX_MAX = CL * 4u;
-    const float2 ni2 = splat2(-p.invT * isl);
     float defect = 0.f;
+    const float2 ni2 = splat2(-p.invT * isl);
+    int e_acc = GRAD_NONE;                                      // scale of the accumulators (see bcjr_lin_bwd.cuh)
+    bool add = p.list != nullptr;                               // gc_part holds something already
+    auto write_acc = [&]() {
+        float *gc = p.gc_part + (size_t)cid * C::S;
+        const float up = grad_up(e_acc);
+#pragma unroll
+        for (int jp = 0; jp < 2; ++jp) {
+            float4 *g0 = reinterpret_cast<float4 *>(gc + (2 * jp) * C::Q + x * 4), *g1 = reinterpret_cast<float4 *>(gc + (2 * jp + 1) * C::Q + x * 4);
+            float4 a = make_float4(up * acc[jp][0].x, up * acc[jp][1].x, up * acc[jp][2].x, up * acc[jp][3].x);
+            float4 b = make_float4(up * acc[jp][0].y, up * acc[jp][1].y, up * acc[jp][2].y, up * acc[jp][3].y);
+            if (add) {
+                const float4 c = *g0, d = *g1;
+                a.x += c.x; a.y += c.y; a.z += c.z; a.w += c.w;
+                b.x += d.x; b.y += d.y; b.z += d.z; b.w += d.w;
+            }
+            *g0 = a; *g1 = b;
+        }
+    };
     // test hook for the waits' abort path: CTA 0 never arms one buffer of its first beta sweep, so that its wait runs out
     const bool drop_hook = CL > 1 && blockIdx.x == 0 && p.diag->drop_history_load != 0;
 
@@ -599,14 +617,35 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
         const int64_t blk = p.list ? (int64_t)p.list[1 + it] : it;
         const float *w = p.W + blk * n, *g = p.g + blk * n, *sf = p.soft + blk * n;
         int outside = 0;
+        uint32_t gmax = 0;
         for (int t = tid; t < n; t += NT) {
             const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
             const float gv = __ldg(g + t), ws = se.wc * sl;
             step[t] = make_float4(ws, (se.wc + 2.f * se.delta) * sl, gv, lin_gs(gv, ws, isl_d, __ldg(sf + t)));
             outside |= se.delta != 0.f;
+            gmax = max(gmax, grad_bits(gv));
         }
         if (tid == 0) step[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+        gmax = __reduce_max_sync(0xffffffffu, gmax);
+        if (C::NWARP > 1 && lane == 0) part[warp] = __uint_as_float(gmax);
         const bool recentre = rb.cta_or(outside) != 0;
+        if (C::NWARP > 1) gmax = __reduce_max_sync(0xffffffffu, lane < C::NWARP ? __float_as_uint(part[lane]) : 0u);
+        const int e_g = grad_exponent(gmax);
+        // the block runs at the accumulators' scale if its gradient is within GRAD_SPAN bits below it
+        if (e_g != GRAD_NONE && (e_g > e_acc || e_g < e_acc - GRAD_SPAN)) {
+            if (ACC && e_acc != GRAD_NONE) {
+                if (active) write_acc();
+                add = true;
+#pragma unroll
+                for (int jp = 0; jp < 2; ++jp)
+#pragma unroll
+                    for (int l = 0; l < K; ++l) acc[jp][l] = make_float2(0.f, 0.f);
+            }
+            e_acc = e_g + GRAD_ROOM;
+        }
+        const float down = grad_down(e_acc);
+        for (int t = tid; t < n; t += NT) { step[t].z *= down; step[t].w *= down; }
+        rb.cta_sync();
         auto run = [&](auto lin_tag, auto rc_tag) {
             constexpr bool LIN = decltype(lin_tag)::value, RC = decltype(rc_tag)::value;
             // ================= alpha sweep
@@ -794,7 +833,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
                 } else {
                     a0 = sums[t].x; a2 = sums[t].y; az = sums[t].z;
                 }
-                const float i0 = 1.f / a0;
+                const float i0 = grad_up(e_acc) / a0;
                 p.gW[blk * n + t] = (__ldg(g + t) - az * i0) + (a2 * i0) * (__ldg(w + t) - __ldg(sf + t)) * p.invT;
                 defect = fmaxf(defect, fabsf(a0 - 1.f));
             }
@@ -804,20 +843,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
         else run(std::true_type{}, std::false_type{});
         rb.block_sync();
     }
-    if (ACC && active) {
-        float *gc = p.gc_part + (size_t)cid * C::S;
-#pragma unroll
-        for (int jp = 0; jp < 2; ++jp) {
-            float4 *g0 = reinterpret_cast<float4 *>(gc + (2 * jp) * C::Q + x * 4), *g1 = reinterpret_cast<float4 *>(gc + (2 * jp + 1) * C::Q + x * 4);
-            float4 a = make_float4(acc[jp][0].x, acc[jp][1].x, acc[jp][2].x, acc[jp][3].x), b = make_float4(acc[jp][0].y, acc[jp][1].y, acc[jp][2].y, acc[jp][3].y);
-            if (p.list) {
-                const float4 c = *g0, d = *g1;
-                a.x += c.x; a.y += c.y; a.z += c.z; a.w += c.w;
-                b.x += d.x; b.y += d.y; b.z += d.z; b.w += d.w;
-            }
-            *g0 = a; *g1 = b;
-        }
-    }
+    if (ACC && active) write_acc();
     defect = warp_max(defect);
     if (lane == 0) diag_max(&p.diag->max_defect, defect);
     if (CL > 1) {

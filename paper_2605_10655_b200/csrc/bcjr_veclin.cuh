@@ -434,8 +434,11 @@ __global__ void __launch_bounds__(Vec2Cfg<NBLK_>::THREADS, 1) bwd_vec_alpha_lin_
             if (!((live >> k) & 1u)) continue;
             const float2 *w = reinterpret_cast<const float2 *>(p.W + (base + k) * n), *g = reinterpret_cast<const float2 *>(p.g + (base + k) * n);
             const float2 *sf = reinterpret_cast<const float2 *>(p.soft + (base + k) * n);
+            const float down = grad_down(grad_scale(p.g_bits[base + k], *p.g_top));
             for (int t = tid; t < nt; t += CT) {
-                const float2 wt = __ldg(w + t), gt = __ldg(g + t), st = __ldg(sf + t);
+                const float2 wt = __ldg(w + t), st = __ldg(sf + t);
+                float2 gt = __ldg(g + t);
+                gt.x *= down; gt.y *= down;
                 step[k * MAX_NT + t] = make_float4(wt.x * sl, wt.y * sl, gt.x * isl, gt.y * isl);
                 gs_s[k * GSTR + t] = vec_gs(gt.x, gt.y, wt.x * sl, wt.y * sl, isl_d, st.x, st.y);
             }
@@ -601,14 +604,34 @@ __global__ void __launch_bounds__(VecBetaLinCfg<NBLK_>::THREADS, 1) bwd_vec_beta
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t tm = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 128);
     const uint32_t tm_acc = tm + 64u;
-    {
+    auto zero_acc = [&]() {
         float2 z[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) z[e] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < UNITS; ++u) tmem_st16(tm_acc + 16u * u, z);
-        vec4_stage_table(tm, p.cb_beta, q0b, sl);                // waits for both
-    }
+        tmem_wait_st();
+    };
+    zero_acc();
+    vec4_stage_table(tm, p.cb_beta, q0b, sl);
+    int e_acc = GRAD_NONE;                                       // scale of the accumulators (see bcjr_lin_bwd.cuh)
+    // the accumulators added to this cluster's partial of the table gradient, in the regrouped layout [b][q][V]
+    auto write_acc = [&]() {
+        float *gc = p.gc_part + (size_t)cid * C::S * 2;
+        const float up = grad_up(e_acc);
+#pragma unroll
+        for (int un = 0; un < UNITS; ++un) {
+            float2 acc[8];
+            tmem_ld16(tm_acc + 16u * un, acc);
+            tmem_wait_ld(acc);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float4 *dst = reinterpret_cast<float4 *>(gc + ((size_t)(4 * un + e) * Q + q0b) * 2);
+                const float4 o = *dst;                           // (z0.x, z0.y, z1.x, z1.y)
+                *dst = make_float4(o.x + up * acc[2 * e].x, o.y + up * acc[2 * e + 1].x, o.z + up * acc[2 * e].y, o.w + up * acc[2 * e + 1].y);
+            }
+        }
+    };
     uint32_t full_phase = 0;
     int ib = 0;
     float defect = 0.f;
@@ -620,138 +643,140 @@ __global__ void __launch_bounds__(VecBetaLinCfg<NBLK_>::THREADS, 1) bwd_vec_beta
 
     int left = range.count;
     for (int64_t base = range.begin; left > 0; base += range.depth, left -= range.depth) {
-        const uint32_t live = vec_live<NBLK>(p.lin_flag, base, left < range.depth ? left : range.depth);   // all four CTAs alike
-        if (live == 0) continue;
-        for (int k = 0; k < range.depth; ++k) {
-            if (!((live >> k) & 1u)) continue;
-            const float2 *w = reinterpret_cast<const float2 *>(p.W + (base + k) * n), *g = reinterpret_cast<const float2 *>(p.g + (base + k) * n);
-            const float2 *sf = reinterpret_cast<const float2 *>(p.soft + (base + k) * n);
-            const int *aux = p.stepO + (size_t)(base + k) * VecAlphaLinCfg<1>::AUX_INTS;
-            for (int t = tid; t < nt; t += CT) {
-                const float2 wt = __ldg(w + t), gt = __ldg(g + t), st = __ldg(sf + t);
-                step[k * MAX_NT + t] = make_float4(wt.x * sl, wt.y * sl, gt.x, gt.y);
-                gso[k * MAX_NT + t] = make_float2(vec_gs(gt.x, gt.y, wt.x * sl, wt.y * sl, isl_d, st.x, st.y), (float)aux[t + 1]);
+        uint32_t todo = vec_live<NBLK>(p.lin_flag, base, left < range.depth ? left : range.depth);   // all four CTAs alike
+        while (todo) {                                           // blocks with gradients of one scale side by side: as a rule all of them
+            int e_g = 0;
+            uint32_t live = 0;
+            for (int k = 0; k < range.depth; ++k) {
+                if (!((todo >> k) & 1u)) continue;
+                const int e = grad_scale(p.g_bits[base + k], *p.g_top);
+                if (live == 0) e_g = e;
+                if (e == e_g) live |= 1u << k;
             }
-            const float m1 = __int_as_float(aux[0]);             // M_nt = 1 / Z, Bt_nt = 0
-            float *m0 = msg + (size_t)(ib * NBLK + k) * 2 * QC;
-            for (int q = tid; q < QC; q += CT) { m0[q] = m1; m0[QC + q] = 0.f; }
-        }
-        // history, requested one turn (block and step) ahead
-        const int k0 = __ffs(live) - 1;
-        float4 H = __ldcg(hist + ((size_t)(base + k0) * nt + nt - 1) * (Q / 2));
-        cluster_sync();
-        // rank 0, warp k: turn the sums of step t of block k (slots of buffer b) into grad_W of that step
-        auto finish_step = [&](int t, int b, int k) {
-            if (rank == 0 && warp == k) {
-                const float *pp = part + (size_t)((b * NBLK + k) * 64) * 4;
-                const float4 s4 = *reinterpret_cast<const float4 *>(pp + lane * 4);
-                const float4 o = *reinterpret_cast<const float4 *>(pp + (lane + 32) * 4);
-                const float v4 = warp_sum4_split(s4.x + o.x, s4.y + o.y, s4.z + o.z, s4.w + o.w, lane);
-                const float a0 = __shfl_sync(0xffffffffu, v4, 0), a2 = __shfl_sync(0xffffffffu, v4, 8);
-                const float z0 = __shfl_sync(0xffffffffu, v4, 16), z1 = __shfl_sync(0xffffffffu, v4, 24);
-                if (lane == 0) {
-                    const int64_t at = (base + k) * n + 2 * (t - 1);
-                    const float2 wt = __ldg(reinterpret_cast<const float2 *>(p.W + at)), gt = __ldg(reinterpret_cast<const float2 *>(p.g + at));
-                    const float2 st = __ldg(reinterpret_cast<const float2 *>(p.soft + at));
-                    const float i0 = 1.f / a0;
-                    *reinterpret_cast<float2 *>(p.gW + at) = make_float2((gt.x - z0 * i0) + (a2 * i0) * (wt.x - st.x) * invT,
-                                                                         (gt.y - z1 * i0) + (a2 * i0) * (wt.y - st.y) * invT);
-                    defect = fmaxf(defect, fabsf(a0 - 1.f));
+            todo &= ~live;
+            if (e_g != e_acc) {
+                if (e_acc != GRAD_NONE) { write_acc(); zero_acc(); }
+                e_acc = e_g;
+            }
+            const float down = grad_down(e_g);
+            for (int k = 0; k < range.depth; ++k) {
+                if (!((live >> k) & 1u)) continue;
+                const float2 *w = reinterpret_cast<const float2 *>(p.W + (base + k) * n), *g = reinterpret_cast<const float2 *>(p.g + (base + k) * n);
+                const float2 *sf = reinterpret_cast<const float2 *>(p.soft + (base + k) * n);
+                const int *aux = p.stepO + (size_t)(base + k) * VecAlphaLinCfg<1>::AUX_INTS;
+                for (int t = tid; t < nt; t += CT) {
+                    const float2 wt = __ldg(w + t), st = __ldg(sf + t);
+                    float2 gt = __ldg(g + t);
+                    gt.x *= down; gt.y *= down;
+                    step[k * MAX_NT + t] = make_float4(wt.x * sl, wt.y * sl, gt.x, gt.y);
+                    gso[k * MAX_NT + t] = make_float2(vec_gs(gt.x, gt.y, wt.x * sl, wt.y * sl, isl_d, st.x, st.y), (float)aux[t + 1]);
                 }
+                const float m1 = __int_as_float(aux[0]);             // M_nt = 1 / Z, Bt_nt = 0
+                float *m0 = msg + (size_t)(ib * NBLK + k) * 2 * QC;
+                for (int q = tid; q < QC; q += CT) { m0[q] = m1; m0[QC + q] = 0.f; }
             }
-        };
-        for (int t = nt; t >= 1; --t) {
-            const int ob = ib == NBUF - 1 ? 0 : ib + 1;
+            // history, requested one turn (block and step) ahead
+            const int k0 = __ffs(live) - 1;
+            float4 H = __ldcg(hist + ((size_t)(base + k0) * nt + nt - 1) * (Q / 2));
+            cluster_sync();
+            // rank 0, warp k: turn the sums of step t of block k (slots of buffer b) into grad_W of that step
+            auto finish_step = [&](int t, int b, int k) {
+                if (rank == 0 && warp == k) {
+                    const float *pp = part + (size_t)((b * NBLK + k) * 64) * 4;
+                    const float4 s4 = *reinterpret_cast<const float4 *>(pp + lane * 4);
+                    const float4 o = *reinterpret_cast<const float4 *>(pp + (lane + 32) * 4);
+                    const float v4 = warp_sum4_split(s4.x + o.x, s4.y + o.y, s4.z + o.z, s4.w + o.w, lane);
+                    const float a0 = __shfl_sync(0xffffffffu, v4, 0), a2 = __shfl_sync(0xffffffffu, v4, 8);
+                    const float z0 = __shfl_sync(0xffffffffu, v4, 16), z1 = __shfl_sync(0xffffffffu, v4, 24);
+                    if (lane == 0) {
+                        const int64_t at = (base + k) * n + 2 * (t - 1);
+                        const float2 wt = __ldg(reinterpret_cast<const float2 *>(p.W + at)), gt = __ldg(reinterpret_cast<const float2 *>(p.g + at));
+                        const float2 st = __ldg(reinterpret_cast<const float2 *>(p.soft + at));
+                        const float i0 = grad_up(e_acc) / a0;
+                        *reinterpret_cast<float2 *>(p.gW + at) = make_float2((gt.x - z0 * i0) + (a2 * i0) * (wt.x - st.x) * invT,
+                                                                             (gt.y - z1 * i0) + (a2 * i0) * (wt.y - st.y) * invT);
+                        defect = fmaxf(defect, fabsf(a0 - 1.f));
+                    }
+                }
+            };
+            for (int t = nt; t >= 1; --t) {
+                const int ob = ib == NBUF - 1 ? 0 : ib + 1;
+#pragma unroll
+                for (int k = 0; k < NBLK; ++k) {
+                    if ((live >> k) & 1u) {
+                        const int si = ib * NBLK + k, so = ob * NBLK + k;
+                        float2 cb[2][8], acc[8];
+                        tmem_ld16(tm, cb[0]);
+                        const float4 sp = step[k * MAX_NT + t - 1];
+                        const float2 so2 = gso[k * MAX_NT + t - 1];
+                        const float2 wx = splat2(sp.x), wy = splat2(sp.y), gx = splat2(sp.z * isl), gy = splat2(sp.w * isl), off2 = splat2(so2.y);
+                        const float2 A2 = make_float2(H.x, H.y), AA2 = make_float2(H.z, H.w), ni2 = splat2(-invT * isl);
+                        const float2 fgx = mul2(A2, splat2(sp.z)), fgy = mul2(A2, splat2(sp.w)), nf = mul2(A2, ni2), nfA = mul2(AA2, ni2);
+                        const uint32_t later = live >> (k + 1) << (k + 1);
+                        const int tn = later ? t : t > 1 ? t - 1 : 1, kn = later ? __ffs(later) - 1 : k0;
+                        H = __ldcg(hist + ((size_t)(base + kn) * nt + tn - 1) * (Q / 2));
+                        if (t < nt) {
+                            wait_inputs(ib, k);
+                            finish_step(t + 1, ib, k);
+                        }
+                        const float *Min = msg + (size_t)si * 2 * QC + 4 * lane, *Bin = Min + QC;           // [b >> 1][x >> 1][b & 1][x & 1], x = 2 lane
+                        if (tid == 0) pr.expect_tx(mbar_full + 8u * so, rank == 0 ? TX_MSG + TX_PART : TX_MSG);
+                        float2 sum = make_float2(0.f, 0.f), ya = sum, Z0 = sum, Z1 = sum;
+#pragma unroll
+                        for (int un = 0; un < UNITS; ++un) {
+                            tmem_ld16(tm_acc + 16u * un, acc);
+                            if (un + 1 < UNITS) tmem_ld16(tm + 16u * (un + 1), cb[(un + 1) & 1]);
+                            if (un == 0) tmem_wait_ld(cb[0]);
+                            tmem_wait_ld(acc);
+                            if (un + 1 < UNITS) tmem_wait_ld(cb[(un + 1) & 1]);
+#pragma unroll
+                            for (int e = 0; e < 4; e += 2) {
+                                const int b = 4 * un + e;
+                                const float4 Mv = *reinterpret_cast<const float4 *>(Min + 128 * (b >> 1));
+                                const float4 Bv = *reinterpret_cast<const float4 *>(Bin + 128 * (b >> 1));
+#pragma unroll
+                                for (int bb = 0; bb < 2; ++bb) {
+                                    const int c = 2 * (e + bb);
+                                    const float2 dx = sub2(cb[un & 1][c], wx), dy = sub2(cb[un & 1][c + 1], wy);
+                                    const float2 ex = ex2n2(fma2(dy, dy, fma2(dx, dx, off2)));
+                                    const float2 y = fma2(gx, dx, fma2(gy, dy, bb == 0 ? make_float2(Bv.x, Bv.y) : make_float2(Bv.z, Bv.w)));   // h - gs + Bt
+                                    const float2 pb = mul2(ex, bb == 0 ? make_float2(Mv.x, Mv.y) : make_float2(Mv.z, Mv.w));
+                                    const float2 r = fma2(nf, y, nfA);                                       // -A r / (T sl)
+                                    const float2 zx = fma2(dx, r, fgx), zy = fma2(dy, r, fgy);               // A (g_v + (w_v - c_v) r / T)
+                                    sum = add2(sum, pb);
+                                    ya = fma2(pb, y, ya);
+                                    Z0 = fma2(pb, zx, Z0); Z1 = fma2(pb, zy, Z1);
+                                    acc[c] = fma2(pb, zx, acc[c]);
+                                    acc[c + 1] = fma2(pb, zy, acc[c + 1]);
+                                }
+                            }
+                            tmem_st16(tm_acc + 16u * un, acc);
+                        }
+                        const float2 outB = fma2(ya, rcpf2(make_float2(fmaxf(sum.x, 1e-37f), fmaxf(sum.y, 1e-37f))), splat2(so2.x));
+                        const uint32_t dst = push_b + (uint32_t)(so * 2 * QC) * 4u;
+                        const float2 mx = vec_pair_x(sum, lane), bx = vec_pair_x(outB, lane);
+                        pr.async_v2(dst, mx.x, mx.y, push_b_mbar + 8u * so);
+                        pr.async_v2(dst + QC * 4u, bx.x, bx.y, push_b_mbar + 8u * so);
+                        const float2 S0 = mul2(A2, sum), S2 = fma2(AA2, sum, mul2(A2, ya));
+                        const float v4 = warp_sum4_split(S0.x + S0.y, S2.x + S2.y, Z0.x + Z0.y, Z1.x + Z1.y, lane);   // lanes 0, 8, 16, 24
+                        if ((lane & 7) == 0)
+                            pr.async_f32(part_dst + (uint32_t)(so * 256 + (lane >> 3)) * 4u, v4, part_mbar + 8u * so);
+                        tmem_wait_st();
+                    }
+                }
+                ib = ob;
+            }
 #pragma unroll
             for (int k = 0; k < NBLK; ++k) {
                 if ((live >> k) & 1u) {
-                    const int si = ib * NBLK + k, so = ob * NBLK + k;
-                    float2 cb[2][8], acc[8];
-                    tmem_ld16(tm, cb[0]);
-                    const float4 sp = step[k * MAX_NT + t - 1];
-                    const float2 so2 = gso[k * MAX_NT + t - 1];
-                    const float2 wx = splat2(sp.x), wy = splat2(sp.y), gx = splat2(sp.z * isl), gy = splat2(sp.w * isl), off2 = splat2(so2.y);
-                    const float2 A2 = make_float2(H.x, H.y), AA2 = make_float2(H.z, H.w), ni2 = splat2(-invT * isl);
-                    const float2 fgx = mul2(A2, splat2(sp.z)), fgy = mul2(A2, splat2(sp.w)), nf = mul2(A2, ni2), nfA = mul2(AA2, ni2);
-                    const uint32_t later = live >> (k + 1) << (k + 1);
-                    const int tn = later ? t : t > 1 ? t - 1 : 1, kn = later ? __ffs(later) - 1 : k0;
-                    H = __ldcg(hist + ((size_t)(base + kn) * nt + tn - 1) * (Q / 2));
-                    if (t < nt) {
-                        wait_inputs(ib, k);
-                        finish_step(t + 1, ib, k);
-                    }
-                    const float *Min = msg + (size_t)si * 2 * QC + 4 * lane, *Bin = Min + QC;           // [b >> 1][x >> 1][b & 1][x & 1], x = 2 lane
-                    if (tid == 0) pr.expect_tx(mbar_full + 8u * so, rank == 0 ? TX_MSG + TX_PART : TX_MSG);
-                    float2 sum = make_float2(0.f, 0.f), ya = sum, Z0 = sum, Z1 = sum;
-#pragma unroll
-                    for (int un = 0; un < UNITS; ++un) {
-                        tmem_ld16(tm_acc + 16u * un, acc);
-                        if (un + 1 < UNITS) tmem_ld16(tm + 16u * (un + 1), cb[(un + 1) & 1]);
-                        if (un == 0) tmem_wait_ld(cb[0]);
-                        tmem_wait_ld(acc);
-                        if (un + 1 < UNITS) tmem_wait_ld(cb[(un + 1) & 1]);
-#pragma unroll
-                        for (int e = 0; e < 4; e += 2) {
-                            const int b = 4 * un + e;
-                            const float4 Mv = *reinterpret_cast<const float4 *>(Min + 128 * (b >> 1));
-                            const float4 Bv = *reinterpret_cast<const float4 *>(Bin + 128 * (b >> 1));
-#pragma unroll
-                            for (int bb = 0; bb < 2; ++bb) {
-                                const int c = 2 * (e + bb);
-                                const float2 dx = sub2(cb[un & 1][c], wx), dy = sub2(cb[un & 1][c + 1], wy);
-                                const float2 ex = ex2n2(fma2(dy, dy, fma2(dx, dx, off2)));
-                                const float2 y = fma2(gx, dx, fma2(gy, dy, bb == 0 ? make_float2(Bv.x, Bv.y) : make_float2(Bv.z, Bv.w)));   // h - gs + Bt
-                                const float2 pb = mul2(ex, bb == 0 ? make_float2(Mv.x, Mv.y) : make_float2(Mv.z, Mv.w));
-                                const float2 r = fma2(nf, y, nfA);                                       // -A r / (T sl)
-                                const float2 zx = fma2(dx, r, fgx), zy = fma2(dy, r, fgy);               // A (g_v + (w_v - c_v) r / T)
-                                sum = add2(sum, pb);
-                                ya = fma2(pb, y, ya);
-                                Z0 = fma2(pb, zx, Z0); Z1 = fma2(pb, zy, Z1);
-                                acc[c] = fma2(pb, zx, acc[c]);
-                                acc[c + 1] = fma2(pb, zy, acc[c + 1]);
-                            }
-                        }
-                        tmem_st16(tm_acc + 16u * un, acc);
-                    }
-                    const float2 outB = fma2(ya, rcpf2(make_float2(fmaxf(sum.x, 1e-37f), fmaxf(sum.y, 1e-37f))), splat2(so2.x));
-                    const uint32_t dst = push_b + (uint32_t)(so * 2 * QC) * 4u;
-                    const float2 mx = vec_pair_x(sum, lane), bx = vec_pair_x(outB, lane);
-                    pr.async_v2(dst, mx.x, mx.y, push_b_mbar + 8u * so);
-                    pr.async_v2(dst + QC * 4u, bx.x, bx.y, push_b_mbar + 8u * so);
-                    const float2 S0 = mul2(A2, sum), S2 = fma2(AA2, sum, mul2(A2, ya));
-                    const float v4 = warp_sum4_split(S0.x + S0.y, S2.x + S2.y, Z0.x + Z0.y, Z1.x + Z1.y, lane);   // lanes 0, 8, 16, 24
-                    if ((lane & 7) == 0)
-                        pr.async_f32(part_dst + (uint32_t)(so * 256 + (lane >> 3)) * 4u, v4, part_mbar + 8u * so);
-                    tmem_wait_st();
+                    wait_inputs(ib, k);                                          // the sums of step 1
+                    finish_step(1, ib, k);
                 }
             }
-            ib = ob;
-        }
-#pragma unroll
-        for (int k = 0; k < NBLK; ++k) {
-            if ((live >> k) & 1u) {
-                wait_inputs(ib, k);                                          // the sums of step 1
-                finish_step(1, ib, k);
-            }
-        }
-        cluster_sync();         // nobody still reads this batch's buffers when the next batch starts
-    }
-    // added to this cluster's partial of the table gradient, in the regrouped layout [b][q][V]
-    {
-        float *gc = p.gc_part + (size_t)cid * C::S * 2;
-#pragma unroll
-        for (int un = 0; un < UNITS; ++un) {
-            float2 acc[8];
-            tmem_ld16(tm_acc + 16u * un, acc);
-            tmem_wait_ld(acc);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                float4 *dst = reinterpret_cast<float4 *>(gc + ((size_t)(4 * un + e) * Q + q0b) * 2);
-                const float4 o = *dst;
-                *dst = make_float4(o.x + acc[2 * e].x, o.y + acc[2 * e + 1].x, o.z + acc[2 * e].y, o.w + acc[2 * e + 1].y);   // (z0.x, z0.y, z1.x, z1.y)
-            }
+            cluster_sync();         // nobody still reads this batch's buffers when the next batch starts
         }
     }
+    if (e_acc != GRAD_NONE) write_acc();
     if (rank == 0 && lane == 0 && warp < NBLK) diag_max(&p.diag->max_defect, defect);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -41,3 +41,71 @@ def test_one_warp_blocks_start_from_their_own_first_step(ctx, Lb, B, messages):
     ref_b = oracle.backward(W, c, g, Lb, 2, T)
     assert parity.rel_inf(got["grad_W"], ref_b["grad_W"]) <= 1e-5          # three float32 steps
     assert parity.rel_inf(got["grad_codebook"], ref_b["grad_codebook"]) <= 1e-5
+
+
+def _gradients(ctx, W, c, g, T, V=1):
+    import torch
+    dev = torch.device("cuda", ctx.device)
+    Lb = (c.shape[0] - 1).bit_length()
+    Wd, cd, gd = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (W, c, g))
+    if V == 2:
+        ctx.bcjr_soft_quantize_vec(Wd, cd, Lb, 2, 2, W.shape[1], T)
+    else:
+        ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, W.shape[1], T)
+    gW, gc = ctx.bcjr_backward(gd)
+    assert ctx.sync_status().device_status == 0
+    return gW.cpu().numpy(), gc.cpu().numpy()
+
+
+# cold calls whose messages reach the ends of float32's range, in the chunked, the vector and the register kernels
+SCALE_CASES = [(16, 1, 256, 1184, 0.0095), (16, 1, 48, 1200, 0.012), (16, 2, 64, 296, 0.0095), (12, 1, 256, 900, 0.02), (9, 1, 100, 900, 0.03),
+               (16, 1, 40, 3, 0.03)]
+
+
+@pytest.mark.parametrize("Lb,V,n,B,T", SCALE_CASES)
+def test_gradients_do_not_depend_on_the_scale_of_the_upstream_gradient(ctx, Lb, V, n, B, T):
+    # The backward pass is linear in the upstream gradient, and a power of two multiplies a float32 number exactly: so it does the
+    # results, bit for bit, as long as neither they nor the gradient leave the normal range (a subnormal result is off by 2^-149 at each
+    # of a few thousand additions).
+    W, c, g = _rand(n, Lb, B, seed=40 + Lb + n)
+    if V == 2:
+        c = np.random.default_rng(41).standard_normal((1 << Lb, 2)).astype(np.float32)
+    g[np.abs(g) < 2.0 ** -20] = 0.5
+    pick = np.unique(np.linspace(0, B - 1, 6).astype(int))
+    gW, gc = _gradients(ctx, W, c, g, T, V)
+    assert np.all(np.isfinite(gW)) and np.all(np.isfinite(gc))
+    if V == 1:
+        ref = oracle.backward(W[pick], c, g[pick], Lb, 2, T)
+        assert parity.rel_inf(gW[pick], ref["grad_W"]) <= parity.GRAD_TOL
+    for e in (20, 60, -30, -60):
+        sW, sc = _gradients(ctx, W, c, np.ldexp(g, e), T, V)
+        np.testing.assert_allclose(sW, np.ldexp(gW, e), rtol=0, atol=2.0 ** -130, err_msg=f"grad_W, gradient times 2^{e}")
+        # a log-domain block flushes what lies 2^-126 below its gradient
+        np.testing.assert_allclose(sc, np.ldexp(gc, e), rtol=0, atol=2.0 ** -126 * max(1.0, float(np.abs(np.ldexp(gc, e)).max())),
+                                   err_msg=f"grad_codebook, gradient times 2^{e}")
+
+
+@pytest.mark.parametrize("Lb,V,n,B,T", SCALE_CASES)
+def test_gradients_of_blocks_at_different_scales(ctx, Lb, V, n, B, T):
+    # Every block at a scale of its own, some without a gradient: grad_W of a block is what it is alone, and grad_codebook is the sum
+    # over the blocks -- here of the blocks at the three largest scales against the same sum with the others' gradients at zero.
+    W, c, g = _rand(n, Lb, B, seed=50 + Lb + n)
+    if V == 2:
+        c = np.random.default_rng(41).standard_normal((1 << Lb, 2)).astype(np.float32)
+    g[np.abs(g) < 2.0 ** -20] = 0.5
+    e = np.random.default_rng(51).permutation(np.resize(np.array([0, 1, 3, -12, -14, -45, -90, 30, 31], dtype=int), B))
+    e[0] = 31
+    zero = np.arange(B) % 5 == 3
+    g[zero] = 0.0
+    gW, _ = _gradients(ctx, W, c, g, T, V)
+    sW, sc = _gradients(ctx, W, c, np.ldexp(g, e[:, None]), T, V)
+    # The scale a block runs at depends on the others' within eight bits, and with it what the coldest messages lose to subnormals: at most
+    # 3e-7 of the block's gradient seen at T = 0.0095, on blocks whose float32 error is 1e-4; nothing at T = 0.012.
+    want = np.ldexp(gW.astype(np.float64), e[:, None])
+    assert np.all(np.abs(sW - want).max(axis=1) <= 2.0 ** -20 * np.abs(want).max(axis=1) + 2.0 ** -130)
+    big = g.copy()
+    big[e < 30] = 0.0
+    _, bc = _gradients(ctx, W, c, np.ldexp(big, e[:, None]), T, V)
+    # what the smaller blocks add is below 2^-27 of the largest; the sums are taken in another order, over up to a few hundred thousand
+    # terms of either sign: a few hundred half-ulps of the largest partial sum
+    assert np.abs(sc - bc).max() <= 2e-5 * np.abs(bc).max()
