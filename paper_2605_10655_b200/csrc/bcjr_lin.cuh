@@ -324,15 +324,14 @@ __global__ void __launch_bounds__(SoloCfg<KB>::THREADS, 1) fwd_lin_kernel(FwdPar
             else issue_chunk(c);
         }
         uint32_t slot = 0;
-        // warp 0: soft of step t from the partial sums of parity b
+        // warp 0: soft of step t from the partial sums of parity b, kept in v_s until the block has its certificate
         auto finish_step = [&](int t, int b) {
             float a = lane < NWARP ? part[(b * 32 + lane) * 2] : 0.f;
             float c = lane < NWARP ? part[(b * 32 + lane) * 2 + 1] : 0.f;
             a = warp_sum(a); c = warp_sum(c);
             if (lane == 0) {
                 const float sw = (float)(((double)w_s[t - 1] + (double)(a / c)) * isl_d);
-                p.soft[blk * n + t - 1] = sw;
-                if (p.soft_copy) p.soft_copy[blk * n + t - 1] = sw;
+                v_s[t - 1] = sw;                                     // (step t is done with its entry)
                 den1 = c;
                 bdef = fmaxf(bdef, fabsf(c - 1.f));
                 bad |= !(fabsf(c - 1.f) <= LIN_DEFECT);
@@ -411,6 +410,7 @@ __global__ void __launch_bounds__(SoloCfg<KB>::THREADS, 1) fwd_lin_kernel(FwdPar
         if (warp == 0) finish_step(1, n & 1);
         if (tid == 0) {
             p.lin_flag[blk] = bad ? 1 : 0;
+            lz[0] = bad ? 1.f : 0.f;
             if (!bad) {
                 const int ez = exp2i(Zs);
                 const float l2z = lg2f(Zs * pow2i(-ez));
@@ -429,6 +429,12 @@ __global__ void __launch_bounds__(SoloCfg<KB>::THREADS, 1) fwd_lin_kernel(FwdPar
             }
         }
         compute_barrier(CT);                                      // part and the messages are free for the next block
+        // soft may be W: written where it stands only, and after everything that reads W
+        if (lz[0] == 0.f)
+            for (int t = tid; t < n; t += CT) {
+                p.soft[blk * n + t] = v_s[t];
+                if (p.soft_copy) p.soft_copy[blk * n + t] = v_s[t];
+            }
     }
     if (tid == 0) {
         diag_max(&p.diag->max_defect, defect);

@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
     const int xl = active ? tid : 0, x = (int)rb.rank * NBC + xl;
     const float sl = sqrtf(p.lam2), NONE = __int_as_float(0xff800000);
     const double isl_d = 1.0 / (double)sl;
-    float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);          // entry t - 1: scaled clamped weight, the same + 2 delta
+    float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);          // entry t - 1: scaled clamped weight, the same + 2 delta, delta, soft
     float4 *sums = step + n + 1;                                           // entry t - 1: numerator, denominator (of this CTA)
     int *O_s = reinterpret_cast<int *>(sums + n);                          // entry t - 1: O_t, t = 1 .. n + 1
     float *part = smem + C::OFF_PART;
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
         int outside = 0;
         for (int t = tid; t < n; t += NT) {
             const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
-            step[t] = make_float4(se.wc * sl, (se.wc + 2.f * se.delta) * sl, 0.f, 0.f);
+            step[t] = make_float4(se.wc * sl, (se.wc + 2.f * se.delta) * sl, se.delta, 0.f);
             outside |= se.delta != 0.f;
         }
         const bool recentre = rb.cta_or(outside) != 0;           // (every CTA of a cluster decides alike)
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
             asm volatile("cp.async.wait_all;" ::: "memory");
             if (C::NWARP > 1 && warp == 0) finish_step(1, n & 1);
             rb.block_sync();
-            // soft codeword, one thread per step
+            // soft codeword, one thread per step (it may overwrite W: written when it stands, after everything that reads W)
             float bdef = 0.f, gap = 0.f;
             for (int t = (int)rb.rank * NT + tid; t < n; t += CL * NT) {
                 float a, c;
@@ -506,15 +506,18 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
                 } else {
                     a = sums[t].x; c = sums[t].y;
                 }
-                const float sw = (float)(((double)step[t].x + (double)(a / c)) * isl_d);
-                p.soft[blk * n + t] = sw;
-                if (p.soft_copy) p.soft_copy[blk * n + t] = sw;
+                step[t].w = (float)(((double)step[t].x + (double)(a / c)) * isl_d);
                 const float df = fabsf(c - 1.f);
                 bad |= LIN && !(df <= LIN_DEFECT);
                 bdef = fmaxf(bdef, df);
                 if (t == 0) gap = fabsf(lg2f(c));                // A_1 is constant: the sums of step 1 are the beta side's Z
             }
             if (LIN && rb.block_or(bad, 16)) return false;
+            for (int t = (int)rb.rank * NT + tid; t < n; t += CL * NT) {
+                const float sw = step[t].w;
+                p.soft[blk * n + t] = sw;
+                if (p.soft_copy) p.soft_copy[blk * n + t] = sw;
+            }
             bdef = rb.block_max(bdef, 24);
             defect = fmaxf(defect, bdef);
             zgap = fmaxf(zgap, gap);
@@ -525,7 +528,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
                     double zshift = 0.0;                         // sum_t lam2 delta_t^2: left out by step_energy
                     if (recentre)
                         for (int t = 0; t < n; ++t) {
-                            const double dl = (double)step_energy(__ldg(w + t), c_lo, c_hi, p.lam2).delta;
+                            const double dl = (double)step[t].z;
                             zshift += (double)p.lam2 * dl * dl;
                         }
                     p.logZ[blk] = (float)(((double)O + (double)l2z - zshift) * 0.6931471805599453);

@@ -231,16 +231,16 @@ __global__ void __launch_bounds__(Vec2Cfg<NBLK_>::THREADS, 1) fwd_vec_lin_kernel
         load_history(nt, 0, Ls);
         float bdef = 0.f, den1 = 1.f;
         cluster_sync();
-        // rank 0, warp k: turn the sums of step t of block k (slots of buffer b) into soft[t]
+        // rank 0, warp k: turn the sums of step t of block k (slots of buffer b) into soft[t], which takes the place of the step's weights
+        // (every warp has read those) until the block has its certificate
         auto finish_step = [&](int t, int b, int k) {
             if (rank == 0 && warp == k) {
                 const float4 s4 = *reinterpret_cast<const float4 *>(part + (size_t)((b * NBLK + k) * SLOTS + lane) * 4);
                 const float den = warp_sum(s4.x), n0 = warp_sum(s4.y), n1 = warp_sum(s4.z);
                 if (lane == 0) {
-                    const float *wk = w_s + k * C::MAX_N + 2 * (t - 1);
+                    float *wk = w_s + k * C::MAX_N + 2 * (t - 1);
                     const float s0 = (float)(((double)wk[0] + (double)(n0 / den)) * isl_d), s1 = (float)(((double)wk[1] + (double)(n1 / den)) * isl_d);
-                    *reinterpret_cast<float2 *>(p.soft + (base + k) * n + 2 * (t - 1)) = make_float2(s0, s1);
-                    if (p.soft_copy) *reinterpret_cast<float2 *>(p.soft_copy + (base + k) * n + 2 * (t - 1)) = make_float2(s0, s1);
+                    *reinterpret_cast<float2 *>(wk) = make_float2(s0, s1);
                     bdef = fmaxf(bdef, fabsf(den - 1.f));
                     bad |= !(fabsf(den - 1.f) <= LIN_DEFECT);
                     den1 = den;
@@ -308,11 +308,20 @@ __global__ void __launch_bounds__(Vec2Cfg<NBLK_>::THREADS, 1) fwd_vec_lin_kernel
                 finish_step(1, ib, k);
             }
         }
-        if (rank == 0 && warp < nact && lane == 0) {
-            p.lin_flag[base + warp] = bad ? 1 : 0;
+        if (rank == 0 && warp < nact) {
+            bad = __shfl_sync(0xffffffffu, (int)bad, 0) != 0;
+            __syncwarp();
+            if (lane == 0) p.lin_flag[base + warp] = bad ? 1 : 0;
             if (!bad) {
-                defect = fmaxf(defect, bdef);
-                zgap = fmaxf(zgap, fabsf(lg2f(den1)));
+                if (lane == 0) {
+                    defect = fmaxf(defect, bdef);
+                    zgap = fmaxf(zgap, fabsf(lg2f(den1)));
+                }
+                const float2 *sw = reinterpret_cast<const float2 *>(w_s + warp * C::MAX_N);
+                for (int t = lane; t < nt; t += 32) {             // (soft may be W)
+                    reinterpret_cast<float2 *>(p.soft + (base + warp) * n)[t] = sw[t];
+                    if (p.soft_copy) reinterpret_cast<float2 *>(p.soft_copy + (base + warp) * n)[t] = sw[t];
+                }
             }
         }
         cluster_sync();         // nobody still reads this batch's buffers when the next batch starts

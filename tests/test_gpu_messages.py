@@ -109,3 +109,25 @@ def test_gradients_of_blocks_at_different_scales(ctx, Lb, V, n, B, T):
     # what the smaller blocks add is below 2^-27 of the largest; the sums are taken in another order, over up to a few hundred thousand
     # terms of either sign: a few hundred half-ulps of the largest partial sum
     assert np.abs(sc - bc).max() <= 2e-5 * np.abs(bc).max()
+
+
+@pytest.mark.parametrize("Lb,k,V,n,B,T", [(16, 2, 1, 12, 1184, 0.009), (16, 3, 1, 10, 1184, 0.009), (16, 2, 2, 12, 300, 0.012), (16, 2, 1, 24, 4, 0.03),
+                                          (14, 2, 1, 24, 9, 0.03), (12, 2, 1, 24, 900, 0.02), (8, 2, 1, 24, 40, 0.05)])
+def test_soft_codeword_may_overwrite_the_weights(ctx, Lb, k, V, n, B, T):
+    # A forward call whose output is its input (nothing is differentiated afterwards): blocks without a certificate are run again, and a
+    # block with weights outside the table adds its share to log Z, both from the weights as they were.
+    import torch
+    W, c, _ = _rand(n, Lb, B, seed=70 + Lb + n)
+    if V == 2:
+        c = np.random.default_rng(71).standard_normal((1 << Lb, 2)).astype(np.float32)
+    W[1] = np.where(np.arange(n) % 2 == 0, 5.0, -5.0)
+    W[B - 1, n // 2] = 9.0
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd = torch.from_numpy(W).to(dev), torch.from_numpy(c).to(dev)
+    run = (lambda w, out: ctx.bcjr_soft_quantize_vec(w, cd, Lb, k, V, n, T, soft=out)) if V == 2 else \
+        (lambda w, out: ctx.bcjr_soft_quantize(w, cd, Lb, k, n, T, soft=out))
+    soft, logZ = run(Wd, None)
+    inplace = Wd.clone()
+    _, logZ2 = run(inplace, inplace)
+    assert ctx.sync_status().device_status == 0
+    assert torch.equal(inplace, soft) and torch.equal(logZ2, logZ)
