@@ -1014,7 +1014,8 @@ bcjr_status launch_bwd_warp2(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
 
 // One butterfly per thread (bcjr_reg.cuh), k = 2 and n <= 1024: calls at Lb = 8 .. 15, and calls of few blocks at
 // Lb = 16 -- forward as many as are resident (0.46 ms for 8 blocks, 0.66 for 16, 0.73 for 32; fwd_lin_kernel takes 1.40 for up
-// to 148), backward two waves of them (0.59 ms for 8, 1.17 for 16; 1.6 ms for up to 148).
+// to 148), and their backward calls (0.59 ms for 8, 1.17 for 16; 1.6 ms for up to 148): the register kernels take their offsets from
+// the step before, the chunked ones from the step itself, and a certificate holds for the gauge it was made in.
 // With log messages (a cold call) the warp-per-block kernels hold more blocks at Lb = 11 .. 13 and win from three quarters of
 // their residency on: 2^12 states, forward 4.23 against 3.68 ms for 4096 blocks, 1.24 against 1.85 for 1000; backward 6.28
 // against 5.80 for 4096.
@@ -1027,7 +1028,7 @@ bool reg_wanted(bcjr_ctx *ctx, int Lb, int k, int n, int64_t B, float lam2, bool
         if (4 * B > 3 * warps * ctx->num_sms) return false;
     }
     const int res = reg_resident_cached(ctx, Lb, n, bwd);
-    return res > 0 && (Lb < 16 || B <= (bwd ? 2 : 1) * (int64_t)res);
+    return res > 0 && (Lb < 16 || bwd || B <= res);             // (bwd: after a forward call of these kernels)
 }
 bcjr_status launch_fwd_reg(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
 {
@@ -1042,10 +1043,6 @@ bcjr_status launch_fwd_reg(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     CU(reg_forward(p, plan, st));
     ctx->launches += 1;
     ctx->fwd_reg = true;
-    if (p.Lb == 16 && lin && !reg_wanted(ctx, 16, 2, p.n, p.B, p.lam2, true)) {   // the backward call will run the chunked kernels
-        if ((rc = lin_make_list(ctx, p.B, st, &p.list))) return rc;
-        ctx->fwd_lin = true;
-    }
     return BCJR_OK;
 }
 bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cudaStream_t st)

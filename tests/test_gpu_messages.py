@@ -131,3 +131,29 @@ def test_soft_codeword_may_overwrite_the_weights(ctx, Lb, k, V, n, B, T):
     _, logZ2 = run(inplace, inplace)
     assert ctx.sync_status().device_status == 0
     assert torch.equal(inplace, soft) and torch.equal(logZ2, logZ)
+
+
+def test_register_forward_calls_are_followed_by_register_backward_calls(ctx):
+    # Few blocks of 2^16 states: the register kernels' gauge lags the chunked kernels' by a step, so that a certificate of the one family says
+    # nothing about the other.  Whatever the number of blocks, a forward call of one or two kernels (the register form: no table range, no
+    # second kernel behind a list) is followed by one kernel and the reduction of grad_codebook, and its gradients are right at the coldest temperature it is used for.
+    import torch
+    n, T = 40, 0.03
+    W, c, g = _rand(n, 16, 40, seed=90)
+    W[::3] *= 1.5
+    dev = torch.device("cuda", ctx.device)
+    cd = torch.from_numpy(c).to(dev)
+    ref = oracle.backward(W, c, g, 16, 2, T)
+    register = 0
+    for B in range(1, 41, 3):
+        Wd, gd = torch.from_numpy(W[:B]).to(dev), torch.from_numpy(g[:B]).to(dev)
+        start = ctx.sync_status().kernel_launches
+        ctx.bcjr_soft_quantize(Wd, cd, 16, 2, n, T)
+        mid = ctx.sync_status().kernel_launches
+        gW, _ = ctx.bcjr_backward(gd)
+        end = ctx.sync_status().kernel_launches
+        if mid - start <= 2:
+            register += 1
+            assert end - mid == 2, f"B={B}"
+        assert parity.rel_inf(gW.cpu().numpy(), ref["grad_W"][:B]) <= parity.GRAD_TOL, f"B={B}"
+    assert 3 <= register < 14                            # both sides of the rule were seen
