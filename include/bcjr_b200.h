@@ -47,7 +47,8 @@ typedef struct {
     float max_posterior_defect;   /* max over blocks and steps of |sum_s gamma_t(s) - 1| (Eq. 6) */
     float max_logz_mismatch;      /* max |log Z (alpha side) - log Z (beta side)|, natural log */
     int32_t kernel_launches;      /* kernels launched by this context since creation */
-    int32_t last_path;            /* kernels used by the last call: 0 = generic, 1 = large-trellis (Lb = 16), 2 = mid-size (Lb = 11..13, k = 2) */
+    int32_t last_path;            /* family of the last call's shape: 1 = large-trellis (Lb = 16), 2 = mid-size (Lb = 11..13, k = 2), 0 = all others
+                                     and the generic kernels; bcjr_last_kernels names the kernels themselves */
 } bcjr_diag;
 
 /* Limits: 1 <= k <= 4, k <= Lb <= 16, Lb - k <= 14, n >= 1, T > 0 and finite.
@@ -96,12 +97,14 @@ bcjr_status bcjr_destroy(bcjr_ctx *ctx);
  *                 m - 1 steps in between inside the beta sweep (1/m of the history traffic to HBM for
  *                 (m-1)/m of an alpha sweep more arithmetic; same results within float32 rounding; Lb = 16, k = 2,
  *                 n <= 512, otherwise the option has no effect)
- *   "messages"    2^16-state kernels: 0 (default) = the messages are carried in float32 themselves where the temperature
- *                 lets them be expected to fit, each block's result is certified on the device, and a block
- *                 without a certificate is run again with log-domain messages; 1 = log-domain messages always.  The same
- *                 holds for viterbi_hard at 2^16 states: 0 = a float32 sweep whose path is proved to be the one of the
- *                 double arithmetic, block by block, and the double kernel for the others; 1 = the double kernel always.
- *                 Same results within float32 rounding.
+ *   "messages"    what the sweeps carry.  0 (default): at Lb = 8..16 with k = 2, Lb = 16 with k = 3 (forward call) and Lb = 16, k = V = 2,
+ *                 the messages themselves in float32 where temperature and weights let them be expected to fit; each block's
+ *                 result is certified on the device -- sum over the states of |error of the posterior| <= 6e-5 at every step,
+ *                 on top of float32 rounding -- and a block without a certificate is run again with log-domain
+ *                 messages.  viterbi_hard at Lb = 10..13 and 16 with k = 2 and Lb = 16 with k = 3: a float32 sweep whose path is
+ *                 proved to be the one of the double arithmetic, block by block, and the double kernel for the others.
+ *                 1: log-domain messages and double metrics always.  2 (test hook): linear messages tried on every block of a
+ *                 shape that has them, whatever the temperature.
  *   "max_ctas"    cap on resident thread blocks (0 = fill the GPU)
  *   "record_block_defect"  1: every scalar forward call also records, per block, max over steps of
  *                 |sum_s gamma_t(s) - 1| (read back with bcjr_block_defects); 0 (default): only the
@@ -276,6 +279,15 @@ bcjr_status bcjr_sync_status(bcjr_ctx *ctx, void *cuda_stream, bcjr_diag *out);
  * (count <= that call's num_blocks, else BCJR_ESTATE) to host_out (host, float32).  A block the
  * kernel in use does not instrument reads NaN (the register-table cluster variant, vector emissions). */
 bcjr_status bcjr_block_defects(bcjr_ctx *ctx, float *host_out, int64_t count, void *cuda_stream);
+
+/* Kernels of the last forward, backward or Viterbi call, in launch order and separated by blanks, auxiliary ones (table
+ * range, lists, reductions) left out: e.g. "fwd_lin fwd_reg fwd_solo".  A kernel that stands behind a list of blocks is named
+ * whether or not the list was empty.  Owned by the context; valid until the next call. */
+const char *bcjr_last_kernels(bcjr_ctx *ctx);
+
+/* Blocks of the saved forward call that were carried with linear messages (option "messages"): 0 where the call ran log-domain kernels
+ * alone.  Synchronises cuda_stream.  BCJR_ESTATE without a saved forward call. */
+bcjr_status bcjr_linear_blocks(bcjr_ctx *ctx, int64_t *count, void *cuda_stream);
 
 /* Scratch bytes currently held by the context. */
 int64_t bcjr_workspace_bytes(const bcjr_ctx *ctx);

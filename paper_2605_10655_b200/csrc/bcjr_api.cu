@@ -71,11 +71,14 @@ struct bcjr_ctx {
                                // cluster kernel, 2 = fused two-CTA TMEM kernel, 3 = fused with skewed slot order, 4 = two-kernel call always
     int opt_fwd_variant = 0;   // 0 = TMEM single-CTA forward kernel where it applies, 1 = cluster forward kernel
     int opt_record_defect = 0; // forward calls record the posterior defect of every block
-    int opt_messages = 0;      // 0 = linear messages where they can be expected to fit float32's range, 1 = log messages always
+    int opt_messages = 0;      // 0 = linear messages where they can be expected to fit float32's range, 1 = log messages always, 2 = linear tried on every block
     int opt_hist_every = 1;    // large-trellis forward call: keep L_t of every m-th step, recompute the others in the beta sweep
     int64_t defect_blocks = 0; // blocks covered by the last recording
     int launches = 0;
     int last_path = 0;
+    const char *ran[12] = {};  // kernels of the last call, in launch order, without the auxiliary ones
+    int num_ran = 0;
+    char ran_text[256] = {};
     std::string cuda_error;
 };
 
@@ -86,6 +89,12 @@ bcjr_status cuda_fail(bcjr_ctx *ctx, cudaError_t e, const char *what)
     ctx->cuda_error = std::string(what) + ": " + cudaGetErrorString(e);
     cudaGetLastError();
     return e == cudaErrorMemoryAllocation ? BCJR_ENOMEM : BCJR_ECUDA;
+}
+
+void note(bcjr_ctx *ctx, const char *kernel)
+{
+    if (ctx->num_ran > 0 && !strcmp(ctx->ran[ctx->num_ran - 1], kernel)) return;     // (chunks repeat)
+    if (ctx->num_ran < (int)(sizeof(ctx->ran) / sizeof(ctx->ran[0]))) ctx->ran[ctx->num_ran++] = kernel;
 }
 
 #define CU(call)                                                        \
@@ -174,6 +183,7 @@ bcjr_status launch_fwd_generic(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     p.stepO = (int *)ctx->stepO.ptr;
     p.msg = gl.msg_global ? (float *)ctx->msg.ptr : nullptr;
     fwd_generic_kernel<KB><<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "fwd_generic");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -195,6 +205,7 @@ bcjr_status launch_bwd_generic(bcjr_ctx *ctx, BwdParams p, float *grad_codebook,
     p.gc_part = (float *)ctx->gc_part.ptr;
     p.msg = gl.msg_global ? (float *)ctx->msg.ptr : nullptr;
     bwd_generic_kernel<KB><<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "bwd_generic");
     ctx->launches += 1;
     CU(cudaGetLastError());
     if (grad_codebook) {
@@ -221,6 +232,7 @@ bcjr_status launch_vit_generic(bcjr_ctx *ctx, VitParams p, cudaStream_t st)
     p.path_ws = (int *)ctx->path_ws.ptr;
     p.msg = gl.msg_global ? (double *)ctx->msg.ptr : nullptr;
     kern<<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "viterbi_generic");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -245,6 +257,7 @@ bcjr_status launch_fwd_vec(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     regroup_table_kernel<<<(SV + 255) / 256, 256, 0, st>>>(p.cb, (float *)ctx->cb_beta.ptr, 1 << p.Lb, KB, V);
     p.cb_beta = (const float *)ctx->cb_beta.ptr;
     fwd_vec_kernel<KB, V><<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "fwd_vec");
     ctx->launches += 2;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -270,6 +283,7 @@ bcjr_status launch_bwd_vec(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     regroup_table_kernel<<<(S * V + 255) / 256, 256, 0, st>>>(p.cb, (float *)ctx->cb_beta.ptr, S, KB, V);
     p.cb_beta = (const float *)ctx->cb_beta.ptr;
     bwd_vec_kernel<KB, V><<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "bwd_vec");
     ctx->launches += 2;
     CU(cudaGetLastError());
     if (grad_codebook) {
@@ -294,6 +308,7 @@ bcjr_status launch_vit_vec(bcjr_ctx *ctx, VitParams p, cudaStream_t st)
     p.path_ws = (int *)ctx->path_ws.ptr;
     p.msg = gl.msg_global ? (double *)ctx->msg.ptr : nullptr;
     viterbi_vec_kernel<KB, V><<<gl.grid, gl.threads, gl.smem, st>>>(p);
+    note(ctx, "viterbi_vec");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -368,6 +383,7 @@ bcjr_status launch_fwd_vec4(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     regroup_table_kernel<<<(C::S * C::V + 255) / 256, 256, 0, st>>>(p.cb, (float *)ctx->cb_beta.ptr, C::S, C::KB, C::V);
     p.hist = (float *)ctx->hist.ptr;
     p.cb_beta = (const float *)ctx->cb_beta.ptr;
+    note(ctx, "fwd_vec4");
     CU(cudaLaunchKernelEx(&cfg, kern, p));
     ctx->launches += 2;
     return BCJR_OK;
@@ -386,6 +402,7 @@ bcjr_status launch_fwd_cluster_t(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     const int ncl = cfg.gridDim.x / CL;
     if ((rc = ensure(ctx, ctx->hist, (size_t)ncl * p.n * C::Q * 4))) return rc;
     p.hist = (float *)ctx->hist.ptr;
+    note(ctx, "fwd_cluster");
     CU(cudaLaunchKernelEx(&cfg, kern, p));
     ctx->launches += 1;
     return BCJR_OK;
@@ -407,6 +424,7 @@ bcjr_status launch_bwd_cluster_t(bcjr_ctx *ctx, BwdParams p, float *grad_codeboo
     if ((rc = ensure(ctx, ctx->gc_part, (size_t)ncl * C::S * 4))) return rc;
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = (float *)ctx->gc_part.ptr;
+    note(ctx, "bwd_cluster");
     CU(cudaLaunchKernelEx(&cfg, kern, p));
     ctx->launches += 1;
     if (grad_codebook) {
@@ -432,6 +450,7 @@ bcjr_status launch_bwd_duo(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = (float *)ctx->gc_part.ptr;
     CU(cudaLaunchKernelEx(&cfg, bwd_duo_kernel<KB>, p));
+    note(ctx, "bwd_duo");
     ctx->launches += 1;
     if (grad_codebook) {
         reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
@@ -457,6 +476,7 @@ bcjr_status launch_bwd_skew(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = ACC ? (float *)ctx->gc_part.ptr : nullptr;
     CU(cudaLaunchKernelEx(&cfg, bwd_skew_kernel<ACC, false>, p));
+    note(ctx, "bwd_skew");
     ctx->launches += 1;
     if (ACC) {
         reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
@@ -491,7 +511,7 @@ int reg_resident_cached(bcjr_ctx *ctx, int Lb, int n, bool bwd)
 //   * The vector trellis: both calls at T = 0.012, 300 blocks 8.08 -> 7.52 ms, 592 14.0 -> 11.7; T = 0.01, 300 blocks 8.05 -> 7.73.
 bool lin_wanted(const bcjr_ctx *ctx, int Lb, float lam2, int64_t B, int V = 1, int k = 2)
 {
-    if (ctx->opt_messages == 1) return false;
+    if (ctx->opt_messages != 0) return ctx->opt_messages == 2;
     const bool many = B >= (Lb == 16 ? 2 : 6) * (int64_t)ctx->num_sms, lots = B >= 8 * (int64_t)ctx->num_sms;
     if (k == 3) return lam2 <= (lots ? 80.2f : 10.f);
     if (ctx->cb_computed && V == 1) return lam2 <= (many ? 15.f : 10.f);
@@ -499,7 +519,7 @@ bool lin_wanted(const bcjr_ctx *ctx, int Lb, float lam2, int64_t B, int V = 1, i
     if (V == 2) return lam2 <= 80.2f;
     return lam2 <= (Lb < 16 ? 36.5f : lots ? 80.2f : 62.2f);
 }
-int lin_exponent(float lam2) { const int x = (int)(1.33f * lam2); return x < LIN_X_MAX ? x : LIN_X_MAX; }
+int lin_exponent(float lam2) { return 1.33f * lam2 < (float)LIN_X_MAX ? (int)(1.33f * lam2) : LIN_X_MAX; }
 bcjr_status lin_buffers(bcjr_ctx *ctx, int64_t B)
 {
     bcjr_status rc = ensure(ctx, ctx->lin_flag, ((size_t)B + 15) / 16 * 16);
@@ -558,11 +578,13 @@ bcjr_status launch_fwd_vec2(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
         p.lin_x = lin_exponent(p.lam2);
         p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
         CU(cudaLaunchKernelEx(&lcfg, fwd_vec_lin_kernel<NBLK>, p));
+        note(ctx, "fwd_vec_lin");
         ctx->launches += 1;
         if ((rc = lin_make_list(ctx, p.B, st, &p.list))) return rc;
         ctx->fwd_lin = true;
     }
     CU(cudaLaunchKernelEx(&cfg, fwd_vec2_kernel<NBLK>, p));
+    note(ctx, "fwd_vec2");
     ctx->launches += 2;
     return BCJR_OK;
 }
@@ -627,12 +649,14 @@ bcjr_status launch_bwd_vec4(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
             acfg.gridDim = dim3((unsigned)(2 * (nb < acl ? nb : acl)), 1, 1);
             bcfg.gridDim = dim3((unsigned)(Bt::CL * (nb < bcl ? nb : bcl)), 1, 1);
             CU(cudaLaunchKernelEx(&acfg, bwd_vec_alpha_lin_kernel<VEC_ALPHA_NBLK>, q));
+            note(ctx, "bwd_vec_lin");
             CU(cudaLaunchKernelEx(&bcfg, bwd_vec_beta_lin_kernel<VEC_BETA_NBLK>, q));
             ctx->launches += 2;
         }
         p.list = (const int *)ctx->lin_list.ptr;
     }
     CU(cudaLaunchKernelEx(&cfg, bwd_vec4_kernel<VEC4_BWD_NBLK>, p));
+    note(ctx, "bwd_vec4");
     ctx->launches += 2;
     if (grad_codebook) {
         reduce_gc_vec_kernel<<<(S * V + 255) / 256, 256, 0, st>>>(p.gc_part, parts, S, KB, V, grad_codebook);
@@ -676,6 +700,7 @@ bcjr_status launch_bwd_split(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
         p.B = nb;
         p.W = W + b0 * p.n; p.g = g + b0 * p.n; p.soft = soft + b0 * p.n; p.gW = gW + b0 * p.n;
         bwd_alpha_kernel<KB><<<(int)nb, A::THREADS, A::SMEM_BYTES, st>>>(p);
+        note(ctx, "bwd_split");
         CU(cudaGetLastError());
         cfg.gridDim = dim3((unsigned)(CL * (nb < ncl ? nb : ncl)), 1, 1);
         CU(cudaLaunchKernelEx(&cfg, beta, p));
@@ -735,6 +760,7 @@ bcjr_status launch_bwd_lin(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
         q.lin_flag = (const uint8_t *)ctx->lin_flag.ptr + b0;
         q.g_bits = p.g_bits + b0;
         bwd_alpha_lin_kernel<2><<<(int)nb, A::THREADS, AlphaLinCfg<2>::SMEM_BYTES, st>>>(q);
+        note(ctx, "bwd_lin");
         CU(cudaGetLastError());
         cfg.gridDim = dim3((unsigned)(C::CL * (nb < ncl ? nb : ncl)), 1, 1);
         CU(cudaLaunchKernelEx(&cfg, bwd_beta_lin_kernel<ACC>, q));
@@ -746,6 +772,7 @@ bcjr_status launch_bwd_lin(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
         q = p;
         q.lin_x = -1;
         CU(reg_backward(q, plan, ACC, st));
+        note(ctx, "bwd_reg");
         ctx->launches += 1;
     }
     q = p;
@@ -753,6 +780,7 @@ bcjr_status launch_bwd_lin(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     for (int64_t b0 = 0; b0 < p.B && (b0 > 0 || p.B > p.list_max); b0 += chunk) {
         q.list_base = (int)b0;
         bwd_alpha_kernel<2><<<(int)chunk, A::THREADS, A::SMEM_BYTES, st>>>(q);
+        note(ctx, "bwd_split");
         CU(cudaGetLastError());
         CU(cudaLaunchKernelEx(&lcfg, bwd_skew_kernel<ACC, true>, q));
         ctx->launches += 2;
@@ -778,6 +806,7 @@ bcjr_status launch_bwd_solo(bcjr_ctx *ctx, BwdParams p, cudaStream_t st)
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = nullptr;
     bwd_solo_kernel<<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "bwd_solo");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -828,6 +857,7 @@ bcjr_status launch_vit_solo(bcjr_ctx *ctx, VitParams p, cudaStream_t st)
         p.hist = (float *)ctx->hist.ptr;
         p.flag = (uint8_t *)ctx->vit_flag.ptr;
         viterbi_fast_kernel<KB><<<(int)grid, F::THREADS, F::SMEM_BYTES, st>>>(p);
+        note(ctx, "viterbi_fast");
         CU(cudaGetLastError());
         lin_list_kernel<<<1, 1024, 0, st>>>(p.flag, p.B, (int *)ctx->vit_list.ptr);
         CU(cudaGetLastError());
@@ -835,6 +865,7 @@ bcjr_status launch_vit_solo(bcjr_ctx *ctx, VitParams p, cudaStream_t st)
         p.list = (const int *)ctx->vit_list.ptr;
     }
     viterbi_solo_kernel<KB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "viterbi_solo");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -853,6 +884,7 @@ bcjr_status launch_fwd_listed(bcjr_ctx *ctx, FwdParams &p, int k, cudaStream_t s
     FwdParams q = p;
     q.lin_x = -1;
     CU(reg_forward(q, plan, st));
+    note(ctx, "fwd_reg");
     ctx->launches += 1;
     return BCJR_OK;
 }
@@ -877,6 +909,7 @@ bcjr_status launch_vit_reg(bcjr_ctx *ctx, VitParams &p, cudaStream_t st)
     p.flag = (uint8_t *)ctx->vit_flag.ptr;
     p.diag = ctx->diag;
     CU(reg_viterbi(p, (int)grid, st));
+    note(ctx, "viterbi_reg");
     lin_list_kernel<<<1, 1024, 0, st>>>(p.flag, p.B, (int *)ctx->vit_list.ptr);
     CU(cudaGetLastError());
     ctx->launches += 2;
@@ -903,6 +936,7 @@ bcjr_status launch_fwd_solo(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
         p.lin_x = lin_exponent(p.lam2);
         p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
         fwd_lin_kernel<KB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+        note(ctx, "fwd_lin");
         CU(cudaGetLastError());
         if ((rc = lin_make_list(ctx, p.B, st, &p.list))) return rc;
         ctx->launches += 1;
@@ -910,6 +944,7 @@ bcjr_status launch_fwd_solo(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
         if ((rc = launch_fwd_listed(ctx, p, KB, st))) return rc;
     }
     fwd_solo_kernel<KB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "fwd_solo");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -929,6 +964,7 @@ bcjr_status launch_fwd_ckpt(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     if (rc) return rc;
     p.hist = (float *)ctx->hist.ptr;
     fwd_ckpt_kernel<KB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "fwd_ckpt");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -953,6 +989,7 @@ bcjr_status launch_fwd_warp(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     p.hist = (float *)ctx->hist.ptr;
     p.stepO = (int *)ctx->stepO.ptr;
     fwd_warp_kernel<LB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "fwd_warp");
     ctx->launches += 1;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -976,6 +1013,7 @@ bcjr_status launch_bwd_warp(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     p.stepO = (int *)ctx->stepO.ptr;
     p.gc_part = ACC ? (float *)ctx->gc_part.ptr : nullptr;
     bwd_warp_kernel<LB, ACC><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "bwd_warp");
     ctx->launches += 1;
     CU(cudaGetLastError());
     if (ACC) {
@@ -1005,6 +1043,7 @@ bcjr_status launch_bwd_warp2(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
     p.stepO = (int *)ctx->stepO.ptr;
     p.gc_part = (float *)ctx->gc_part.ptr;
     bwd_warp2_kernel<LB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
+    note(ctx, "bwd_warp2");
     CU(cudaGetLastError());
     reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)pairs, C::S, grad_codebook);
     ctx->launches += 2;
@@ -1041,6 +1080,7 @@ bcjr_status launch_fwd_reg(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
     p.lin_x = lin ? lin_exponent(p.lam2) : -1;
     CU(reg_forward(p, plan, st));
+    note(ctx, "fwd_reg");
     ctx->launches += 1;
     ctx->fwd_reg = true;
     return BCJR_OK;
@@ -1057,6 +1097,7 @@ bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     p.lin_flag = (const uint8_t *)ctx->lin_flag.ptr;
     p.lin_x = lin_wanted(ctx, p.Lb, p.lam2, p.B) ? lin_exponent(p.lam2) : -1;
     CU(reg_backward(p, plan, grad_codebook != nullptr, st));
+    note(ctx, "bwd_reg");
     ctx->launches += 1;
     if (grad_codebook) {
         reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, plan.parts, S, grad_codebook);
@@ -1092,6 +1133,7 @@ bcjr_status launch_fwd_small(bcjr_ctx *ctx, FwdParams p, int k, cudaStream_t st)
     if (rc) return rc;
     p.hist = (float *)ctx->hist.ptr;
     CU(small_forward(p, k, plan, grid, st));
+    note(ctx, "fwd_small");
     ctx->launches += 1;
     return BCJR_OK;
 }
@@ -1106,6 +1148,7 @@ bcjr_status launch_bwd_small(bcjr_ctx *ctx, BwdParams p, int k, float *grad_code
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = grad_codebook ? (float *)ctx->gc_part.ptr : nullptr;
     CU(small_backward(p, k, plan, grid, st));
+    note(ctx, "bwd_small");
     ctx->launches += 1;
     if (grad_codebook) {
         reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, grid, S, grad_codebook);
@@ -1287,7 +1330,7 @@ bcjr_status bcjr_set_option(bcjr_ctx *ctx, const char *name, int64_t value)
         return BCJR_OK;
     }
     if (!strcmp(name, "messages")) {
-        if (value < 0 || value > 1) return BCJR_EINVAL;
+        if (value < 0 || value > 2) return BCJR_EINVAL;
         ctx->opt_messages = (int)value;
         return BCJR_OK;
     }
@@ -1316,6 +1359,7 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = false;
+    ctx->num_ran = 0;
     ctx->cb_computed = codebook == nullptr;
     if (num_blocks == 0) {
         ctx->W = W; ctx->cb = codebook; ctx->Lb = Lb; ctx->k = k; ctx->n = n; ctx->B = 0; ctx->T = T;
@@ -1392,6 +1436,7 @@ bcjr_status bcjr_backward(bcjr_ctx *ctx, const float *grad_soft, float *grad_W, 
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int S = 1 << ctx->Lb;
+    ctx->num_ran = 0;
     if (ctx->B == 0) {
         if (grad_codebook) CU(cudaMemsetAsync(grad_codebook, 0, (size_t)S * ctx->V * 4, st));
         return BCJR_OK;
@@ -1478,6 +1523,7 @@ bcjr_status viterbi_hard(bcjr_ctx *ctx, const float *W, const float *codebook, i
         if (ctx->have_fwd && saved_computed && ctx->Lb != Lb) ctx->have_fwd = false;
         if ((rc = computed_table(ctx, Lb, st, &codebook))) return rc;
     }
+    ctx->num_ran = 0;
     VitParams p{};
     p.W = W; p.cb = codebook; p.path_bits = path_bits; p.path_stride = path_stride_bytes;
     p.states = states; p.hard = hard; p.B = num_blocks; p.Lb = Lb; p.n = n;
@@ -1522,6 +1568,7 @@ bcjr_status bcjr_soft_quantize_vec(bcjr_ctx *ctx, const float *W, const float *c
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = false;
+    ctx->num_ran = 0;
     if (num_blocks > 0) {
         if ((rc = ensure(ctx, ctx->soft_copy, (size_t)num_blocks * n * 4))) return rc;
         FwdParams p{};
@@ -1566,6 +1613,7 @@ bcjr_status viterbi_hard_vec(bcjr_ctx *ctx, const float *W, const float *codeboo
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
+    ctx->num_ran = 0;
     VitParams p{};
     p.W = W; p.cb = codebook; p.path_bits = path_bits; p.path_stride = path_stride_bytes;
     p.states = states; p.hard = hard; p.B = num_blocks; p.Lb = Lb; p.n = n;
@@ -1790,6 +1838,37 @@ bcjr_status bcjr_block_defects(bcjr_ctx *ctx, float *host_out, int64_t count, vo
     if (!guard.ok) return BCJR_ECUDA;
     CU(cudaStreamSynchronize((cudaStream_t)cuda_stream));
     CU(cudaMemcpy(host_out, ctx->blk_defect.ptr, (size_t)count * 4, cudaMemcpyDeviceToHost));
+    return BCJR_OK;
+}
+
+const char *bcjr_last_kernels(bcjr_ctx *ctx)
+{
+    if (!ctx) return "";
+    size_t at = 0;
+    ctx->ran_text[0] = 0;
+    for (int i = 0; i < ctx->num_ran; ++i) {
+        const int len = snprintf(ctx->ran_text + at, sizeof(ctx->ran_text) - at, "%s%s", i ? " " : "", ctx->ran[i]);
+        if (len < 0 || at + (size_t)len >= sizeof(ctx->ran_text)) break;
+        at += (size_t)len;
+    }
+    return ctx->ran_text;
+}
+
+bcjr_status bcjr_linear_blocks(bcjr_ctx *ctx, int64_t *count, void *cuda_stream)
+{
+    if (!ctx || !count) return BCJR_EINVAL;
+    if (!ctx->have_fwd) return BCJR_ESTATE;
+    *count = 0;
+    if (!(ctx->fwd_lin || ctx->fwd_reg) || ctx->B == 0) return BCJR_OK;
+    DeviceGuard guard(ctx->device);
+    if (!guard.ok) return BCJR_ECUDA;
+    CU(cudaStreamSynchronize((cudaStream_t)cuda_stream));
+    uint8_t part[4096];
+    for (int64_t b = 0; b < ctx->B; b += (int64_t)sizeof(part)) {
+        const int64_t m = ctx->B - b < (int64_t)sizeof(part) ? ctx->B - b : (int64_t)sizeof(part);
+        CU(cudaMemcpy(part, (const uint8_t *)ctx->lin_flag.ptr + b, (size_t)m, cudaMemcpyDeviceToHost));
+        for (int64_t i = 0; i < m; ++i) *count += part[i] == 0;
+    }
     return BCJR_OK;
 }
 

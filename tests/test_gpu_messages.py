@@ -157,3 +157,35 @@ def test_register_forward_calls_are_followed_by_register_backward_calls(ctx):
             assert end - mid == 2, f"B={B}"
         assert parity.rel_inf(gW.cpu().numpy(), ref["grad_W"][:B]) <= parity.GRAD_TOL, f"B={B}"
     assert 3 <= register < 14                            # both sides of the rule were seen
+
+
+@pytest.mark.parametrize("Lb,k,n,B,T,options,forward,backward,linear", [
+    (16, 2, 6, 4, 0.1, {}, ["fwd_reg"], ["bwd_reg"], 4),
+    (16, 2, 6, 70, 0.1, {}, ["fwd_lin", "fwd_reg", "fwd_solo"], ["bwd_lin", "bwd_reg", "bwd_split"], 70),
+    (16, 2, 6, 70, 0.01, {}, ["fwd_solo"], ["bwd_split"], 0),
+    (16, 2, 6, 70, 0.01, {"messages": 2}, ["fwd_lin", "fwd_reg", "fwd_solo"], ["bwd_lin", "bwd_reg", "bwd_split"], 70),
+    (16, 2, 6, 4, 0.1, {"messages": 1}, ["fwd_reg"], ["bwd_reg"], 0),
+    (16, 3, 6, 4, 0.3, {}, ["fwd_lin", "fwd_solo"], ["bwd_split"], 4),
+    (15, 2, 6, 4, 0.3, {}, ["fwd_reg"], ["bwd_reg"], 4),
+    (12, 2, 6, 4, 0.1, {"path": 1}, ["fwd_generic"], ["bwd_generic"], 0),
+    (12, 2, 1100, 2, 0.1, {}, ["fwd_warp"], ["bwd_warp2"], 0),
+    (9, 3, 6, 4, 0.3, {}, ["fwd_small"], ["bwd_small"], 0),
+    (13, 3, 6, 4, 0.3, {}, ["fwd_generic"], ["bwd_generic"], 0),
+])
+def test_a_call_reports_its_kernels_and_its_linear_blocks(ctx, Lb, k, n, B, T, options, forward, backward, linear):
+    import torch
+    W, c, g = _rand(n, Lb, B, seed=30)
+    W *= 0.3                                             # weights every state can follow: each block has its certificate
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(a).to(dev) for a in (W, c, g))
+    try:
+        for name, value in options.items():
+            ctx.set_option(name, value)
+        ctx.bcjr_soft_quantize(Wd, cd, Lb, k, n, T)
+        assert ctx.last_kernels() == forward and ctx.linear_blocks() == linear
+        ctx.bcjr_backward(gd)
+        assert ctx.last_kernels() == backward
+        assert ctx.sync_status().device_status == 0
+    finally:
+        for name in options:
+            ctx.set_option(name, 0)
