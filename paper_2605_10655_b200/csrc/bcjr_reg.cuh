@@ -52,7 +52,7 @@ struct RegCfg {
     static constexpr int OFF_PART = OFF_CMAX + 32;             // [2][16][4]
     static constexpr int OFF_RED = OFF_PART + 128;             // [64]: sums and flags between the sweeps
     static constexpr int OFF_MBAR = OFF_RED + 64;              // uint64 [4]
-    static constexpr int OFF_FLAG = OFF_MBAR + 8;              // abort flag of the waits
+    static constexpr int OFF_FLAG = OFF_MBAR + 8;              // abort flag of the waits, then two words of the backward kernel
     static constexpr int OFF_STEP = OFF_FLAG + 4;              // float4 [n + 1], then float4 [n] sums, then int [n + 2] offsets
     static size_t smem_bytes(int n) { return (size_t)(OFF_STEP + 4 * (n + 1) + 4 * n + n + 2 + 2) * 4; }
     static_assert(LB >= 8 && NBC <= 512, "sixteen butterflies at least, 512 threads at most");
@@ -595,11 +595,14 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
     constexpr uint32_t TX_MSG = (uint32_t)C::BUF * 4u, TX_MAX = CL * 4u;
     float defect = 0.f;
     const float2 ni2 = splat2(-p.invT * isl);
-    int e_acc = GRAD_NONE;                                      // scale of the accumulators (see bcjr_lin_bwd.cuh)
-    bool add = p.list != nullptr;                               // gc_part holds something already
+    // scale of the accumulators (see bcjr_lin_bwd.cuh), and whether gc_part holds something already: the sweeps have no registers for them
+    int *scale_s = reinterpret_cast<int *>(smem + C::OFF_FLAG + 1);
+    if (tid == 0) { scale_s[0] = GRAD_NONE; scale_s[1] = p.list != nullptr; }
+    rb.cta_sync();
     auto write_acc = [&]() {
         float *gc = p.gc_part + (size_t)cid * C::S;
-        const float up = grad_up(e_acc);
+        const float up = grad_up(scale_s[0]);
+        const bool add = scale_s[1] != 0;
 #pragma unroll
         for (int jp = 0; jp < 2; ++jp) {
             float4 *g0 = reinterpret_cast<float4 *>(gc + (2 * jp) * C::Q + x * 4), *g1 = reinterpret_cast<float4 *>(gc + (2 * jp + 1) * C::Q + x * 4);
@@ -619,26 +622,15 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
     for (int64_t it = cid; it < nblk; it += ncid) {
         const int64_t blk = p.list ? (int64_t)p.list[1 + it] : it;
         const float *w = p.W + blk * n, *g = p.g + blk * n, *sf = p.soft + blk * n;
-        int outside = 0;
-        uint32_t gmax = 0;
-        for (int t = tid; t < n; t += NT) {
-            const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
-            const float gv = __ldg(g + t), ws = se.wc * sl;
-            step[t] = make_float4(ws, (se.wc + 2.f * se.delta) * sl, gv, lin_gs(gv, ws, isl_d, __ldg(sf + t)));
-            outside |= se.delta != 0.f;
-            gmax = max(gmax, grad_bits(gv));
-        }
-        if (tid == 0) step[n] = make_float4(0.f, 0.f, 0.f, 0.f);
-        gmax = __reduce_max_sync(0xffffffffu, gmax);
-        if (C::NWARP > 1 && lane == 0) part[warp] = __uint_as_float(gmax);
-        const bool recentre = rb.cta_or(outside) != 0;
-        if (C::NWARP > 1) gmax = __reduce_max_sync(0xffffffffu, lane < C::NWARP ? __float_as_uint(part[lane]) : 0u);
-        const int e_g = grad_exponent(gmax);
+        uint32_t gmax = 0;                                         // (each warp looks at all of it)
+        for (int t = lane; t < n; t += 32) gmax = max(gmax, grad_bits(__ldg(g + t)));
+        const int e_g = grad_exponent(__reduce_max_sync(0xffffffffu, gmax));
         // the block runs at the accumulators' scale if its gradient is within GRAD_SPAN bits below it
+        int e_acc = ACC ? scale_s[0] : GRAD_NONE, first = 0;
         if (e_g != GRAD_NONE && (e_g > e_acc || e_g < e_acc - GRAD_SPAN)) {
             if (ACC && e_acc != GRAD_NONE) {
                 if (active) write_acc();
-                add = true;
+                first = 1;
 #pragma unroll
                 for (int jp = 0; jp < 2; ++jp)
 #pragma unroll
@@ -647,8 +639,16 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
             e_acc = e_g + GRAD_ROOM;
         }
         const float down = grad_down(e_acc);
-        for (int t = tid; t < n; t += NT) { step[t].z *= down; step[t].w *= down; }
-        rb.cta_sync();
+        int outside = 0;
+        for (int t = tid; t < n; t += NT) {
+            const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
+            const float gv = __ldg(g + t) * down, ws = se.wc * sl;
+            step[t] = make_float4(ws, (se.wc + 2.f * se.delta) * sl, gv, lin_gs(gv, ws, isl_d, __ldg(sf + t)));
+            outside |= se.delta != 0.f;
+        }
+        if (tid == 0) step[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool recentre = rb.cta_or(outside) != 0;
+        if (tid == 0) { scale_s[0] = e_acc; if (first) scale_s[1] = 1; }
         auto run = [&](auto lin_tag, auto rc_tag) {
             constexpr bool LIN = decltype(lin_tag)::value, RC = decltype(rc_tag)::value;
             // ================= alpha sweep
@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
                 } else {
                     a0 = sums[t].x; a2 = sums[t].y; az = sums[t].z;
                 }
-                const float i0 = grad_up(e_acc) / a0;
+                const float i0 = grad_up(scale_s[0]) / a0;
                 p.gW[blk * n + t] = (__ldg(g + t) - az * i0) + (a2 * i0) * (__ldg(w + t) - __ldg(sf + t)) * p.invT;
                 defect = fmaxf(defect, fabsf(a0 - 1.f));
             }
