@@ -55,6 +55,8 @@ struct bcjr_ctx {
     // saved by bcjr_soft_quantize for bcjr_backward
     bool have_fwd = false;
     bool fwd_reg = false;      // the saved forward call ran a one-butterfly-per-thread kernel (lin_flag belongs to it)
+    bool fwd_judged = false;   // ... or the warp-per-block kernel behind it: lin_list[0] against judged_max says which
+    int judged_max = 0;
     struct { int n = 0, count = 0; } vit_res[17];      // the same for viterbi_reg_kernel (CTAs)
     struct { int n = 0, count = 0; } reg_res[2][17];   // resident clusters of those kernels by call kind and Lb, for the n asked last
     bool fwd_lin = false;      // lin_flag and lin_list belong to the saved forward call
@@ -496,19 +498,24 @@ int reg_resident_cached(bcjr_ctx *ctx, int Lb, int n, bool bwd)
 }
 
 // Linear messages (bcjr_lin.cuh).  A block without a certificate runs twice: another 0.5 ms (forward) and 0.65 ms (backward) at
-// least with 2^16 states, a second pass in place with fewer.  Measured shares of N(0,1) blocks of 2^16 states without one: 0 at
-// T = 0.03, 0.3 % at 0.015, 1.6 % at 0.012, 5.5 % at 0.01; of heavy-tailed ones (four degrees of freedom) 15 % at 0.02.  lam2 = log2(e) / 2T.
+// least with 2^16 states, a second pass in place with fewer.  lin_wanted says where N(0,1) weights gain; the weights themselves are judged
+// on the device (lin_demand_limit, lin_failures_allowed), which leaves a call or a block to the log domain.  Measured shares of N(0,1) blocks
+// of 2^16 states without a certificate: 0 at T = 0.03, 0.3 % at 0.015, 1.6 % at 0.012, 5.5 % at 0.01.  lam2 = log2(e) / 2T.  Log -> linear:
 //   * Few blocks, less than two waves (six of the smaller trellises): one failure doubles the call, so only where there is hardly any.
 //     Forward, 300 blocks of 2^10 states, T = 0.05 0.28 -> 0.265 ms, T = 0.02 0.26 -> 0.42; 8 of 2^12 0.265 -> 0.244 at T = 0.02 but
-//     0.49 at 0.0145; 24 of 2^16 0.79 -> 0.70 at T = 0.02, heavy-tailed 1.45.
-//   * Many blocks: the share counts.  600 blocks of 2^16, T = 0.0145, both calls 22.6 -> 18.5 ms, heavy-tailed at T = 0.02 23.3 -> 23.1;
-//     3000 of 2^12 at T = 0.02 8.0 -> 6.2, heavy-tailed 8.0 -> 7.9; 4096 of 2^12 at T = 0.01 3.68 -> 4.61 (13 % fail); 1977 blocks of
-//     501 weights and 2^11 states at T = 0.0143 4.46 -> 4.94.
-//   * At k = 3 only fwd_solo_kernel can run them, 1.7 ms for the first: heavy tails have some from T = 0.05 down (482 blocks 6.69 ->
-//     7.37 ms; 2500 at T = 0.01 28.5 -> 26.9).
+//     0.49 at 0.0145; 24 of 2^16 0.79 -> 0.70 at T = 0.02.
+//   * Many blocks: the share counts.  600 blocks of 2^16, T = 0.0145, both calls 22.6 -> 18.5 ms; 3000 of 2^12 at T = 0.02 8.0 -> 6.2; 4096
+//     of 2^12 at T = 0.01 3.68 -> 4.61 (13 % fail); 1977 blocks of 501 weights and 2^11 states at T = 0.0143 4.46 -> 4.94.
+//   * At k = 3 only fwd_solo_kernel can run them again, 1.7 ms for the first (482 blocks, heavy tails, T = 0.05 6.69 -> 7.37 ms; 2500 at
+//     T = 0.01 28.5 -> 26.9).
 //   * The monotone table of the computed emission needs more range: both calls at T = 0.1 / 0.05 / 0.02, 300 blocks of 2^16 states 13.4 ->
 //     10.1 / 11.2 / 18.4 ms; 8 of 2^12 0.57 -> 0.49 / 0.50 / 0.79; 3000 of 2^12 7.7 -> 6.2 / 6.6 / 9.4.
 //   * The vector trellis: both calls at T = 0.012, 300 blocks 8.08 -> 7.52 ms, 592 14.0 -> 11.7; T = 0.01, 300 blocks 8.05 -> 7.73.
+// With the judging, over 24 .. 4096 blocks of 128 .. 512 weights, N(0,1) and heavy-tailed (four degrees of freedom), 2^8 .. 2^16 states, k = 2,
+// 3, V = 2, T = 0.1 .. 0.01, both calls: the worst is 2.4 % above messages = 1 (2000 heavy-tailed blocks of 512 weights and 2^12 states at T =
+// 0.05, 9.43 -> 9.66 ms), the next 1.7 % (300 vector blocks, T = 0.01, left to the log domain).  By temperature alone heavy tails lost
+// up to 45 %: 4096 blocks at T = 0.01 137 -> 191 ms (now 137), 600 of 512 weights at T = 0.0145 46.5 -> 65.1 (46.6), 300 of 2^10 states at T =
+// 0.05 0.535 -> 0.672 (0.512), 4096 of 2^12 with the computed emission at T = 0.05 9.07 -> 13.1 (9.09).
 bool lin_wanted(const bcjr_ctx *ctx, int Lb, float lam2, int64_t B, int V = 1, int k = 2)
 {
     if (ctx->opt_messages != 0) return ctx->opt_messages == 2;
@@ -518,6 +525,57 @@ bool lin_wanted(const bcjr_ctx *ctx, int Lb, float lam2, int64_t B, int V = 1, i
     if (!many) return lam2 <= (Lb <= 10 ? 15.f : 25.f);
     if (V == 2) return lam2 <= 80.2f;
     return lam2 <= (Lb < 16 ? 36.5f : lots ? 80.2f : 62.2f);
+}
+// The largest demand of a block that is tried (lin_demand).  From a float32 emulation of the certificate on the CPU, N(0,1) and heavy-tailed
+// weights, n = 256, T = 0.3 .. 0.01:
+//   * calls judged as a whole: the share of blocks beyond the limit is about the share that fails, for either kind of weights (k = 2, 2^16
+//     states: limits of 64 / 54 / 48 / 43 at T = 0.03 / 0.02 / 0.0145 / 0.01, shares of heavy-tailed blocks that fail 5 to 12 / 23 / 46 /
+//     63 %, of N(0,1) 0 / 0 / 1 / 8 %); strict, where a single failure costs more than all the others gain: ten bits less.
+//   * register kernels, which judge block by block: where a block in three beyond it fails (2^12 states: 60 / 44 / 36 at T = 0.05 / 0.03 /
+//     0.02); strict, where all blocks run at once and the last one decides: eight bits less (ten with the computed emission).
+// Warm calls have no failures to expect.  The vector kernels do not re-centre the energies, so that an outlier alone can end a block.
+float lin_demand_limit(const bcjr_ctx *ctx, int Lb, int k, int V, float lam2, bool by_block, bool strict = false)
+{
+    const bool computed = ctx->cb_computed && V == 1;
+    if (ctx->opt_messages == 2 || lam2 < (computed || V == 2 ? 2.f : 7.f)) return INFINITY;
+    if (by_block) return computed ? 1.5f * Lb + 150.f / lam2 + (strict ? -4.f : 6.f) : 1.3f * Lb + 590.f / lam2 + (strict ? -4.f : 4.f);
+    float d = computed ? 36.f + 100.f / lam2 : k == 3 ? 55.f + 550.f / lam2 : 33.f + 750.f / lam2;
+    if (V == 2) d = fminf(32.f + 350.f / lam2, 45.f + 130.f / lam2);
+    return strict ? d - 10.f : d;
+}
+// How many blocks may fail before both calls with linear messages take longer than with log messages (2^16 states; waves of 148 blocks).  k = 2:
+// a wave gains 0.48 ms forward and 0.3 backward; up to 16 failures cost 1.15 ms, up to 48 3.1 ms (register kernels; of those counted
+// fewer fail), a wave of them 3.8.  k = 3: 0.31 ms forward, 1.7 for a wave of failures.  V = 2: 0.0069 ms a block, 0.024 a failure and
+// 2 ms for the first.
+int lin_failures_allowed(const bcjr_ctx *ctx, int k, int V, int64_t B)
+{
+    const double waves = std::ceil((double)B / ctx->num_sms);
+    if (V == 2) return 0.0069 * (double)B > 2.0 ? (int)(0.284 * (double)B) : 0;
+    const double gain = k == 3 ? 0.31 * waves : 0.78 * waves, rerun = k == 3 ? 1.7 : 3.8;
+    if (gain >= rerun) return (int)(gain / rerun) * ctx->num_sms;
+    return k == 3 || gain < 1.15 ? 0 : gain < 2.2 ? 16 : 48;
+}
+// Count the call's blocks that are not expected to have a certificate (3 us), for kernels that take the call as a whole.
+bcjr_status lin_count_unlikely(bcjr_ctx *ctx, FwdParams &p, cudaStream_t st)
+{
+    p.unlikely = nullptr;
+    if (std::isinf(p.demand)) return BCJR_OK;
+    int *count = (int *)ctx->lin_list.ptr;                       // (a list is made after the kernels have read it)
+    CU(cudaMemsetAsync(count, 0, 4, st));
+    int64_t grid = (p.B + 7) / 8;
+    if (grid > (int64_t)ctx->num_sms * 8) grid = (int64_t)ctx->num_sms * 8;
+    lin_judge_kernel<<<(int)grid, 256, 0, st>>>(p, count);
+    ctx->launches += 1;
+    CU(cudaGetLastError());
+    p.unlikely = count;
+    return BCJR_OK;
+}
+bcjr_status lin_judge(bcjr_ctx *ctx, FwdParams &p, int k, int V, cudaStream_t st)
+{
+    p.unlikely_max = lin_failures_allowed(ctx, k, V, p.B);
+    p.demand = lin_demand_limit(ctx, p.Lb, k, V, p.lam2, false, p.unlikely_max == 0);
+    p.window = (p.Lb + k * V - 1) / (k * V) * V;
+    return lin_count_unlikely(ctx, p, st);
 }
 int lin_exponent(float lam2) { return 1.33f * lam2 < (float)LIN_X_MAX ? (int)(1.33f * lam2) : LIN_X_MAX; }
 bcjr_status lin_buffers(bcjr_ctx *ctx, int64_t B)
@@ -577,6 +635,7 @@ bcjr_status launch_fwd_vec2(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     if (lin) {
         p.lin_x = lin_exponent(p.lam2);
         p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
+        if ((rc = lin_judge(ctx, p, C::KB / C::V, C::V, st))) return rc;
         CU(cudaLaunchKernelEx(&lcfg, fwd_vec_lin_kernel<NBLK>, p));
         note(ctx, "fwd_vec_lin");
         ctx->launches += 1;
@@ -935,6 +994,7 @@ bcjr_status launch_fwd_solo(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
         CU(cudaFuncSetAttribute(fwd_lin_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin));
         p.lin_x = lin_exponent(p.lam2);
         p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
+        if ((rc = lin_judge(ctx, p, KB, 1, st))) return rc;
         fwd_lin_kernel<KB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
         note(ctx, "fwd_lin");
         CU(cudaGetLastError());
@@ -1017,7 +1077,7 @@ bcjr_status launch_bwd_warp(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     ctx->launches += 1;
     CU(cudaGetLastError());
     if (ACC) {
-        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)warps, C::S, grad_codebook);
+        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)warps, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -1045,11 +1105,14 @@ bcjr_status launch_bwd_warp2(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
     bwd_warp2_kernel<LB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
     note(ctx, "bwd_warp2");
     CU(cudaGetLastError());
-    reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)pairs, C::S, grad_codebook);
+    reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)pairs, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
     ctx->launches += 2;
     CU(cudaGetLastError());
     return BCJR_OK;
 }
+
+bcjr_status launch_fwd_warp_any(bcjr_ctx *ctx, FwdParams p, cudaStream_t st);
+bcjr_status launch_bwd_warp_any(bcjr_ctx *ctx, BwdParams p, float *gc, cudaStream_t st);
 
 // One butterfly per thread (bcjr_reg.cuh), k = 2 and n <= 1024: calls at Lb = 8 .. 15, and calls of few blocks at
 // Lb = 16 -- forward as many as are resident (0.46 ms for 8 blocks, 0.66 for 16, 0.73 for 32; fwd_lin_kernel takes 1.40 for up
@@ -1058,13 +1121,25 @@ bcjr_status launch_bwd_warp2(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
 // With log messages (a cold call) the warp-per-block kernels hold more blocks at Lb = 11 .. 13 and win from three quarters of
 // their residency on: 2^12 states, forward 4.23 against 3.68 ms for 4096 blocks, 1.24 against 1.85 for 1000; backward 6.28
 // against 5.80 for 4096.
+bool warp_better(const bcjr_ctx *ctx, int Lb, int64_t B, bool bwd)
+{
+    const int64_t warps = Lb == 13 ? (bwd ? 4 : 8) : bwd ? 8 : 16;           // blocks on an SM of those kernels
+    return Lb >= 11 && Lb <= 13 && 4 * B > 3 * warps * ctx->num_sms;
+}
+// Calls of such sizes with linear messages: the register kernels take them unless more than a quarter of the blocks are not expected to
+// have a certificate (their log-domain form costs 11 % more than the warp-per-block kernels, their linear form 11 % less); the
+// device decides, and the warp-per-block kernels stand behind in both directions.  4096 heavy-tailed blocks of 2^12 states at T = 0.02,
+// both calls 10.2 -> 9.5 ms.
+bool reg_judged(const bcjr_ctx *ctx, int Lb, int64_t B, float lam2)
+{
+    return warp_better(ctx, Lb, B, false) && ctx->opt_path == 0 && ctx->opt_messages == 0 && !std::isinf(lin_demand_limit(ctx, Lb, 2, 1, lam2, true));
+}
 bool reg_wanted(bcjr_ctx *ctx, int Lb, int k, int n, int64_t B, float lam2, bool bwd)
 {
     if (k != 2 || ctx->opt_path == 1 || ctx->opt_fwd_variant != 0 || ctx->opt_hist_every != 1) return false;
     if (ctx->opt_path == 2 && Lb != 16) return false;
     if (Lb >= 11 && Lb <= 13 && !lin_wanted(ctx, Lb, lam2, B)) {
-        const int64_t warps = Lb == 13 ? (bwd ? 4 : 8) : bwd ? 8 : 16;       // blocks on an SM of those kernels
-        if (4 * B > 3 * warps * ctx->num_sms) return false;
+        if (warp_better(ctx, Lb, B, bwd)) return false;
     }
     const int res = reg_resident_cached(ctx, Lb, n, bwd);
     return res > 0 && (Lb < 16 || bwd || B <= res);             // (bwd: after a forward call of these kernels)
@@ -1079,11 +1154,19 @@ bcjr_status launch_fwd_reg(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
     p.hist = (float *)ctx->hist.ptr;
     p.lin_flag = (uint8_t *)ctx->lin_flag.ptr;
     p.lin_x = lin ? lin_exponent(p.lam2) : -1;
+    p.demand = lin_demand_limit(ctx, p.Lb, 2, 1, p.lam2, true, p.B < 6 * (int64_t)ctx->num_sms);
+    p.window = (p.Lb + 1) / 2;
+    if (lin && reg_judged(ctx, p.Lb, p.B, p.lam2)) {
+        p.unlikely_max = (int)(p.B / 4);
+        if ((rc = lin_count_unlikely(ctx, p, st))) return rc;
+        ctx->fwd_judged = true;
+        ctx->judged_max = p.unlikely_max;
+    }
     CU(reg_forward(p, plan, st));
     note(ctx, "fwd_reg");
     ctx->launches += 1;
     ctx->fwd_reg = true;
-    return BCJR_OK;
+    return ctx->fwd_judged ? launch_fwd_warp_any(ctx, p, st) : BCJR_OK;
 }
 bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cudaStream_t st)
 {
@@ -1095,16 +1178,17 @@ bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     p.hist = (float *)ctx->hist.ptr;
     p.gc_part = (float *)ctx->gc_part.ptr;
     p.lin_flag = (const uint8_t *)ctx->lin_flag.ptr;
-    p.lin_x = lin_wanted(ctx, p.Lb, p.lam2, p.B) ? lin_exponent(p.lam2) : -1;
+    p.lin_x = ctx->opt_messages == 1 ? -1 : lin_exponent(p.lam2);     // (the flags say which blocks)
+    if (ctx->fwd_judged) { p.unlikely = (const int *)ctx->lin_list.ptr; p.unlikely_max = ctx->judged_max; }
     CU(reg_backward(p, plan, grad_codebook != nullptr, st));
     note(ctx, "bwd_reg");
     ctx->launches += 1;
     if (grad_codebook) {
-        reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, plan.parts, S, grad_codebook);
+        reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, plan.parts, S, grad_codebook, p.unlikely, p.unlikely_max, false);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
-    return BCJR_OK;
+    return ctx->fwd_judged ? launch_bwd_warp_any(ctx, p, grad_codebook, st) : BCJR_OK;
 }
 
 // One warp per block, or for several (bcjr_small.cuh): 2^4 .. 2^10 states where bcjr_reg.cuh has no kernel.  At 2^10 states and k = 1 a
@@ -1358,7 +1442,7 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = false;
+    ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = ctx->fwd_judged = false;
     ctx->num_ran = 0;
     ctx->cb_computed = codebook == nullptr;
     if (num_blocks == 0) {
@@ -1377,7 +1461,11 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
 #ifndef BCJR_NO_CLUSTER
     use_reg = reg_wanted(ctx, Lb, k, n, num_blocks, p.lam2, false);           // (these kernels find c_lo, c_hi themselves)
 #endif
-    if (!use_reg) {
+    bool range = !use_reg;
+#ifndef BCJR_NO_CLUSTER
+    range = range || reg_judged(ctx, Lb, num_blocks, p.lam2);                 // (nor do they when they leave the call to the others)
+#endif
+    if (range) {
         table_range_kernel<<<1, 1024, 0, st>>>(codebook, 1 << Lb, ctx->diag); // c_lo, c_hi for step_energy, this call's and its backward's
         ctx->launches += 1;
     }
@@ -1567,7 +1655,7 @@ bcjr_status bcjr_soft_quantize_vec(bcjr_ctx *ctx, const float *W, const float *c
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = false;
+    ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = ctx->fwd_judged = false;
     ctx->num_ran = 0;
     if (num_blocks > 0) {
         if ((rc = ensure(ctx, ctx->soft_copy, (size_t)num_blocks * n * 4))) return rc;

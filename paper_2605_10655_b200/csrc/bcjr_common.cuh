@@ -165,6 +165,10 @@ struct FwdParams {
     int hist_every;          // checkpointing kernels: L_t is kept for every hist_every-th step (1 = every step)
     int lin_x;               // linear-message kernels: exponent the largest forward message is scaled to
     uint8_t *lin_flag;       // linear-message kernels: [B] 1 = the block has no certificate (bcjr_lin.cuh)
+    float demand;            // a block whose weights demand more (lin_demand) is not expected to have one; infinity: not looked at
+    int window;              // consecutive weights that share a state's bits
+    const int *unlikely;     // number of such blocks in the call: above unlikely_max no block is tried, and the log-domain kernel that
+    int unlikely_max;        // stands behind (bcjr_warp.cuh) runs the call.  null: not counted, the kernel runs
     const int *list;         // log-domain kernels behind them: list[0] blocks to run, list[1 ...] their indices; null = all B blocks
     int list_max;            // listed blocks up to this number belong to fwd_reg_kernel, more to fwd_solo_kernel
 };
@@ -187,6 +191,8 @@ struct BwdParams {
     float invT;              // 1/T
     int lin_x;               // linear-message kernels: exponent the largest forward message is scaled to
     const uint8_t *lin_flag; // linear-message kernels: [B] 1 = not certified, left to the log-domain kernel
+    const int *unlikely;     // as in FwdParams: what the forward call decided
+    int unlikely_max;
     const uint32_t *g_bits;  // chunked linear-message kernels: [B] bit pattern of the block's largest |g| (grad_bits_kernel)
     const uint32_t *g_top;   // the largest of them all
     const int *list;         // log-domain kernels behind them: list[0] blocks to run, list[1 ...] their indices; null = all B blocks

@@ -73,6 +73,42 @@ __device__ __forceinline__ float2 ex2n_poly2(float2 a)
     return p;
 }
 
+// Which blocks can be expected to have a certificate.  A state is what the last Lb / k steps left in it, so those steps' weights share its
+// Lb bits.  A weight near the middle of the table is served by half the states, one in its tail by a few, and a window of weights that
+// together ask for many more bits than there are is served by paths that were poor prefixes: that excess over the best prefix, times lam2, is
+// the range float32 lacks.  The measure: bits a weight asks for, -log2 of the normal tail beyond it (the quadratic is within 0.3 bits up to 7
+// sigma, its tangent from there on), summed over the window, maximum over the block.  N(0,1) blocks of 256 weights and 2^16 states: 32 in the
+// median, 41 at the 99th percentile; heavy-tailed ones (four degrees of freedom) 40 and 100.  The limits are in the dispatch
+// (lin_demand_limit).  A misjudged block costs time only.
+__device__ __forceinline__ float lin_demand(const float *__restrict__ w, int t, int n, int window)
+{
+    float s = 0.f;
+    for (int i = t; i < t + window && i < n; ++i) {
+        const float a = fabsf(__ldg(w + i)), m = fminf(a, 7.3f);
+        s += fmaf(10.2f, a - m, fmaf(m, fmaf(0.63f, m, 1.05f), 1.f));
+    }
+    return s;
+}
+// *count (zero before the call): blocks beyond p.demand, a warp per block
+static __global__ void __launch_bounds__(256) lin_judge_kernel(FwdParams p, int *count)
+{
+    const int lane = threadIdx.x & 31;
+    int mine = 0;
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < p.B; b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        float d = 0.f;
+        for (int t = lane; t < p.n; t += 32) d = fmaxf(d, lin_demand(p.W + b * p.n, t, p.n, p.window));
+        mine += warp_max(d) > p.demand;
+    }
+    if (lane == 0 && mine) atomicAdd(count, mine);
+}
+// calls judged as a whole: true if no block is tried (all are flagged then)
+__device__ __forceinline__ bool lin_given_up(const FwdParams &p)
+{
+    if (!p.unlikely || *p.unlikely <= p.unlikely_max) return false;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < p.B; b += (int64_t)gridDim.x * blockDim.x) p.lin_flag[b] = 1;
+    return true;
+}
+
 // Backward kernels (see bcjr_lin_bwd.cuh): exponent of a gradient from the bit pattern of its largest |g| (NaN sorts above infinity);
 // GRAD_NONE: all zero.  The bounds keep both factors normal numbers.
 constexpr int GRAD_LEVEL = 2, GRAD_SPAN = 8, GRAD_ROOM = 2, GRAD_NONE = -1000;
@@ -162,6 +198,7 @@ __global__ void __launch_bounds__(SoloCfg<KB>::THREADS, 1) fwd_lin_kernel(FwdPar
     using C = SoloCfg<KB>;
     constexpr int K = C::K, NB = C::NB, Q = C::Q, BPT = C::BPT, NWARP = C::NWARP, CT = C::CTHREADS, NCH = C::NCH, RD = C::RD;
     constexpr int UNITS = C::UNITS, HPU = C::HPU, NU = BPT * UNITS;
+    if (lin_given_up(p)) return;
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.n, X = p.lin_x;

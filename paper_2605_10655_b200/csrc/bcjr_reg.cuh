@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
     const int cid = blockIdx.x / CL, ncid = gridDim.x / CL;
     const int64_t nblk = p.list ? (int64_t)p.list[0] : p.B;
     if (cid >= nblk || (p.list && nblk > p.list_max)) return;
+    if (lin_given_up(p)) return;
     extern __shared__ __align__(16) float smem[];
     RegBlock<C> rb{smem, (int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5, CL > 1 ? cluster_ctarank() : 0u,
                    Proto{1u, reinterpret_cast<volatile int *>(smem + C::OFF_FLAG), p.diag}, 0u};
@@ -336,7 +337,15 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
             outside |= se.delta != 0.f;
         }
         const bool recentre = rb.cta_or(outside) != 0;           // (every CTA of a cluster decides alike)
+        bool likely = X >= 0;
+        if (likely && p.demand < __int_as_float(0x7f800000)) {
+            int beyond = 0;
+            for (int t = tid; t < n; t += NT) beyond |= lin_demand(w, t, n, p.window) > p.demand;
+            likely = rb.cta_or(beyond) == 0;
+        }
         // both sweeps in one message domain; true if the result stands
+        int Ofin = 0;
+        float l2zf = 0.f, bdef = 0.f, gap = 0.f;
         auto run = [&](auto lin_tag, auto rc_tag) -> bool {
             constexpr bool LIN = decltype(lin_tag)::value, RC = decltype(rc_tag)::value;
             int bad = 0;
@@ -492,8 +501,8 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
             asm volatile("cp.async.wait_all;" ::: "memory");
             if (C::NWARP > 1 && warp == 0) finish_step(1, n & 1);
             rb.block_sync();
-            // soft codeword, one thread per step (it may overwrite W: written when it stands, after everything that reads W)
-            float bdef = 0.f, gap = 0.f;
+            // soft codeword, one thread per step, kept until it stands
+            bdef = gap = 0.f;
             for (int t = (int)rb.rank * NT + tid; t < n; t += CL * NT) {
                 float a, c;
                 if (CL > 1) {
@@ -512,35 +521,35 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
                 bdef = fmaxf(bdef, df);
                 if (t == 0) gap = fabsf(lg2f(c));                // A_1 is constant: the sums of step 1 are the beta side's Z
             }
-            if (LIN && rb.block_or(bad, 16)) return false;
-            for (int t = (int)rb.rank * NT + tid; t < n; t += CL * NT) {
-                const float sw = step[t].w;
-                p.soft[blk * n + t] = sw;
-                if (p.soft_copy) p.soft_copy[blk * n + t] = sw;
-            }
-            bdef = rb.block_max(bdef, 24);
-            defect = fmaxf(defect, bdef);
-            zgap = fmaxf(zgap, gap);
-            if (rb.rank == 0 && tid == 0) {
-                p.lin_flag[blk] = LIN ? 0 : 1;
-                if (p.blk_defect) p.blk_defect[blk] = bdef;
-                if (p.logZ) {
-                    double zshift = 0.0;                         // sum_t lam2 delta_t^2: left out by step_energy
-                    if (recentre)
-                        for (int t = 0; t < n; ++t) {
-                            const double dl = (double)step[t].z;
-                            zshift += (double)p.lam2 * dl * dl;
-                        }
-                    p.logZ[blk] = (float)(((double)O + (double)l2z - zshift) * 0.6931471805599453);
-                }
-            }
-            return true;
+            Ofin = O; l2zf = l2z;
+            return !(LIN && rb.block_or(bad, 16));
         };
         bool done = false;
-        if (X >= 0) done = recentre ? run(std::true_type{}, std::true_type{}) : run(std::true_type{}, std::false_type{});
+        if (likely) done = recentre ? run(std::true_type{}, std::true_type{}) : run(std::true_type{}, std::false_type{});
         if (!done) {
             rb.block_sync();
             run(std::false_type{}, std::true_type{});
+        }
+        bdef = rb.block_max(bdef, 24);
+        defect = fmaxf(defect, bdef);
+        zgap = fmaxf(zgap, gap);
+        for (int t = (int)rb.rank * NT + tid; t < n; t += CL * NT) {   // (it may overwrite W, which nothing below reads)
+            const float sw = step[t].w;
+            p.soft[blk * n + t] = sw;
+            if (p.soft_copy) p.soft_copy[blk * n + t] = sw;
+        }
+        if (rb.rank == 0 && tid == 0) {
+            p.lin_flag[blk] = done ? 0 : 1;
+            if (p.blk_defect) p.blk_defect[blk] = bdef;
+            if (p.logZ) {
+                double zshift = 0.0;                             // sum_t lam2 delta_t^2: left out by step_energy
+                if (recentre)
+                    for (int t = 0; t < n; ++t) {
+                        const double dl = (double)step[t].z;
+                        zshift += (double)p.lam2 * dl * dl;
+                    }
+                p.logZ[blk] = (float)(((double)Ofin + (double)l2zf - zshift) * 0.6931471805599453);
+            }
         }
         rb.block_sync();
     }
@@ -565,6 +574,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, 
     const int cid = blockIdx.x / CL, ncid = gridDim.x / CL;
     const int64_t nblk = p.list ? (int64_t)p.list[0] : p.B;
     if (cid >= nblk || (p.list && nblk > p.list_max)) return;
+    if (p.unlikely && *p.unlikely > p.unlikely_max) return;
     extern __shared__ __align__(16) float smem[];
     RegBlock<C> rb{smem, (int)threadIdx.x, (int)threadIdx.x & 31, (int)threadIdx.x >> 5, CL > 1 ? cluster_ctarank() : 0u,
                    Proto{1u, reinterpret_cast<volatile int *>(smem + C::OFF_FLAG), p.diag}, 0u};

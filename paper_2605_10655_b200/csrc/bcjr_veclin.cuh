@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(Vec2Cfg<NBLK_>::THREADS, 1) fwd_vec_lin_kernel
     constexpr int NBLK = C::NBLK, OSTR = C::MAX_NT + 4, PP = C::PP;
     constexpr uint32_t TX_ALPHA = QC * 4u + SLOTS * 4u;          // half of the messages + gauge slots
     constexpr uint32_t TX_BETA = QC * 4u, TX_PART = SLOTS * 16u; // half of the messages; posterior sums (rank 0 only)
+    if (lin_given_up(p)) return;                                 // (every CTA alike)
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rank = cluster_ctarank();

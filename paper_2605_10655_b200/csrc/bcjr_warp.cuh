@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(WarpCfg<LB, false>::THREADS, 1) fwd_warp_kerne
 {
     using C = WarpCfg<LB, false>;
     constexpr int K = C::K, NB = C::NB, Q = C::Q, BPT = C::BPT, RD = C::RD;
+    if (p.unlikely && *p.unlikely <= p.unlikely_max) return;      // the register kernel has run the call
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.n;
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(WarpCfg<LB, true>::THREADS, 1) bwd_warp_kernel
 {
     using C = WarpCfg<LB, true>;
     constexpr int K = C::K, NB = C::NB, Q = C::Q, BPT = C::BPT, RD = C::RD;
+    if (p.unlikely && *p.unlikely <= p.unlikely_max) return;      // the register kernel has run the call
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.n;
@@ -531,6 +533,7 @@ __global__ void __launch_bounds__(Warp2Cfg<LB>::THREADS, 1) bwd_warp2_kernel(Bwd
 {
     using C = Warp2Cfg<LB>;
     constexpr int K = C::K, NB = C::NB, Q = C::Q, BPT = C::BPT, RD = C::RD;
+    if (p.unlikely && *p.unlikely <= p.unlikely_max) return;      // the register kernel has run the call
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pw = warp & 1, pair = warp >> 1;
     const int n = p.n;

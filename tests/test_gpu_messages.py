@@ -189,3 +189,104 @@ def test_a_call_reports_its_kernels_and_its_linear_blocks(ctx, Lb, k, n, B, T, o
     finally:
         for name in options:
             ctx.set_option(name, 0)
+
+
+def _heavy(rng, B, n):
+    return (rng.standard_normal((B, n)) / np.sqrt((rng.standard_normal((4, B, n)) ** 2).mean(0)) / np.sqrt(2.0)).astype(np.float32)
+
+
+def _demand(W, window):
+    a = np.abs(W.astype(np.float64))
+    m = np.minimum(a, 7.3)
+    bits = np.pad(1.0 + m * (1.05 + 0.63 * m) + 10.2 * (a - m), ((0, 0), (0, window - 1)))
+    return np.lib.stride_tricks.sliding_window_view(bits, window, axis=1).sum(-1).max(1)
+
+
+@pytest.mark.parametrize("Lb,k,V,n,B,T,computed", [(16, 2, 1, 256, 600, 0.0145, False), (16, 2, 1, 256, 300, 0.0145, False), (16, 2, 1, 512, 148, 0.03, False),
+                                                   (16, 2, 2, 256, 400, 0.02, False), (16, 3, 1, 256, 1200, 0.0095, False), (16, 2, 1, 256, 300, 0.07, True),
+                                                   (12, 2, 1, 256, 1800, 0.02, False), (13, 2, 1, 256, 1000, 0.1, True), (11, 2, 1, 300, 1999, 0.02, False)])
+def test_calls_whose_blocks_would_fail_do_not_try_linear_messages(ctx, Lb, k, V, n, B, T, computed):
+    # The same shape and temperature: nearly all N(0,1) blocks have a certificate; of heavy-tailed ones so many have none that running those
+    # again costs more than the others gain, and the call is left to the log-domain kernels.
+    import torch
+    rng = np.random.default_rng(200 + B)
+    dev = torch.device("cuda", ctx.device)
+    c = torch.from_numpy(rng.standard_normal((1 << Lb, V) if V > 1 else 1 << Lb).astype(np.float32)).to(dev)
+    for W, heavy in ((rng.standard_normal((B, n)).astype(np.float32), False), (_heavy(rng, B, n), True)):
+        Wd = torch.from_numpy(W).to(dev)
+        if V > 1:
+            ctx.bcjr_soft_quantize_vec(Wd, c, Lb, k, V, n, T)
+        else:
+            ctx.bcjr_soft_quantize(Wd, None if computed else c, Lb, k, n, T)
+        linear = ctx.linear_blocks()
+        assert ctx.sync_status().device_status == 0
+        if k == 3:                                       # hardly any fail: both kinds of weights are tried
+            assert linear >= 0.8 * B
+        else:
+            assert linear == 0 if heavy else linear >= 0.9 * B, f"heavy={heavy}: {linear} of {B}"
+
+
+@pytest.mark.parametrize("Lb,n,B,T", [(10, 256, 300, 0.05), (12, 300, 1000, 0.02), (9, 100, 50, 0.05), (14, 256, 10, 0.04), (16, 128, 20, 0.03)])
+def test_register_kernels_judge_block_by_block(ctx, Lb, n, B, T):
+    import torch
+    rng = np.random.default_rng(300 + Lb)
+    W = np.concatenate([rng.standard_normal((B - B // 2, n)).astype(np.float32), _heavy(rng, B // 2, n)])
+    W = np.ascontiguousarray(W[rng.permutation(B)])
+    W[0, :] = 0.0
+    W[0, 3:3 + Lb // 2] = 7.0                            # one window that asks for everything
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd = torch.from_numpy(W).to(dev), torch.from_numpy(rng.standard_normal(1 << Lb).astype(np.float32)).to(dev)
+    lam2 = 1.4426950408889634 / (2.0 * T)
+    strict = 4.0 if B < 888 else -4.0                    # fewer than six blocks an SM: the last one decides
+    likely = int((_demand(W, (Lb + 1) // 2) <= 1.3 * Lb + 590.0 / lam2 - strict + 1e-3).sum())
+    soft, _ = ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, n, T)
+    linear = ctx.linear_blocks()
+    assert 0.9 * likely <= linear <= likely < B, (linear, likely, B)
+    ctx.set_option("messages", 2)
+    try:
+        tried, _ = ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, n, T)
+        assert linear <= ctx.linear_blocks() <= B
+    finally:
+        ctx.set_option("messages", 0)
+    assert ctx.sync_status().device_status == 0
+    assert parity.rel_inf(soft.cpu().numpy(), tried.cpu().numpy()) <= parity.SOFT_TOL
+
+
+@pytest.mark.parametrize("Lb,B,T,heavy", [(12, 1800, 0.02, True), (12, 1800, 0.02, False), (11, 1801, 0.02, True), (13, 900, 0.03, True), (13, 900, 0.03, False)])
+def test_mid_size_calls_judged_as_a_whole(ctx, Lb, B, T, heavy):
+    # The register kernels and the warp-per-block kernels are both launched and one of them runs the call.  A call left to the second is
+    # the call of messages = 1, bit for bit, in both directions; the other agrees with it within float32's rounding.
+    import torch
+    n = 24
+    rng = np.random.default_rng(400 + Lb + heavy)
+    W = _heavy(rng, B, n) * 2 if heavy else rng.standard_normal((B, n)).astype(np.float32) * np.float32(0.8)
+    g = rng.standard_normal((B, n)).astype(np.float32)
+    c = rng.standard_normal(1 << Lb).astype(np.float32)
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (W, c, g))
+    out = []
+    for messages in (0, 1):
+        ctx.set_option("messages", messages)
+        try:
+            soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, n, T)
+            forward, linear = ctx.last_kernels(), ctx.linear_blocks()
+            gW, gc = ctx.bcjr_backward(gd)
+            backward = ctx.last_kernels()
+            gW2, _ = ctx.bcjr_backward(gd, want_grad_codebook=False)
+            assert ctx.sync_status().device_status == 0
+        finally:
+            ctx.set_option("messages", 0)
+        if messages == 0:
+            assert forward == ["fwd_reg", "fwd_warp"] and backward[0] == "bwd_reg" and backward[1].startswith("bwd_warp")
+            assert linear == 0 if heavy else linear > 0.9 * B
+        else:
+            assert forward == ["fwd_warp"] and linear == 0
+        out.append([x.cpu().numpy() for x in (soft, logZ, gW, gc, gW2)])
+    for x, r, tol in zip(out[0], out[1], (parity.SOFT_TOL, 1e-5, parity.GRAD_TOL, parity.GRAD_TOL, parity.GRAD_TOL)):
+        if heavy:
+            np.testing.assert_array_equal(x, r)
+        else:
+            assert parity.rel_inf(x, r) <= tol
+    pick = np.array([0, 1, B // 2, B - 1])
+    ref = oracle.soft_quantize(W[pick], c, Lb, 2, T)
+    assert parity.rel_inf(out[0][0][pick], ref["soft"]) <= parity.SOFT_TOL
