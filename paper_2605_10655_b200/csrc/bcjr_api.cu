@@ -1136,7 +1136,8 @@ bool reg_judged(const bcjr_ctx *ctx, int Lb, int64_t B, float lam2)
 }
 bool reg_wanted(bcjr_ctx *ctx, int Lb, int k, int n, int64_t B, float lam2, bool bwd)
 {
-    if (k != 2 || ctx->opt_path == 1 || ctx->opt_fwd_variant != 0 || ctx->opt_hist_every != 1) return false;
+    if (k != 2 || ctx->opt_path == 1 || ctx->opt_fwd_variant != 0) return false;
+    if (ctx->opt_hist_every != 1 && Lb == 16 && n <= CkptCfg<2>::MAX_N) return false;   // fwd_ckpt_kernel's shapes: the option is for no other
     if (ctx->opt_path == 2 && Lb != 16) return false;
     if (Lb >= 11 && Lb <= 13 && !lin_wanted(ctx, Lb, lam2, B)) {
         if (warp_better(ctx, Lb, B, bwd)) return false;

@@ -290,3 +290,26 @@ def test_mid_size_calls_judged_as_a_whole(ctx, Lb, B, T, heavy):
     pick = np.array([0, 1, B // 2, B - 1])
     ref = oracle.soft_quantize(W[pick], c, Lb, 2, T)
     assert parity.rel_inf(out[0][0][pick], ref["soft"]) <= parity.SOFT_TOL
+
+
+@pytest.mark.parametrize("Lb,n,B", [(9, 20, 5), (12, 20, 5), (15, 20, 2), (16, 600, 2)])
+def test_history_every_m_leaves_other_shapes_alone(ctx, Lb, n, B):
+    # The option is for 2^16 states, k = 2 and up to 512 weights; elsewhere a call runs the kernels it would run without it.
+    import torch
+    W, c, g = _rand(n, Lb, B, seed=500 + Lb)
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(a).to(dev) for a in (W, c, g))
+    out = []
+    for m in (1, 4):
+        ctx.set_option("history_every_m", m)
+        try:
+            soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, n, 0.2)
+            assert ctx.last_kernels() == ["fwd_reg"], f"m={m}"
+            gW, gc = ctx.bcjr_backward(gd)
+            assert ctx.last_kernels() == ["bwd_reg"], f"m={m}"
+        finally:
+            ctx.set_option("history_every_m", 1)
+        out.append((soft, logZ, gW, gc))
+    assert ctx.sync_status().device_status == 0
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
