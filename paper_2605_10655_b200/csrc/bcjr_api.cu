@@ -395,7 +395,7 @@ template <int LB, int KB, int CL, int THREADS>
 bcjr_status launch_fwd_cluster_t(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
 {
     using C = ClusterCfg<LB, KB, CL, THREADS>;
-    if (p.n > C::MAX_N) return BCJR_EUNSUPPORTED;
+    if (p.n > C::MAX_N || ((uintptr_t)p.cb & 15u)) return BCJR_EUNSUPPORTED;     // (the table is read four entries at a time)
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     auto kern = fwd_cluster_kernel<LB, KB, CL, THREADS>;
@@ -415,7 +415,7 @@ bcjr_status launch_bwd_cluster_t(bcjr_ctx *ctx, BwdParams p, float *grad_codeboo
 {
     using C = ClusterCfg<LB, KB, CL, THREADS>;
     using BC = BwdClusterCfg<LB, KB, CL, THREADS>;
-    if (p.n > BC::MAX_N) return BCJR_EUNSUPPORTED;
+    if (p.n > BC::MAX_N || ((uintptr_t)p.cb & 15u)) return BCJR_EUNSUPPORTED;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     auto kern = bwd_cluster_kernel<LB, KB, CL, THREADS>;
@@ -1621,7 +1621,8 @@ bcjr_status viterbi_hard(bcjr_ctx *ctx, const float *W, const float *codebook, i
     use_large = ctx->opt_path != 1 && Lb == 16 && (k == 2 || k == 3);
     if (ctx->opt_path == 2 && !use_large) return BCJR_EUNSUPPORTED;
     if (use_large) {
-        rc = k == 2 ? launch_vit_solo<2>(ctx, p, st) : launch_vit_solo<3>(ctx, p, st);
+        // (the double kernel reads the table four entries at a time; a table that starts elsewhere is the generic kernel's)
+        rc = ((uintptr_t)codebook & 15u) ? BCJR_EUNSUPPORTED : k == 2 ? launch_vit_solo<2>(ctx, p, st) : launch_vit_solo<3>(ctx, p, st);
         if (rc == BCJR_EUNSUPPORTED && ctx->opt_path != 2) { use_large = false; rc = BCJR_OK; }
     }
 #else

@@ -313,3 +313,30 @@ def test_history_every_m_leaves_other_shapes_alone(ctx, Lb, n, B):
     assert ctx.sync_status().device_status == 0
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("Lb,k,n,B", [(16, 2, 7, 3), (16, 3, 5, 2), (16, 2, 20, 40), (16, 2, 1030, 1), (12, 2, 9, 5), (12, 2, 9, 2000), (9, 2, 9, 3), (9, 3, 9, 3)])
+def test_tables_and_weights_at_any_float_address(ctx, Lb, k, n, B):
+    # A slice of a tensor starts at any multiple of four bytes: table, weights and gradient one float past a 16-byte boundary.
+    import torch
+    W, c, g = _rand(n, Lb, B, seed=600 + Lb + k)
+    dev = torch.device("cuda", ctx.device)
+
+    def shifted(a):
+        buf = torch.zeros(a.size + 1, device=dev)
+        buf[1:] = torch.from_numpy(a.reshape(-1)).to(dev)
+        return buf[1:]
+    calls = []
+    for place in (lambda a: torch.from_numpy(a.reshape(-1)).to(dev), shifted):
+        Wd, cd, gd = place(W), place(c), place(g)
+        bits, states, hard = ctx.viterbi_hard(Wd, cd, Lb, k, n)
+        soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, k, n, 0.2)
+        gW, gc = ctx.bcjr_backward(gd)
+        assert ctx.sync_status().device_status == 0
+        calls.append((bits, states, hard, soft, logZ, gW, gc))
+    for i, (a, b) in enumerate(zip(*calls)):
+        if i < 3 or n <= 1024:
+            assert torch.equal(a, b)
+        else:                                            # longer blocks: another kernel where the table does not start on 16 bytes
+            assert parity.rel_inf(a.cpu().numpy(), b.cpu().numpy()) <= (parity.SOFT_TOL if i < 5 else parity.GRAD_TOL)
+    assert cd.data_ptr() % 16 == 4
