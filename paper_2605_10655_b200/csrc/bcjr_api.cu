@@ -114,6 +114,16 @@ bcjr_status ensure(bcjr_ctx *ctx, Buffer &b, size_t bytes)
     return BCJR_OK;
 }
 
+// Scratch of a faster kernel that a slower one with less scratch can stand in for: *got = false where it cannot be had.
+bcjr_status ensure_or_do_without(bcjr_ctx *ctx, Buffer &b, size_t bytes, bool *got)
+{
+    const bcjr_status rc = ensure(ctx, b, bytes);
+    *got = rc == BCJR_OK;
+    if (rc != BCJR_ENOMEM) return rc;
+    ctx->cuda_error.clear();
+    return BCJR_OK;
+}
+
 // Computed Gaussian emission (a NULL codebook): the context keeps a table of it, written by gaussian_table_kernel at every call (3 us),
 // which the kernels read like any other.  (Evaluating the entries in each kernel while it stages them cost 0.15 ms a staging at
 // 2^16 states: 148 blocks of 136 weights forward 1.16 -> 0.84 ms, backward 1.59 -> 1.26.)
@@ -664,7 +674,7 @@ bcjr_status launch_bwd_vec4(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     using Bt = VecBetaLinCfg<VEC_BETA_NBLK>;
     constexpr int S = C::F::S, V = 2, KB = 4;
     if (p.n > C::MAX_N || ((uintptr_t)p.cb & 15u)) return BCJR_EUNSUPPORTED;
-    const bool lin = ctx->fwd_lin && ctx->opt_messages != 1 && p.n <= A::MAX_N;
+    bool lin = ctx->fwd_lin && ctx->opt_messages != 1 && p.n <= A::MAX_N;
     cudaLaunchConfig_t cfg{}, acfg{}, bcfg{};
     cudaLaunchAttribute attr[1], aattr[1], battr[1];
     bcjr_status rc = plan_cluster(ctx, bwd_vec4_kernel<VEC4_BWD_NBLK>, C::CL, C::THREADS, C::SMEM_BYTES, p.B, &cfg, attr, st);
@@ -682,8 +692,11 @@ bcjr_status launch_bwd_vec4(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
         const int64_t wave = (int64_t)acl * VEC_ALPHA_NBLK, waves = (int64_t)(5e9 / (4.0 * (double)row)) / wave;
         chunk = wave * (waves > 1 ? waves : 1);
         if (chunk > p.B) chunk = p.B;
-        if (row * (size_t)chunk > hist) hist = row * (size_t)chunk;
-        if ((rc = ensure(ctx, ctx->stepO, (size_t)chunk * A::AUX_INTS * 4))) return rc;
+        // (5 GB of history against 0.3 for the log-domain kernel, which runs the call where they do not fit)
+        const size_t more = row * (size_t)chunk > hist ? row * (size_t)chunk : hist;
+        if ((rc = ensure_or_do_without(ctx, ctx->hist, more * 4, &lin))) return rc;
+        if (lin && (rc = ensure(ctx, ctx->stepO, (size_t)chunk * A::AUX_INTS * 4))) return rc;
+        if (!lin) parts = ncl;
     }
     if ((rc = ensure(ctx, ctx->hist, hist * 4))) return rc;
     if ((rc = ensure(ctx, ctx->gc_part, (size_t)parts * S * V * 4))) return rc;
@@ -907,10 +920,12 @@ bcjr_status launch_vit_solo(bcjr_ctx *ctx, VitParams p, cudaStream_t st)
     p.diag = ctx->diag;
     // Float32 first, the double kernel for what that cannot prove -- except with the computed emission, which is monotone in the state:
     // paths that differ in old bits cost almost the same, no block is proved, and both kernels would run (740 blocks 5.32 -> 6.97 ms).
-    if (p.n <= VitFastCfg<KB>::MAX_N && ctx->opt_messages != 1 && !ctx->cb_computed) {
+    // The float32 kernel's stored messages are 1.7 GB at n = 256 (the double kernel's back pointers 0.3): where they do not fit, the double one.
+    bool fast = p.n <= VitFastCfg<KB>::MAX_N && ctx->opt_messages != 1 && !ctx->cb_computed;
+    if (fast && (rc = ensure_or_do_without(ctx, ctx->hist, (size_t)grid * VitFastCfg<KB>::hist_floats(p.n) * 4, &fast))) return rc;
+    if (fast) {
         using F = VitFastCfg<KB>;
         CU(cudaFuncSetAttribute(viterbi_fast_kernel<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->max_smem_optin));
-        if ((rc = ensure(ctx, ctx->hist, (size_t)grid * F::hist_floats(p.n) * 4))) return rc;
         if ((rc = ensure(ctx, ctx->vit_flag, ((size_t)p.B + 15) / 16 * 16))) return rc;
         if ((rc = ensure(ctx, ctx->vit_list, ((size_t)p.B + 1) * 4))) return rc;
         p.hist = (float *)ctx->hist.ptr;
@@ -938,7 +953,9 @@ bcjr_status launch_fwd_listed(bcjr_ctx *ctx, FwdParams &p, int k, cudaStream_t s
     const int res = k == 2 && ctx->opt_max_ctas == 0 ? reg_resident_cached(ctx, p.Lb, p.n, false) : 0;
     if (res == 0) return BCJR_OK;
     const RegPlan plan = reg_plan(p.Lb, p.n, p.B, false, res, 0);
-    if (plan.hist_floats * 4 > ctx->hist.bytes) return BCJR_OK;          // (never: the history of a linear call is larger)
+    bcjr_status rc = ensure(ctx, ctx->hist, plan.hist_floats * 4);       // (the linear call's history is as large or larger)
+    if (rc) return rc;
+    p.hist = (float *)ctx->hist.ptr;
     p.list_max = 2 * res;
     FwdParams q = p;
     q.lin_x = -1;
@@ -961,7 +978,8 @@ bcjr_status launch_vit_reg(bcjr_ctx *ctx, VitParams &p, cudaStream_t st)
     if (ctx->opt_max_ctas > 0 && grid > ctx->opt_max_ctas) grid = ctx->opt_max_ctas;
     if (grid > p.B) grid = p.B;
     bcjr_status rc;
-    if ((rc = ensure(ctx, ctx->hist, (size_t)grid * reg_viterbi_hist_floats(p.Lb, p.n) * 4))) return rc;
+    bool fits = false;
+    if ((rc = ensure_or_do_without(ctx, ctx->hist, (size_t)grid * reg_viterbi_hist_floats(p.Lb, p.n) * 4, &fits)) || !fits) return rc;
     if ((rc = ensure(ctx, ctx->vit_flag, ((size_t)p.B + 15) / 16 * 16))) return rc;
     if ((rc = ensure(ctx, ctx->vit_list, ((size_t)p.B + 1) * 4))) return rc;
     p.hist = (float *)ctx->hist.ptr;

@@ -340,3 +340,46 @@ def test_tables_and_weights_at_any_float_address(ctx, Lb, k, n, B):
         else:                                            # longer blocks: another kernel where the table does not start on 16 bytes
             assert parity.rel_inf(a.cpu().numpy(), b.cpu().numpy()) <= (parity.SOFT_TOL if i < 5 else parity.GRAD_TOL)
     assert cd.data_ptr() % 16 == 4
+
+
+@pytest.mark.parametrize("shape", ["viterbi", "vector"])
+def test_calls_that_lack_scratch_run_the_kernels_that_need_less(shape):
+    # The float32 Viterbi sweep and the chunked vector backward call hold 1.7 and 4.7 GB of scratch for these calls; with less to be had the
+    # kernels behind them run, which hold a few hundred MB.  A context of its own, so that nothing is held already.
+    import torch
+    from paper_2605_10655_b200 import Context
+    dev = torch.device("cuda", 0)
+    rng = np.random.default_rng(700)
+    fresh, hold = Context(0), None
+    try:
+        if shape == "viterbi":
+            W = torch.from_numpy(rng.standard_normal((150, 256)).astype(np.float32)).to(dev)
+            c = torch.from_numpy(rng.standard_normal(1 << 16).astype(np.float32)).to(dev)
+            run, want, less = (lambda: fresh.viterbi_hard(W, c, 16, 2, 256)), ["viterbi_fast", "viterbi_solo"], ["viterbi_solo"]
+            free_bytes = 1200 << 20
+        else:
+            W = torch.from_numpy(rng.standard_normal((1184, 256)).astype(np.float32)).to(dev)
+            g = torch.from_numpy(rng.standard_normal((1184, 256)).astype(np.float32)).to(dev)
+            c = torch.from_numpy(rng.standard_normal((1 << 16, 2)).astype(np.float32)).to(dev)
+            fresh.bcjr_soft_quantize_vec(W, c, 16, 2, 2, 256, 0.3)
+            run, want, less = (lambda: fresh.bcjr_backward(g)), ["bwd_vec_lin", "bwd_vec4"], ["bwd_vec4"]
+            free_bytes = 2000 << 20
+        fresh.sync_status()
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info(0)
+        hold = torch.empty(free - free_bytes, dtype=torch.uint8, device=dev)
+        first = run()
+        assert fresh.last_kernels() == less and fresh.sync_status().device_status == 0
+        hold = None
+        torch.cuda.empty_cache()
+        second = run()
+        assert fresh.last_kernels() == want and fresh.sync_status().device_status == 0
+        for a, b in zip(first, second):
+            if shape == "viterbi":
+                assert torch.equal(a, b)
+            else:
+                assert parity.rel_inf(a.cpu().numpy(), b.cpu().numpy()) <= parity.GRAD_TOL
+    finally:
+        hold = None
+        torch.cuda.empty_cache()
+        fresh.close()
