@@ -383,3 +383,175 @@ def test_calls_that_lack_scratch_run_the_kernels_that_need_less(shape):
         hold = None
         torch.cuda.empty_cache()
         fresh.close()
+
+
+def _planted(n, B, listed, seed, V=1):
+    # every weight near the middle of the table but for the listed blocks, which jump from one end of it to the other at every step
+    W, c, g = _rand(n, 16, B, seed)
+    W *= 0.3
+    jump = np.where((np.arange(n) // V) % 2 == 0, 5.0, -5.0).astype(np.float32)
+    W[listed] = jump
+    return W, c, g
+
+
+def _forced(ctx, W, c, g, k, T, V=1, want_gc=True):
+    import torch
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (W, c, g))
+    Lb, n = (c.shape[0] - 1).bit_length(), W.shape[1]
+    ctx.set_option("messages", 2)
+    try:
+        if V > 1:
+            soft, logZ = ctx.bcjr_soft_quantize_vec(Wd, cd, Lb, k, V, n, T)
+        else:
+            soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, k, n, T)
+        kernels, linear = [ctx.last_kernels()], ctx.linear_blocks()
+        gW, gc = ctx.bcjr_backward(gd, want_grad_codebook=want_gc)
+        kernels.append(ctx.last_kernels())
+        st = ctx.sync_status()
+        assert st.device_status == 0 and st.max_posterior_defect < 1e-3
+    finally:
+        ctx.set_option("messages", 0)
+    return soft.cpu().numpy(), logZ.cpu().numpy(), gW.cpu().numpy(), gc.cpu().numpy() if want_gc else None, kernels, linear
+
+
+def _grad_err(x, r):
+    # A block that jumps has one path left and no gradient but float32's rounding, (w - c) / T of 250 times 2^-24 at a step: where all do, the
+    # scale is a twentieth of the upstream gradient's.
+    return float(np.abs(np.asarray(x, dtype=np.float64) - r).max() / max(np.abs(r).max(), 0.05))
+
+
+@pytest.mark.parametrize("k,n,B,T,count", [(2, 5, 600, 0.02, 400), (2, 7, 600, 0.009, 149), (2, 6, 450, 0.02, 61), (2, 6, 450, 0.02, 50), (2, 4, 300, 0.02, 300),
+                                           (3, 6, 400, 0.012, 170)])
+def test_many_blocks_without_a_certificate(ctx, k, n, B, T, count):
+    # Behind the chunked linear kernels: the register kernels up to two (forward) and four (backward) residencies of listed blocks, above
+    # that the log-domain kernels, the backward ones in chunks of one block an SM -- several, whole and ragged, with gradients of listed
+    # and other blocks added into the same partial tables.
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(800 + B + count)
+    listed = np.sort(rng.permutation(B)[:count])
+    W, c, g = _planted(n, B, listed, seed=801)
+    edge = [listed[0], listed[-1], listed[min(count - 1, sms - 1)], listed[min(count - 1, sms)], listed[count // 2]]
+    others = np.setdiff1d(np.arange(B), listed)
+    pick = np.unique(np.concatenate([edge, others[[0, len(others) // 2, -1]] if len(others) else []]).astype(int))
+    z = np.zeros_like(g); z[pick] = g[pick]
+    soft, logZ, gW, gc, kernels, linear = _forced(ctx, W, c, z, k, T)
+    assert linear == B - count
+    if k == 2:
+        assert kernels == [["fwd_lin", "fwd_reg", "fwd_solo"], ["bwd_lin", "bwd_reg", "bwd_split"]]
+    ref_f, ref_b = oracle.soft_quantize(W[pick], c, 16, k, T), oracle.backward(W[pick], c, g[pick], 16, k, T)
+    parity.assert_forward_backward({"soft": soft[pick], "logZ": logZ[pick]}, ref_f, what=f"{count} of {B} listed")
+    assert _grad_err(gW[pick], ref_b["grad_W"]) <= parity.GRAD_TOL and _grad_err(gc, ref_b["grad_codebook"]) <= parity.GRAD_TOL
+    rest = np.setdiff1d(np.arange(B), pick)
+    assert np.all(np.isfinite(soft)) and np.all(gW[rest] == 0.0)
+    if k == 2:                                           # the same without grad_codebook
+        gW2 = _forced(ctx, W, c, z, k, T, want_gc=False)[2]
+        assert _grad_err(gW2[pick], ref_b["grad_W"]) <= parity.GRAD_TOL
+
+
+@pytest.mark.parametrize("n,B,T,count", [(8, 400, 0.02, 300), (12, 300, 0.012, 37), (6, 75, 0.02, 75)])
+def test_many_vector_blocks_without_a_certificate(ctx, n, B, T, count):
+    # Two weights a step: several listed blocks per cluster in either direction, beside the others.
+    rng = np.random.default_rng(900 + B)
+    listed = np.sort(rng.permutation(B)[:count])
+    W, _, g = _planted(n, B, listed, seed=901, V=2)
+    c = rng.standard_normal((1 << 16, 2)).astype(np.float32)
+    others = np.setdiff1d(np.arange(B), listed)
+    pick = np.unique(np.concatenate([listed[[0, count // 2, -1]], others[[0, -1]] if len(others) else []]).astype(int))
+    z = np.zeros_like(g); z[pick] = g[pick]
+    soft, logZ, gW, gc, kernels, linear = _forced(ctx, W, c, z, 2, T, V=2)
+    assert linear == B - count and kernels == [["fwd_vec_lin", "fwd_vec2"], ["bwd_vec_lin", "bwd_vec4"]]
+    rf = oracle.soft_quantize_vec(W[pick], c, 16, 4, 2, T)
+    rb = oracle.backward_vec(W[pick], c, g[pick], 16, 4, 2, T)
+    assert parity.rel_inf(soft[pick], rf["soft"]) <= parity.SOFT_TOL
+    np.testing.assert_allclose(logZ[pick], rf["logZ"], rtol=1e-5, atol=1e-3)
+    assert _grad_err(gW[pick], rb["grad_W"]) <= parity.GRAD_TOL
+    assert _grad_err(gc, np.asarray(rb["grad_codebook"]).reshape(gc.shape)) <= parity.GRAD_TOL
+
+
+@pytest.mark.parametrize("k,n,B,T", [(2, 1, 70, 0.5), (2, 2, 70, 0.02), (2, 3, 150, 0.3), (2, 40, 149, 0.02), (2, 61, 70, 0.02), (2, 256, 70, 0.012), (2, 255, 35, 0.1),
+                                     (3, 1, 2, 0.5), (3, 41, 3, 0.02), (3, 256, 3, 0.012)])
+def test_linear_messages_tried_at_any_temperature(ctx, k, n, B, T):
+    # messages = 2: the chunked kernels themselves, cold and warm, shortest and full blocks, weights outside the table, and one block of
+    # jumps between the table's ends that has no certificate where the trellis is cold.  Against the oracle, with both domains seen to run.
+    W, c, g = _rand(n, 16, B, seed=1000 + n + k)
+    W[B - 1, n // 2] = 6.0
+    jump = n >= 8 and T < 0.05
+    if jump:
+        W[1] = 0.3
+        W[1, 2:8] = [5, -5, 5, -5, 5, -5]
+    pick = np.unique([0, 1, B // 2, B - 1])
+    z = np.zeros_like(g); z[pick] = g[pick]
+    soft, logZ, gW, gc, kernels, linear = _forced(ctx, W, c, z, k, T)
+    assert kernels[0][0] == "fwd_lin" and kernels[1][0] == ("bwd_lin" if k == 2 else "bwd_split")
+    assert 0.85 * B - 1 <= linear <= B - jump
+    ref_f, ref_b = oracle.soft_quantize(W[pick], c, 16, k, T), oracle.backward(W[pick], c, g[pick], 16, k, T)
+    parity.assert_forward_backward({"soft": soft[pick], "logZ": logZ[pick], "grad_W": gW[pick], "grad_codebook": gc}, ref_f, ref_b, f"k={k} n={n} B={B} T={T}")
+
+
+@pytest.mark.parametrize("Lb,n,B,T", [(8, 33, 130, 0.02), (9, 40, 7, 0.02), (10, 64, 3, 0.02), (10, 40, 900, 0.0145), (11, 30, 9, 0.02), (12, 70, 5, 0.015), (13, 30, 600, 0.02),
+                                      (14, 40, 150, 0.02), (15, 24, 2, 0.02), (16, 30, 31, 0.02)])
+def test_register_kernels_fall_back_in_place(ctx, Lb, n, B, T):
+    # messages = 2: most blocks keep their linear messages; block 1 jumps between the table's ends for a while, has no certificate, and is run
+    # in the log domain by the same thread block, between blocks that are not.
+    W, c, g = _rand(n, Lb, B, seed=1100 + Lb + n)
+    W *= 0.7
+    W[1] = 0.3
+    W[1, 2:10] = [5, -5, 5, -5, 5, -5, 5, -5]
+    pick = np.arange(B) if B <= 200 else np.unique(np.linspace(0, B - 1, 40).astype(int)).clip(1)
+    pick = np.unique(np.append(pick, 1))
+    z = np.zeros_like(g); z[pick] = g[pick]
+    soft, logZ, gW, gc, kernels, linear = _forced(ctx, W, c, z, 2, T)
+    assert kernels == [["fwd_reg"], ["bwd_reg"]]
+    assert 0.9 * B - 1 <= linear <= B - 1
+    ref_f, ref_b = oracle.soft_quantize(W[pick], c, Lb, 2, T), oracle.backward(W[pick], c, g[pick], Lb, 2, T)
+    parity.assert_forward_backward({"soft": soft[pick], "logZ": logZ[pick], "grad_W": gW[pick], "grad_codebook": gc}, ref_f, ref_b, f"Lb={Lb} n={n} B={B} T={T}")
+
+
+@pytest.mark.parametrize("Lb,k,n,B,T,want_gc,options,forward,backward", [
+    (11, 2, 9, 1800, 0.02, True, {"messages": 1}, "fwd_warp", "bwd_warp"),
+    (11, 2, 9, 1800, 0.02, False, {"messages": 1}, "fwd_warp", "bwd_warp"),
+    (12, 2, 9, 1800, 0.02, True, {"messages": 1}, "fwd_warp", "bwd_warp2"),
+    (12, 2, 9, 1800, 0.02, True, {"messages": 1, "bwd_variant": 1}, "fwd_warp", "bwd_warp"),
+    (12, 2, 9, 1800, 0.02, False, {"messages": 1}, "fwd_warp", "bwd_warp"),
+    (13, 2, 9, 900, 0.02, True, {"messages": 1}, "fwd_warp", "bwd_warp2"),
+    (13, 2, 9, 900, 0.02, True, {"messages": 1, "bwd_variant": 1}, "fwd_warp", "bwd_warp"),
+    (13, 2, 9, 900, 0.02, False, {"messages": 1}, "fwd_warp", "bwd_warp"),
+    (16, 2, 1, 60, 0.02, False, {"messages": 1}, "fwd_solo", "bwd_solo"),
+    (16, 2, 37, 60, 0.02, False, {"messages": 1}, "fwd_solo", "bwd_solo"),
+    (16, 2, 9, 160, 0.02, False, {"messages": 1, "max_ctas": 50}, "fwd_solo", "bwd_solo"),
+    (16, 2, 9, 160, 0.02, True, {"messages": 1}, "fwd_solo", "bwd_split"),
+    (16, 2, 9, 60, 0.02, True, {"messages": 1, "bwd_variant": 2}, "fwd_solo", "bwd_duo"),
+    (16, 2, 9, 60, 0.02, True, {"messages": 1, "bwd_variant": 3}, "fwd_solo", "bwd_skew"),
+    (16, 2, 9, 60, 0.02, True, {"fwd_variant": 1, "bwd_variant": 1}, "fwd_cluster", "bwd_cluster"),
+    (16, 3, 9, 60, 0.02, True, {"bwd_variant": 1}, "fwd_solo", "bwd_cluster"),
+    (16, 3, 9, 160, 0.02, True, {}, "fwd_solo", "bwd_split"),
+])
+def test_every_log_domain_kernel_is_reached(ctx, Lb, k, n, B, T, want_gc, options, forward, backward):
+    # Register and linear kernels have taken many shapes over; what still stands behind them is run here, seen to be run, and compared.
+    import torch
+    W, c, g = _rand(n, Lb, B, seed=1200 + Lb + n)
+    W[1, n // 2] = 6.0
+    pick = np.unique(np.linspace(0, B - 1, 12).astype(int))
+    pick[1] = 1
+    z = np.zeros_like(g); z[pick] = g[pick]
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in (W, c, z))
+    try:
+        for name, value in options.items():
+            ctx.set_option(name, value)
+        soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, k, n, T)
+        assert ctx.last_kernels() == [forward]
+        gW, gc = ctx.bcjr_backward(gd, want_grad_codebook=want_gc)
+        assert ctx.last_kernels() == [backward]
+        st = ctx.sync_status()
+        assert st.device_status == 0 and st.max_posterior_defect < 1e-3
+    finally:
+        for name in options:
+            ctx.set_option(name, 0)
+    ref_f, ref_b = oracle.soft_quantize(W[pick], c, Lb, k, T), oracle.backward(W[pick], c, g[pick], Lb, k, T)
+    parity.assert_forward_backward({"soft": soft.cpu().numpy()[pick], "logZ": logZ.cpu().numpy()[pick]}, ref_f, what=f"{forward} Lb={Lb}")
+    assert parity.rel_inf(gW.cpu().numpy()[pick], ref_b["grad_W"]) <= parity.GRAD_TOL
+    if want_gc:
+        assert parity.rel_inf(gc.cpu().numpy(), ref_b["grad_codebook"]) <= parity.GRAD_TOL
