@@ -59,11 +59,16 @@ typedef struct {
  *                         four-CTA register kernel (about 1.7x slower per weight), and anything longer
  *                         the generic one-CTA kernels (more than 10x slower per weight at Lb = 16).
  *                         k = 2: few blocks (up to about 30, n <= 1024) run one butterfly per thread, a block on eight SMs.
+ *                         A table that does not start on 16 bytes: Viterbi, and what n > 1024 would run, generic.
  *   Lb = 8..15, k = 2:    one butterfly (16 states) per thread, table and gradient accumulators in registers, a block on a warp
  *                         or CTA (Lb <= 13) or a cluster of two or four CTAs (n <= 1024).
- *   Lb = 11..13, k = 2:   longer blocks, and many blocks at low temperatures: one warp per block, sixteen (forward) or eight
+ *   Lb = 11..13, k = 2:   longer blocks, and many blocks at low temperatures or with weights that float32 messages cannot be expected
+ *                         to carry: one warp per block, sixteen (forward) or eight
  *                         (backward) blocks per SM at Lb = 12, table in tensor memory.  The backward call with grad_codebook at
  *                         Lb = 12, 13 gives a block to two warps ("bwd_variant" = 1: one warp).
+ *   Lb = 10..13, k = 2:   viterbi_hard in float32 with one butterfly per thread where the path can be proved (n <= 1024).
+ *   Lb = 4..10, other k, and k = 2 up to Lb = 7: one warp per block, or up to 32 blocks a warp (n <= 1024; at Lb = 10, k = 1 with more
+ *                         blocks than SMs).
  *   V = 2, Lb = 16, k = 2: forward on clusters of two CTAs (n <= 2048), backward on clusters of four (table and
  *                         gradient accumulators are 1 MB of tensor memory; n <= 1024); longer blocks and every
  *                         other V = 2 shape run the one-CTA vector kernels.
@@ -120,15 +125,14 @@ bcjr_status bcjr_set_option(bcjr_ctx *ctx, const char *name, int64_t value);
 
 /*
  * Soft codeword (Eq. 3 / Eq. 7): soft[t] = sum_s codebook[s] * p_T(s_t = s | w), with the
- * marginals from the temperature-T forward-backward recursions of Eq. 5-6 carried in the
- * log domain.
+ * marginals from the temperature-T forward-backward recursions of Eq. 5-6 (option "messages":
+ * what they carry).
  *   W         device in   [num_blocks * n] float32
  *   codebook  device in   [2^Lb] float32, or NULL for the computed Gaussian emission of Section 3.1,
- *                         codebook[s] = Phi^-1((s + 1/2) / 2^Lb) (what bcjr_gaussian_codebook writes out): at
- *                         Lb = 16, k = 2 or 3 the kernels then evaluate the entries themselves while filling
- *                         their tensor-memory slices and no table is read; other shapes use a table the
- *                         context keeps.  viterbi_hard and bcjr_ste_forward take NULL the same way.
- *   soft      device out  [num_blocks * n] float32
+ *                         codebook[s] = Phi^-1((s + 1/2) / 2^Lb) (what bcjr_gaussian_codebook writes out): the
+ *                         kernels read a table that the context keeps and writes at every call.  viterbi_hard and
+ *                         bcjr_ste_forward take NULL the same way.
+ *   soft      device out  [num_blocks * n] float32; may be W where no backward call follows
  *   logZ      device out  [num_blocks] float32, natural log of Z_T per block (sum over legal
  *                         paths of exp(-E/T), no prior constant); may be NULL
  * Saves, for bcjr_backward: the W and codebook POINTERS (borrowed: keep them valid and

@@ -119,10 +119,13 @@ def path_bytes(Lb: int, k: int, n: int) -> int:
 
 # The calls of a small layer are bound by the host (four of them for a rotation of 256 x 2048 weights), so the marshalling is kept
 # short: plain integers for pointers (the argtypes convert them), no Stream object where the current stream is meant.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # (not public: the Stream object where it is missing)
+
+
 def _stream_ptr(stream):
-    if stream is not None:
-        return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if stream is None and _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def _dev(t, dtype, numel=None, name="tensor"):
