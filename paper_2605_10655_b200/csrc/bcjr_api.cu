@@ -1134,7 +1134,7 @@ bcjr_status launch_bwd_warp_any(bcjr_ctx *ctx, BwdParams p, float *gc, cudaStrea
 
 // One butterfly per thread (bcjr_reg.cuh), k = 2 and n <= 1024: calls at Lb = 8 .. 15, and calls of few blocks at
 // Lb = 16 -- forward as many as are resident (0.46 ms for 8 blocks, 0.66 for 16, 0.73 for 32; fwd_lin_kernel takes 1.40 for up
-// to 148), and their backward calls (0.59 ms for 8, 1.17 for 16; 1.6 ms for up to 148): the register kernels take their offsets from
+// to 148), and their backward calls (0.54 ms for 8, 1.06 for 16, 1.57 for 31; the chunked kernels 1.6 for up to 148): the register kernels take their offsets from
 // the step before, the chunked ones from the step itself, and a certificate holds for the gauge it was made in.
 // With log messages (a cold call) the warp-per-block kernels hold more blocks at Lb = 11 .. 13 and win from three quarters of
 // their residency on: 2^12 states, forward 4.23 against 3.68 ms for 4096 blocks, 1.24 against 1.85 for 1000; backward 6.28

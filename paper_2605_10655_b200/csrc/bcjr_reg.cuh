@@ -9,8 +9,8 @@
 //   * Throughput at mid sizes: several CTAs share an SM and fill each other's barriers.
 // Messages are linear where float32's range allows, with the certificate of bcjr_lin.cuh; a block without one, or a call at a
 // temperature where most would fail, takes the log-domain form of the same sweeps, in the same kernel.
-// Forward + backward at T = 0.1, n = 256: 16 blocks of 2^16 states 1.40 + 1.60 -> 0.66 + 1.15 ms, one block of them
-// 1.37 + 1.60 -> 0.47 + 0.58; 4096 blocks of 2^12 states 3.68 + 5.80 (a warp or two per block) -> 3.31 + 5.13, 16 of them 1.85 +
+// Forward + backward at T = 0.1, n = 256: 16 blocks of 2^16 states 1.40 + 1.60 -> 0.66 + 1.06 ms, one block of them
+// 1.37 + 1.60 -> 0.47 + 0.54; 4096 blocks of 2^12 states 3.68 + 5.80 (a warp or two per block) -> 3.18 + 5.24, 16 of them 1.85 +
 // 1.45 -> 0.24 + 0.27.
 //
 // Pairs.  All state pairs are (j, j+1) for one l (= b): the table is loaded once per launch, and the alpha sweep's inputs
