@@ -11,7 +11,7 @@ from pathlib import Path
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libbcjr_b200.so"
-SOURCES = [CSRC / "bcjr_api.cu", CSRC / "bcjr_reg.cu", CSRC / "bcjr_small.cu", CSRC / "bcjr_static.cu", CSRC / "bcjr_microbench.cu"]
+SOURCES = [CSRC / "bcjr_api.cu", CSRC / "bcjr_reg.cu", CSRC / "bcjr_meet.cu", CSRC / "bcjr_meet_bwd.cu", CSRC / "bcjr_small.cu", CSRC / "bcjr_static.cu", CSRC / "bcjr_microbench.cu"]
 HEADERS = sorted(CSRC.glob("*.cuh")) + sorted(CSRC.glob("*.h")) + sorted((PKG.parent / "include").glob("*.h"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

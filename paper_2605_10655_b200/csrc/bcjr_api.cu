@@ -25,6 +25,7 @@
 #include "bcjr_alpha.cuh"
 #include "bcjr_lin_bwd.cuh"
 #include "bcjr_reg.h"
+#include "bcjr_meet.h"
 #include "bcjr_small.h"
 #include "bcjr_bsolo.cuh"
 #include "bcjr_ckpt.cuh"
@@ -59,6 +60,9 @@ struct bcjr_ctx {
     int judged_max = 0;
     struct { int n = 0, count = 0; } vit_res[17];      // the same for viterbi_reg_kernel (CTAs)
     struct { int n = 0, count = 0; } reg_res[2][17];   // resident clusters of those kernels by call kind and Lb, for the n asked last
+    int64_t meet_from = -1;    // blocks from here on ran the two-ended kernels (bcjr_meet.h): first those of the second form, then of the
+    int64_t meet_count[MEET_FORMS] = {};   // first; -1: none did
+    struct { int n = 0, count = 0; } meet_res[MEET_FORMS][2][17];   // sides in flight of those, for the n asked last
     bool fwd_lin = false;      // lin_flag and lin_list belong to the saved forward call
     bool cb_computed = false;  // the call in flight (and the saved forward state) uses the computed Gaussian emission
     const float *W = nullptr, *cb = nullptr;
@@ -1210,6 +1214,199 @@ bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     return ctx->fwd_judged ? launch_bwd_warp_any(ctx, p, grad_codebook, st) : BCJR_OK;
 }
 
+// Few blocks, k = 2: the register kernels from both ends of a block (bcjr_meet.cuh).
+int meet_sides(bcjr_ctx *ctx, int form, int Lb, int n)
+{
+    int least = 0;
+    for (int bwd = 0; bwd < 2; ++bwd) {
+        auto &r = ctx->meet_res[form][bwd][Lb];
+        if (r.n != n) { r.count = bwd ? meet_bwd_resident(Lb, form, n, ctx->num_sms) : meet_fwd_resident(Lb, form, n, ctx->num_sms); r.n = n; }
+        if (bwd == 0 || r.count < least) least = r.count;
+    }
+    return least;
+}
+// Which form takes how many of B blocks (count), or false where the one-ended kernels are as good.  Both calls of 256 weights at T = 0.3, one-ended
+// -> two-ended:
+//   * 2^8 states: always; 1 .. 64 blocks 259 -> 144 us, 600 363 -> 243, 8000 2282 -> 1704.  2^9: 16 265 -> 167, 600 349 -> 302, 1200 482 -> 508.
+//   * 2^10, 2^11: a block an SM, 148 378 -> 224 and 394 -> 280 us; 300 464 -> 480 and 540 -> 603.
+//   * 2^12: an SM per side while there are that many, 64 482 -> 331 (on one SM 396); then on one, 148 484 -> 404, 300 946 -> 1081.
+//   * 2^13 .. 2^15: as many as are in flight at once, 74 blocks 716 -> 439, 37 1062 -> 611, 16 1042 -> 620; 50 of 2^14 1080 -> 1181.
+//   * 2^16: clusters of eight while all sides are in flight, 7 blocks 1019 -> 595.  Clusters of four up to three waves of them, the last blocks on
+//     clusters of eight if those can take them: 8 1019 -> 926, 16 1754 -> 937, 33 2360 -> 1846, 40 2932 -> 2442, 49 2933 -> 2745.  Between,
+//     where the one-ended kernels need two waves as well, they keep the call (24 blocks 1779 us against 1814, 17 1754 against 1533).
+// With log messages the same (T = 0.015: 16 blocks of 2^16 2053 -> 1094, 49 3832 -> 3214, 148 of 2^12 558 -> 477).
+// last: the last blocks of a call, instead of a wave of the chunked kernels that they do not fill (both calls, 149 blocks 6626 -> 4418 us, 171
+// 6645 -> 5374, 197 6805 -> 6608, 600 17846 -> 15983).
+bool meet_count(bcjr_ctx *ctx, int Lb, int n, int64_t B, bool last, int64_t count[MEET_FORMS])
+{
+    count[0] = count[1] = 0;
+    const int s0 = meet_sides(ctx, 0, Lb, n), s1 = meet_sides(ctx, 1, Lb, n);
+    if (s0 == 0) return false;
+    if (Lb <= 11) { count[0] = B; return Lb == 8 || B <= (Lb == 9 ? 4 : 1) * (int64_t)ctx->num_sms; }
+    if (Lb == 12 && 2 * B <= s1) { count[1] = B; return true; }
+    if (2 * B <= s0) { count[0] = B; return true; }
+    if (Lb < 16 || s1 == 0) return false;
+    for (int w = 1; w <= 3; ++w) {
+        const int64_t full = (int64_t)(w - 1) * s1 / 2;
+        if (w == 2 && !last && B <= 2 * reg_resident_cached(ctx, Lb, n, true)) return false;
+        if (w > 1 && 2 * (B - full) <= s0) { count[1] = full; count[0] = B - full; return true; }
+        if (2 * B <= (int64_t)w * s1) { count[1] = B; return true; }
+    }
+    return false;
+}
+// Where the two-ended kernels take over: the whole call (*from = 0), its last blocks, or none (false).
+bool meet_wanted(bcjr_ctx *ctx, const FwdParams &p, int k, int64_t *from, int64_t count[MEET_FORMS])
+{
+    if (k != 2 || p.Lb < 8 || ctx->opt_path == 1 || (ctx->opt_path == 2 && p.Lb != 16) || ctx->opt_fwd_variant != 0) return false;
+    if (ctx->opt_hist_every != 1 && p.Lb == 16 && p.n <= CkptCfg<2>::MAX_N) return false;
+    *from = 0;
+    const bool few = p.Lb < 16 || p.B <= reg_resident_cached(ctx, p.Lb, p.n, false);
+    if (!few && ctx->opt_messages != 0) return false;            // (the option names the chunked kernels' messages)
+    if (meet_count(ctx, p.Lb, p.n, p.B, false, count)) return true;
+    if (p.Lb < 16 || p.B <= ctx->num_sms || p.n > SkewCfg::MAX_N || ctx->opt_max_ctas != 0) return false;
+    const int64_t left = p.B % ctx->num_sms;
+    *from = p.B - left;
+    return left > 0 && meet_count(ctx, p.Lb, p.n, left, true, count);
+}
+// Option max_ctas: the split form in launches of as many blocks as that leaves room for, the CTA form on fewer CTAs.
+int64_t meet_chunk(const bcjr_ctx *ctx, const MeetPlan &plan, int64_t B)
+{
+    if (!plan.split || ctx->opt_max_ctas == 0) return B;
+    const int64_t fit = ctx->opt_max_ctas / (plan.grid / B);
+    return fit < 1 ? 1 : fit < B ? fit : B;
+}
+MeetPlan meet_part(const bcjr_ctx *ctx, const MeetPlan &plan, int64_t B, int64_t nb)
+{
+    MeetPlan part = plan;
+    if (plan.split) part.grid = (int)(plan.grid / B * nb);
+    else if (ctx->opt_max_ctas > 0 && part.grid > ctx->opt_max_ctas) { part.grid = ctx->opt_max_ctas; part.parts = 2 * part.grid; }
+    return part;
+}
+// blocks of p by the two-ended kernels; *ran = false where their scratch cannot be had
+bcjr_status launch_fwd_meet(bcjr_ctx *ctx, FwdParams p, int form, bool *ran, cudaStream_t st)
+{
+    const MeetPlan plan = meet_fwd_plan(p.Lb, form, p.n, p.B, meet_sides(ctx, form, p.Lb, p.n));
+    const bool lin = lin_wanted(ctx, p.Lb, p.lam2, p.B);
+    RegPlan behind;
+    size_t hist = plan.hist_floats;
+    if (plan.split && lin) {
+        behind = reg_plan(p.Lb, p.n, p.B, false, reg_resident_cached(ctx, p.Lb, p.n, false), ctx->opt_max_ctas);
+        if (behind.hist_floats > hist) hist = behind.hist_floats;
+    }
+    bcjr_status rc = ensure_or_do_without(ctx, ctx->hist, hist * 4, ran);
+    if (rc || !*ran) return rc;
+    if ((rc = ensure(ctx, ctx->stepO, plan.aux_ints * 4))) return rc;
+    p.hist = (float *)ctx->hist.ptr;
+    p.lin_x = lin ? 0 : -1;                                      // (any exponent: the kernels have their own)
+    p.demand = lin_demand_limit(ctx, p.Lb, 2, 1, p.lam2, true, p.B < 6 * (int64_t)ctx->num_sms);
+    p.window = (p.Lb + 1) / 2;
+    const int64_t chunk = meet_chunk(ctx, plan, p.B);
+    for (int64_t b0 = 0; b0 < p.B; b0 += chunk) {
+        FwdParams q = p;
+        q.B = p.B - b0 < chunk ? p.B - b0 : chunk;
+        q.W = p.W + b0 * p.n; q.soft = p.soft + b0 * p.n;
+        if (p.soft_copy) q.soft_copy = p.soft_copy + b0 * p.n;
+        if (p.logZ) q.logZ = p.logZ + b0;
+        if (p.blk_defect) q.blk_defect = p.blk_defect + b0;
+        q.lin_flag = p.lin_flag + b0;
+        CU(meet_forward(q, form, meet_part(ctx, plan, p.B, q.B), (int *)ctx->stepO.ptr, st));
+        ctx->launches += plan.split ? 2 : 1;
+    }
+    note(ctx, "fwd_reg");
+    if (plan.split && lin) {
+        p.lin_x = -1;
+        p.only_flagged = true;
+        CU(reg_forward(p, behind, st));
+        ctx->launches += 1;
+    }
+    return BCJR_OK;
+}
+// Blocks from `from` on, count[] of them by form.  Where scratch is short the call ends with *ran = false and has run none of them or some.
+bcjr_status launch_fwd_meets(bcjr_ctx *ctx, const FwdParams &p, int64_t from, const int64_t count[MEET_FORMS], bool *ran, cudaStream_t st)
+{
+    bcjr_status rc = lin_buffers(ctx, from + count[0] + count[1]);
+    if (rc) return rc;
+    *ran = true;
+    int64_t b0 = from;
+    // the split form writes one side's part of soft before the other side has its certificate: over the weights, by way of the copy
+    const bool in_place = p.Lb >= 12 && p.soft_copy && p.soft < p.W + p.B * p.n && p.W < p.soft + p.B * p.n;
+    for (int form = MEET_FORMS - 1; form >= 0 && *ran; --form) {
+        if (count[form] == 0) continue;
+        FwdParams q = p;
+        q.B = count[form];
+        q.W = p.W + b0 * p.n; q.soft = p.soft + b0 * p.n;
+        if (p.soft_copy) q.soft_copy = p.soft_copy + b0 * p.n;
+        if (in_place) q.soft = q.soft_copy;
+        if (p.logZ) q.logZ = p.logZ + b0;
+        if (p.blk_defect) q.blk_defect = p.blk_defect + b0;
+        q.lin_flag = (uint8_t *)ctx->lin_flag.ptr + b0;
+        if ((rc = launch_fwd_meet(ctx, q, form, ran, st))) return rc;
+        b0 += count[form];
+    }
+    if (*ran) {
+        if (in_place) CU(cudaMemcpyAsync(p.soft + from * p.n, p.soft_copy + from * p.n, (size_t)(b0 - from) * p.n * 4, cudaMemcpyDeviceToDevice, st));
+        ctx->meet_from = from;
+        for (int f = 0; f < MEET_FORMS; ++f) ctx->meet_count[f] = count[f];
+    }
+    return BCJR_OK;
+}
+// The blocks behind ctx->meet_from; grad_codebook is added to where others have left theirs in it.
+bcjr_status launch_bwd_meets(bcjr_ctx *ctx, const BwdParams &p, float *grad_codebook, cudaStream_t st)
+{
+    const int S = 1 << p.Lb;
+    int64_t b0 = ctx->meet_from;
+    for (int form = MEET_FORMS - 1; form >= 0; --form) {
+        const int64_t B = ctx->meet_count[form];
+        if (B == 0) continue;
+        BwdParams q = p;
+        q.B = B;
+        q.W = p.W + b0 * p.n; q.g = p.g + b0 * p.n; q.soft = p.soft + b0 * p.n; q.gW = p.gW + b0 * p.n;
+        q.lin_flag = (const uint8_t *)ctx->lin_flag.ptr + b0;
+        q.lin_x = ctx->opt_messages == 1 ? -1 : 0;               // (the flags say which blocks)
+        const MeetPlan plan = meet_bwd_plan(p.Lb, form, p.n, B, meet_sides(ctx, form, p.Lb, p.n));
+        bool got = false;
+        bcjr_status rc = ensure_or_do_without(ctx, ctx->hist, plan.hist_floats * 4, &got);
+        if (rc) return rc;
+        int parts = plan.parts;
+        RegPlan other;
+        if (!got) {                                              // log messages need no gauge in common with the forward call
+            other = reg_plan(p.Lb, p.n, B, true, reg_resident_cached(ctx, p.Lb, p.n, true), ctx->opt_max_ctas);
+            parts = other.parts;
+            if ((rc = ensure(ctx, ctx->hist, other.hist_floats * 4))) return rc;
+        }
+        if ((rc = ensure(ctx, ctx->stepO, plan.aux_ints * 4))) return rc;
+        if (grad_codebook && (rc = ensure(ctx, ctx->gc_part, (size_t)parts * S * 4))) return rc;
+        q.hist = (float *)ctx->hist.ptr;
+        q.gc_part = (float *)ctx->gc_part.ptr;
+        if (got) {
+            const int64_t chunk = meet_chunk(ctx, plan, B);
+            for (int64_t c0 = 0; c0 < B; c0 += chunk) {
+                BwdParams c = q;
+                c.B = B - c0 < chunk ? B - c0 : chunk;
+                c.W = q.W + c0 * p.n; c.g = q.g + c0 * p.n; c.soft = q.soft + c0 * p.n; c.gW = q.gW + c0 * p.n;
+                c.lin_flag = q.lin_flag + c0;
+                c.gc_part = q.gc_part + (size_t)2 * c0 * S;
+                const MeetPlan part = meet_part(ctx, plan, B, c.B);
+                CU(meet_backward(c, form, part, (int *)ctx->stepO.ptr, grad_codebook != nullptr, st));
+                ctx->launches += plan.split ? 2 : 1;
+                parts = part.parts;
+            }
+        } else {
+            q.lin_x = -1;
+            CU(reg_backward(q, other, grad_codebook != nullptr, st));
+            ctx->launches += 1;
+        }
+        note(ctx, "bwd_reg");
+        if (grad_codebook) {
+            reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(q.gc_part, parts, S, grad_codebook, nullptr, 0, false, b0 > 0);
+            ctx->launches += 1;
+            CU(cudaGetLastError());
+        }
+        b0 += B;
+    }
+    return BCJR_OK;
+}
+
 // One warp per block, or for several (bcjr_small.cuh): 2^4 .. 2^10 states where bcjr_reg.cuh has no kernel.  At 2^10 states and k = 1 a
 // lane's sixteen groups take longer than a CTA's barrier while there is an SM for every block: both calls 0.72 ms in the generic kernels
 // against 0.95 for 2 blocks of 256 weights, 1.47 against 1.00 for 200.
@@ -1347,6 +1544,98 @@ cudaError_t launch_fwht_cols(int b, float *W, const RhtSigns &s, int lm, int o, 
         return cudaGetLastError();
     }
 }
+// Forward call of p.B blocks by whichever kernels take them, the two-ended ones aside.
+bcjr_status forward_blocks(bcjr_ctx *ctx, const FwdParams &p, int k, cudaStream_t st)
+{
+    const int Lb = p.Lb, n = p.n;
+    const int64_t num_blocks = p.B;
+    const float *codebook = p.cb;
+    bcjr_status rc = BCJR_OK;
+    bool use_reg = false;
+#ifndef BCJR_NO_CLUSTER
+    use_reg = reg_wanted(ctx, Lb, k, n, num_blocks, p.lam2, false);           // (these kernels find c_lo, c_hi themselves)
+#endif
+    bool range = !use_reg;
+#ifndef BCJR_NO_CLUSTER
+    range = range || reg_judged(ctx, Lb, num_blocks, p.lam2);                 // (nor do they when they leave the call to the others)
+#endif
+    if (range) {
+        table_range_kernel<<<1, 1024, 0, st>>>(codebook, 1 << Lb, ctx->diag); // c_lo, c_hi for step_energy, this call's and its backward's
+        ctx->launches += 1;
+    }
+    bool use_cluster = false;
+#ifndef BCJR_NO_CLUSTER
+    use_cluster = ctx->opt_path != 1 && cluster_supported(Lb, k);
+    if (ctx->opt_path == 2 && !use_cluster) return BCJR_EUNSUPPORTED;
+    if (use_reg) {
+        rc = launch_fwd_reg(ctx, p, st);
+    } else if (use_cluster) {
+        rc = launch_fwd_cluster(ctx, p, k, st);
+        if (rc == BCJR_EUNSUPPORTED && ctx->opt_path != 2) { use_cluster = false; rc = BCJR_OK; }   // e.g. n too long
+    }
+    bool use_warp = !use_cluster && ctx->opt_path == 0 && warp_supported(Lb, k);
+    if (use_warp && !use_reg) rc = launch_fwd_warp_any(ctx, p, st);
+#else
+    if (ctx->opt_path == 2) return BCJR_EUNSUPPORTED;
+    const bool use_warp = false;
+#endif
+    bool use_small = false;
+#ifndef BCJR_NO_CLUSTER
+    use_small = !use_cluster && !use_warp && !use_reg && small_wanted(ctx, Lb, k, n, num_blocks);
+    if (use_small && (rc = launch_fwd_small(ctx, p, k, st)) == BCJR_EUNSUPPORTED) { use_small = false; rc = BCJR_OK; }
+#endif
+    if (!use_cluster && !use_warp && !use_reg && !use_small) {
+        switch (k) {
+            case 1: rc = launch_fwd_generic<1>(ctx, p, st); break;
+            case 2: rc = launch_fwd_generic<2>(ctx, p, st); break;
+            case 3: rc = launch_fwd_generic<3>(ctx, p, st); break;
+            default: rc = launch_fwd_generic<4>(ctx, p, st); break;
+        }
+    }
+    if (rc) return rc;
+    ctx->last_path = use_cluster ? 1 : use_warp ? 2 : 0;
+    return BCJR_OK;
+}
+
+// Backward call of the first p.B blocks of the saved forward call.
+bcjr_status backward_blocks(bcjr_ctx *ctx, const BwdParams &p, float *grad_codebook, cudaStream_t st)
+{
+    bcjr_status rc = BCJR_OK;
+    bool use_cluster = false;
+#ifndef BCJR_NO_CLUSTER
+    use_cluster = ctx->opt_path != 1 && cluster_supported(ctx->Lb, ctx->k);
+    if (ctx->opt_path == 2 && !use_cluster) return BCJR_EUNSUPPORTED;
+    const bool use_reg = ctx->fwd_reg && ctx->opt_bwd_variant == 0 && reg_wanted(ctx, ctx->Lb, ctx->k, ctx->n, p.B, p.lam2, true);
+    if (use_reg) {
+        rc = launch_bwd_reg(ctx, p, grad_codebook, st);
+    } else if (use_cluster) {
+        rc = launch_bwd_cluster(ctx, p, ctx->k, grad_codebook, st);
+        if (rc == BCJR_EUNSUPPORTED && ctx->opt_path != 2) { use_cluster = false; rc = BCJR_OK; }
+    }
+    const bool use_warp = !use_cluster && ctx->opt_path == 0 && warp_supported(ctx->Lb, ctx->k);
+    if (use_warp && !use_reg) rc = launch_bwd_warp_any(ctx, p, grad_codebook, st);
+#else
+    if (ctx->opt_path == 2) return BCJR_EUNSUPPORTED;
+    const bool use_warp = false, use_reg = false;
+#endif
+    bool use_small = false;
+#ifndef BCJR_NO_CLUSTER
+    use_small = !use_cluster && !use_warp && !use_reg && small_wanted(ctx, ctx->Lb, ctx->k, ctx->n, p.B);
+    if (use_small && (rc = launch_bwd_small(ctx, p, ctx->k, grad_codebook, st)) == BCJR_EUNSUPPORTED) { use_small = false; rc = BCJR_OK; }
+#endif
+    if (!use_cluster && !use_warp && !use_reg && !use_small) {
+        switch (ctx->k) {
+            case 1: rc = launch_bwd_generic<1>(ctx, p, grad_codebook, st); break;
+            case 2: rc = launch_bwd_generic<2>(ctx, p, grad_codebook, st); break;
+            case 3: rc = launch_bwd_generic<3>(ctx, p, grad_codebook, st); break;
+            default: rc = launch_bwd_generic<4>(ctx, p, grad_codebook, st); break;
+        }
+    }
+    if (rc) return rc;
+    ctx->last_path = use_cluster ? 1 : use_warp ? 2 : 0;
+    return BCJR_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1462,6 +1751,7 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = ctx->fwd_judged = false;
+    ctx->meet_from = -1;
     ctx->num_ran = 0;
     ctx->cb_computed = codebook == nullptr;
     if (num_blocks == 0) {
@@ -1476,18 +1766,6 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
     p.W = W; p.cb = codebook; p.soft = soft; p.soft_copy = (float *)ctx->soft_copy.ptr; p.logZ = logZ;
     p.diag = ctx->diag; p.B = num_blocks; p.Lb = Lb; p.n = n;
     p.lam2 = (float)(1.4426950408889634 / (2.0 * (double)T));
-    bool use_reg = false;
-#ifndef BCJR_NO_CLUSTER
-    use_reg = reg_wanted(ctx, Lb, k, n, num_blocks, p.lam2, false);           // (these kernels find c_lo, c_hi themselves)
-#endif
-    bool range = !use_reg;
-#ifndef BCJR_NO_CLUSTER
-    range = range || reg_judged(ctx, Lb, num_blocks, p.lam2);                 // (nor do they when they leave the call to the others)
-#endif
-    if (range) {
-        table_range_kernel<<<1, 1024, 0, st>>>(codebook, 1 << Lb, ctx->diag); // c_lo, c_hi for step_energy, this call's and its backward's
-        ctx->launches += 1;
-    }
     ctx->defect_blocks = 0;
     if (ctx->opt_record_defect) {
         if ((rc = ensure(ctx, ctx->blk_defect, (size_t)num_blocks * 4))) return rc;
@@ -1495,37 +1773,22 @@ bcjr_status bcjr_soft_quantize(bcjr_ctx *ctx, const float *W, const float *codeb
         p.blk_defect = (float *)ctx->blk_defect.ptr;
         ctx->defect_blocks = num_blocks;
     }
-    bool use_cluster = false;
+    bool ran = false;
 #ifndef BCJR_NO_CLUSTER
-    use_cluster = ctx->opt_path != 1 && cluster_supported(Lb, k);
-    if (ctx->opt_path == 2 && !use_cluster) return BCJR_EUNSUPPORTED;
-    if (use_reg) {
-        rc = launch_fwd_reg(ctx, p, st);
-    } else if (use_cluster) {
-        rc = launch_fwd_cluster(ctx, p, k, st);
-        if (rc == BCJR_EUNSUPPORTED && ctx->opt_path != 2) { use_cluster = false; rc = BCJR_OK; }   // e.g. n too long
-    }
-    bool use_warp = !use_cluster && ctx->opt_path == 0 && warp_supported(Lb, k);
-    if (use_warp && !use_reg) rc = launch_fwd_warp_any(ctx, p, st);
-#else
-    if (ctx->opt_path == 2) return BCJR_EUNSUPPORTED;
-    const bool use_warp = false;
-#endif
-    bool use_small = false;
-#ifndef BCJR_NO_CLUSTER
-    use_small = !use_cluster && !use_warp && !use_reg && small_wanted(ctx, Lb, k, n, num_blocks);
-    if (use_small && (rc = launch_fwd_small(ctx, p, k, st)) == BCJR_EUNSUPPORTED) { use_small = false; rc = BCJR_OK; }
-#endif
-    if (!use_cluster && !use_warp && !use_reg && !use_small) {
-        switch (k) {
-            case 1: rc = launch_fwd_generic<1>(ctx, p, st); break;
-            case 2: rc = launch_fwd_generic<2>(ctx, p, st); break;
-            case 3: rc = launch_fwd_generic<3>(ctx, p, st); break;
-            default: rc = launch_fwd_generic<4>(ctx, p, st); break;
+    int64_t from = 0, count[MEET_FORMS] = {};
+    if (meet_wanted(ctx, p, k, &from, count)) {
+        if (from > 0) {                                            // the last blocks are left out here
+            if ((rc = lin_buffers(ctx, num_blocks))) return rc;
+            FwdParams q = p;
+            q.B = from;
+            if ((rc = forward_blocks(ctx, q, k, st))) return rc;
         }
+        if ((rc = launch_fwd_meets(ctx, p, from, count, &ran, st))) return rc;
+        if (!ran) ctx->fwd_lin = ctx->fwd_reg = ctx->fwd_judged = false;
+        ctx->last_path = Lb == 16 ? 1 : warp_supported(Lb, k) ? 2 : 0;
     }
-    if (rc) return rc;
-    ctx->last_path = use_cluster ? 1 : use_warp ? 2 : 0;
+#endif
+    if (!ran && (rc = forward_blocks(ctx, p, k, st))) return rc;
     ctx->W = W; ctx->cb = codebook; ctx->Lb = Lb; ctx->k = k; ctx->n = n; ctx->B = num_blocks; ctx->T = T;
     ctx->V = 1;
     ctx->have_fwd = true;
@@ -1573,39 +1836,22 @@ bcjr_status bcjr_backward(bcjr_ctx *ctx, const float *grad_soft, float *grad_W, 
         ctx->last_path = large ? 1 : 0;
         return BCJR_OK;
     }
-    bool use_cluster = false;
 #ifndef BCJR_NO_CLUSTER
-    use_cluster = ctx->opt_path != 1 && cluster_supported(ctx->Lb, ctx->k);
-    if (ctx->opt_path == 2 && !use_cluster) return BCJR_EUNSUPPORTED;
-    const bool use_reg = ctx->fwd_reg && ctx->opt_bwd_variant == 0 && reg_wanted(ctx, ctx->Lb, ctx->k, ctx->n, ctx->B, p.lam2, true);
-    if (use_reg) {
-        rc = launch_bwd_reg(ctx, p, grad_codebook, st);
-    } else if (use_cluster) {
-        rc = launch_bwd_cluster(ctx, p, ctx->k, grad_codebook, st);
-        if (rc == BCJR_EUNSUPPORTED && ctx->opt_path != 2) { use_cluster = false; rc = BCJR_OK; }
-    }
-    const bool use_warp = !use_cluster && ctx->opt_path == 0 && warp_supported(ctx->Lb, ctx->k);
-    if (use_warp && !use_reg) rc = launch_bwd_warp_any(ctx, p, grad_codebook, st);
-#else
-    if (ctx->opt_path == 2) return BCJR_EUNSUPPORTED;
-    const bool use_warp = false, use_reg = false;
-#endif
-    bool use_small = false;
-#ifndef BCJR_NO_CLUSTER
-    use_small = !use_cluster && !use_warp && !use_reg && small_wanted(ctx, ctx->Lb, ctx->k, ctx->n, ctx->B);
-    if (use_small && (rc = launch_bwd_small(ctx, p, ctx->k, grad_codebook, st)) == BCJR_EUNSUPPORTED) { use_small = false; rc = BCJR_OK; }
-#endif
-    if (!use_cluster && !use_warp && !use_reg && !use_small) {
-        switch (ctx->k) {
-            case 1: rc = launch_bwd_generic<1>(ctx, p, grad_codebook, st); break;
-            case 2: rc = launch_bwd_generic<2>(ctx, p, grad_codebook, st); break;
-            case 3: rc = launch_bwd_generic<3>(ctx, p, grad_codebook, st); break;
-            default: rc = launch_bwd_generic<4>(ctx, p, grad_codebook, st); break;
+    if (ctx->meet_from >= 0) {
+        if (ctx->opt_path == 2 && !cluster_supported(ctx->Lb, ctx->k)) return BCJR_EUNSUPPORTED;
+        if (ctx->opt_bwd_variant == 0 && ctx->opt_fwd_variant == 0 && ctx->opt_path != 1) {
+            if (ctx->meet_from > 0) {
+                BwdParams q = p;
+                q.B = ctx->meet_from;
+                if ((rc = backward_blocks(ctx, q, grad_codebook, st))) return rc;
+            }
+            ctx->last_path = ctx->Lb == 16 ? 1 : warp_supported(ctx->Lb, ctx->k) ? 2 : 0;
+            return launch_bwd_meets(ctx, p, grad_codebook, st);
         }
+        ctx->fwd_lin = false;                                      // certificates of two gauges: all blocks in the log domain
     }
-    if (rc) return rc;
-    ctx->last_path = use_cluster ? 1 : use_warp ? 2 : 0;
-    return BCJR_OK;
+#endif
+    return backward_blocks(ctx, p, grad_codebook, st);
 }
 
 bcjr_status viterbi_hard(bcjr_ctx *ctx, const float *W, const float *codebook, int Lb, int k, int n,
@@ -1676,6 +1922,7 @@ bcjr_status bcjr_soft_quantize_vec(bcjr_ctx *ctx, const float *W, const float *c
     if (!guard.ok) return BCJR_ECUDA;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     ctx->have_fwd = ctx->fwd_lin = ctx->fwd_reg = ctx->fwd_judged = false;
+    ctx->meet_from = -1;
     ctx->num_ran = 0;
     if (num_blocks > 0) {
         if ((rc = ensure(ctx, ctx->soft_copy, (size_t)num_blocks * n * 4))) return rc;
@@ -1967,12 +2214,13 @@ bcjr_status bcjr_linear_blocks(bcjr_ctx *ctx, int64_t *count, void *cuda_stream)
     if (!ctx || !count) return BCJR_EINVAL;
     if (!ctx->have_fwd) return BCJR_ESTATE;
     *count = 0;
-    if (!(ctx->fwd_lin || ctx->fwd_reg) || ctx->B == 0) return BCJR_OK;
+    if (!(ctx->fwd_lin || ctx->fwd_reg || ctx->meet_from >= 0) || ctx->B == 0) return BCJR_OK;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return BCJR_ECUDA;
     CU(cudaStreamSynchronize((cudaStream_t)cuda_stream));
     uint8_t part[4096];
-    for (int64_t b = 0; b < ctx->B; b += (int64_t)sizeof(part)) {
+    const int64_t first = ctx->meet_from > 0 && !ctx->fwd_lin ? ctx->meet_from : 0;      // (no flags of log-domain calls)
+    for (int64_t b = first; b < ctx->B; b += (int64_t)sizeof(part)) {
         const int64_t m = ctx->B - b < (int64_t)sizeof(part) ? ctx->B - b : (int64_t)sizeof(part);
         CU(cudaMemcpy(part, (const uint8_t *)ctx->lin_flag.ptr + b, (size_t)m, cudaMemcpyDeviceToHost));
         for (int64_t i = 0; i < m; ++i) *count += part[i] == 0;

@@ -171,6 +171,7 @@ struct FwdParams {
     int unlikely_max;        // stands behind (bcjr_warp.cuh) runs the call.  null: not counted, the kernel runs
     const int *list;         // log-domain kernels behind them: list[0] blocks to run, list[1 ...] their indices; null = all B blocks
     int list_max;            // listed blocks up to this number belong to fwd_reg_kernel, more to fwd_solo_kernel
+    bool only_flagged;       // fwd_reg_kernel behind the two-ended kernels (bcjr_meet.cuh): blocks with lin_flag set
 };
 
 struct BwdParams {

@@ -339,14 +339,15 @@ __global__ void __launch_bounds__(GEN_MAX_THREADS, KB == 2 ? 2 : 1) bwd_generic_
 
 // Deterministic (fixed-order) sum of the per-CTA partial codebook gradients.
 // unlikely: this sum is wanted if (*unlikely > unlikely_max) == given_up (FwdParams); null: always.
-static __global__ void reduce_gc_kernel(const float *part, int nparts, int S, float *out, const int *unlikely = nullptr, int unlikely_max = 0, bool given_up = false)
+static __global__ void reduce_gc_kernel(const float *part, int nparts, int S, float *out, const int *unlikely = nullptr, int unlikely_max = 0, bool given_up = false,
+                                        bool add = false)
 {
     if (unlikely && (*unlikely > unlikely_max) != given_up) return;
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= S) return;
     float acc = 0.f;
     for (int i = 0; i < nparts; ++i) acc += part[(size_t)i * S + u];
-    out[u] = acc;
+    out[u] = add ? out[u] + acc : acc;
 }
 
 // --------------------------------------------------------------------------------------

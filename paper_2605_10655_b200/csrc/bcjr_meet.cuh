@@ -1,0 +1,1103 @@
+// The register kernels' sweeps (bcjr_reg.cuh: k = 2, butterflies in registers) from both ends of a block at once.
+//
+// The alpha and the beta sweep of a block do not depend on each other until their messages are multiplied.  bcjr_reg.cuh runs one
+// behind the other, 2 n dependent steps, and with few blocks those steps' latency is all a call takes (a step of 2^16 states on
+// eight SMs 0.93 us, of which 0.27 are arithmetic; of 2^8 states in a warp 0.28 us with every pipe below 9 %).  Here one set of threads
+// (dir 0) runs the alpha steps 1 .. m, m = n / 2, while another (dir 1) runs the beta steps n .. m + 1; both keep their messages.  Then
+// each goes on through the other half and forms the posterior of every step from its own message and the kept one of the
+// other side: n dependent steps instead of 2 n, the same arithmetic, the same bytes of history.
+//   * CTA form (PHASE 0): both directions in one thread block, a barrier of its own for each, two of the whole block.
+//   * Split form (PHASE 1 and 2): a cluster of CL CTAs per direction and block; the end of the first launch is where the sides meet.  The
+//     first leaves A_{m+1}, M_m and the offsets in global memory.
+// A thread has BPT whole butterflies (G = 4) or half of one (G = 2: two of its four outputs, eight states).
+// Which form for which trellis, and what it measured: bcjr_meet_launch.cuh.
+//
+// A step of a cluster pays 330 clocks of latency and one clock per 20 bytes that a CTA sends, whatever the width of the
+// stores as long as a warp's lanes are side by side (32-byte gaps halve the rate; bulk copies and plain remote stores are slower):
+// hence butterflies STR apart in a thread with two.
+//
+// Gauge.  Either side scales its messages to 2^X_MEET by its own largest message (a step behind, see bcjr_reg.cuh); where a
+// side starts its second half the offset is taken from the message itself.  With S_t = sum A_t E M_t unnormalised,
+// Z = S_t 2^(O + P): Z comes from the products at the meeting point, kappa_t = 2^(O + P) / Z multiplies one factor of every posterior.
+// X_MEET = 50 on both sides keeps products below 2^123 and leaves 176 bits below the largest message.
+// Certificate (bcjr_lin.cuh): the alpha side adds what flushing can take from an output, the beta side flushes, and every S_t / Z
+// has to be within 3/4 of LIN_DEFECT of one (Z is that of the middle here, not the alpha side's, which doubles one of the three parts of
+// the bound), with kappa_t below 2^KAP_MEET (the backward call multiplies messages of up to 2^54 by it).
+#pragma once
+#include <type_traits>
+
+#include "bcjr_reg.cuh"
+
+namespace bcjr {
+
+constexpr int X_MEET = 50, KAP_MEET = 50;
+constexpr float MEET_DEFECT = 0.75f * LIN_DEFECT;
+
+template <int LB_, int CL_, int G_, int BPT_, bool BWD_, bool SPLIT_>
+struct MeetCfg {
+    static constexpr int LB = LB_, CL = CL_, G = G_, BPT = BPT_, K = 4, S = 1 << LB, Q = S >> 2, NB = S >> 4;
+    static constexpr bool BWD = BWD_, SPLIT = SPLIT_;
+    static constexpr int NBC = NB / CL;                        // butterflies of a CTA and direction
+    static constexpr int STR = NBC / BPT;                      // from one butterfly of a thread to its next
+    static constexpr int NT = NBC * (4 / G) / BPT, NWARP = NT / 32, NDIR = SPLIT ? 1 : 2, THREADS = NT * NDIR;
+    static constexpr int ARR = BWD ? 2 : 1;
+    static constexpr int NBUF = CL == 8 ? 4 : CL > 1 ? 3 : 2;  // clusters of up to four: a CTA's inputs come from all of them, one step back is enough
+    static constexpr int BUF = ARR * 4 * NBC;
+    static constexpr int RD = BWD && BPT > 1 ? 2 : 4;          // history staging depth in steps
+    static constexpr int PW = BWD ? 4 : 2, PROWS = 64;         // posterior sums of the warps, by step
+    static constexpr int MAX_N = 1024;
+    static constexpr int REGS = BWD || SPLIT ? 128 : 96;       // budget of a thread
+    static constexpr int FIT = 65536 / REGS / THREADS;
+    static constexpr int MIN_CTAS = FIT < 1 ? 1 : FIT > 16 ? 16 : FIT;
+    static constexpr int OFF_MSG = 0;
+    static constexpr int OFF_RING = OFF_MSG + NBUF * BUF;      // float4 [RD][ARR][BPT][NT]
+    static constexpr int OFF_PSUM = OFF_RING + RD * ARR * BPT * NT * 4;
+    static constexpr int OFF_WMAX = OFF_PSUM + (NWARP > 1 ? PROWS * NWARP * PW : 0);   // [4][16]
+    static constexpr int OFF_CMAX = OFF_WMAX + 64;             // [4][8]
+    static constexpr int OFF_RED = OFF_CMAX + 32;              // [6][24]: warps' and CTAs' values of a reduction
+    static constexpr int OFF_MBAR = OFF_RED + 144;             // uint64 [4]
+    static constexpr int DIR_FLOATS = OFF_MBAR + 8;
+    static constexpr int OFF_FLAG = NDIR * DIR_FLOATS;         // abort flag of the waits, then two words of the backward kernel
+    static constexpr int OFF_STEP = OFF_FLAG + 4;              // float4 [n + 1], float4 [n] sums, int O [n + 2], int P [n + 2]
+    static size_t smem_bytes(int n) { return (size_t)(OFF_STEP + 4 * (n + 1) + 4 * n + 2 * (n + 2)) * 4; }
+    // per block: rows of history; split form: then A_{m+1} and M_m by group
+    __host__ __device__ static constexpr size_t block_floats(int n) { return (size_t)(SPLIT ? n + 2 : n) * ARR * Q; }
+    static_assert(LB >= 8 && NT % 32 == 0 && NT <= 512 && THREADS <= 1024, "whole warps");
+    static_assert((G == 4 || (G == 2 && BPT == 1)) && (CL == 1 || (SPLIT && G == 4)) && (BPT == 1 || (BPT == 2 && CL == 4)), "forms");
+    static_assert(DIR_FLOATS % 4 == 0 && OFF_MBAR % 2 == 0, "alignment");
+};
+
+// One direction's threads.
+template <typename C>
+struct MeetUnit {
+    float *base;                                               // the direction's shared memory
+    int dir, i, lane, warp;                                    // thread of the direction
+    uint32_t rank;
+    Proto pr;
+    uint32_t phase;
+    int xl, x, h;                                              // first butterfly (in the CTA, in the block), half of it
+    static constexpr uint32_t TX_MSG = (uint32_t)C::BUF * 4u, TX_MAX = C::CL * 4u;
+    __device__ __forceinline__ float *msg(int s) const { return base + C::OFF_MSG + s * C::BUF; }
+    __device__ __forceinline__ uint32_t mbar(int s) const { return smem_u32(base + C::OFF_MBAR) + 8u * s; }
+    __device__ __forceinline__ void sync() const
+    {
+        if (C::NWARP == 1) __syncwarp();
+        else if (C::SPLIT) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + dir), "n"(C::NT) : "memory");
+    }
+    __device__ __forceinline__ void wait_inputs(int s)
+    {
+        if (C::CL > 1) { pr.wait(mbar(s), (phase >> s) & 1u); phase ^= 1u << s; }
+    }
+    // sum or maximum over the direction; every use between two block-wide barriers has a region of its own
+    template <bool MAX>
+    __device__ __forceinline__ float reduce(float v, int region) const
+    {
+        float *red = base + C::OFF_RED + region * 24;
+        const float none = MAX ? __int_as_float(0xff800000) : 0.f;
+        v = MAX ? warp_max(v) : warp_sum(v);
+        if (C::NWARP > 1) {
+            if (lane == 0) red[warp] = v;
+            sync();
+            v = lane < C::NWARP ? red[lane] : none;
+            v = MAX ? warp_max(v) : warp_sum(v);
+        }
+        if (C::CL > 1) {
+            if (i < C::CL) st_cluster_f32(mapa_u32(smem_u32(red + 16 + (int)rank), (uint32_t)i), v);
+            cluster_sync();
+            v = red[16];
+#pragma unroll
+            for (int r = 1; r < C::CL; ++r) v = MAX ? fmaxf(v, red[16 + r]) : v + red[16 + r];
+        }
+        return v;
+    }
+    // largest message of the step before (see reg_seen_max); v: step of the sweep, from one
+    __device__ __forceinline__ float seen_max(int v) const
+    {
+        const float none = __int_as_float(0xff800000);
+        if (C::CL > 1) return warp_max(lane < C::CL ? base[C::OFF_CMAX + (v & 3) * 8 + lane] : none);
+        if (C::NWARP == 1) return base[C::OFF_WMAX + (v & 3) * 16];
+        return warp_max(lane < C::NWARP ? base[C::OFF_WMAX + (v & 3) * 16 + lane] : none);
+    }
+    template <bool LIN>
+    __device__ __forceinline__ int offset(int v, int off, int lev0) const
+    {
+        const int o = (v <= 2 ? lev0 : reg_level<LIN>(seen_max(v), X_MEET)) - (v == 1 ? 0 : off);
+        return LIN && o < -LIN_STEP_DROP ? -LIN_STEP_DROP : o;
+    }
+    __device__ __forceinline__ void post_max(int v, float tmax) const
+    {
+        tmax = warp_max(tmax);
+        if (lane == 0) base[C::OFF_WMAX + ((v + 2) & 3) * 16 + warp] = tmax;
+    }
+    __device__ __forceinline__ void push_max(int v, int next) const
+    {
+        if (C::CL > 1 && warp == 0) {
+            const float none = __int_as_float(0xff800000);
+            const float m = warp_max(lane < C::NWARP ? base[C::OFF_WMAX + ((v + 1) & 3) * 16 + lane] : none);
+            if (lane < C::CL && pr.live)
+                st_async_f32(mapa_u32(smem_u32(base + C::OFF_CMAX + ((v + 1) & 3) * 8 + (int)rank), (uint32_t)lane), m, mapa_u32(mbar(next), (uint32_t)lane));
+        }
+    }
+    // start of step v with outputs into buffer nxt
+    __device__ __forceinline__ void arm(int v, int nxt, bool hook) const
+    {
+        if (C::CL > 1) {
+            if (i == 0 && !hook) pr.expect_tx(mbar(nxt), TX_MSG + (v > 1 ? TX_MAX : 0u));
+            if (v > 1) push_max(v, nxt);
+        }
+    }
+    // posterior sums of step v (width values, in lanes 0, 32 / width, ...): kept by warp, added up 32 steps at a time, each warp some rows
+    __device__ __forceinline__ void put_sums(int v, float4 *sum_of_step, float s, int width) const
+    {
+        const int span = 32 / width;
+        if ((lane % span) == 0 && lane / span < (C::BWD ? 3 : 2)) {
+            if (C::NWARP > 1) base[C::OFF_PSUM + ((v & (C::PROWS - 1)) * C::NWARP + warp) * C::PW + lane / span] = s;
+            else reinterpret_cast<float *>(sum_of_step)[lane / span] = s;
+        }
+    }
+    template <typename F>
+    __device__ __forceinline__ void add_rows(int v0, int v1, F sum_of_step) const
+    {
+        if constexpr (C::NWARP > 1) {
+            for (int v = v0 + warp; v <= v1; v += C::NWARP) {
+                const float *row = base + C::OFF_PSUM + (v & (C::PROWS - 1)) * C::NWARP * C::PW;
+                const int w = lane & 15, which = lane >> 4;
+                float a = w < C::NWARP ? row[w * C::PW + which] : 0.f, b = 0.f;
+                if (C::BWD) b = w < C::NWARP && which == 0 ? row[w * C::PW + 2] : 0.f;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) {
+                    a += __shfl_xor_sync(0xffffffffu, a, o);
+                    if (C::BWD) b += __shfl_xor_sync(0xffffffffu, b, o);
+                }
+                float *to = reinterpret_cast<float *>(sum_of_step(v));
+                if ((lane & 15) == 0) to[which] = a;
+                if (C::BWD && lane == 0) to[2] = b;
+            }
+        }
+    }
+    // end of step v of cnt: sums of the 32 steps before, where they are complete
+    template <typename F>
+    __device__ __forceinline__ void end_step(int v, bool comb, F sum_of_step) const
+    {
+        sync();
+        if (comb && (v & 31) == 1 && v > 1) add_rows(v - 32, v - 1, sum_of_step);
+    }
+};
+
+// Thread's table entries, 2 G pairs a butterfly, each (j, j + 1) of one l: alpha tab[jp G + l], l of the thread's half; beta
+// tab[jp 4 + b], j of its half.
+template <typename C>
+__device__ __forceinline__ int meet_entry(const MeetUnit<C> &un, int u, int e)
+{
+    const int j = un.dir == 0 ? 2 * (e / C::G) : 2 * (e / 4) + un.h * C::G, l = un.dir == 0 ? e % C::G + un.h * C::G : e % 4;
+    return j * C::Q + (un.x + u * C::STR) * 4 + (C::G == 4 ? e % 4 : l);
+}
+template <typename C>
+__device__ __forceinline__ void meet_load_table(const float *cb, const MeetUnit<C> &un, float2 (&tab)[C::BPT][2 * C::G])
+{
+#pragma unroll
+    for (int u = 0; u < C::BPT; ++u)
+#pragma unroll
+        for (int e = 0; e < 2 * C::G; ++e) {
+            const int at = meet_entry<C>(un, u, e);
+            tab[u][e] = make_float2(__ldg(cb + at), __ldg(cb + at + C::Q));
+        }
+}
+template <typename C>
+__device__ __forceinline__ void meet_table_range(const MeetUnit<C> &un, const float2 (&tab)[C::BPT][2 * C::G], float *lo_out, float *hi_out)
+{
+    float lo = tab[0][0].x, hi = lo;
+#pragma unroll
+    for (int u = 0; u < C::BPT; ++u)
+#pragma unroll
+        for (int e = 0; e < 2 * C::G; ++e) { lo = fminf(lo, fminf(tab[u][e].x, tab[u][e].y)); hi = max3f(hi, tab[u][e].x, tab[u][e].y); }
+    *lo_out = -un.template reduce<true>(-lo, 0);
+    *hi_out = un.template reduce<true>(hi, 1);
+}
+
+// Where a thread's outputs go (see RegDest).  The beta outputs of a thread's second butterfly go to the same CTAs as those of the first,
+// STR further on (two butterflies only where a CTA has a quarter of the block: output j is CTA j's).
+template <typename C>
+struct MeetDest {
+    uint32_t a[C::BPT], abar[C::BPT], b[C::G], bbar[C::G];
+    static constexpr uint32_t STEP_B = (uint32_t)(C::STR * C::ARR) * (C::CL > 1 ? 4u : 1u);
+    __device__ __forceinline__ explicit MeetDest(const MeetUnit<C> &un)
+    {
+        const uint32_t msg0 = smem_u32(un.base + C::OFF_MSG), mb0 = un.mbar(0);
+#pragma unroll
+        for (int u = 0; u < C::BPT; ++u) {
+            const int x = un.x + u * C::STR;
+            const int xa = (4 * x) % C::NB, ja = (4 * x) / C::NB, ata = ja * C::NBC + xa % C::NBC + (C::G == 2 ? 2 * un.h : 0);
+            a[u] = C::CL > 1 ? mapa_u32(msg0 + (uint32_t)ata * 4u, (uint32_t)(xa / C::NBC)) : (uint32_t)ata;
+            abar[u] = C::CL > 1 ? mapa_u32(mb0, (uint32_t)(xa / C::NBC)) : 0u;
+        }
+#pragma unroll
+        for (int o = 0; o < C::G; ++o) {
+            const int j = o + (C::G == 2 ? 2 * un.h : 0), x1 = j * (C::NB / 4) + un.x / 4, at = ((x1 % C::NBC) * 4 + (un.x & 3)) * C::ARR;
+            b[o] = C::CL > 1 ? mapa_u32(msg0 + (uint32_t)at * 4u, (uint32_t)(x1 / C::NBC)) : (uint32_t)at;
+            bbar[o] = C::CL > 1 ? mapa_u32(mb0, (uint32_t)(x1 / C::NBC)) : 0u;
+        }
+    }
+};
+
+// Z = 2^ez / iz (linear) or 2^(ez + lz); both are set in either domain's terms, lz for log Z
+struct MeetZ {
+    int ez;
+    float iz, lz;
+    // kappa_t (linear) or its log2, e = O + P
+    template <bool LIN>
+    __device__ __forceinline__ float kappa(int e) const
+    {
+        const int d = e - ez;
+        return LIN ? pow2i(d < -126 ? -126 : d > 127 ? 127 : d) * iz : (float)d - lz;
+    }
+};
+
+template <typename C>
+__device__ __forceinline__ MeetUnit<C> meet_unit(float *smem, DeviceDiag *diag)
+{
+    const int tid = (int)threadIdx.x, dir = C::SPLIT ? ((int)blockIdx.x / C::CL) & 1 : tid / C::NT, i = C::SPLIT ? tid : tid % C::NT;
+    const uint32_t rank = C::CL > 1 ? cluster_ctarank() : 0u;
+    MeetUnit<C> un{smem + (C::SPLIT ? 0 : dir * C::DIR_FLOATS), dir, i, i & 31, i >> 5, rank,
+                   Proto{1u, reinterpret_cast<volatile int *>(smem + C::OFF_FLAG), diag}, 0u, 0, 0, 0};
+    constexpr int PER = C::NBC / C::BPT;
+    un.xl = i % PER; un.h = i / PER;
+    un.x = (int)rank * C::NBC + un.xl;
+    if (C::CL > 1) {
+        volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_FLAG);
+        if (tid == 0) {
+            for (int s = 0; s < C::NBUF; ++s) mbar_init(un.mbar(s), 1);
+            *abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        cluster_sync();
+    }
+    return un;
+}
+
+// Z from the products of the two sides' messages at the meeting point; e: sum of their offsets.  false: not representable.
+template <bool LIN, typename C, typename FA, typename FB>
+__device__ __forceinline__ bool meet_z(const MeetUnit<C> &un, int count, FA a, FB b, int e, MeetZ *z)
+{
+    if (LIN) {
+        float v = 0.f;
+        for (int f = un.i; f < count; f += C::NT) v = fmaf(a(f), b(f), v);
+        const float s = un.template reduce<false>(v, 2);
+        const int ez = exp2i(s);
+        const float mz = s * pow2i(ez < -126 ? 126 : ez > 126 ? -126 : -ez);
+        z->ez = e + ez; z->iz = 1.f / mz; z->lz = lg2f(mz);
+        return s > 8.6e-19f && s < 4.2e37f;                      // 2^-60 .. 2^125
+    }
+    float v = __int_as_float(0xff800000);
+    for (int f = un.i; f < count; f += C::NT) v = fmaxf(v, a(f) + b(f));
+    const float m = un.template reduce<true>(v, 2);
+    v = 0.f;
+    for (int f = un.i; f < count; f += C::NT) v += ex2f(a(f) + b(f) - m);
+    z->ez = e; z->iz = 1.f;
+    z->lz = m + lg2f(un.template reduce<false>(v, 3));
+    return true;
+}
+
+// scratch of the split form
+struct MeetScratch {
+    int *aux;                                                    // [B][2][n + 2]: O_t, P_t
+};
+
+// History rows of the other side, staged RD - 1 steps ahead.
+template <typename C>
+struct MeetRing {
+    uint32_t to;
+    const float4 *from, *src;
+    __device__ __forceinline__ MeetRing(const MeetUnit<C> &un, const float4 *ring, const float4 *hist)
+        : to(smem_u32(ring) + (uint32_t)un.i * 16u), from(ring + un.i), src(hist + un.x) {}
+    __device__ __forceinline__ void issue(int t, bool want) const
+    {
+        if (want) {
+#pragma unroll
+            for (int e = 0; e < C::ARR * C::BPT; ++e)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (uint32_t)(((t % C::RD) * C::ARR * C::BPT + e) * C::NT * 16)),
+                             "l"(src + (size_t)(t - 1) * (C::ARR * C::NB) + (e / C::BPT) * C::NB + (e % C::BPT) * C::STR) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    __device__ __forceinline__ void wait() const { asm volatile("cp.async.wait_group %0;" ::"n"(C::RD - 1) : "memory"); }
+    __device__ __forceinline__ float4 row(int t, int arr, int u) const { return from[((t % C::RD) * C::ARR * C::BPT + arr * C::BPT + u) * C::NT]; }
+};
+
+// ---------------------------------------------------------------------------- forward
+template <typename C, int PHASE>
+__global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdParams p, MeetScratch ms)
+{
+    constexpr int CL = C::CL, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS;
+    extern __shared__ __align__(16) float smem[];
+    const int tid = (int)threadIdx.x;
+    MeetUnit<C> un = meet_unit<C>(smem, p.diag);
+    const int n = p.n, m = n / 2;
+    const float sl = sqrtf(p.lam2), NONE = __int_as_float(0xff800000);
+    const double isl_d = 1.0 / (double)sl;
+    float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);          // entry t - 1: scaled clamped weight, the same + 2 delta, delta, soft
+    float4 *sums = step + n + 1;                                           // entry t - 1: numerator, denominator (of this CTA)
+    int *O_s = reinterpret_cast<int *>(sums + n), *P_s = O_s + n + 2;      // entry t: A_t 2^O_t, M_t 2^P_t
+    float2 tab[BPT][2 * G];
+    meet_load_table<C>(p.cb, un, tab);
+    float c_lo, c_hi;
+    if (PHASE == 2) { c_lo = p.diag->c_lo; c_hi = p.diag->c_hi; }
+    else {
+        meet_table_range<C>(un, tab, &c_lo, &c_hi);
+        if (blockIdx.x == 0 && tid == 0) { p.diag->c_lo = c_lo; p.diag->c_hi = c_hi; }
+    }
+#pragma unroll
+    for (int u = 0; u < BPT; ++u)
+#pragma unroll
+        for (int e = 0; e < 2 * G; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; }
+    const MeetDest<C> dst(un);
+    float defect = 0.f, zgap = 0.f;
+    const int64_t first = C::SPLIT ? (int64_t)(blockIdx.x / (2 * CL)) : (int64_t)blockIdx.x;
+    const int64_t stride = C::SPLIT ? p.B : (int64_t)gridDim.x;
+
+    for (int64_t blk = first; blk < p.B; blk += stride) {
+        float *area = p.hist + (size_t)(C::SPLIT ? blk : (int64_t)blockIdx.x) * C::block_floats(n);
+        float4 *hist4 = reinterpret_cast<float4 *>(area);                  // row t - 1: [NB], A_t up to the middle, M_t behind it
+        float *endA = area + (size_t)n * C::Q, *endM = endA + C::Q;        // split form
+        int *aux = C::SPLIT ? ms.aux + blk * 2 * (n + 2) : nullptr;
+        const MeetRing<C> ring(un, reinterpret_cast<const float4 *>(un.base + C::OFF_RING), hist4);
+        const float *w = p.W + blk * n;
+        int outside = 0, beyond = 0;
+        for (int t = tid; t < n; t += TH) {
+            const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
+            step[t] = make_float4(se.wc * sl, (se.wc + 2.f * se.delta) * sl, se.delta, 0.f);
+            outside |= se.delta != 0.f;
+        }
+        const bool judge = p.lin_x >= 0 && p.demand < __int_as_float(0x7f800000);
+        if (judge)
+            for (int t = tid; t < n; t += TH) beyond |= lin_demand(w, t, n, p.window) > p.demand;
+        const bool recentre = __syncthreads_or(outside) != 0;             // (every CTA decides alike)
+        const bool likely = p.lin_x >= 0 && !(judge && __syncthreads_or(beyond) != 0);
+        MeetZ z{0, 1.f, 0.f};
+        float bdef = 0.f, gap = 0.f;
+        bool stands = true;
+        // steps whose results this CTA writes
+        const int out0 = C::SPLIT ? (un.dir == 0 ? m : 0) + (int)un.rank * NT + tid : tid, out1 = C::SPLIT && un.dir == 1 ? m : n;
+
+        auto run = [&](auto lin_tag, auto rc_tag) {
+            constexpr bool LIN = decltype(lin_tag)::value, RC = decltype(rc_tag)::value;
+            const int X = LIN ? X_MEET : 0;
+            // alpha steps t0 .. t0 + cnt - 1, the messages of step v in buffer (ub + v - 1) % NBUF
+            auto alpha = [&](auto comb_tag, int t0, int cnt, int ub, int lev0) {
+                constexpr bool COMB = decltype(comb_tag)::value;
+                auto sum_of = [&](int v) { return sums + (t0 + v - 2); };
+                int off = 0, O = O_s[t0];
+                float pn = 0.f, pd = 0.f;
+                if (COMB)
+                    for (int c = 0; c < C::RD - 1; ++c) ring.issue(t0 + c, c < cnt);
+                for (int v = 1; v <= cnt; ++v) {
+                    const int t = t0 + v - 1, cur = (ub + v - 1) % C::NBUF, nxt = (ub + v) % C::NBUF;
+                    const bool send = !COMB || v < cnt;
+                    if (COMB) { ring.issue(t + C::RD - 1, v + C::RD - 1 <= cnt); ring.wait(); }
+                    if (v > 1) un.wait_inputs(cur);
+                    if (send) un.arm(v, nxt, false);
+                    const float *in = un.msg(cur) + un.xl;
+                    float4 a4[BPT];
+#pragma unroll
+                    for (int u = 0; u < BPT; ++u) {
+                        const int at = u * C::STR;
+                        a4[u] = make_float4(in[at], in[NBC + at], in[2 * NBC + at], in[3 * NBC + at]);
+                    }
+                    const float4 sp = step[t - 1];
+                    off = un.template offset<LIN>(v, off, lev0);
+                    O += off;
+                    if (un.i == 0) O_s[t + 1] = O;
+                    const float kap = COMB ? z.kappa<LIN>(O + P_s[t]) : 0.f;
+                    if (!COMB && (G == 4 || un.h == 0)) {
+#pragma unroll
+                        for (int u = 0; u < BPT; ++u) hist4[(size_t)(t - 1) * C::NB + un.x + u * C::STR] = a4[u];
+                    }
+                    if (COMB && v > 1) un.put_sums(v - 1, sum_of(v - 1), warp_sum2_split(pn, pd, un.lane), 2);   // (beside this step's arithmetic)
+                    pn = pd = 0.f;
+                    const float2 w2 = splat2(sp.x), v2 = splat2(sp.y), off2 = splat2((float)off);
+                    float tmax = NONE;
+#pragma unroll
+                    for (int u = 0; u < BPT; ++u) {
+                        const float2 A0 = make_float2(a4[u].x, a4[u].y), A1 = make_float2(a4[u].z, a4[u].w);
+                        const float floor1 = LIN ? lin_floor((a4[u].x + a4[u].y) + (a4[u].z + a4[u].w)) : 0.f;
+                        float Ml[4] = {0.f, 0.f, 0.f, 0.f};
+                        if (COMB) { const float4 m4 = ring.row(t, 0, u); Ml[0] = m4.x; Ml[1] = m4.y; Ml[2] = m4.z; Ml[3] = m4.w; }
+                        if (G == 2 && un.h) { Ml[0] = Ml[2]; Ml[1] = Ml[3]; }
+                        float out[G];
+#pragma unroll
+                        for (int l = 0; l < G; ++l) {
+                            const float2 c0 = tab[u][l], c1 = tab[u][G + l];
+                            const float2 d0 = sub2(c0, w2), d1 = sub2(c1, w2);
+                            const float2 r0 = RC ? sub2(c0, v2) : d0, r1 = RC ? sub2(c1, v2) : d1;
+                            if (LIN) {
+                                const float2 e0 = ex2n2(fma2(d0, r0, off2)), e1 = ex2n2(fma2(d1, r1, off2));
+                                if (COMB) {
+                                    const float2 p0 = mul2(e0, A0), p1 = mul2(e1, A1), s = add2(p0, p1), ds = fma2(p1, d1, mul2(p0, d0));
+                                    const float f = Ml[l] * kap;
+                                    out[l] = (s.x + s.y) + floor1;
+                                    pd = fmaf(f, out[l], pd);
+                                    pn = fmaf(f, ds.x + ds.y, pn);
+                                } else {
+                                    const float2 s = fma2(e1, A1, fma2(e0, A0, make_float2(floor1, 0.f)));
+                                    out[l] = s.x + s.y;
+                                }
+                            } else {
+                                const float2 u0 = sub2(A0, mul2(d0, r0)), u1 = sub2(A1, mul2(d1, r1));
+                                const float mx = max3f(fmaxf(u0.x, u0.y), u1.x, u1.y);
+                                const float2 e0 = ex2f2(sub2(u0, splat2(mx))), e1 = ex2f2(sub2(u1, splat2(mx))), s = add2(e0, e1);
+                                const float sum = s.x + s.y, top = mx - off2.x;
+                                out[l] = top + lg2f(sum);
+                                if (COMB) {
+                                    const float2 ds = fma2(e1, d1, mul2(e0, d0));
+                                    const float f = ex2f(top + Ml[l] + kap);
+                                    pd = fmaf(f, sum, pd);
+                                    pn = fmaf(f, ds.x + ds.y, pn);
+                                }
+                            }
+                            tmax = fmaxf(tmax, out[l]);
+                        }
+                        if (send) {
+                            if constexpr (CL > 1) {
+                                if (un.pr.live) st_async_v4(dst.a[u] + (uint32_t)nxt * un.TX_MSG, out[0], out[1], out[G - 2], out[G - 1], dst.abar[u] + 8u * nxt);
+                            } else if constexpr (G == 4) *reinterpret_cast<float4 *>(un.msg(nxt) + dst.a[u]) = make_float4(out[0], out[1], out[2], out[3]);
+                            else *reinterpret_cast<float2 *>(un.msg(nxt) + dst.a[u]) = make_float2(out[0], out[1]);
+                        }
+                    }
+                    un.post_max(v, tmax);
+                    un.end_step(v, COMB, sum_of);
+                }
+                if (COMB && cnt > 0) {
+                    un.put_sums(cnt, sum_of(cnt), warp_sum2_split(pn, pd, un.lane), 2);
+                    un.sync();
+                    un.add_rows((cnt - 1) / 32 * 32 + 1, cnt, sum_of);
+                }
+            };
+            // beta steps tb .. tb - cnt + 1
+            auto beta = [&](auto comb_tag, int tb, int cnt, int ub, int lev0) {
+                constexpr bool COMB = decltype(comb_tag)::value;
+                auto sum_of = [&](int v) { return sums + (tb - v); };
+                int off = 0, P = P_s[tb];
+                float pn = 0.f, pd = 0.f;
+                if (COMB)
+                    for (int c = 0; c < C::RD - 1; ++c) ring.issue(tb - c, c < cnt);
+                for (int v = 1; v <= cnt; ++v) {
+                    const int t = tb - v + 1, cur = (ub + v - 1) % C::NBUF, nxt = (ub + v) % C::NBUF;
+                    const bool send = !COMB || v < cnt;
+                    if (COMB) { ring.issue(t - (C::RD - 1), v + C::RD - 1 <= cnt); ring.wait(); }
+                    if (v > 1) un.wait_inputs(cur);
+                    if (send) un.arm(v, nxt, false);
+                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + un.xl;
+                    const float4 sp = step[t - 1];
+                    off = un.template offset<LIN>(v, off, lev0);
+                    P += off;
+                    if (un.i == 0) P_s[t - 1] = P;
+                    const float kap = COMB ? z.kappa<LIN>(O_s[t] + P) : 0.f;
+                    if (COMB && v > 1) un.put_sums(v - 1, sum_of(v - 1), warp_sum2_split(pn, pd, un.lane), 2);
+                    const float2 w2 = splat2(sp.x), v2 = splat2(sp.y), off2 = splat2((float)off);
+                    float2 num2 = make_float2(0.f, 0.f), den2 = num2;
+                    float tmax = NONE;
+#pragma unroll
+                    for (int u = 0; u < BPT; ++u) {
+                        const float4 m4 = in[u * C::STR];
+                        if (!COMB && (G == 4 || un.h == 0)) hist4[(size_t)(t - 1) * C::NB + un.x + u * C::STR] = m4;
+                        const float Mb[4] = {m4.x, m4.y, m4.z, m4.w};
+                        float2 Ah[2];
+                        if (COMB) {
+                            const float4 a4 = ring.row(t, 0, u);
+                            Ah[0] = make_float2(a4.x, a4.y); Ah[1] = make_float2(a4.z, a4.w);
+                            if (G == 2 && un.h) Ah[0] = Ah[1];
+                        }
+                        float out[G];
+#pragma unroll
+                        for (int jp = 0; jp < G / 2; ++jp) {
+                            float2 sum, ds, f, o;
+                            if (LIN) {
+#pragma unroll
+                                for (int b = 0; b < 4; ++b) {
+                                    const float2 c = tab[u][jp * 4 + b], d = sub2(c, w2);
+                                    const float2 pb = mul2(ex2n2(fma2(d, RC ? sub2(c, v2) : d, off2)), splat2(Mb[b]));
+                                    sum = b == 0 ? pb : add2(sum, pb);
+                                    if (COMB) ds = b == 0 ? mul2(pb, d) : fma2(pb, d, ds);
+                                }
+                                o = sum;
+                                if (COMB) f = mul2(Ah[jp], splat2(kap));
+                            } else {
+                                float2 d[4], uu[4];
+#pragma unroll
+                                for (int b = 0; b < 4; ++b) {
+                                    const float2 c = tab[u][jp * 4 + b];
+                                    d[b] = sub2(c, w2);
+                                    uu[b] = sub2(splat2(Mb[b] - off2.x), mul2(d[b], RC ? sub2(c, v2) : d[b]));
+                                }
+                                const float2 mx = max_pairs<4>(uu);
+#pragma unroll
+                                for (int b = 0; b < 4; ++b) {
+                                    const float2 pb = ex2f2(sub2(uu[b], mx));
+                                    sum = b == 0 ? pb : add2(sum, pb);
+                                    if (COMB) ds = b == 0 ? mul2(pb, d[b]) : fma2(pb, d[b], ds);
+                                }
+                                o = add2(mx, lg2f2(sum));
+                                if (COMB) f = ex2f2(add2(add2(Ah[jp], mx), splat2(kap)));
+                            }
+                            out[2 * jp] = o.x; out[2 * jp + 1] = o.y;
+                            if (COMB) { num2 = fma2(f, ds, num2); den2 = fma2(f, sum, den2); }
+                            tmax = max3f(tmax, o.x, o.y);
+                        }
+                        if (send) {
+#pragma unroll
+                            for (int o = 0; o < G; ++o) {
+                                if constexpr (CL > 1) {
+                                    if (un.pr.live) st_async_f32(dst.b[o] + u * dst.STEP_B + (uint32_t)nxt * un.TX_MSG, out[o], dst.bbar[o] + 8u * nxt);
+                                } else {
+                                    un.msg(nxt)[dst.b[o] + u * dst.STEP_B] = out[o];
+                                }
+                            }
+                        }
+                    }
+                    if (COMB) { pn = num2.x + num2.y; pd = den2.x + den2.y; }
+                    un.post_max(v, tmax);
+                    un.end_step(v, COMB, sum_of);
+                }
+                if (COMB && cnt > 0) {
+                    un.put_sums(cnt, sum_of(cnt), warp_sum2_split(pn, pd, un.lane), 2);
+                    un.sync();
+                    un.add_rows((cnt - 1) / 32 * 32 + 1, cnt, sum_of);
+                }
+            };
+            constexpr std::true_type YES{};
+            constexpr std::false_type NO{};
+            // ================= from either end to the middle
+            if (PHASE != 2) {
+                for (int f = un.i; f < C::BUF; f += NT) un.msg(0)[f] = LIN ? pow2i(X_MEET) : 0.f;
+                if (tid == 0) { O_s[1] = -X; P_s[n] = -X; }
+                if (CL > 1) cluster_sync(); else __syncthreads();
+                if (un.dir == 0) alpha(NO, 1, m, 0, 0);
+                else beta(NO, n, n - m, 0, 0);
+            }
+            const int fin = un.dir == 0 ? m : n - m;             // steps done so far
+            if (PHASE == 1) {
+                if (fin > 0) un.wait_inputs(fin % C::NBUF);
+                const float *last = un.msg(fin % C::NBUF);
+                for (int f = un.i; f < C::BUF; f += NT) {
+                    if (un.dir == 0) endA[(f / NBC) * C::NB + (int)un.rank * NBC + f % NBC] = last[f];
+                    else endM[(int)un.rank * C::BUF + f] = last[f];
+                }
+                if (un.rank == 0) {
+                    if (un.dir == 0) for (int t = 1 + tid; t <= m + 1; t += NT) aux[t] = O_s[t];
+                    else for (int t = m + tid; t <= n; t += NT) aux[n + 2 + t] = P_s[t];
+                }
+                return;
+            }
+            // ================= the sides meet
+            const int ub = PHASE == 2 ? 0 : fin;
+            if (PHASE == 2) {
+                for (int t = 1 + tid; t <= m + 1; t += NT) O_s[t] = aux[t];
+                for (int t = m + tid; t <= n; t += NT) P_s[t] = aux[n + 2 + t];
+                for (int f = un.i; f < C::BUF; f += NT)
+                    un.msg(0)[f] = un.dir == 0 ? endA[(f / NBC) * C::NB + (int)un.rank * NBC + f % NBC] : endM[(int)un.rank * C::BUF + f];
+            }
+            __syncthreads();
+            const int e = O_s[m + 1] + P_s[m];
+            bool ok;
+            if (PHASE == 2) {
+                const int q0 = (int)un.rank * (C::Q / CL);
+                ok = meet_z<LIN>(un, C::Q / CL, [&](int f) { return endA[q0 + f]; }, [&](int f) { return endM[q0 + f]; }, e, &z);
+            } else {
+                const float *a = smem + C::OFF_MSG + (m % C::NBUF) * C::BUF, *b = smem + C::DIR_FLOATS + C::OFF_MSG + ((n - m) % C::NBUF) * C::BUF;
+                ok = meet_z<LIN>(un, C::Q, [&](int f) { return a[f]; }, [&](int f) { return b[f]; }, e, &z);
+            }
+            stands = ok || !LIN;
+            float mv = NONE;
+            for (int f = un.i; f < C::BUF; f += NT) mv = fmaxf(mv, un.msg(ub % C::NBUF)[f]);
+            const int lev0 = reg_level<LIN>(un.template reduce<true>(mv, 4), X_MEET);
+            if (PHASE == 0) __syncthreads();                     // (the sweeps overwrite what the other side has just read)
+            if (stands) {                                        // (both sides and every CTA decide alike)
+                if (un.dir == 0) alpha(YES, m + 1, n - m, ub, lev0);
+                else beta(YES, m, m, ub, lev0);
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            if (CL > 1) cluster_sync(); else __syncthreads();
+            // soft codeword, one thread per step, kept until it stands
+            int bad = !stands;
+            bdef = gap = 0.f;
+            if (stands)
+                for (int t = out0; t < out1; t += CL * TH) {
+                    float a, c;
+                    if (CL > 1) {
+                        a = c = 0.f;
+#pragma unroll
+                        for (int r = 0; r < CL; ++r) {
+                            const float2 s = ld_cluster_f2(mapa_u32(smem_u32(sums + t), (uint32_t)r));
+                            a += s.x; c += s.y;
+                        }
+                    } else {
+                        a = sums[t].x; c = sums[t].y;
+                    }
+                    step[t].w = (float)(((double)step[t].x + (double)(a / c)) * isl_d);
+                    const float df = fabsf(c - 1.f);
+                    const int ke = (t >= m ? O_s[t + 2] + P_s[t + 1] : O_s[t + 1] + P_s[t]) - z.ez;
+                    bad |= LIN && (!(df <= MEET_DEFECT) || ke > KAP_MEET);
+                    bdef = fmaxf(bdef, df);
+                    if (t == 0 || t == n - 1) gap = fmaxf(gap, fabsf(lg2f(c)));   // M_n and A_1 are constant: Z of either side
+                }
+            if (!LIN && un.rank == 0 && tid == 0) diag_check_finite(p.diag, z.lz);
+            stands = __syncthreads_or(bad) == 0;
+        };
+        bool done = false;
+        if (likely) {
+            if (recentre) run(std::true_type{}, std::true_type{});
+            else run(std::true_type{}, std::false_type{});
+            done = stands;
+        }
+        if (C::SPLIT) {
+            // a block without a certificate is run again by fwd_reg_kernel, behind these launches
+            if (p.lin_x < 0) run(std::false_type{}, std::true_type{});
+            if (PHASE == 1) {
+                if (un.dir == 0 && un.rank == 0 && tid == 0) {
+                    p.lin_flag[blk] = likely ? 0 : 1;
+                    if (p.blk_defect) p.blk_defect[blk] = 0.f;
+                }
+                break;
+            }
+            if (p.lin_x >= 0 && !done) {
+                if (likely && tid == 0) p.lin_flag[blk] = 1;
+                break;
+            }
+        } else if (!done) {
+            __syncthreads();
+            run(std::false_type{}, std::true_type{});
+        }
+        defect = fmaxf(defect, bdef);
+        zgap = fmaxf(zgap, gap);
+        for (int t = out0; t < out1; t += CL * TH) {             // (the CTA form may overwrite W, which nothing below reads)
+            const float sw = step[t].w;
+            p.soft[blk * n + t] = sw;
+            if (p.soft_copy) p.soft_copy[blk * n + t] = sw;
+        }
+        if (p.blk_defect) {
+            if (!C::SPLIT) {
+                if (tid == 0) p.blk_defect[blk] = 0.f;
+                __syncthreads();
+            }
+            bdef = warp_max(bdef);
+            if (un.lane == 0) atomicMax(reinterpret_cast<unsigned *>(p.blk_defect + blk), __float_as_uint(bdef));
+        }
+        if (un.dir == 0 && un.rank == 0 && tid == 0) {
+            if (!C::SPLIT) p.lin_flag[blk] = done ? 0 : 1;
+            if (p.logZ) {
+                double zshift = 0.0;                             // sum_t lam2 delta_t^2: left out by step_energy
+                if (recentre)
+                    for (int t = 0; t < n; ++t) {
+                        const double dl = (double)step[t].z;
+                        zshift += (double)p.lam2 * dl * dl;
+                    }
+                p.logZ[blk] = (float)(((double)z.ez + (double)z.lz - zshift) * 0.6931471805599453);
+            }
+        }
+        if (!C::SPLIT) __syncthreads();
+    }
+    if (PHASE != 1) {
+        defect = warp_max(defect); zgap = warp_max(zgap);
+        if (un.lane == 0) {
+            diag_max(&p.diag->max_defect, defect);
+            diag_max(&p.diag->max_logz_gap, zgap);
+        }
+    }
+    if (CL > 1) {
+        cluster_sync();                                          // no CTA leaves while a peer may still address its shared memory
+        if (*un.pr.abort_flag) settle_after_abort();
+    }
+}
+
+// ---------------------------------------------------------------------------- backward
+// (A, AA) and (M, Bt) as in bwd_reg_kernel, L and At in the log domain.  The second half of either sweep forms gradients from both: with
+// r = h + At + Bt the state's gradient is gamma (g + (w - c) r / T), on the alpha side E [A g + (w - c) (A (h + Bt) + AA) / T] times M kappa.
+// p.gc_part: one partial per direction of a thread block (CTA form) or per cluster (split form), the states' sums over its half.
+template <typename C, bool ACC, int PHASE>
+__global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdParams p, MeetScratch ms)
+{
+    constexpr int CL = C::CL, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS, ARR = 2;
+    extern __shared__ __align__(16) float smem[];
+    const int tid = (int)threadIdx.x;
+    MeetUnit<C> un = meet_unit<C>(smem, p.diag);
+    const int n = p.n, m = n / 2;
+    const float sl = sqrtf(p.lam2), isl = 1.f / sl, NONE = __int_as_float(0xff800000);
+    const double isl_d = 1.0 / (double)sl;
+    float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);          // entry t - 1: scaled clamped weight, the same + 2 delta, g, gs
+    float4 *sums = step + n + 1;                                           // entry t - 1: the three posterior sums (of this CTA)
+    int *O_s = reinterpret_cast<int *>(sums + n), *P_s = O_s + n + 2;
+    const float c_lo = p.diag->c_lo, c_hi = p.diag->c_hi;                  // left by the forward call
+    float2 tab[BPT][2 * G], acc[BPT][2 * G];
+    meet_load_table<C>(p.cb, un, tab);
+#pragma unroll
+    for (int u = 0; u < BPT; ++u)
+#pragma unroll
+        for (int e = 0; e < 2 * G; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; acc[u][e] = make_float2(0.f, 0.f); }
+    const MeetDest<C> dst(un);
+    constexpr int PL = 4 * NBC;                                             // floats from A to AA in an alpha message
+    float defect = 0.f;
+    const float2 ni2 = splat2(-p.invT * isl);
+    // scale of the accumulators (see bcjr_lin_bwd.cuh), and whether gc_part holds something already
+    int *scale_s = reinterpret_cast<int *>(smem + C::OFF_FLAG + 1);
+    if (tid == 0) { scale_s[0] = GRAD_NONE; scale_s[1] = 0; }
+    __syncthreads();
+    auto write_acc = [&]() {
+        float *gc = p.gc_part + (size_t)(C::SPLIT ? (int)blockIdx.x / CL : 2 * (int)blockIdx.x + un.dir) * C::S;
+        const float up = grad_up(scale_s[0]);
+        const bool add = scale_s[1] != 0;
+#pragma unroll
+        for (int u = 0; u < BPT; ++u)
+#pragma unroll
+            for (int e = 0; e < 2 * G; ++e) {
+                float *to = gc + meet_entry<C>(un, u, e);
+                to[0] = up * acc[u][e].x + (add ? to[0] : 0.f);
+                to[C::Q] = up * acc[u][e].y + (add ? to[C::Q] : 0.f);
+            }
+    };
+    // test hook for the waits' abort path: CTA 0 never arms one buffer of its first sweep, so that its wait runs out
+    const bool drop_hook = CL > 1 && blockIdx.x == 0 && p.diag->drop_history_load != 0;
+    const int64_t first = C::SPLIT ? (int64_t)(blockIdx.x / (2 * CL)) : (int64_t)blockIdx.x;
+    const int64_t stride = C::SPLIT ? p.B : (int64_t)gridDim.x;
+
+    for (int64_t blk = first; blk < p.B; blk += stride) {
+        float *area = p.hist + (size_t)(C::SPLIT ? blk : (int64_t)blockIdx.x) * C::block_floats(n);
+        float4 *hist4 = reinterpret_cast<float4 *>(area);                  // row t - 1: [2][NB]: A, AA up to the middle, M, Bt behind it
+        float *endA = area + (size_t)n * ARR * C::Q, *endM = endA + ARR * C::Q;
+        int *aux = C::SPLIT ? ms.aux + blk * 2 * (n + 2) : nullptr;
+        const MeetRing<C> ring(un, reinterpret_cast<const float4 *>(un.base + C::OFF_RING), hist4);
+        const float *w = p.W + blk * n, *g = p.g + blk * n, *sf = p.soft + blk * n;
+        uint32_t gmax = 0;                                                 // (each warp looks at all of it)
+        for (int t = un.lane; t < n; t += 32) gmax = max(gmax, grad_bits(__ldg(g + t)));
+        const int e_g = grad_exponent(__reduce_max_sync(0xffffffffu, gmax));
+        // the block runs at the accumulators' scale if its gradient is within GRAD_SPAN bits below it
+        int e_acc = ACC ? scale_s[0] : GRAD_NONE, wrote = 0;
+        if (e_g != GRAD_NONE && (e_g > e_acc || e_g < e_acc - GRAD_SPAN)) {
+            if (ACC && e_acc != GRAD_NONE) {
+                write_acc();
+                wrote = 1;
+#pragma unroll
+                for (int u = 0; u < BPT; ++u)
+#pragma unroll
+                    for (int e = 0; e < 2 * G; ++e) acc[u][e] = make_float2(0.f, 0.f);
+            }
+            e_acc = e_g + GRAD_ROOM;
+        }
+        const float down = grad_down(e_acc);
+        int outside = 0;
+        for (int t = tid; t < n; t += TH) {
+            const StepEnergy se = step_energy(__ldg(w + t), c_lo, c_hi, p.lam2);
+            const float gv = __ldg(g + t) * down, ws = se.wc * sl;
+            step[t] = make_float4(ws, (se.wc + 2.f * se.delta) * sl, gv, lin_gs(gv, ws, isl_d, __ldg(sf + t)));
+            outside |= se.delta != 0.f;
+        }
+        if (tid == 0) step[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool recentre = __syncthreads_or(outside) != 0;
+        if (tid == 0) { scale_s[0] = e_acc; if (wrote) scale_s[1] = 1; }
+        MeetZ z{0, 1.f, 0.f};
+        const int out0 = C::SPLIT ? (un.dir == 0 ? m : 0) + (int)un.rank * NT + tid : tid, out1 = C::SPLIT && un.dir == 1 ? m : n;
+
+        auto run = [&](auto lin_tag, auto rc_tag) {
+            constexpr bool LIN = decltype(lin_tag)::value, RC = decltype(rc_tag)::value;
+            const int X = LIN ? X_MEET : 0;
+            auto alpha = [&](auto comb_tag, int t0, int cnt, int ub, int lev0) {
+                constexpr bool COMB = decltype(comb_tag)::value;
+                auto sum_of = [&](int v) { return sums + (t0 + v - 2); };
+                int off = 0, O = O_s[t0];
+                float s0 = 0.f, s2 = 0.f, sz = 0.f;
+                if (COMB)
+                    for (int c = 0; c < C::RD - 1; ++c) ring.issue(t0 + c, c < cnt);
+                for (int v = 1; v <= cnt; ++v) {
+                    const int t = t0 + v - 1, cur = (ub + v - 1) % C::NBUF, nxt = (ub + v) % C::NBUF;
+                    const bool send = !COMB || v < cnt;
+                    if (COMB) { ring.issue(t + C::RD - 1, v + C::RD - 1 <= cnt); ring.wait(); }
+                    if (v > 1) un.wait_inputs(cur);
+                    if (send) un.arm(v, nxt, drop_hook && PHASE != 2 && v == 1);
+                    const float *in = un.msg(cur) + un.xl;
+                    const float4 sp = step[t - 1];
+                    const float gsn = step[t].w;
+                    off = un.template offset<LIN>(v, off, lev0);
+                    O += off;
+                    if (un.i == 0) O_s[t + 1] = O;
+                    const float kap = COMB ? z.kappa<LIN>(O + P_s[t]) : 0.f;
+                    if (COMB && v > 1) un.put_sums(v - 1, sum_of(v - 1), warp_sum3_split(s0, s2, sz, un.lane), 4);
+                    s0 = s2 = sz = 0.f;
+                    const float2 w2 = splat2(sp.x), v2 = splat2(sp.y), off2 = splat2((float)off), gd2 = splat2(sp.z * isl), g2 = splat2(sp.z);
+                    const float2 u2 = splat2(0.5f * (sp.x + sp.y));   // scaled weight + delta
+                    float tmax = NONE;
+#pragma unroll
+                    for (int u = 0; u < BPT; ++u) {
+                        const int at = u * C::STR;
+                        const float4 a4 = make_float4(in[at], in[NBC + at], in[2 * NBC + at], in[3 * NBC + at]);
+                        const float4 b4 = make_float4(in[PL + at], in[PL + NBC + at], in[PL + 2 * NBC + at], in[PL + 3 * NBC + at]);
+                        if (!COMB && (G == 4 || un.h == 0)) {
+                            float4 *row = hist4 + (size_t)(t - 1) * (ARR * C::NB) + un.x + at;
+                            row[0] = a4; row[C::NB] = b4;
+                        }
+                        const float2 A0 = make_float2(a4.x, a4.y), A1 = make_float2(a4.z, a4.w);
+                        const float2 B0 = make_float2(b4.x, b4.y), B1 = make_float2(b4.z, b4.w);
+                        const float2 q0 = LIN ? mul2(A0, gd2) : gd2, q1 = LIN ? mul2(A1, gd2) : gd2;
+                        float2 G0 = g2, G1 = g2;
+                        float Ml[4] = {0.f, 0.f, 0.f, 0.f}, Yl[4] = {0.f, 0.f, 0.f, 0.f};
+                        if (COMB) {
+                            const float4 m4 = ring.row(t, 0, u), y4 = ring.row(t, 1, u);
+                            Ml[0] = m4.x; Ml[1] = m4.y; Ml[2] = m4.z; Ml[3] = m4.w;
+                            Yl[0] = y4.x; Yl[1] = y4.y; Yl[2] = y4.z; Yl[3] = y4.w;
+                            if (G == 2 && un.h) { Ml[0] = Ml[2]; Ml[1] = Ml[3]; Yl[0] = Yl[2]; Yl[1] = Yl[3]; }
+                            if (LIN) { G0 = mul2(A0, g2); G1 = mul2(A1, g2); }
+                        }
+                        float oa[G], ob[G];
+#pragma unroll
+                        for (int l = 0; l < G; ++l) {
+                            const float2 c0 = tab[u][l], c1 = tab[u][G + l];
+                            const float2 d0 = sub2(c0, w2), d1 = sub2(c1, w2);
+                            const float2 r0 = RC ? sub2(c0, v2) : d0, r1 = RC ? sub2(c1, v2) : d1;
+                            const float2 y0 = fma2(d0, q0, B0), y1 = fma2(d1, q1, B1);
+                            float2 e0, e1;
+                            float top = 0.f;
+                            if (LIN) {
+                                e0 = ex2n2(fma2(d0, r0, off2)); e1 = ex2n2(fma2(d1, r1, off2));
+                            } else {
+                                const float2 u0 = sub2(A0, mul2(d0, r0)), u1 = sub2(A1, mul2(d1, r1));
+                                const float mx = max3f(fmaxf(u0.x, u0.y), u1.x, u1.y);
+                                e0 = ex2f2(sub2(u0, splat2(mx))); e1 = ex2f2(sub2(u1, splat2(mx)));
+                                top = mx - off2.x;
+                            }
+                            const float2 s = LIN ? fma2(e1, A1, mul2(e0, A0)) : add2(e0, e1), ax = fma2(e1, y1, mul2(e0, y0));
+                            const float sum = s.x + s.y, axs = ax.x + ax.y;
+                            if (LIN) { oa[l] = sum; ob[l] = fmaf(sum, gsn, axs); }
+                            else { oa[l] = top + lg2f(sum); ob[l] = fmaf(axs, rcpf(sum), gsn); }
+                            if (COMB) {
+                                const float f = LIN ? Ml[l] * kap : ex2f(top + Ml[l] + kap);
+                                const float2 Y2 = splat2(Yl[l]), f2 = splat2(f);
+                                const float2 h0 = LIN ? fma2(A0, Y2, y0) : add2(y0, Y2), h1 = LIN ? fma2(A1, Y2, y1) : add2(y1, Y2);
+                                const float2 z0 = fma2(mul2(RC ? sub2(c0, u2) : d0, ni2), h0, G0), z1 = fma2(mul2(RC ? sub2(c1, u2) : d1, ni2), h1, G1);
+                                const float2 x0 = mul2(e0, z0), x1 = mul2(e1, z1), xs = add2(x0, x1);
+                                if (ACC) { acc[u][l] = fma2(x0, f2, acc[u][l]); acc[u][G + l] = fma2(x1, f2, acc[u][G + l]); }
+                                s0 = fmaf(f, sum, s0);
+                                s2 = fmaf(f, fmaf(Yl[l], sum, axs), s2);
+                                sz = fmaf(f, xs.x + xs.y, sz);
+                            }
+                            tmax = fmaxf(tmax, oa[l]);
+                        }
+                        if (send) {
+                            if constexpr (CL > 1) {
+                                if (un.pr.live) {
+                                    const uint32_t to = dst.a[u] + (uint32_t)nxt * un.TX_MSG;
+                                    st_async_v4(to, oa[0], oa[1], oa[G - 2], oa[G - 1], dst.abar[u] + 8u * nxt);
+                                    st_async_v4(to + PL * 4u, ob[0], ob[1], ob[G - 2], ob[G - 1], dst.abar[u] + 8u * nxt);
+                                }
+                            } else if constexpr (G == 4) {
+                                float *to = un.msg(nxt) + dst.a[u];
+                                *reinterpret_cast<float4 *>(to) = make_float4(oa[0], oa[1], oa[2], oa[3]);
+                                *reinterpret_cast<float4 *>(to + PL) = make_float4(ob[0], ob[1], ob[2], ob[3]);
+                            } else {
+                                float *to = un.msg(nxt) + dst.a[u];
+                                *reinterpret_cast<float2 *>(to) = make_float2(oa[0], oa[1]);
+                                *reinterpret_cast<float2 *>(to + PL) = make_float2(ob[0], ob[1]);
+                            }
+                        }
+                    }
+                    un.post_max(v, tmax);
+                    un.end_step(v, COMB, sum_of);
+                }
+                if (COMB && cnt > 0) {
+                    un.put_sums(cnt, sum_of(cnt), warp_sum3_split(s0, s2, sz, un.lane), 4);
+                    un.sync();
+                    un.add_rows((cnt - 1) / 32 * 32 + 1, cnt, sum_of);
+                }
+            };
+            auto beta = [&](auto comb_tag, int tb, int cnt, int ub, int lev0) {
+                constexpr bool COMB = decltype(comb_tag)::value;
+                auto sum_of = [&](int v) { return sums + (tb - v); };
+                int off = 0, P = P_s[tb];
+                float s0 = 0.f, s2 = 0.f, sz = 0.f;
+                if (COMB)
+                    for (int c = 0; c < C::RD - 1; ++c) ring.issue(tb - c, c < cnt);
+                for (int v = 1; v <= cnt; ++v) {
+                    const int t = tb - v + 1, cur = (ub + v - 1) % C::NBUF, nxt = (ub + v) % C::NBUF;
+                    const bool send = !COMB || v < cnt;
+                    if (COMB) { ring.issue(t - (C::RD - 1), v + C::RD - 1 <= cnt); ring.wait(); }
+                    if (v > 1) un.wait_inputs(cur);
+                    if (send) un.arm(v, nxt, drop_hook && PHASE != 2 && v == 1);
+                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + 2 * un.xl;
+                    const float4 sp = step[t - 1];
+                    off = un.template offset<LIN>(v, off, lev0);
+                    P += off;
+                    if (un.i == 0) P_s[t - 1] = P;
+                    const float kap = COMB ? z.kappa<LIN>(O_s[t] + P) : 0.f;
+                    if (COMB && v > 1) un.put_sums(v - 1, sum_of(v - 1), warp_sum3_split(s0, s2, sz, un.lane), 4);
+                    const float2 w2 = splat2(sp.x), v2 = splat2(sp.y), off2 = splat2((float)off), gd2 = splat2(sp.z * isl), g2 = splat2(sp.z), gs2 = splat2(sp.w);
+                    const float2 u2 = splat2(0.5f * (sp.x + sp.y));
+                    float2 S0 = make_float2(0.f, 0.f), S2 = S0, ZS = S0;
+                    float tmax = NONE;
+#pragma unroll
+                    for (int u = 0; u < BPT; ++u) {
+                        const float4 m01 = in[2 * u * C::STR], m23 = in[2 * u * C::STR + 1];
+                        const float Mb[4] = {m01.x, m01.z, m23.x, m23.z}, Yb[4] = {m01.y, m01.w, m23.y, m23.w};
+                        if (!COMB && (G == 4 || un.h == 0)) {
+                            float4 *row = hist4 + (size_t)(t - 1) * (ARR * C::NB) + un.x + u * C::STR;
+                            row[0] = make_float4(Mb[0], Mb[1], Mb[2], Mb[3]); row[C::NB] = make_float4(Yb[0], Yb[1], Yb[2], Yb[3]);
+                        }
+                        float2 Ah[2], Bh[2];
+                        if (COMB) {
+                            const float4 a4 = ring.row(t, 0, u), b4 = ring.row(t, 1, u);
+                            Ah[0] = make_float2(a4.x, a4.y); Ah[1] = make_float2(a4.z, a4.w);
+                            Bh[0] = make_float2(b4.x, b4.y); Bh[1] = make_float2(b4.z, b4.w);
+                            if (G == 2 && un.h) { Ah[0] = Ah[1]; Bh[0] = Bh[1]; }
+                        }
+                        float oM[G], oB[G];
+#pragma unroll
+                        for (int jp = 0; jp < G / 2; ++jp) {
+                            float2 d[4], e[4], mx = make_float2(0.f, 0.f);
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                const float2 c = tab[u][jp * 4 + b];
+                                d[b] = sub2(c, w2);
+                                const float2 r = RC ? sub2(c, v2) : d[b];
+                                e[b] = LIN ? mul2(ex2n2(fma2(d[b], r, off2)), splat2(Mb[b])) : sub2(splat2(Mb[b] - off2.x), mul2(d[b], r));
+                            }
+                            if (!LIN) {
+                                mx = max_pairs<4>(e);
+#pragma unroll
+                                for (int b = 0; b < 4; ++b) e[b] = ex2f2(sub2(e[b], mx));
+                            }
+                            float2 f, fA, fg, nf, nfA;
+                            if (COMB) {
+                                f = LIN ? mul2(Ah[jp], splat2(kap)) : ex2f2(add2(add2(Ah[jp], mx), splat2(kap)));
+                                fA = LIN ? mul2(Bh[jp], splat2(kap)) : mul2(f, Bh[jp]);
+                                fg = mul2(f, g2); nf = mul2(f, ni2); nfA = mul2(fA, ni2);
+                            }
+                            float2 sum, ya, zs;
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                const float2 y = fma2(gd2, d[b], splat2(Yb[b]));
+                                sum = b == 0 ? e[b] : add2(sum, e[b]);
+                                ya = b == 0 ? mul2(e[b], y) : fma2(e[b], y, ya);
+                                if (COMB) {
+                                    const float2 zz = fma2(RC ? sub2(tab[u][jp * 4 + b], u2) : d[b], fma2(nf, y, nfA), fg);
+                                    zs = b == 0 ? mul2(e[b], zz) : fma2(e[b], zz, zs);
+                                    if (ACC) acc[u][jp * 4 + b] = fma2(e[b], zz, acc[u][jp * 4 + b]);
+                                }
+                            }
+                            const float2 om = LIN ? sum : add2(mx, lg2f2(sum));
+                            const float2 obt = fma2(ya, rcpf2(make_float2(fmaxf(sum.x, 1e-37f), fmaxf(sum.y, 1e-37f))), gs2);
+                            oM[2 * jp] = om.x; oM[2 * jp + 1] = om.y;
+                            oB[2 * jp] = obt.x; oB[2 * jp + 1] = obt.y;
+                            if (COMB) {
+                                S0 = fma2(f, sum, S0);
+                                S2 = fma2(fA, sum, fma2(f, ya, S2));
+                                ZS = add2(ZS, zs);
+                            }
+                            tmax = max3f(tmax, om.x, om.y);
+                        }
+                        if (send) {
+#pragma unroll
+                            for (int o = 0; o < G; ++o) {
+                                if constexpr (CL > 1) {
+                                    if (un.pr.live) st_async_v2(dst.b[o] + u * dst.STEP_B + (uint32_t)nxt * un.TX_MSG, oM[o], oB[o], dst.bbar[o] + 8u * nxt);
+                                } else {
+                                    *reinterpret_cast<float2 *>(un.msg(nxt) + dst.b[o] + u * dst.STEP_B) = make_float2(oM[o], oB[o]);
+                                }
+                            }
+                        }
+                    }
+                    if (COMB) { s0 = S0.x + S0.y; s2 = S2.x + S2.y; sz = ZS.x + ZS.y; }
+                    un.post_max(v, tmax);
+                    un.end_step(v, COMB, sum_of);
+                }
+                if (COMB && cnt > 0) {
+                    un.put_sums(cnt, sum_of(cnt), warp_sum3_split(s0, s2, sz, un.lane), 4);
+                    un.sync();
+                    un.add_rows((cnt - 1) / 32 * 32 + 1, cnt, sum_of);
+                }
+            };
+            constexpr std::true_type YES{};
+            constexpr std::false_type NO{};
+            if (PHASE != 2) {
+                if (un.dir == 0) {
+                    const float a1 = LIN ? pow2i(X_MEET) : 0.f, aa1 = LIN ? step[0].w * a1 : step[0].w;
+                    for (int f = un.i; f < PL; f += NT) { un.msg(0)[f] = a1; un.msg(0)[PL + f] = aa1; }
+                } else {
+                    const float m1 = LIN ? pow2i(X_MEET) : 0.f;
+                    for (int f = un.i; f < C::BUF; f += NT) un.msg(0)[f] = (f & 1) ? 0.f : m1;      // M_n, Bt_n = 0
+                }
+                if (tid == 0) { O_s[1] = -X; P_s[n] = -X; }
+                if (CL > 1) cluster_sync(); else __syncthreads();
+                if (un.dir == 0) alpha(NO, 1, m, 0, 0);
+                else beta(NO, n, n - m, 0, 0);
+            }
+            const int fin = un.dir == 0 ? m : n - m;
+            if (PHASE == 1) {
+                if (fin > 0) un.wait_inputs(fin % C::NBUF);
+                const float *last = un.msg(fin % C::NBUF);
+                for (int f = un.i; f < C::BUF; f += NT) {
+                    if (un.dir == 0) endA[(f / NBC) * C::NB + (int)un.rank * NBC + f % NBC] = last[f];     // (AA follows A: Q = 4 NB)
+                    else endM[(int)un.rank * C::BUF + f] = last[f];
+                }
+                if (un.rank == 0) {
+                    if (un.dir == 0) for (int t = 1 + tid; t <= m + 1; t += NT) aux[t] = O_s[t];
+                    else for (int t = m + tid; t <= n; t += NT) aux[n + 2 + t] = P_s[t];
+                }
+                return;
+            }
+            const int ub = PHASE == 2 ? 0 : fin;
+            if (PHASE == 2) {
+                for (int t = 1 + tid; t <= m + 1; t += NT) O_s[t] = aux[t];
+                for (int t = m + tid; t <= n; t += NT) P_s[t] = aux[n + 2 + t];
+                for (int f = un.i; f < C::BUF; f += NT)
+                    un.msg(0)[f] = un.dir == 0 ? endA[(f / NBC) * C::NB + (int)un.rank * NBC + f % NBC] : endM[(int)un.rank * C::BUF + f];
+            }
+            __syncthreads();
+            const int e = O_s[m + 1] + P_s[m];
+            if (PHASE == 2) {
+                const int q0 = (int)un.rank * (C::Q / CL);
+                meet_z<LIN>(un, C::Q / CL, [&](int f) { return endA[q0 + f]; }, [&](int f) { return endM[2 * (q0 + f)]; }, e, &z);
+            } else {
+                const float *a = smem + C::OFF_MSG + (m % C::NBUF) * C::BUF, *b = smem + C::DIR_FLOATS + C::OFF_MSG + ((n - m) % C::NBUF) * C::BUF;
+                meet_z<LIN>(un, C::Q, [&](int f) { return a[f]; }, [&](int f) { return b[2 * f]; }, e, &z);
+            }
+            float mv = NONE;
+            for (int f = un.i; f < PL; f += NT) mv = fmaxf(mv, un.msg(ub % C::NBUF)[un.dir == 0 ? f : 2 * f]);
+            const int lev0 = reg_level<LIN>(un.template reduce<true>(mv, 4), X_MEET);
+            if (PHASE == 0) __syncthreads();                     // (the sweeps overwrite what the other side has just read)
+            if (!LIN && un.rank == 0 && un.i == 0) diag_check_finite(p.diag, z.lz);
+            if (un.dir == 0) alpha(YES, m + 1, n - m, ub, lev0);
+            else beta(YES, m, m, ub, lev0);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            if (CL > 1) cluster_sync(); else __syncthreads();
+            for (int t = out0; t < out1; t += CL * TH) {
+                float a0, a2, az;
+                if (CL > 1) {
+                    a0 = a2 = az = 0.f;
+#pragma unroll
+                    for (int r = 0; r < CL; ++r) {
+                        const uint32_t at = mapa_u32(smem_u32(sums + t), (uint32_t)r);
+                        const float2 s = ld_cluster_f2(at), q = ld_cluster_f2(at + 8u);
+                        a0 += s.x; a2 += s.y; az += q.x;
+                    }
+                } else {
+                    a0 = sums[t].x; a2 = sums[t].y; az = sums[t].z;
+                }
+                const float i0 = grad_up(scale_s[0]) / a0;
+                p.gW[blk * n + t] = (__ldg(g + t) - az * i0) + (a2 * i0) * (__ldg(w + t) - __ldg(sf + t)) * p.invT;
+                defect = fmaxf(defect, fabsf(a0 - 1.f));
+            }
+        };
+        if (p.lin_x < 0 || p.lin_flag[blk]) run(std::false_type{}, std::true_type{});
+        else if (recentre) run(std::true_type{}, std::true_type{});
+        else run(std::true_type{}, std::false_type{});
+        if (!C::SPLIT) __syncthreads();
+    }
+    if (PHASE != 1) {
+        if (ACC) write_acc();
+        defect = warp_max(defect);
+        if (un.lane == 0) diag_max(&p.diag->max_defect, defect);
+    }
+    if (CL > 1) {
+        cluster_sync();                                          // no CTA leaves while a peer may still address its shared memory
+        if (*un.pr.abort_flag) settle_after_abort();
+    }
+}
+
+}  // namespace bcjr

@@ -1,0 +1,139 @@
+// What the launches of the two-ended kernels share (bcjr_meet.cu: forward, bcjr_meet_bwd.cu: backward).
+#pragma once
+#include "bcjr_meet.h"
+
+#include "bcjr_meet.cuh"
+
+namespace bcjr {
+namespace {
+
+// configuration of a trellis: CTAs of a cluster, outputs of a butterfly per thread, butterflies per thread, split form
+template <int LB, int FORM, bool BWD>
+struct MeetOf { using C = void; };
+template <bool BWD> struct MeetOf<8, 0, BWD> { using C = MeetCfg<8, 1, 2, 1, BWD, false>; };
+template <bool BWD> struct MeetOf<9, 0, BWD> { using C = MeetCfg<9, 1, 4, 1, BWD, false>; };
+template <bool BWD> struct MeetOf<10, 0, BWD> { using C = MeetCfg<10, 1, 2, 1, BWD, false>; };
+template <bool BWD> struct MeetOf<11, 0, BWD> { using C = MeetCfg<11, 1, 4, 1, BWD, false>; };
+template <bool BWD> struct MeetOf<12, 0, BWD> { using C = MeetCfg<12, 1, 4, 1, BWD, false>; };
+template <bool BWD> struct MeetOf<12, 1, BWD> { using C = MeetCfg<12, 1, 2, 1, BWD, true>; };
+template <bool BWD> struct MeetOf<13, 0, BWD> { using C = MeetCfg<13, 1, 4, 1, BWD, true>; };
+template <bool BWD> struct MeetOf<14, 0, BWD> { using C = MeetCfg<14, 2, 4, 1, BWD, true>; };
+template <bool BWD> struct MeetOf<15, 0, BWD> { using C = MeetCfg<15, 4, 4, 1, BWD, true>; };
+template <bool BWD> struct MeetOf<16, 0, BWD> { using C = MeetCfg<16, 8, 4, 1, BWD, true>; };
+template <bool BWD> struct MeetOf<16, 1, BWD> { using C = MeetCfg<16, 4, 4, 2, BWD, true>; };
+
+template <typename C, typename Kern>
+cudaError_t config(Kern kern, size_t smem, int grid, cudaStream_t st, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr)
+{
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C::CL;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg->gridDim = dim3((unsigned)grid, 1, 1);
+    cfg->blockDim = dim3((unsigned)C::THREADS, 1, 1);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = st;
+    cfg->attrs = attr;
+    cfg->numAttrs = C::CL > 1 ? 1 : 0;
+    return cudaSuccess;
+}
+
+// f(C{}) with the configuration of (Lb, form)
+template <int LB, int FORM, bool BWD, typename F>
+cudaError_t with(F f)
+{
+    using C = typename MeetOf<LB, FORM, BWD>::C;
+    if constexpr (std::is_void_v<C>) return cudaErrorInvalidValue;
+    else return f(C{});
+}
+template <bool BWD, int FORM, typename F>
+cudaError_t dispatch_form(int Lb, F f)
+{
+    switch (Lb) {
+        case 8: return with<8, FORM, BWD>(f);
+        case 9: return with<9, FORM, BWD>(f);
+        case 10: return with<10, FORM, BWD>(f);
+        case 11: return with<11, FORM, BWD>(f);
+        case 12: return with<12, FORM, BWD>(f);
+        case 13: return with<13, FORM, BWD>(f);
+        case 14: return with<14, FORM, BWD>(f);
+        case 15: return with<15, FORM, BWD>(f);
+        case 16: return with<16, FORM, BWD>(f);
+    }
+    return cudaErrorInvalidValue;
+}
+template <bool BWD, typename F>
+cudaError_t dispatch(int Lb, int form, F f)
+{
+    return form == 0 ? dispatch_form<BWD, 0>(Lb, f) : dispatch_form<BWD, 1>(Lb, f);
+}
+
+template <typename C>
+auto last_kernel()
+{
+    constexpr int PHASE = C::SPLIT ? 2 : 0;
+    if constexpr (C::BWD) return meet_bwd_kernel<C, true, PHASE>;
+    else return meet_fwd_kernel<C, PHASE>;
+}
+
+template <typename C>
+cudaError_t resident(int n, int num_sms, int *sides)
+{
+    auto kern = last_kernel<C>();
+    const size_t smem = C::smem_bytes(n);
+    *sides = 0;
+    if (smem > 232448 || n > C::MAX_N) return cudaSuccess;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cudaError_t e = config<C>(kern, smem, C::CL * num_sms, nullptr, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    int units = 0;
+    if (C::CL > 1) e = cudaOccupancyMaxActiveClusters(&units, kern, &cfg);
+    else {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&units, kern, C::THREADS, smem);
+        units *= num_sms;
+    }
+    *sides = C::SPLIT ? units : 2 * units;
+    return e;
+}
+
+template <typename C, typename Kern, typename P>
+cudaError_t launch(Kern kern, const P &p, const MeetPlan &plan, const MeetScratch &ms, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    const cudaError_t e = config<C>(kern, plan.smem, plan.grid, st, &cfg, attr);
+    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, kern, p, ms);
+}
+
+// sides in flight of (Lb, form); plan of a call
+template <bool BWD>
+int meet_resident_of(int Lb, int form, int n, int num_sms)
+{
+    int sides = 0;
+    const cudaError_t e = dispatch<BWD>(Lb, form, [&](auto c) { return resident<decltype(c)>(n, num_sms, &sides); });
+    if (e != cudaSuccess) { cudaGetLastError(); return 0; }
+    return sides;
+}
+template <bool BWD>
+MeetPlan meet_plan_of(int Lb, int form, int n, int64_t B, int resident)
+{
+    MeetPlan plan;
+    dispatch<BWD>(Lb, form, [&](auto c) {
+        using C = decltype(c);
+        plan.split = C::SPLIT;
+        const int64_t blocks = C::SPLIT || 2 * B < resident ? B : resident / 2;    // (the split form's launches have a cluster for every side)
+        plan.grid = (int)(blocks * (C::SPLIT ? 2 * C::CL : 1));
+        plan.parts = (int)(2 * blocks);
+        plan.smem = C::smem_bytes(n);
+        plan.hist_floats = (size_t)blocks * C::block_floats(n);
+        plan.aux_ints = C::SPLIT ? (size_t)B * 2 * (n + 2) : 0;
+        return cudaSuccess;
+    });
+    return plan;
+}
+
+}  // namespace
+}  // namespace bcjr

@@ -283,7 +283,8 @@ struct RegDest {
 };
 
 // ---------------------------------------------------------------------------- forward
-// p.lin_x < 0: log-domain messages.  With p.list the kernel runs the listed blocks, provided their number is at most p.list_max.
+// p.lin_x < 0: log-domain messages.  With p.list the kernel runs the listed blocks, provided their number is at most p.list_max; with
+// p.only_flagged those whose p.lin_flag is set.
 template <int LB, int CL>
 __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL, false>::MIN_CTAS) fwd_reg_kernel(FwdParams p)
 {
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
     float2 tab[2][4];
     reg_load_table<C>(p.cb, x, tab);
     float c_lo, c_hi;
-    if (p.list) { c_lo = p.diag->c_lo; c_hi = p.diag->c_hi; }
+    if (p.list || p.only_flagged) { c_lo = p.diag->c_lo; c_hi = p.diag->c_hi; }
     else {
         reg_table_range<C>(p, rb, tab, &c_lo, &c_hi);
         if (blockIdx.x == 0 && tid == 0) { p.diag->c_lo = c_lo; p.diag->c_hi = c_hi; }
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
 
     for (int64_t it = cid; it < nblk; it += ncid) {
         const int64_t blk = p.list ? (int64_t)p.list[1 + it] : it;
+        if (p.only_flagged && !p.lin_flag[blk]) continue;           // (a cluster's CTAs alike)
         const float *w = p.W + blk * n;
         int outside = 0;
         for (int t = tid; t < n; t += NT) {
