@@ -1636,6 +1636,27 @@ bcjr_status backward_blocks(bcjr_ctx *ctx, const BwdParams &p, float *grad_codeb
     return BCJR_OK;
 }
 
+template <int B, bool SIGNS>
+cudaError_t launch_fwht_next_t(float *W, const RhtSigns &s, int lt, float scale, cudaStream_t st)
+{
+    const size_t smem = B > 5 ? RHT_TILE_SMEM : 0;
+    if (B > 5) {
+        const cudaError_t e = cudaFuncSetAttribute(fwht_next_kernel<B, SIGNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    const unsigned grid = B > 5 ? 1u << (lt - RHT_TILE_BITS) : 1u << (lt - B - 8);
+    fwht_next_kernel<B, SIGNS><<<grid, B > 5 ? RHT_THREADS : 256, smem, st>>>(W, s, scale);
+    return cudaGetLastError();
+}
+template <int B>
+cudaError_t launch_fwht_next(int b, float *W, const RhtSigns &s, int lt, float scale, bool signs, cudaStream_t st)
+{
+    if constexpr (B < 1) return cudaErrorInvalidValue;
+    else {
+        if (b != B) return launch_fwht_next<B - 1>(b, W, s, lt, scale, signs, st);
+        return signs ? launch_fwht_next_t<B, true>(W, s, lt, scale, st) : launch_fwht_next_t<B, false>(W, s, lt, scale, st);
+    }
+}
 }  // namespace
 
 extern "C" {
@@ -2086,14 +2107,16 @@ bcjr_status bcjr_rht(bcjr_ctx *ctx, const float *W, float *out, int m, int n, co
     }
     // the low 14 index bits, then the remaining row-index bits in passes of at most ten
     int o = RHT_TILE_BITS - ln;
-    CU(cudaFuncSetAttribute(fwht_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RHT_TILE_SMEM));
-    fwht_tile_kernel<<<1u << (lt - RHT_TILE_BITS), RHT_THREADS, RHT_TILE_SMEM, st>>>(W, out, s, o == lm ? scale : 1.f, !inverse ? 1 : o == lm ? 2 : 0);
+    auto tile = !inverse ? fwht_tile_kernel<1> : o == lm ? fwht_tile_kernel<2> : fwht_tile_kernel<0>;
+    CU(cudaFuncSetAttribute(tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RHT_TILE_SMEM));
+    tile<<<1u << (lt - RHT_TILE_BITS), RHT_THREADS, RHT_TILE_SMEM, st>>>(W, out, s, o == lm ? scale : 1.f);
     CU(cudaGetLastError());
     ctx->launches += 1;
     for (int passes = (lm - o + 9) / 10; passes > 0; --passes) {
         const int b = (lm - o + passes - 1) / passes;
         const bool last = passes == 1;
-        CU(launch_fwht_cols<10>(b, out, s, lm, o, last ? scale : 1.f, inverse && last ? 2 : 0, st));
+        if (o + ln == RHT_TILE_BITS) CU(launch_fwht_next<10>(b, out, s, lt, last ? scale : 1.f, inverse && last, st));
+        else CU(launch_fwht_cols<10>(b, out, s, lm, o, last ? scale : 1.f, inverse && last ? 2 : 0, st));
         ctx->launches += 1;
         o += b;
     }

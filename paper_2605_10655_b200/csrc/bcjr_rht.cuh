@@ -9,16 +9,31 @@
 // Fast Walsh-Hadamard transform.  The rotation of a row-major matrix is ONE transform over the bits of the linear index, and
 // any subset of the bits can be taken in any order.  A matrix of 2^14 elements or more takes two kernels: the low 14 bits
 // (the row transform and the lowest column bits: contiguous tiles of 64 KB, fwht_tile_kernel), then the remaining row-index bits,
-// ten at a time (tiles of 2^B rows x 16 columns or more, fwht_cols_kernel).  Each reads and writes the matrix once.  A thread
+// ten at a time (tiles of 2^B rows x 16 columns or more: fwht_next_kernel, beyond 2^24 elements then fwht_cols_kernel).  Each reads and writes the matrix once.  A thread
 // holds 32 elements and runs five butterfly stages on them in registers, so that a tile passes through shared memory twice
 // in the first kernel and once in the second.  Smaller matrices are one radix-8 transform in shared memory
 // (fwht_small_kernel).  8192 x 2048, rotation and its inverse with group scales between: 313 -> 170 us
-// (a pass over the matrix for every three bits before).
+// (a pass over the matrix for every three bits before), 160 with addresses that are constants, 146 with streaming loads (rht_stream4).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace bcjr {
+
+// Four floats that this kernel is the last to want for a while: their lines go first when the L2 needs room, so that what the kernel
+// writes is still there for the next one (a 67 MB matrix and its image do not both fit 126 MB).
+__device__ __forceinline__ uint64_t rht_stream_policy()
+{
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
+}
+__device__ __forceinline__ float4 rht_stream4(const float4 *p, uint64_t policy)
+{
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(policy) : "memory");
+    return v;
+}
 
 // stages for bits s with first <= s < 3 of an 8-point transform (first = 0: all three)
 template <typename T>
@@ -107,26 +122,30 @@ constexpr size_t RHT_TILE_SMEM = ((size_t)(1 << RHT_TILE_BITS) + (1 << (RHT_TILE
 // four floats of padding per 128: the lanes of the second pass differ in bits 0, 1 and 7 .. 9
 __device__ __forceinline__ int rht_tile_pad(int e) { return e + ((e >> 7) << 2); }
 
-// Index bits 0 .. 13 of tile blockIdx.x (2^14 consecutive elements).  sign_mode 1: inputs times their signs; 2: outputs.
-__global__ void __launch_bounds__(RHT_THREADS, 2) fwht_tile_kernel(const float *in, float *out, RhtSigns s, float scale, int sign_mode)
+// Index bits 0 .. 13 of tile blockIdx.x (2^14 consecutive elements).  MODE 1: inputs times their signs; 2: outputs.
+template <int MODE>
+__global__ void __launch_bounds__(RHT_THREADS, 2) fwht_tile_kernel(const float *in, float *out, RhtSigns s, float scale)
 {
     extern __shared__ __align__(16) float tile[];
     const int t = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x << RHT_TILE_BITS;
+    const uint64_t policy = rht_stream_policy();
     float v[32];
     // bits 0, 1 (inside a float4) and 11 .. 13: element 4 (t + 512 i) + j
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const float4 f = reinterpret_cast<const float4 *>(in + base)[t + 512 * i];
+        const float4 f = rht_stream4(reinterpret_cast<const float4 *>(in + base) + t + 512 * i, policy);
         v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
     }
-    if (sign_mode == 1) {
-        const int64_t cm = ((int64_t)1 << s.ln) - 1;
+    if (MODE == 1) {
+        const int cm = (1 << s.ln) - 1;
+        const float *rows = s.rows + (base >> s.ln);             // (a tile starts with a row, or inside one: then it has no other)
+        const int in_row = (int)(base & cm);
+        float4 c = __ldg(reinterpret_cast<const float4 *>(s.cols + ((in_row + 4 * t) & cm)));
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int64_t at = base + 4 * (t + 512 * i);
-            const float4 c = __ldg(reinterpret_cast<const float4 *>(s.cols + (at & cm)));
-            const float r = __ldg(s.rows + (at >> s.ln));
+            if (i > 0 && s.ln > 11) c = __ldg(reinterpret_cast<const float4 *>(s.cols + ((in_row + 4 * t + 2048 * i) & cm)));
+            const float r = __ldg(rows + ((in_row + 4 * t + 2048 * i) >> s.ln));
             v[4 * i] *= c.x * r; v[4 * i + 1] *= c.y * r; v[4 * i + 2] *= c.z * r; v[4 * i + 3] *= c.w * r;
         }
     }
@@ -155,12 +174,62 @@ __global__ void __launch_bounds__(RHT_THREADS, 2) fwht_tile_kernel(const float *
 #pragma unroll
         for (int j = 0; j < 16; ++j) u[j] = p3[j * (128 + 4) + x * (8192 + 256)];
         fwht_reg<4>(u);
-        if (sign_mode == 2) {
+        if (MODE == 2) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) u[j] *= s.of(base + e0 + (j << 7) + (x << 13));
         }
 #pragma unroll
         for (int j = 0; j < 16; ++j) q[(j << 7) + (x << 13)] = u[j] * scale;
+    }
+}
+
+// Index bits [14, 14 + B), in place: the pass behind the tile kernel.  A block takes 2^B elements 2^14 apart x 2^(14 - B) side by side
+// (B > 5: the top five bits, then the others, through shared memory) or a thread 2^B (B <= 5, in registers).  The distance is
+// a constant here, so that an element's address is the thread's plus a constant: with the distance in a register (fwht_cols_kernel) the
+// addresses were most of the instructions, 36.5 -> 25.6 us for 2^24 elements, a copy of which takes 28.1.
+template <int B, bool SIGNS>
+__global__ void __launch_bounds__(B > 5 ? RHT_THREADS : 256, 2) fwht_next_kernel(float *W, RhtSigns s, float scale)
+{
+    constexpr int LT = RHT_TILE_BITS;
+    constexpr int64_t ST = (int64_t)1 << LT;
+    const int t = threadIdx.x;
+    auto sign = [&](int64_t at) { return SIGNS ? scale * __ldg(s.rows + (at >> s.ln)) : scale; };
+    if constexpr (B <= 5) {
+        const int64_t q = (int64_t)blockIdx.x * blockDim.x + t;
+        const int64_t base = (q & (ST - 1)) | ((q >> LT) << (LT + B));
+        float v[1 << B], *p = W + base;
+#pragma unroll
+        for (int j = 0; j < (1 << B); ++j) v[j] = p[j * ST];
+        fwht_reg<B>(v);
+        if (SIGNS) scale *= __ldg(s.cols + (base & (((int64_t)1 << s.ln) - 1)));
+#pragma unroll
+        for (int j = 0; j < (1 << B); ++j) p[j * ST] = v[j] * sign(base + j * ST);
+    } else {
+        constexpr int L = B - 5, LC = LT - B, C = 1 << LC, PITCH = (1 << (L + LC)) + 16;     // (see fwht_cols_kernel)
+        extern __shared__ __align__(16) float tile[];
+        const int cl = t & (C - 1), r = t >> LC;
+        const int64_t base = (int64_t)(blockIdx.x & ((1 << B) - 1)) * C + ((int64_t)(blockIdx.x >> B) << (LT + B)) + cl;
+        float v[32];
+        const float *p = W + base + r * ST;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = p[j * (ST << L)];
+        fwht_reg<5>(v);
+        float *p1 = tile + (r << LC) + cl;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) p1[j * PITCH] = v[j];
+        __syncthreads();
+        if (SIGNS) scale *= __ldg(s.cols + (base & (((int64_t)1 << s.ln) - 1)));
+#pragma unroll
+        for (int q = 0; q < (32 >> L); ++q) {
+            const int rh = r + (q << L);
+            const int64_t at = base + (int64_t)rh * (ST << L);
+            float u[1 << L], *o = W + at;
+#pragma unroll
+            for (int j = 0; j < (1 << L); ++j) u[j] = tile[rh * PITCH + (j << LC) + cl];
+            fwht_reg<L>(u);
+#pragma unroll
+            for (int j = 0; j < (1 << L); ++j) o[j * ST] = u[j] * sign(at + j * ST);
+        }
     }
 }
 
@@ -230,8 +299,9 @@ __global__ void __launch_bounds__(B > 5 ? RHT_THREADS : 256, 2) fwht_cols_kernel
 __global__ void __launch_bounds__(256) group_scale_kernel(const float *W, float *scales, float *out, int64_t groups)
 {
     const int64_t quads = 4 * groups, step = (int64_t)gridDim.x * blockDim.x;
+    const uint64_t policy = rht_stream_policy();
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < quads; q += step) {      // (whole groups of lanes: quads and step are multiples of 4)
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(W) + q);
+        const float4 v = rht_stream4(reinterpret_cast<const float4 *>(W) + q, policy);
         const unsigned mask = __activemask();
         float ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
         ss += __shfl_xor_sync(mask, ss, 1);
@@ -247,8 +317,9 @@ __global__ void __launch_bounds__(256) group_scale_kernel(const float *W, float 
 __global__ void __launch_bounds__(256) group_unscale_kernel(const float *Ws, const float *scales, float *out, int64_t groups)
 {
     const int64_t quads = 4 * groups, step = (int64_t)gridDim.x * blockDim.x;
+    const uint64_t policy = rht_stream_policy();
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < quads; q += step) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(Ws) + q);
+        const float4 v = rht_stream4(reinterpret_cast<const float4 *>(Ws) + q, policy);
         const float sc = __ldg(scales + (q >> 2));
         reinterpret_cast<float4 *>(out)[q] = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
     }

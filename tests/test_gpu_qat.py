@@ -161,3 +161,31 @@ def test_group_scales_and_their_inverse(ctx):
     back = ctx.bcjr_group_unscale(Ws, scales)
     ctx.sync_status()
     np.testing.assert_allclose(back.cpu().numpy(), W, rtol=3e-7, atol=0)
+
+
+@pytest.mark.parametrize("m,n", [(128, 4096), (256, 4096), (512, 4096), (8192, 512), (1024, 8192), (4096, 4096), (8192, 4096), (8192, 8), (1 << 20, 32)])
+def test_rotation_of_larger_matrices(ctx, m, n):
+    # 2^16 to 2^25 elements: every number of bits the pass behind the tiles takes (2 to 10, and two passes), in registers and through shared
+    # memory, against a transform in float64; the sums have up to 25 terms' rounding, a few 2^-24 of the result's scale.
+    import torch
+    dev = torch.device("cuda", ctx.device)
+    gen = torch.Generator(device="cuda").manual_seed(m + n)
+    W = torch.randn(m, n, generator=gen, device=dev)
+    sL, sR = (torch.where(torch.rand(k, generator=gen, device=dev) < 0.5, -1.0, 1.0) for k in (m, n))
+
+    def wht(x):                                          # over all bits of the linear index
+        x = x.reshape(-1)
+        h = 1
+        while h < x.numel():
+            y = x.reshape(-1, 2, h)
+            x = torch.stack((y[:, 0] + y[:, 1], y[:, 0] - y[:, 1]), dim=1).reshape(-1)
+            h *= 2
+        return x.reshape(m, n) / (float(m) * n) ** 0.5
+    signs = sL.double()[:, None] * sR.double()[None, :]
+    ref = wht(W.double() * signs)
+    out = ctx.bcjr_rht(W, sL, sR)
+    assert float((out.double() - ref).abs().max()) <= 25 * 2.0 ** -24 * float(ref.abs().max())
+    back = ctx.bcjr_rht(out, sL, sR, inverse=True)
+    ref = wht(out.double()) * signs
+    assert float((back.double() - ref).abs().max()) <= 25 * 2.0 ** -24 * float(ref.abs().max())
+    assert ctx.sync_status().device_status == 0
