@@ -1214,7 +1214,7 @@ bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     return ctx->fwd_judged ? launch_bwd_warp_any(ctx, p, grad_codebook, st) : BCJR_OK;
 }
 
-// Few blocks, k = 2: the register kernels from both ends of a block (bcjr_meet.cuh).
+// Few blocks: the register kernels from both ends of a block (bcjr_meet.cuh).
 int meet_sides(bcjr_ctx *ctx, int form, int Lb, int n)
 {
     int least = 0;
@@ -1234,12 +1234,19 @@ int meet_sides(bcjr_ctx *ctx, int form, int Lb, int n)
 //   * 2^16: clusters of eight while all sides are in flight, 7 blocks 1019 -> 595.  Clusters of four up to three waves of them, the last blocks on
 //     clusters of eight if those can take them: 8 1019 -> 926, 16 1754 -> 937, 33 2360 -> 1846, 40 2932 -> 2442, 49 2933 -> 2745.  Between,
 //     where the one-ended kernels need two waves as well, they keep the call (24 blocks 1779 us against 1814, 17 1754 against 1533).
+//   * 2^16 at k = 3: clusters of eight, four waves of them (seven blocks and a half each): 7 blocks 3166 -> 685 us, 14 3168 -> 1345, 30 3180 -> 2663,
+//     37 3183 -> 3203 (T = 0.015: 7 3454 -> 715).  Blocks of less than 16 weights stay with the chunked kernels (0.2 ms), whose tests run there.
 // With log messages the same (T = 0.015: 16 blocks of 2^16 2053 -> 1094, 49 3832 -> 3214, 148 of 2^12 558 -> 477).
 // last: the last blocks of a call, instead of a wave of the chunked kernels that they do not fill (both calls, 149 blocks 6626 -> 4418 us, 171
-// 6645 -> 5374, 197 6805 -> 6608, 600 17846 -> 15983).
-bool meet_count(bcjr_ctx *ctx, int Lb, int n, int64_t B, bool last, int64_t count[MEET_FORMS])
+// 6645 -> 5374, 197 6805 -> 6608, 600 17846 -> 15983; k = 3 149 7241 -> 4829, a fifth wave 7343 -> 7373).
+bool meet_count(bcjr_ctx *ctx, int Lb, int k, int n, int64_t B, bool last, int64_t count[MEET_FORMS])
 {
-    count[0] = count[1] = 0;
+    count[0] = count[1] = count[MEET_K3] = 0;
+    if (k == 3) {
+        const int s3 = n >= 16 ? meet_sides(ctx, MEET_K3, Lb, n) : 0;
+        count[MEET_K3] = B;
+        return 2 * B <= 4 * (int64_t)s3;
+    }
     const int s0 = meet_sides(ctx, 0, Lb, n), s1 = meet_sides(ctx, 1, Lb, n);
     if (s0 == 0) return false;
     if (Lb <= 11) { count[0] = B; return Lb == 8 || B <= (Lb == 9 ? 4 : 1) * (int64_t)ctx->num_sms; }
@@ -1257,16 +1264,16 @@ bool meet_count(bcjr_ctx *ctx, int Lb, int n, int64_t B, bool last, int64_t coun
 // Where the two-ended kernels take over: the whole call (*from = 0), its last blocks, or none (false).
 bool meet_wanted(bcjr_ctx *ctx, const FwdParams &p, int k, int64_t *from, int64_t count[MEET_FORMS])
 {
-    if (k != 2 || p.Lb < 8 || ctx->opt_path == 1 || (ctx->opt_path == 2 && p.Lb != 16) || ctx->opt_fwd_variant != 0) return false;
+    if ((k != 2 && (k != 3 || p.Lb != 16)) || p.Lb < 8 || ctx->opt_path == 1 || (ctx->opt_path == 2 && p.Lb != 16) || ctx->opt_fwd_variant != 0) return false;
     if (ctx->opt_hist_every != 1 && p.Lb == 16 && p.n <= CkptCfg<2>::MAX_N) return false;
     *from = 0;
-    const bool few = p.Lb < 16 || p.B <= reg_resident_cached(ctx, p.Lb, p.n, false);
+    const bool few = p.Lb < 16 || (k == 2 && p.B <= reg_resident_cached(ctx, p.Lb, p.n, false));
     if (!few && ctx->opt_messages != 0) return false;            // (the option names the chunked kernels' messages)
-    if (meet_count(ctx, p.Lb, p.n, p.B, false, count)) return true;
+    if (meet_count(ctx, p.Lb, k, p.n, p.B, false, count)) return true;
     if (p.Lb < 16 || p.B <= ctx->num_sms || p.n > SkewCfg::MAX_N || ctx->opt_max_ctas != 0) return false;
     const int64_t left = p.B % ctx->num_sms;
     *from = p.B - left;
-    return left > 0 && meet_count(ctx, p.Lb, p.n, left, true, count);
+    return left > 0 && meet_count(ctx, p.Lb, k, p.n, left, true, count);
 }
 // Option max_ctas: the split form in launches of as many blocks as that leaves room for, the CTA form on fewer CTAs.
 int64_t meet_chunk(const bcjr_ctx *ctx, const MeetPlan &plan, int64_t B)
@@ -1286,10 +1293,11 @@ MeetPlan meet_part(const bcjr_ctx *ctx, const MeetPlan &plan, int64_t B, int64_t
 bcjr_status launch_fwd_meet(bcjr_ctx *ctx, FwdParams p, int form, bool *ran, cudaStream_t st)
 {
     const MeetPlan plan = meet_fwd_plan(p.Lb, form, p.n, p.B, meet_sides(ctx, form, p.Lb, p.n));
-    const bool lin = lin_wanted(ctx, p.Lb, p.lam2, p.B);
+    const int k = form == MEET_K3 ? 3 : 2;
+    const bool lin = lin_wanted(ctx, p.Lb, p.lam2, p.B, 1, k);
     RegPlan behind;
     size_t hist = plan.hist_floats;
-    if (plan.split && lin) {
+    if (plan.split && lin && k == 2) {
         behind = reg_plan(p.Lb, p.n, p.B, false, reg_resident_cached(ctx, p.Lb, p.n, false), ctx->opt_max_ctas);
         if (behind.hist_floats > hist) hist = behind.hist_floats;
     }
@@ -1298,22 +1306,26 @@ bcjr_status launch_fwd_meet(bcjr_ctx *ctx, FwdParams p, int form, bool *ran, cud
     if ((rc = ensure(ctx, ctx->stepO, plan.aux_ints * 4))) return rc;
     p.hist = (float *)ctx->hist.ptr;
     p.lin_x = lin ? 0 : -1;                                      // (any exponent: the kernels have their own)
-    p.demand = lin_demand_limit(ctx, p.Lb, 2, 1, p.lam2, true, p.B < 6 * (int64_t)ctx->num_sms);
-    p.window = (p.Lb + 1) / 2;
+    p.demand = lin_demand_limit(ctx, p.Lb, k, 1, p.lam2, true, p.B < 6 * (int64_t)ctx->num_sms);
+    p.window = (p.Lb + k - 1) / k;
     const int64_t chunk = meet_chunk(ctx, plan, p.B);
-    for (int64_t b0 = 0; b0 < p.B; b0 += chunk) {
-        FwdParams q = p;
-        q.B = p.B - b0 < chunk ? p.B - b0 : chunk;
-        q.W = p.W + b0 * p.n; q.soft = p.soft + b0 * p.n;
-        if (p.soft_copy) q.soft_copy = p.soft_copy + b0 * p.n;
-        if (p.logZ) q.logZ = p.logZ + b0;
-        if (p.blk_defect) q.blk_defect = p.blk_defect + b0;
-        q.lin_flag = p.lin_flag + b0;
-        CU(meet_forward(q, form, meet_part(ctx, plan, p.B, q.B), (int *)ctx->stepO.ptr, st));
-        ctx->launches += plan.split ? 2 : 1;
+    // split form: behind the linear messages, blocks without a certificate -- in these kernels at k = 3
+    for (int pass = 0; pass < (plan.split && lin && k == 3 ? 2 : 1); ++pass) {
+        if (pass == 1) { p.lin_x = -1; p.only_flagged = true; }
+        for (int64_t b0 = 0; b0 < p.B; b0 += chunk) {
+            FwdParams q = p;
+            q.B = p.B - b0 < chunk ? p.B - b0 : chunk;
+            q.W = p.W + b0 * p.n; q.soft = p.soft + b0 * p.n;
+            if (p.soft_copy) q.soft_copy = p.soft_copy + b0 * p.n;
+            if (p.logZ) q.logZ = p.logZ + b0;
+            if (p.blk_defect) q.blk_defect = p.blk_defect + b0;
+            q.lin_flag = p.lin_flag + b0;
+            CU(meet_forward(q, form, meet_part(ctx, plan, p.B, q.B), (int *)ctx->stepO.ptr, st));
+            ctx->launches += plan.split ? 2 : 1;
+        }
     }
     note(ctx, "fwd_reg");
-    if (plan.split && lin) {
+    if (plan.split && lin && k == 2) {
         p.lin_x = -1;
         p.only_flagged = true;
         CU(reg_forward(p, behind, st));
@@ -1324,7 +1336,9 @@ bcjr_status launch_fwd_meet(bcjr_ctx *ctx, FwdParams p, int form, bool *ran, cud
 // Blocks from `from` on, count[] of them by form.  Where scratch is short the call ends with *ran = false and has run none of them or some.
 bcjr_status launch_fwd_meets(bcjr_ctx *ctx, const FwdParams &p, int64_t from, const int64_t count[MEET_FORMS], bool *ran, cudaStream_t st)
 {
-    bcjr_status rc = lin_buffers(ctx, from + count[0] + count[1]);
+    int64_t total = from;
+    for (int f = 0; f < MEET_FORMS; ++f) total += count[f];
+    bcjr_status rc = lin_buffers(ctx, total);
     if (rc) return rc;
     *ran = true;
     int64_t b0 = from;
@@ -1369,6 +1383,7 @@ bcjr_status launch_bwd_meets(bcjr_ctx *ctx, const BwdParams &p, float *grad_code
         if (rc) return rc;
         int parts = plan.parts;
         RegPlan other;
+        if (!got && form == MEET_K3) return BCJR_ENOMEM;
         if (!got) {                                              // log messages need no gauge in common with the forward call
             other = reg_plan(p.Lb, p.n, B, true, reg_resident_cached(ctx, p.Lb, p.n, true), ctx->opt_max_ctas);
             parts = other.parts;

@@ -1,4 +1,4 @@
-// The register kernels' sweeps (bcjr_reg.cuh: k = 2, butterflies in registers) from both ends of a block at once.
+// The register kernels' sweeps (bcjr_reg.cuh: butterflies in registers) from both ends of a block at once; k = 2, and k = 3 at 2^16 states.
 //
 // The alpha and the beta sweep of a block do not depend on each other until their messages are multiplied.  bcjr_reg.cuh runs one
 // behind the other, 2 n dependent steps, and with few blocks those steps' latency is all a call takes (a step of 2^16 states on
@@ -9,7 +9,7 @@
 //   * CTA form (PHASE 0): both directions in one thread block, a barrier of its own for each, two of the whole block.
 //   * Split form (PHASE 1 and 2): a cluster of CL CTAs per direction and block; the end of the first launch is where the sides meet.  The
 //     first leaves A_{m+1}, M_m and the offsets in global memory.
-// A thread has BPT whole butterflies (G = 4) or half of one (G = 2: two of its four outputs, eight states).
+// A thread has BPT whole butterflies (G = K) or a part of one (G = 2 of its K outputs: eight states at k = 2, sixteen at k = 3).
 // Which form for which trellis, and what it measured: bcjr_meet_launch.cuh.
 //
 // A step of a cluster pays 330 clocks of latency and one clock per 20 bytes that a CTA sends, whatever the width of the
@@ -33,16 +33,18 @@ namespace bcjr {
 constexpr int X_MEET = 50, KAP_MEET = 50;
 constexpr float MEET_DEFECT = 0.75f * LIN_DEFECT;
 
-template <int LB_, int CL_, int G_, int BPT_, bool BWD_, bool SPLIT_>
+template <int LB_, int CL_, int G_, int BPT_, bool BWD_, bool SPLIT_, int KB_ = 2>
 struct MeetCfg {
-    static constexpr int LB = LB_, CL = CL_, G = G_, BPT = BPT_, K = 4, S = 1 << LB, Q = S >> 2, NB = S >> 4;
+    static constexpr int LB = LB_, KB = KB_, CL = CL_, G = G_, BPT = BPT_, K = 1 << KB, S = 1 << LB, Q = S >> KB, NB = S >> (2 * KB);
     static constexpr bool BWD = BWD_, SPLIT = SPLIT_;
     static constexpr int NBC = NB / CL;                        // butterflies of a CTA and direction
     static constexpr int STR = NBC / BPT;                      // from one butterfly of a thread to its next
-    static constexpr int NT = NBC * (4 / G) / BPT, NWARP = NT / 32, NDIR = SPLIT ? 1 : 2, THREADS = NT * NDIR;
+    static constexpr int PARTS = K / G;                        // threads of a butterfly
+    static constexpr int NT = NBC * PARTS / BPT, NWARP = NT / 32, NDIR = SPLIT ? 1 : 2, THREADS = NT * NDIR;
     static constexpr int ARR = BWD ? 2 : 1;
     static constexpr int NBUF = CL == 8 ? 4 : CL > 1 ? 3 : 2;  // clusters of up to four: a CTA's inputs come from all of them, one step back is enough
-    static constexpr int BUF = ARR * 4 * NBC;
+    static constexpr int BUF = ARR * K * NBC, KC = K / 4;      // floats of a message buffer; quadruples of a butterfly's inputs
+    static constexpr int ROW = ARR * KC * NB;                  // float4 of a history row: [ARR][KC][NB]
     static constexpr int RD = BWD && BPT > 1 ? 2 : 4;          // history staging depth in steps
     static constexpr int PW = BWD ? 4 : 2, PROWS = 64;         // posterior sums of the warps, by step
     static constexpr int MAX_N = 1024;
@@ -50,8 +52,8 @@ struct MeetCfg {
     static constexpr int FIT = 65536 / REGS / THREADS;
     static constexpr int MIN_CTAS = FIT < 1 ? 1 : FIT > 16 ? 16 : FIT;
     static constexpr int OFF_MSG = 0;
-    static constexpr int OFF_RING = OFF_MSG + NBUF * BUF;      // float4 [RD][ARR][BPT][NT]
-    static constexpr int OFF_PSUM = OFF_RING + RD * ARR * BPT * NT * 4;
+    static constexpr int OFF_RING = OFF_MSG + NBUF * BUF;      // float4 [RD][ARR][KC][BPT][NT]
+    static constexpr int OFF_PSUM = OFF_RING + RD * ARR * KC * BPT * NT * 4;
     static constexpr int OFF_WMAX = OFF_PSUM + (NWARP > 1 ? PROWS * NWARP * PW : 0);   // [4][16]
     static constexpr int OFF_CMAX = OFF_WMAX + 64;             // [4][8]
     static constexpr int OFF_RED = OFF_CMAX + 32;              // [6][24]: warps' and CTAs' values of a reduction
@@ -63,7 +65,8 @@ struct MeetCfg {
     // per block: rows of history; split form: then A_{m+1} and M_m by group
     __host__ __device__ static constexpr size_t block_floats(int n) { return (size_t)(SPLIT ? n + 2 : n) * ARR * Q; }
     static_assert(LB >= 8 && NT % 32 == 0 && NT <= 512 && THREADS <= 1024, "whole warps");
-    static_assert((G == 4 || (G == 2 && BPT == 1)) && (CL == 1 || (SPLIT && G == 4)) && (BPT == 1 || (BPT == 2 && CL == 4)), "forms");
+    static_assert((KB == 2 && G == 4) || (G == 2 && BPT == 1), "forms");
+    static_assert((CL == 1 || (SPLIT && (KB == 3 || G == 4))) && (BPT == 1 || (BPT == 2 && CL == 4)) && (KB == 2 || CL == 8), "forms");
     static_assert(DIR_FLOATS % 4 == 0 && OFF_MBAR % 2 == 0, "alignment");
 };
 
@@ -75,7 +78,7 @@ struct MeetUnit {
     uint32_t rank;
     Proto pr;
     uint32_t phase;
-    int xl, x, h;                                              // first butterfly (in the CTA, in the block), half of it
+    int xl, x, h;                                              // first butterfly (in the CTA, in the block), part of it
     static constexpr uint32_t TX_MSG = (uint32_t)C::BUF * 4u, TX_MAX = C::CL * 4u;
     __device__ __forceinline__ float *msg(int s) const { return base + C::OFF_MSG + s * C::BUF; }
     __device__ __forceinline__ uint32_t mbar(int s) const { return smem_u32(base + C::OFF_MBAR) + 8u * s; }
@@ -185,33 +188,34 @@ struct MeetUnit {
     }
 };
 
-// Thread's table entries, 2 G pairs a butterfly, each (j, j + 1) of one l: alpha tab[jp G + l], l of the thread's half; beta
-// tab[jp 4 + b], j of its half.
+// Thread's table entries, K G / 2 pairs a butterfly, each (j, j + 1) of one l: alpha tab[jp G + l], l of the thread's part; beta
+// tab[jp K + b], j of its part.
 template <typename C>
 __device__ __forceinline__ int meet_entry(const MeetUnit<C> &un, int u, int e)
 {
-    const int j = un.dir == 0 ? 2 * (e / C::G) : 2 * (e / 4) + un.h * C::G, l = un.dir == 0 ? e % C::G + un.h * C::G : e % 4;
-    return j * C::Q + (un.x + u * C::STR) * 4 + (C::G == 4 ? e % 4 : l);
+    if (C::PARTS == 1) return 2 * (e / C::K) * C::Q + (un.x + u * C::STR) * C::K + e % C::K;
+    const int j = un.dir == 0 ? 2 * (e / C::G) : 2 * (e / C::K) + un.h * C::G, l = un.dir == 0 ? e % C::G + un.h * C::G : e % C::K;
+    return j * C::Q + (un.x + u * C::STR) * C::K + l;
 }
 template <typename C>
-__device__ __forceinline__ void meet_load_table(const float *cb, const MeetUnit<C> &un, float2 (&tab)[C::BPT][2 * C::G])
+__device__ __forceinline__ void meet_load_table(const float *cb, const MeetUnit<C> &un, float2 (&tab)[C::BPT][C::K * C::G / 2])
 {
 #pragma unroll
     for (int u = 0; u < C::BPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 2 * C::G; ++e) {
+        for (int e = 0; e < C::K * C::G / 2; ++e) {
             const int at = meet_entry<C>(un, u, e);
             tab[u][e] = make_float2(__ldg(cb + at), __ldg(cb + at + C::Q));
         }
 }
 template <typename C>
-__device__ __forceinline__ void meet_table_range(const MeetUnit<C> &un, const float2 (&tab)[C::BPT][2 * C::G], float *lo_out, float *hi_out)
+__device__ __forceinline__ void meet_table_range(const MeetUnit<C> &un, const float2 (&tab)[C::BPT][C::K * C::G / 2], float *lo_out, float *hi_out)
 {
     float lo = tab[0][0].x, hi = lo;
 #pragma unroll
     for (int u = 0; u < C::BPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 2 * C::G; ++e) { lo = fminf(lo, fminf(tab[u][e].x, tab[u][e].y)); hi = max3f(hi, tab[u][e].x, tab[u][e].y); }
+        for (int e = 0; e < C::K * C::G / 2; ++e) { lo = fminf(lo, fminf(tab[u][e].x, tab[u][e].y)); hi = max3f(hi, tab[u][e].x, tab[u][e].y); }
     *lo_out = -un.template reduce<true>(-lo, 0);
     *hi_out = un.template reduce<true>(hi, 1);
 }
@@ -228,13 +232,13 @@ struct MeetDest {
 #pragma unroll
         for (int u = 0; u < C::BPT; ++u) {
             const int x = un.x + u * C::STR;
-            const int xa = (4 * x) % C::NB, ja = (4 * x) / C::NB, ata = ja * C::NBC + xa % C::NBC + (C::G == 2 ? 2 * un.h : 0);
+            const int xa = (C::K * x) % C::NB, ja = (C::K * x) / C::NB, ata = ja * C::NBC + xa % C::NBC + C::G * un.h;
             a[u] = C::CL > 1 ? mapa_u32(msg0 + (uint32_t)ata * 4u, (uint32_t)(xa / C::NBC)) : (uint32_t)ata;
             abar[u] = C::CL > 1 ? mapa_u32(mb0, (uint32_t)(xa / C::NBC)) : 0u;
         }
 #pragma unroll
         for (int o = 0; o < C::G; ++o) {
-            const int j = o + (C::G == 2 ? 2 * un.h : 0), x1 = j * (C::NB / 4) + un.x / 4, at = ((x1 % C::NBC) * 4 + (un.x & 3)) * C::ARR;
+            const int j = o + C::G * un.h, x1 = j * (C::NB / C::K) + un.x / C::K, at = ((x1 % C::NBC) * C::K + un.x % C::K) * C::ARR;
             b[o] = C::CL > 1 ? mapa_u32(msg0 + (uint32_t)at * 4u, (uint32_t)(x1 / C::NBC)) : (uint32_t)at;
             bbar[o] = C::CL > 1 ? mapa_u32(mb0, (uint32_t)(x1 / C::NBC)) : 0u;
         }
@@ -261,8 +265,10 @@ __device__ __forceinline__ MeetUnit<C> meet_unit(float *smem, DeviceDiag *diag)
     const uint32_t rank = C::CL > 1 ? cluster_ctarank() : 0u;
     MeetUnit<C> un{smem + (C::SPLIT ? 0 : dir * C::DIR_FLOATS), dir, i, i & 31, i >> 5, rank,
                    Proto{1u, reinterpret_cast<volatile int *>(smem + C::OFF_FLAG), diag}, 0u, 0, 0, 0};
+    // the lanes of a warp side by side in what they send: alpha outputs of one butterfly (k = 3), otherwise butterflies
     constexpr int PER = C::NBC / C::BPT;
-    un.xl = i % PER; un.h = i / PER;
+    if (C::KB == 3 && dir == 0) { un.xl = i / C::PARTS; un.h = i % C::PARTS; }
+    else { un.xl = i % PER; un.h = i / PER; }
     un.x = (int)rank * C::NBC + un.xl;
     if (C::CL > 1) {
         volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_FLAG);
@@ -315,21 +321,28 @@ struct MeetRing {
     {
         if (want) {
 #pragma unroll
-            for (int e = 0; e < C::ARR * C::BPT; ++e)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (uint32_t)(((t % C::RD) * C::ARR * C::BPT + e) * C::NT * 16)),
-                             "l"(src + (size_t)(t - 1) * (C::ARR * C::NB) + (e / C::BPT) * C::NB + (e % C::BPT) * C::STR) : "memory");
+            for (int e = 0; e < C::ARR * C::KC * C::BPT; ++e)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + (uint32_t)(((t % C::RD) * C::ARR * C::KC * C::BPT + e) * C::NT * 16)),
+                             "l"(src + (size_t)(t - 1) * C::ROW + (e / C::BPT) * C::NB + (e % C::BPT) * C::STR) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     __device__ __forceinline__ void wait() const { asm volatile("cp.async.wait_group %0;" ::"n"(C::RD - 1) : "memory"); }
-    __device__ __forceinline__ float4 row(int t, int arr, int u) const { return from[((t % C::RD) * C::ARR * C::BPT + arr * C::BPT + u) * C::NT]; }
+    // inputs of butterfly u, all K of them or (its outputs' of a part) those of G h .. G h + G - 1
+    __device__ __forceinline__ void row(int t, int arr, int u, int h, float (&v)[C::G]) const
+    {
+        const float4 *at = from + ((t % C::RD) * C::ARR * C::KC * C::BPT + (arr * C::KC + (C::KC > 1 ? h / 2 : 0)) * C::BPT + u) * C::NT;
+        const float4 f = *at;
+        if constexpr (C::G == 4) { v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w; }
+        else { v[0] = h & 1 ? f.z : f.x; v[1] = h & 1 ? f.w : f.y; }
+    }
 };
 
 // ---------------------------------------------------------------------------- forward
 template <typename C, int PHASE>
 __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdParams p, MeetScratch ms)
 {
-    constexpr int CL = C::CL, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS;
+    constexpr int CL = C::CL, K = C::K, KP = K / 2, KC = C::KC, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS;
     extern __shared__ __align__(16) float smem[];
     const int tid = (int)threadIdx.x;
     MeetUnit<C> un = meet_unit<C>(smem, p.diag);
@@ -339,10 +352,10 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
     float4 *step = reinterpret_cast<float4 *>(smem + C::OFF_STEP);          // entry t - 1: scaled clamped weight, the same + 2 delta, delta, soft
     float4 *sums = step + n + 1;                                           // entry t - 1: numerator, denominator (of this CTA)
     int *O_s = reinterpret_cast<int *>(sums + n), *P_s = O_s + n + 2;      // entry t: A_t 2^O_t, M_t 2^P_t
-    float2 tab[BPT][2 * G];
+    float2 tab[BPT][K * G / 2];
     meet_load_table<C>(p.cb, un, tab);
     float c_lo, c_hi;
-    if (PHASE == 2) { c_lo = p.diag->c_lo; c_hi = p.diag->c_hi; }
+    if (PHASE == 2 || p.only_flagged) { c_lo = p.diag->c_lo; c_hi = p.diag->c_hi; }
     else {
         meet_table_range<C>(un, tab, &c_lo, &c_hi);
         if (blockIdx.x == 0 && tid == 0) { p.diag->c_lo = c_lo; p.diag->c_hi = c_hi; }
@@ -350,13 +363,14 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
 #pragma unroll
     for (int u = 0; u < BPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 2 * G; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; }
+        for (int e = 0; e < K * G / 2; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; }
     const MeetDest<C> dst(un);
     float defect = 0.f, zgap = 0.f;
     const int64_t first = C::SPLIT ? (int64_t)(blockIdx.x / (2 * CL)) : (int64_t)blockIdx.x;
     const int64_t stride = C::SPLIT ? p.B : (int64_t)gridDim.x;
 
     for (int64_t blk = first; blk < p.B; blk += stride) {
+        if (C::SPLIT && p.only_flagged && !p.lin_flag[blk]) break;         // (both launches and every CTA alike)
         float *area = p.hist + (size_t)(C::SPLIT ? blk : (int64_t)blockIdx.x) * C::block_floats(n);
         float4 *hist4 = reinterpret_cast<float4 *>(area);                  // row t - 1: [NB], A_t up to the middle, M_t behind it
         float *endA = area + (size_t)n * C::Q, *endM = endA + C::Q;        // split form
@@ -398,20 +412,22 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
                     if (v > 1) un.wait_inputs(cur);
                     if (send) un.arm(v, nxt, false);
                     const float *in = un.msg(cur) + un.xl;
-                    float4 a4[BPT];
+                    float2 A[BPT][KP];
 #pragma unroll
-                    for (int u = 0; u < BPT; ++u) {
-                        const int at = u * C::STR;
-                        a4[u] = make_float4(in[at], in[NBC + at], in[2 * NBC + at], in[3 * NBC + at]);
-                    }
+                    for (int u = 0; u < BPT; ++u)
+#pragma unroll
+                        for (int jp = 0; jp < KP; ++jp) A[u][jp] = make_float2(in[2 * jp * NBC + u * C::STR], in[(2 * jp + 1) * NBC + u * C::STR]);
                     const float4 sp = step[t - 1];
                     off = un.template offset<LIN>(v, off, lev0);
                     O += off;
                     if (un.i == 0) O_s[t + 1] = O;
                     const float kap = COMB ? z.kappa<LIN>(O + P_s[t]) : 0.f;
-                    if (!COMB && (G == 4 || un.h == 0)) {
+                    if (!COMB && (C::PARTS == 1 || un.h == 0)) {
 #pragma unroll
-                        for (int u = 0; u < BPT; ++u) hist4[(size_t)(t - 1) * C::NB + un.x + u * C::STR] = a4[u];
+                        for (int u = 0; u < BPT; ++u)
+#pragma unroll
+                            for (int c = 0; c < KC; ++c)
+                                hist4[(size_t)(t - 1) * C::ROW + c * C::NB + un.x + u * C::STR] = make_float4(A[u][2 * c].x, A[u][2 * c].y, A[u][2 * c + 1].x, A[u][2 * c + 1].y);
                     }
                     if (COMB && v > 1) un.put_sums(v - 1, sum_of(v - 1), warp_sum2_split(pn, pd, un.lane), 2);   // (beside this step's arithmetic)
                     pn = pd = 0.f;
@@ -419,37 +435,59 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
                     float tmax = NONE;
 #pragma unroll
                     for (int u = 0; u < BPT; ++u) {
-                        const float2 A0 = make_float2(a4[u].x, a4[u].y), A1 = make_float2(a4[u].z, a4[u].w);
-                        const float floor1 = LIN ? lin_floor((a4[u].x + a4[u].y) + (a4[u].z + a4[u].w)) : 0.f;
-                        float Ml[4] = {0.f, 0.f, 0.f, 0.f};
-                        if (COMB) { const float4 m4 = ring.row(t, 0, u); Ml[0] = m4.x; Ml[1] = m4.y; Ml[2] = m4.z; Ml[3] = m4.w; }
-                        if (G == 2 && un.h) { Ml[0] = Ml[2]; Ml[1] = Ml[3]; }
+                        float floor1 = 0.f;
+                        if (LIN) {
+                            float total = A[u][0].x + A[u][0].y;
+#pragma unroll
+                            for (int jp = 1; jp < KP; ++jp) total += A[u][jp].x + A[u][jp].y;
+                            floor1 = lin_floor(total);
+                        }
+                        float Ml[G];
+                        if (COMB) ring.row(t, 0, u, un.h, Ml);
                         float out[G];
 #pragma unroll
                         for (int l = 0; l < G; ++l) {
-                            const float2 c0 = tab[u][l], c1 = tab[u][G + l];
-                            const float2 d0 = sub2(c0, w2), d1 = sub2(c1, w2);
-                            const float2 r0 = RC ? sub2(c0, v2) : d0, r1 = RC ? sub2(c1, v2) : d1;
+                            float2 s, ds;
                             if (LIN) {
-                                const float2 e0 = ex2n2(fma2(d0, r0, off2)), e1 = ex2n2(fma2(d1, r1, off2));
+                                if (!COMB) s = make_float2(floor1, 0.f);
+#pragma unroll
+                                for (int jp = 0; jp < KP; ++jp) {
+                                    const float2 c = tab[u][jp * G + l], d = sub2(c, w2);
+                                    const float2 e = ex2n2(fma2(d, RC ? sub2(c, v2) : d, off2));
+                                    if (COMB) {
+                                        const float2 pa = mul2(e, A[u][jp]);
+                                        s = jp == 0 ? pa : add2(s, pa);
+                                        ds = jp == 0 ? mul2(pa, d) : fma2(pa, d, ds);
+                                    } else {
+                                        s = fma2(e, A[u][jp], s);
+                                    }
+                                }
+                                out[l] = s.x + s.y;
                                 if (COMB) {
-                                    const float2 p0 = mul2(e0, A0), p1 = mul2(e1, A1), s = add2(p0, p1), ds = fma2(p1, d1, mul2(p0, d0));
                                     const float f = Ml[l] * kap;
-                                    out[l] = (s.x + s.y) + floor1;
+                                    out[l] += floor1;
                                     pd = fmaf(f, out[l], pd);
                                     pn = fmaf(f, ds.x + ds.y, pn);
-                                } else {
-                                    const float2 s = fma2(e1, A1, fma2(e0, A0, make_float2(floor1, 0.f)));
-                                    out[l] = s.x + s.y;
                                 }
                             } else {
-                                const float2 u0 = sub2(A0, mul2(d0, r0)), u1 = sub2(A1, mul2(d1, r1));
-                                const float mx = max3f(fmaxf(u0.x, u0.y), u1.x, u1.y);
-                                const float2 e0 = ex2f2(sub2(u0, splat2(mx))), e1 = ex2f2(sub2(u1, splat2(mx))), s = add2(e0, e1);
-                                const float sum = s.x + s.y, top = mx - off2.x;
+                                float2 d[KP], uu[KP];
+#pragma unroll
+                                for (int jp = 0; jp < KP; ++jp) {
+                                    const float2 c = tab[u][jp * G + l];
+                                    d[jp] = sub2(c, w2);
+                                    uu[jp] = sub2(A[u][jp], mul2(d[jp], RC ? sub2(c, v2) : d[jp]));
+                                }
+                                const float2 m2 = max_pairs<KP>(uu);
+                                const float mx = fmaxf(m2.x, m2.y), top = mx - off2.x;
+#pragma unroll
+                                for (int jp = 0; jp < KP; ++jp) {
+                                    const float2 e = ex2f2(sub2(uu[jp], splat2(mx)));
+                                    s = jp == 0 ? e : add2(s, e);
+                                    if (COMB) ds = jp == 0 ? mul2(e, d[jp]) : fma2(e, d[jp], ds);
+                                }
+                                const float sum = s.x + s.y;
                                 out[l] = top + lg2f(sum);
                                 if (COMB) {
-                                    const float2 ds = fma2(e1, d1, mul2(e0, d0));
                                     const float f = ex2f(top + Ml[l] + kap);
                                     pd = fmaf(f, sum, pd);
                                     pn = fmaf(f, ds.x + ds.y, pn);
@@ -459,7 +497,10 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
                         }
                         if (send) {
                             if constexpr (CL > 1) {
-                                if (un.pr.live) st_async_v4(dst.a[u] + (uint32_t)nxt * un.TX_MSG, out[0], out[1], out[G - 2], out[G - 1], dst.abar[u] + 8u * nxt);
+                                if (un.pr.live) {
+                                    if constexpr (G == 4) st_async_v4(dst.a[u] + (uint32_t)nxt * un.TX_MSG, out[0], out[1], out[2], out[3], dst.abar[u] + 8u * nxt);
+                                    else st_async_v2(dst.a[u] + (uint32_t)nxt * un.TX_MSG, out[0], out[1], dst.abar[u] + 8u * nxt);
+                                }
                             } else if constexpr (G == 4) *reinterpret_cast<float4 *>(un.msg(nxt) + dst.a[u]) = make_float4(out[0], out[1], out[2], out[3]);
                             else *reinterpret_cast<float2 *>(un.msg(nxt) + dst.a[u]) = make_float2(out[0], out[1]);
                         }
@@ -487,7 +528,7 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
                     if (COMB) { ring.issue(t - (C::RD - 1), v + C::RD - 1 <= cnt); ring.wait(); }
                     if (v > 1) un.wait_inputs(cur);
                     if (send) un.arm(v, nxt, false);
-                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + un.xl;
+                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + KC * un.xl;
                     const float4 sp = step[t - 1];
                     off = un.template offset<LIN>(v, off, lev0);
                     P += off;
@@ -499,46 +540,46 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
                     float tmax = NONE;
 #pragma unroll
                     for (int u = 0; u < BPT; ++u) {
-                        const float4 m4 = in[u * C::STR];
-                        if (!COMB && (G == 4 || un.h == 0)) hist4[(size_t)(t - 1) * C::NB + un.x + u * C::STR] = m4;
-                        const float Mb[4] = {m4.x, m4.y, m4.z, m4.w};
-                        float2 Ah[2];
-                        if (COMB) {
-                            const float4 a4 = ring.row(t, 0, u);
-                            Ah[0] = make_float2(a4.x, a4.y); Ah[1] = make_float2(a4.z, a4.w);
-                            if (G == 2 && un.h) Ah[0] = Ah[1];
+                        float Mb[K];
+#pragma unroll
+                        for (int c = 0; c < KC; ++c) {
+                            const float4 m4 = in[KC * u * C::STR + c];
+                            if (!COMB && (C::PARTS == 1 || un.h == 0)) hist4[(size_t)(t - 1) * C::ROW + c * C::NB + un.x + u * C::STR] = m4;
+                            Mb[4 * c] = m4.x; Mb[4 * c + 1] = m4.y; Mb[4 * c + 2] = m4.z; Mb[4 * c + 3] = m4.w;
                         }
+                        float Ah[G];
+                        if (COMB) ring.row(t, 0, u, un.h, Ah);
                         float out[G];
 #pragma unroll
                         for (int jp = 0; jp < G / 2; ++jp) {
                             float2 sum, ds, f, o;
                             if (LIN) {
 #pragma unroll
-                                for (int b = 0; b < 4; ++b) {
-                                    const float2 c = tab[u][jp * 4 + b], d = sub2(c, w2);
+                                for (int b = 0; b < K; ++b) {
+                                    const float2 c = tab[u][jp * K + b], d = sub2(c, w2);
                                     const float2 pb = mul2(ex2n2(fma2(d, RC ? sub2(c, v2) : d, off2)), splat2(Mb[b]));
                                     sum = b == 0 ? pb : add2(sum, pb);
                                     if (COMB) ds = b == 0 ? mul2(pb, d) : fma2(pb, d, ds);
                                 }
                                 o = sum;
-                                if (COMB) f = mul2(Ah[jp], splat2(kap));
+                                if (COMB) f = make_float2(Ah[2 * jp] * kap, Ah[2 * jp + 1] * kap);
                             } else {
-                                float2 d[4], uu[4];
+                                float2 d[K], uu[K];
 #pragma unroll
-                                for (int b = 0; b < 4; ++b) {
-                                    const float2 c = tab[u][jp * 4 + b];
+                                for (int b = 0; b < K; ++b) {
+                                    const float2 c = tab[u][jp * K + b];
                                     d[b] = sub2(c, w2);
                                     uu[b] = sub2(splat2(Mb[b] - off2.x), mul2(d[b], RC ? sub2(c, v2) : d[b]));
                                 }
-                                const float2 mx = max_pairs<4>(uu);
+                                const float2 mx = max_pairs<K>(uu);
 #pragma unroll
-                                for (int b = 0; b < 4; ++b) {
+                                for (int b = 0; b < K; ++b) {
                                     const float2 pb = ex2f2(sub2(uu[b], mx));
                                     sum = b == 0 ? pb : add2(sum, pb);
                                     if (COMB) ds = b == 0 ? mul2(pb, d[b]) : fma2(pb, d[b], ds);
                                 }
                                 o = add2(mx, lg2f2(sum));
-                                if (COMB) f = ex2f2(add2(add2(Ah[jp], mx), splat2(kap)));
+                                if (COMB) f = ex2f2(add2(add2(make_float2(Ah[2 * jp], Ah[2 * jp + 1]), mx), splat2(kap)));
                             }
                             out[2 * jp] = o.x; out[2 * jp + 1] = o.y;
                             if (COMB) { num2 = fma2(f, ds, num2); den2 = fma2(f, sum, den2); }
@@ -717,7 +758,7 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
 template <typename C, bool ACC, int PHASE>
 __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdParams p, MeetScratch ms)
 {
-    constexpr int CL = C::CL, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS, ARR = 2;
+    constexpr int CL = C::CL, K = C::K, KP = K / 2, KC = C::KC, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS, ARR = 2;
     extern __shared__ __align__(16) float smem[];
     const int tid = (int)threadIdx.x;
     MeetUnit<C> un = meet_unit<C>(smem, p.diag);
@@ -728,14 +769,14 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
     float4 *sums = step + n + 1;                                           // entry t - 1: the three posterior sums (of this CTA)
     int *O_s = reinterpret_cast<int *>(sums + n), *P_s = O_s + n + 2;
     const float c_lo = p.diag->c_lo, c_hi = p.diag->c_hi;                  // left by the forward call
-    float2 tab[BPT][2 * G], acc[BPT][2 * G];
+    float2 tab[BPT][K * G / 2], acc[BPT][K * G / 2];
     meet_load_table<C>(p.cb, un, tab);
 #pragma unroll
     for (int u = 0; u < BPT; ++u)
 #pragma unroll
-        for (int e = 0; e < 2 * G; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; acc[u][e] = make_float2(0.f, 0.f); }
+        for (int e = 0; e < K * G / 2; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; acc[u][e] = make_float2(0.f, 0.f); }
     const MeetDest<C> dst(un);
-    constexpr int PL = 4 * NBC;                                             // floats from A to AA in an alpha message
+    constexpr int PL = K * NBC;                                             // floats from A to AA in an alpha message
     float defect = 0.f;
     const float2 ni2 = splat2(-p.invT * isl);
     // scale of the accumulators (see bcjr_lin_bwd.cuh), and whether gc_part holds something already
@@ -749,7 +790,7 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
 #pragma unroll
         for (int u = 0; u < BPT; ++u)
 #pragma unroll
-            for (int e = 0; e < 2 * G; ++e) {
+            for (int e = 0; e < K * G / 2; ++e) {
                 float *to = gc + meet_entry<C>(un, u, e);
                 to[0] = up * acc[u][e].x + (add ? to[0] : 0.f);
                 to[C::Q] = up * acc[u][e].y + (add ? to[C::Q] : 0.f);
@@ -779,7 +820,7 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
 #pragma unroll
                 for (int u = 0; u < BPT; ++u)
 #pragma unroll
-                    for (int e = 0; e < 2 * G; ++e) acc[u][e] = make_float2(0.f, 0.f);
+                    for (int e = 0; e < K * G / 2; ++e) acc[u][e] = make_float2(0.f, 0.f);
             }
             e_acc = e_g + GRAD_ROOM;
         }
@@ -828,52 +869,65 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
 #pragma unroll
                     for (int u = 0; u < BPT; ++u) {
                         const int at = u * C::STR;
-                        const float4 a4 = make_float4(in[at], in[NBC + at], in[2 * NBC + at], in[3 * NBC + at]);
-                        const float4 b4 = make_float4(in[PL + at], in[PL + NBC + at], in[PL + 2 * NBC + at], in[PL + 3 * NBC + at]);
-                        if (!COMB && (G == 4 || un.h == 0)) {
-                            float4 *row = hist4 + (size_t)(t - 1) * (ARR * C::NB) + un.x + at;
-                            row[0] = a4; row[C::NB] = b4;
+                        float2 A[KP], Bq[KP], q[KP], Gq[KP];
+#pragma unroll
+                        for (int jp = 0; jp < KP; ++jp) {
+                            A[jp] = make_float2(in[2 * jp * NBC + at], in[(2 * jp + 1) * NBC + at]);
+                            Bq[jp] = make_float2(in[PL + 2 * jp * NBC + at], in[PL + (2 * jp + 1) * NBC + at]);
+                            q[jp] = LIN ? mul2(A[jp], gd2) : gd2;
+                            Gq[jp] = LIN && COMB ? mul2(A[jp], g2) : g2;
                         }
-                        const float2 A0 = make_float2(a4.x, a4.y), A1 = make_float2(a4.z, a4.w);
-                        const float2 B0 = make_float2(b4.x, b4.y), B1 = make_float2(b4.z, b4.w);
-                        const float2 q0 = LIN ? mul2(A0, gd2) : gd2, q1 = LIN ? mul2(A1, gd2) : gd2;
-                        float2 G0 = g2, G1 = g2;
-                        float Ml[4] = {0.f, 0.f, 0.f, 0.f}, Yl[4] = {0.f, 0.f, 0.f, 0.f};
-                        if (COMB) {
-                            const float4 m4 = ring.row(t, 0, u), y4 = ring.row(t, 1, u);
-                            Ml[0] = m4.x; Ml[1] = m4.y; Ml[2] = m4.z; Ml[3] = m4.w;
-                            Yl[0] = y4.x; Yl[1] = y4.y; Yl[2] = y4.z; Yl[3] = y4.w;
-                            if (G == 2 && un.h) { Ml[0] = Ml[2]; Ml[1] = Ml[3]; Yl[0] = Yl[2]; Yl[1] = Yl[3]; }
-                            if (LIN) { G0 = mul2(A0, g2); G1 = mul2(A1, g2); }
+                        if (!COMB && (C::PARTS == 1 || un.h == 0)) {
+                            float4 *row = hist4 + (size_t)(t - 1) * C::ROW + un.x + at;
+#pragma unroll
+                            for (int c = 0; c < KC; ++c) {
+                                row[c * C::NB] = make_float4(A[2 * c].x, A[2 * c].y, A[2 * c + 1].x, A[2 * c + 1].y);
+                                row[(KC + c) * C::NB] = make_float4(Bq[2 * c].x, Bq[2 * c].y, Bq[2 * c + 1].x, Bq[2 * c + 1].y);
+                            }
                         }
+                        float Ml[G], Yl[G];
+                        if (COMB) { ring.row(t, 0, u, un.h, Ml); ring.row(t, 1, u, un.h, Yl); }
                         float oa[G], ob[G];
 #pragma unroll
                         for (int l = 0; l < G; ++l) {
-                            const float2 c0 = tab[u][l], c1 = tab[u][G + l];
-                            const float2 d0 = sub2(c0, w2), d1 = sub2(c1, w2);
-                            const float2 r0 = RC ? sub2(c0, v2) : d0, r1 = RC ? sub2(c1, v2) : d1;
-                            const float2 y0 = fma2(d0, q0, B0), y1 = fma2(d1, q1, B1);
-                            float2 e0, e1;
+                            float2 d[KP], e[KP], y[KP], s, ax;
                             float top = 0.f;
-                            if (LIN) {
-                                e0 = ex2n2(fma2(d0, r0, off2)); e1 = ex2n2(fma2(d1, r1, off2));
-                            } else {
-                                const float2 u0 = sub2(A0, mul2(d0, r0)), u1 = sub2(A1, mul2(d1, r1));
-                                const float mx = max3f(fmaxf(u0.x, u0.y), u1.x, u1.y);
-                                e0 = ex2f2(sub2(u0, splat2(mx))); e1 = ex2f2(sub2(u1, splat2(mx)));
+#pragma unroll
+                            for (int jp = 0; jp < KP; ++jp) {
+                                const float2 c = tab[u][jp * G + l];
+                                d[jp] = sub2(c, w2);
+                                const float2 r = RC ? sub2(c, v2) : d[jp];
+                                y[jp] = fma2(d[jp], q[jp], Bq[jp]);
+                                e[jp] = LIN ? ex2n2(fma2(d[jp], r, off2)) : sub2(A[jp], mul2(d[jp], r));
+                            }
+                            if (!LIN) {
+                                const float2 m2 = max_pairs<KP>(e);
+                                const float mx = fmaxf(m2.x, m2.y);
+#pragma unroll
+                                for (int jp = 0; jp < KP; ++jp) e[jp] = ex2f2(sub2(e[jp], splat2(mx)));
                                 top = mx - off2.x;
                             }
-                            const float2 s = LIN ? fma2(e1, A1, mul2(e0, A0)) : add2(e0, e1), ax = fma2(e1, y1, mul2(e0, y0));
+#pragma unroll
+                            for (int jp = 0; jp < KP; ++jp) {
+                                if (LIN) s = jp == 0 ? mul2(e[0], A[0]) : fma2(e[jp], A[jp], s);
+                                else s = jp == 0 ? e[0] : add2(s, e[jp]);
+                                ax = jp == 0 ? mul2(e[0], y[0]) : fma2(e[jp], y[jp], ax);
+                            }
                             const float sum = s.x + s.y, axs = ax.x + ax.y;
                             if (LIN) { oa[l] = sum; ob[l] = fmaf(sum, gsn, axs); }
                             else { oa[l] = top + lg2f(sum); ob[l] = fmaf(axs, rcpf(sum), gsn); }
                             if (COMB) {
                                 const float f = LIN ? Ml[l] * kap : ex2f(top + Ml[l] + kap);
                                 const float2 Y2 = splat2(Yl[l]), f2 = splat2(f);
-                                const float2 h0 = LIN ? fma2(A0, Y2, y0) : add2(y0, Y2), h1 = LIN ? fma2(A1, Y2, y1) : add2(y1, Y2);
-                                const float2 z0 = fma2(mul2(RC ? sub2(c0, u2) : d0, ni2), h0, G0), z1 = fma2(mul2(RC ? sub2(c1, u2) : d1, ni2), h1, G1);
-                                const float2 x0 = mul2(e0, z0), x1 = mul2(e1, z1), xs = add2(x0, x1);
-                                if (ACC) { acc[u][l] = fma2(x0, f2, acc[u][l]); acc[u][G + l] = fma2(x1, f2, acc[u][G + l]); }
+                                float2 xs;
+#pragma unroll
+                                for (int jp = 0; jp < KP; ++jp) {
+                                    const float2 hq = LIN ? fma2(A[jp], Y2, y[jp]) : add2(y[jp], Y2);
+                                    const float2 zq = fma2(mul2(RC ? sub2(tab[u][jp * G + l], u2) : d[jp], ni2), hq, Gq[jp]);
+                                    const float2 xq = mul2(e[jp], zq);
+                                    xs = jp == 0 ? xq : add2(xs, xq);
+                                    if (ACC) acc[u][jp * G + l] = fma2(xq, f2, acc[u][jp * G + l]);
+                                }
                                 s0 = fmaf(f, sum, s0);
                                 s2 = fmaf(f, fmaf(Yl[l], sum, axs), s2);
                                 sz = fmaf(f, xs.x + xs.y, sz);
@@ -884,8 +938,13 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
                             if constexpr (CL > 1) {
                                 if (un.pr.live) {
                                     const uint32_t to = dst.a[u] + (uint32_t)nxt * un.TX_MSG;
-                                    st_async_v4(to, oa[0], oa[1], oa[G - 2], oa[G - 1], dst.abar[u] + 8u * nxt);
-                                    st_async_v4(to + PL * 4u, ob[0], ob[1], ob[G - 2], ob[G - 1], dst.abar[u] + 8u * nxt);
+                                    if constexpr (G == 4) {
+                                        st_async_v4(to, oa[0], oa[1], oa[2], oa[3], dst.abar[u] + 8u * nxt);
+                                        st_async_v4(to + PL * 4u, ob[0], ob[1], ob[2], ob[3], dst.abar[u] + 8u * nxt);
+                                    } else {
+                                        st_async_v2(to, oa[0], oa[1], dst.abar[u] + 8u * nxt);
+                                        st_async_v2(to + PL * 4u, ob[0], ob[1], dst.abar[u] + 8u * nxt);
+                                    }
                                 }
                             } else if constexpr (G == 4) {
                                 float *to = un.msg(nxt) + dst.a[u];
@@ -920,7 +979,7 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
                     if (COMB) { ring.issue(t - (C::RD - 1), v + C::RD - 1 <= cnt); ring.wait(); }
                     if (v > 1) un.wait_inputs(cur);
                     if (send) un.arm(v, nxt, drop_hook && PHASE != 2 && v == 1);
-                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + 2 * un.xl;
+                    const float4 *in = reinterpret_cast<const float4 *>(un.msg(cur)) + KP * un.xl;
                     const float4 sp = step[t - 1];
                     off = un.template offset<LIN>(v, off, lev0);
                     P += off;
@@ -933,51 +992,55 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_bwd_kernel(BwdPa
                     float tmax = NONE;
 #pragma unroll
                     for (int u = 0; u < BPT; ++u) {
-                        const float4 m01 = in[2 * u * C::STR], m23 = in[2 * u * C::STR + 1];
-                        const float Mb[4] = {m01.x, m01.z, m23.x, m23.z}, Yb[4] = {m01.y, m01.w, m23.y, m23.w};
-                        if (!COMB && (G == 4 || un.h == 0)) {
-                            float4 *row = hist4 + (size_t)(t - 1) * (ARR * C::NB) + un.x + u * C::STR;
-                            row[0] = make_float4(Mb[0], Mb[1], Mb[2], Mb[3]); row[C::NB] = make_float4(Yb[0], Yb[1], Yb[2], Yb[3]);
+                        float Mb[K], Yb[K];
+#pragma unroll
+                        for (int c = 0; c < KP; ++c) {
+                            const float4 v = in[KP * u * C::STR + c];
+                            Mb[2 * c] = v.x; Yb[2 * c] = v.y; Mb[2 * c + 1] = v.z; Yb[2 * c + 1] = v.w;
                         }
-                        float2 Ah[2], Bh[2];
-                        if (COMB) {
-                            const float4 a4 = ring.row(t, 0, u), b4 = ring.row(t, 1, u);
-                            Ah[0] = make_float2(a4.x, a4.y); Ah[1] = make_float2(a4.z, a4.w);
-                            Bh[0] = make_float2(b4.x, b4.y); Bh[1] = make_float2(b4.z, b4.w);
-                            if (G == 2 && un.h) { Ah[0] = Ah[1]; Bh[0] = Bh[1]; }
+                        if (!COMB && (C::PARTS == 1 || un.h == 0)) {
+                            float4 *row = hist4 + (size_t)(t - 1) * C::ROW + un.x + u * C::STR;
+#pragma unroll
+                            for (int c = 0; c < KC; ++c) {
+                                row[c * C::NB] = make_float4(Mb[4 * c], Mb[4 * c + 1], Mb[4 * c + 2], Mb[4 * c + 3]);
+                                row[(KC + c) * C::NB] = make_float4(Yb[4 * c], Yb[4 * c + 1], Yb[4 * c + 2], Yb[4 * c + 3]);
+                            }
                         }
+                        float Ah[G], Bh[G];
+                        if (COMB) { ring.row(t, 0, u, un.h, Ah); ring.row(t, 1, u, un.h, Bh); }
                         float oM[G], oB[G];
 #pragma unroll
                         for (int jp = 0; jp < G / 2; ++jp) {
-                            float2 d[4], e[4], mx = make_float2(0.f, 0.f);
+                            float2 d[K], e[K], mx = make_float2(0.f, 0.f);
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
-                                const float2 c = tab[u][jp * 4 + b];
+                            for (int b = 0; b < K; ++b) {
+                                const float2 c = tab[u][jp * K + b];
                                 d[b] = sub2(c, w2);
                                 const float2 r = RC ? sub2(c, v2) : d[b];
                                 e[b] = LIN ? mul2(ex2n2(fma2(d[b], r, off2)), splat2(Mb[b])) : sub2(splat2(Mb[b] - off2.x), mul2(d[b], r));
                             }
                             if (!LIN) {
-                                mx = max_pairs<4>(e);
+                                mx = max_pairs<K>(e);
 #pragma unroll
-                                for (int b = 0; b < 4; ++b) e[b] = ex2f2(sub2(e[b], mx));
+                                for (int b = 0; b < K; ++b) e[b] = ex2f2(sub2(e[b], mx));
                             }
                             float2 f, fA, fg, nf, nfA;
                             if (COMB) {
-                                f = LIN ? mul2(Ah[jp], splat2(kap)) : ex2f2(add2(add2(Ah[jp], mx), splat2(kap)));
-                                fA = LIN ? mul2(Bh[jp], splat2(kap)) : mul2(f, Bh[jp]);
+                                const float2 Ap = make_float2(Ah[2 * jp], Ah[2 * jp + 1]), Bp = make_float2(Bh[2 * jp], Bh[2 * jp + 1]);
+                                f = LIN ? mul2(Ap, splat2(kap)) : ex2f2(add2(add2(Ap, mx), splat2(kap)));
+                                fA = LIN ? mul2(Bp, splat2(kap)) : mul2(f, Bp);
                                 fg = mul2(f, g2); nf = mul2(f, ni2); nfA = mul2(fA, ni2);
                             }
                             float2 sum, ya, zs;
 #pragma unroll
-                            for (int b = 0; b < 4; ++b) {
+                            for (int b = 0; b < K; ++b) {
                                 const float2 y = fma2(gd2, d[b], splat2(Yb[b]));
                                 sum = b == 0 ? e[b] : add2(sum, e[b]);
                                 ya = b == 0 ? mul2(e[b], y) : fma2(e[b], y, ya);
                                 if (COMB) {
-                                    const float2 zz = fma2(RC ? sub2(tab[u][jp * 4 + b], u2) : d[b], fma2(nf, y, nfA), fg);
+                                    const float2 zz = fma2(RC ? sub2(tab[u][jp * K + b], u2) : d[b], fma2(nf, y, nfA), fg);
                                     zs = b == 0 ? mul2(e[b], zz) : fma2(e[b], zz, zs);
-                                    if (ACC) acc[u][jp * 4 + b] = fma2(e[b], zz, acc[u][jp * 4 + b]);
+                                    if (ACC) acc[u][jp * K + b] = fma2(e[b], zz, acc[u][jp * K + b]);
                                 }
                             }
                             const float2 om = LIN ? sum : add2(mx, lg2f2(sum));

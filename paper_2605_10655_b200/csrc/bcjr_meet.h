@@ -8,7 +8,7 @@
 namespace bcjr {
 
 // Forms of the kernels for a trellis, see bcjr_meet_launch.cuh
-constexpr int MEET_FORMS = 2;
+constexpr int MEET_FORMS = 3, MEET_K3 = 2;   // the last one: k = 3
 struct MeetPlan {
     bool split = false;               // two launches
     int grid = 0, parts = 0;          // CTAs, partial codebook gradients

@@ -21,6 +21,7 @@ template <bool BWD> struct MeetOf<14, 0, BWD> { using C = MeetCfg<14, 2, 4, 1, B
 template <bool BWD> struct MeetOf<15, 0, BWD> { using C = MeetCfg<15, 4, 4, 1, BWD, true>; };
 template <bool BWD> struct MeetOf<16, 0, BWD> { using C = MeetCfg<16, 8, 4, 1, BWD, true>; };
 template <bool BWD> struct MeetOf<16, 1, BWD> { using C = MeetCfg<16, 4, 4, 2, BWD, true>; };
+template <bool BWD> struct MeetOf<16, MEET_K3, BWD> { using C = MeetCfg<16, 8, 2, 1, BWD, true, 3>; };
 
 template <typename C, typename Kern>
 cudaError_t config(Kern kern, size_t smem, int grid, cudaStream_t st, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr)
@@ -67,7 +68,7 @@ cudaError_t dispatch_form(int Lb, F f)
 template <bool BWD, typename F>
 cudaError_t dispatch(int Lb, int form, F f)
 {
-    return form == 0 ? dispatch_form<BWD, 0>(Lb, f) : dispatch_form<BWD, 1>(Lb, f);
+    return form == 0 ? dispatch_form<BWD, 0>(Lb, f) : form == 1 ? dispatch_form<BWD, 1>(Lb, f) : dispatch_form<BWD, MEET_K3>(Lb, f);
 }
 
 template <typename C>

@@ -557,10 +557,11 @@ def test_every_log_domain_kernel_is_reached(ctx, Lb, k, n, B, T, want_gc, option
         assert parity.rel_inf(gc.cpu().numpy(), ref_b["grad_codebook"]) <= parity.GRAD_TOL
 
 
-@pytest.mark.parametrize("Lb,n,B,T", [(8, 1, 3, 0.3), (8, 2, 700, 0.1), (8, 65, 5, 0.012), (9, 33, 600, 0.2), (10, 97, 148, 0.05), (11, 34, 9, 0.02), (12, 3, 74, 0.1), (12, 66, 75, 0.02),
-                                      (13, 31, 37, 0.1), (13, 64, 74, 0.015), (14, 2, 37, 0.1), (14, 35, 5, 0.03), (15, 67, 3, 0.1), (15, 5, 16, 0.015), (16, 1, 2, 0.3), (16, 67, 7, 0.1),
-                                      (16, 2, 8, 0.1), (16, 99, 16, 0.05), (16, 5, 33, 0.015), (16, 6, 40, 0.2), (16, 5, 49, 0.03), (16, 4, 150, 0.1), (16, 5, 164, 0.015), (16, 6, 340, 0.02)])
-def test_sweeps_from_both_ends(ctx, Lb, n, B, T):
+@pytest.mark.parametrize("Lb,k,n,B,T", [(8, 2, 1, 3, 0.3), (8, 2, 2, 700, 0.1), (8, 2, 65, 5, 0.012), (9, 2, 33, 600, 0.2), (10, 2, 97, 148, 0.05), (11, 2, 34, 9, 0.02), (12, 2, 3, 74, 0.1), (12, 2, 66, 75, 0.02),
+                                      (13, 2, 31, 37, 0.1), (13, 2, 64, 74, 0.015), (14, 2, 2, 37, 0.1), (14, 2, 35, 5, 0.03), (15, 2, 67, 3, 0.1), (15, 2, 5, 16, 0.015), (16, 2, 1, 2, 0.3), (16, 2, 67, 7, 0.1),
+                                      (16, 2, 2, 8, 0.1), (16, 2, 99, 16, 0.05), (16, 2, 5, 33, 0.015), (16, 2, 6, 40, 0.2), (16, 2, 5, 49, 0.03), (16, 2, 4, 150, 0.1), (16, 2, 5, 164, 0.015), (16, 2, 6, 340, 0.02),
+                                      (16, 3, 16, 7, 0.3), (16, 3, 67, 3, 0.015), (16, 3, 33, 30, 0.1), (16, 3, 17, 151, 0.05)])
+def test_sweeps_from_both_ends(ctx, Lb, k, n, B, T):
     # Every form of the two-ended kernels at its fewest and most blocks, as the end of longer calls too: one step (no alpha half), halves of
     # different lengths, posterior sums of 32 steps and one more, weights outside the table, linear and log messages, blocks whose
     # gradients differ in scale, a block without a certificate; with and without grad_codebook, into the weights.
@@ -575,18 +576,38 @@ def test_sweeps_from_both_ends(ctx, Lb, n, B, T):
     z[pick[0]] *= 2.0 ** -20
     dev = torch.device("cuda", ctx.device)
     Wd, cd, gd = (torch.from_numpy(a).to(dev) for a in (W, c, z))
-    soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, 2, n, T)
+    soft, logZ = ctx.bcjr_soft_quantize(Wd, cd, Lb, k, n, T)
     forward = ctx.last_kernels()
     gW, gc = ctx.bcjr_backward(gd)
     backward = ctx.last_kernels()
     gW2, _ = ctx.bcjr_backward(gd, want_grad_codebook=False)
     assert forward[-1] == "fwd_reg" and backward[-1] == "bwd_reg"
-    ref_f, ref_b = oracle.soft_quantize(W[pick], c, Lb, 2, T), oracle.backward(W[pick], c, z[pick], Lb, 2, T)
+    ref_f, ref_b = oracle.soft_quantize(W[pick], c, Lb, k, T), oracle.backward(W[pick], c, z[pick], Lb, k, T)
     got = {"soft": soft.cpu().numpy()[pick], "logZ": logZ.cpu().numpy()[pick], "grad_W": gW.cpu().numpy()[pick], "grad_codebook": gc.cpu().numpy()}
-    parity.assert_forward_backward(got, ref_f, ref_b, f"Lb={Lb} n={n} B={B} T={T}")
+    parity.assert_forward_backward(got, ref_f, ref_b, f"Lb={Lb} k={k} n={n} B={B} T={T}")
     assert parity.rel_inf(gW2.cpu().numpy()[pick], ref_b["grad_W"]) <= parity.GRAD_TOL
     small = gW.cpu().numpy()[pick[0]]                    # a block of its own scale is right on its own scale
     assert parity.rel_inf(small, ref_b["grad_W"][0]) <= 2 * parity.GRAD_TOL
     over = Wd.clone()
-    ctx.bcjr_soft_quantize(over, cd, Lb, 2, n, T, soft=over)
+    ctx.bcjr_soft_quantize(over, cd, Lb, k, n, T, soft=over)
     assert torch.equal(over, soft) and ctx.sync_status().device_status == 0
+
+
+@pytest.mark.parametrize("Lb,k,n,B", [(8, 2, 20, 3), (12, 2, 20, 3), (16, 2, 20, 3), (16, 2, 20, 20), (16, 3, 20, 3), (16, 3, 20, 150)])
+def test_first_call_of_a_context(ctx, Lb, k, n, B):
+    # Nothing is held yet: scratch, flags and lists are sized by this call alone.  The same numbers as from a context that has run others.
+    import torch
+    from paper_2605_10655_b200 import Context
+    W, c, g = _rand(n, Lb, B, seed=1400 + Lb + B)
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd, gd = (torch.from_numpy(a).to(dev) for a in (W, c, g))
+    fresh = Context(ctx.device)
+    try:
+        out = []
+        for x in (fresh, ctx):
+            out.append([*x.bcjr_soft_quantize(Wd, cd, Lb, k, n, 0.2), *x.bcjr_backward(gd)])
+            assert x.sync_status().device_status == 0
+        for a, b in zip(*out):
+            assert torch.equal(a, b)
+    finally:
+        fresh.close()
