@@ -59,7 +59,7 @@ struct bcjr_ctx {
     bool fwd_judged = false;   // ... or the warp-per-block kernel behind it: lin_list[0] against judged_max says which
     int judged_max = 0;
     struct { int n = 0, count = 0; } vit_res[17];      // the same for viterbi_reg_kernel (CTAs)
-    struct { int n = 0, count = 0; } reg_res[2][17];   // resident clusters of those kernels by call kind and Lb, for the n asked last
+    struct { int n = 0, count = 0; } reg_res[3][17];   // resident clusters of those kernels by call kind and Lb, for the n asked last
     int64_t meet_from = -1;    // blocks from here on ran the two-ended kernels (bcjr_meet.h): first those of the second form, then of the
     int64_t meet_count[MEET_FORMS] = {};   // first; -1: none did
     struct { int n = 0, count = 0; } meet_res[MEET_FORMS][2][17];   // sides in flight of those, for the n asked last
@@ -503,11 +503,12 @@ bcjr_status launch_bwd_skew(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
 }
 
 // One butterfly per thread (bcjr_reg.cuh): clusters resident at once.
-int reg_resident_cached(bcjr_ctx *ctx, int Lb, int n, bool bwd)
+int reg_resident_cached(bcjr_ctx *ctx, int Lb, int n, bool bwd, bool want_gc = true)
 {
+    const RegKind kind = !bwd ? REG_FWD : want_gc ? REG_BWD : REG_BWD_FIXED;
     if (Lb < 8 || Lb > 16) return 0;
-    auto &r = ctx->reg_res[bwd][Lb];
-    if (r.n != n) { r.count = reg_resident(Lb, n, bwd, ctx->num_sms); r.n = n; }
+    auto &r = ctx->reg_res[kind][Lb];
+    if (r.n != n) { r.count = reg_resident(Lb, n, kind, ctx->num_sms); r.n = n; }
     return r.count;
 }
 
@@ -1193,7 +1194,7 @@ bcjr_status launch_fwd_reg(bcjr_ctx *ctx, FwdParams p, cudaStream_t st)
 }
 bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cudaStream_t st)
 {
-    const RegPlan plan = reg_plan(p.Lb, p.n, p.B, true, reg_resident_cached(ctx, p.Lb, p.n, true), ctx->opt_max_ctas);
+    const RegPlan plan = reg_plan(p.Lb, p.n, p.B, true, reg_resident_cached(ctx, p.Lb, p.n, true, grad_codebook != nullptr), ctx->opt_max_ctas);
     const int S = 1 << p.Lb;
     bcjr_status rc;
     if ((rc = ensure(ctx, ctx->hist, plan.hist_floats * 4))) return rc;

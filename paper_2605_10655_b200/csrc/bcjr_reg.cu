@@ -62,13 +62,14 @@ cudaError_t dispatch(int Lb, F f)
 
 }  // namespace
 
-int reg_resident(int Lb, int n, bool bwd, int num_sms)
+int reg_resident(int Lb, int n, RegKind kind, int num_sms)
 {
     if (Lb < 8 || Lb > 16 || n > RegCfg<8, 1, true>::MAX_N) return 0;
     int cl = 0;
     const cudaError_t e = dispatch(Lb, [&](auto lb) {
         constexpr int LB = decltype(lb)::value, CL = ClusterOf<LB>::CL;
-        return bwd ? resident<RegCfg<LB, CL, true>>(bwd_reg_kernel<LB, CL, true>, n, num_sms, &cl)
+        return kind == REG_BWD ? resident<RegCfg<LB, CL, true>>(bwd_reg_kernel<LB, CL, true>, n, num_sms, &cl)
+             : kind == REG_BWD_FIXED ? resident<RegCfg<LB, CL, true>>(bwd_reg_kernel<LB, CL, false>, n, num_sms, &cl)
                    : resident<RegCfg<LB, CL, false>>(fwd_reg_kernel<LB, CL>, n, num_sms, &cl);
     });
     if (e != cudaSuccess) cudaGetLastError();

@@ -42,9 +42,13 @@ struct RegCfg {
     static constexpr int RD = 4;                               // history staging depth in steps
     static constexpr int BUF = ARR * K * NBC;                  // floats of one message buffer
     static constexpr int MAX_N = 1024;
-    // resident CTAs the register budget is set for
-    static constexpr int MIN_CTAS = BWD ? (THREADS >= 512 ? 1 : 512 / THREADS > 16 ? 16 : 512 / THREADS)
-                                        : (THREADS >= 512 ? 2 : 1024 / THREADS > 24 ? 24 : 1024 / THREADS);
+    // Resident CTAs the register budget is set for.  Threads of an SM: forward 1024 with 64 registers; at 2^10 states 768 with 80 (8000 blocks 1765
+    // -> 1544 us; 2^11 and 2^12 gain nothing).  Backward 512 with 128; without accumulators 640 with 95 at 2^11 states (4096 blocks 2457 ->
+    // 2305 us, 600 at T = 0.015 590 -> 518).  At 2^12 768 win or lose by how the blocks fill the waves (1000 blocks 1397 -> 1289, 700 of 500 weights
+    // 1769 -> 2014); with accumulators they spill (5122 -> 5402).
+    static constexpr int fit(int threads, int most) { return THREADS >= 512 ? threads / 512 : threads / THREADS > most ? most : threads / THREADS; }
+    static constexpr int MIN_CTAS = BWD ? fit(512, 16) : fit(LB == 10 ? 768 : 1024, 24);
+    static constexpr int MIN_CTAS_FIXED = LB == 11 ? fit(640, 16) : MIN_CTAS;      // backward, no grad_codebook
     static constexpr int OFF_MSG = 0;
     static constexpr int OFF_RING = OFF_MSG + NBUF * BUF;      // float4 [RD][ARR][THREADS]
     static constexpr int OFF_WMAX = OFF_RING + RD * ARR * THREADS * 4;   // [4][16]
@@ -569,7 +573,7 @@ __global__ void __launch_bounds__(RegCfg<LB, CL, false>::THREADS, RegCfg<LB, CL,
 // alpha sweep carrying (A, AA) and beta sweep carrying (M, Bt), see bcjr_lin_bwd.cuh; in the log domain (L, At + gs) and
 // (M, Bt).  p.gc_part: [clusters][S], written once at the end (added to, for listed blocks).
 template <int LB, int CL, bool ACC>
-__global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, RegCfg<LB, CL, true>::MIN_CTAS) bwd_reg_kernel(BwdParams p)
+__global__ void __launch_bounds__(RegCfg<LB, CL, true>::THREADS, ACC ? RegCfg<LB, CL, true>::MIN_CTAS : RegCfg<LB, CL, true>::MIN_CTAS_FIXED) bwd_reg_kernel(BwdParams p)
 {
     using C = RegCfg<LB, CL, true>;
     constexpr int K = C::K, NBC = C::NBC, RD = C::RD, NT = C::THREADS;

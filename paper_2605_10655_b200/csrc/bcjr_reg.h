@@ -13,7 +13,8 @@ struct RegPlan {
 };
 
 // Clusters of the kernel that can be resident at once; 0 if the shape is not covered.
-int reg_resident(int Lb, int n, bool bwd, int num_sms);
+enum RegKind { REG_FWD = 0, REG_BWD = 1, REG_BWD_FIXED = 2 };   // the last: without grad_codebook
+int reg_resident(int Lb, int n, RegKind kind, int num_sms);
 RegPlan reg_plan(int Lb, int n, int64_t B, bool bwd, int resident, int max_ctas);
 cudaError_t reg_forward(const FwdParams &p, const RegPlan &plan, cudaStream_t st);
 cudaError_t reg_backward(const BwdParams &p, const RegPlan &plan, bool want_gc, cudaStream_t st);
