@@ -10,7 +10,8 @@
 //   * Split form (PHASE 1 and 2): a cluster of CL CTAs per direction and block; the end of the first launch is where the sides meet.  The
 //     first leaves A_{m+1}, M_m and the offsets in global memory.
 // A thread has BPT whole butterflies (G = K) or a part of one (G = 2 of its K outputs: eight states at k = 2, sixteen at k = 3).
-// Which form for which trellis, and what it measured: bcjr_meet_launch.cuh.
+// Which form for which trellis: bcjr_meet_launch.cuh; for how many blocks, and what they measured: meet_count in bcjr_api.cu.  What bounds a step
+// of a cluster is the exchange and its latency (issue 34 to 53 %, special-function unit 19 to 41 %), of a warp or CTA fixed latencies.
 //
 // A step of a cluster pays 330 clocks of latency and one clock per 20 bytes that a CTA sends, whatever the width of the
 // stores as long as a warp's lanes are side by side (32-byte gaps halve the rate; bulk copies and plain remote stores are slower):
@@ -343,6 +344,9 @@ template <typename C, int PHASE>
 __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdParams p, MeetScratch ms)
 {
     constexpr int CL = C::CL, K = C::K, KP = K / 2, KC = C::KC, G = C::G, BPT = C::BPT, NT = C::NT, NBC = C::NBC, TH = C::THREADS;
+    const int64_t first = C::SPLIT ? (int64_t)(blockIdx.x / (2 * CL)) : (int64_t)blockIdx.x;
+    const int64_t stride = C::SPLIT ? p.B : (int64_t)gridDim.x;
+    if (C::SPLIT && p.only_flagged && !p.lin_flag[first]) return;          // (both launches and every CTA alike)
     extern __shared__ __align__(16) float smem[];
     const int tid = (int)threadIdx.x;
     MeetUnit<C> un = meet_unit<C>(smem, p.diag);
@@ -366,11 +370,8 @@ __global__ void __launch_bounds__(C::THREADS, C::MIN_CTAS) meet_fwd_kernel(FwdPa
         for (int e = 0; e < K * G / 2; ++e) { tab[u][e].x *= sl; tab[u][e].y *= sl; }
     const MeetDest<C> dst(un);
     float defect = 0.f, zgap = 0.f;
-    const int64_t first = C::SPLIT ? (int64_t)(blockIdx.x / (2 * CL)) : (int64_t)blockIdx.x;
-    const int64_t stride = C::SPLIT ? p.B : (int64_t)gridDim.x;
 
     for (int64_t blk = first; blk < p.B; blk += stride) {
-        if (C::SPLIT && p.only_flagged && !p.lin_flag[blk]) break;         // (both launches and every CTA alike)
         float *area = p.hist + (size_t)(C::SPLIT ? blk : (int64_t)blockIdx.x) * C::block_floats(n);
         float4 *hist4 = reinterpret_cast<float4 *>(area);                  // row t - 1: [NB], A_t up to the middle, M_t behind it
         float *endA = area + (size_t)n * C::Q, *endM = endA + C::Q;        // split form

@@ -7,7 +7,10 @@
 namespace bcjr {
 namespace {
 
-// configuration of a trellis: CTAs of a cluster, outputs of a butterfly per thread, butterflies per thread, split form
+// Configuration of a trellis: CTAs of a cluster, outputs of a butterfly per thread, butterflies per thread, split form.  Half butterflies
+// where they fill warps that would be half empty (2^8 states) or shorten the step by more than the larger barrier costs (both calls, 16 blocks
+// of 256 weights: 2^10 210 us against 226 with whole ones; 2^9 195 against 167, 2^11 288 against 263, where they do not).  2^12 states on one SM
+// per side, and on one SM for both where there are more blocks than that (331 and 396 us for 64 blocks).
 template <int LB, int FORM, bool BWD>
 struct MeetOf { using C = void; };
 template <bool BWD> struct MeetOf<8, 0, BWD> { using C = MeetCfg<8, 1, 2, 1, BWD, false>; };

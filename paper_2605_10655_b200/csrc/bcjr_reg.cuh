@@ -3,7 +3,7 @@
 // A butterfly is sixteen states: its sixteen table entries, and in the backward kernel its sixteen gradient accumulators,
 // are a few dozen registers, so neither tensor memory nor a table read from cache is needed.  NB = 2^(Lb-4) threads hold a
 // block: a warp at Lb = 8, 9, a CTA up to Lb = 13, a cluster of CL CTAs of 512 threads above (2 at Lb = 14, 4 at 15, 8 at 16).
-//   * Latency.  A step is one butterfly per thread and one exchange.  At Lb = 16 that spreads a block over eight SMs: the
+//   * Latency (the fewest blocks run bcjr_meet.cuh, the same sweeps from both ends).  A step is one butterfly per thread and one exchange.  At Lb = 16 that spreads a block over eight SMs: the
 //     kernels of bcjr_solo.cuh / bcjr_lin.cuh do eight butterflies per thread and step on one SM, which is the better use of
 //     a full GPU and eight times the latency when there are fewer blocks than SMs.
 //   * Throughput at mid sizes: several CTAs share an SM and fill each other's barriers.
