@@ -32,10 +32,12 @@ struct VitFastCfg : SoloCfg<KB_> {
     static constexpr int OFF_G = OFF_MSG + 2 * Q;              // double [2][MAX_SEG + 1]: offset of the messages at a segment's start, of the last ones
     static constexpr int OFF_SECOND = OFF_G + 4 * (MAX_SEG + 1);   // double [MAX_SEG]: best alternative of a segment
     static constexpr int OFF_PATH = OFF_SECOND + 2 * MAX_SEG;  // int [MAX_N]
-    static constexpr int OFF_W = OFF_PATH + MAX_N;             // [MAX_N] weights of the block being swept
-    static constexpr int OFF_RED = OFF_W + MAX_N;              // [NWARP][4]: best, its index, second
-    static constexpr int OFF_FIN = OFF_RED + 4 * NWARP;        // [2][4]: the same over all warps, per parity
-    static constexpr int OFF_WMIN = OFF_FIN + 8;               // [2][32]
+    static constexpr int OFF_ALT = OFF_PATH + MAX_N;           // int [MAX_N], double [2][MAX_SEG]: see VitWork
+    static constexpr int OFF_ALT_SECOND = OFF_ALT + MAX_N;
+    static constexpr int OFF_W = OFF_ALT_SECOND + 4 * MAX_SEG; // [MAX_N] weights of the block being swept
+    static constexpr int OFF_RED = OFF_W + MAX_N;              // VitLast [NWARP], eight words each
+    static constexpr int OFF_FIN = OFF_RED + 8 * NWARP;        // [2]: the same over all warps, per parity
+    static constexpr int OFF_WMIN = OFF_FIN + 16;              // [2][32]
     static constexpr int OFF_MBAR = OFF_WMIN + 64;             // uint64: ready[2], done[2]
     static constexpr int OFF_TMEM = OFF_MBAR + 8;
     static constexpr int OFF_FLAG = OFF_TMEM + 2;
@@ -43,7 +45,7 @@ struct VitFastCfg : SoloCfg<KB_> {
     static constexpr size_t SMEM_BYTES = (size_t)SMEM_FLOATS * 4;
     __host__ __device__ static constexpr int segments(int n) { return (n + SEG - 1) / SEG; }
     __host__ __device__ static constexpr size_t hist_floats(int n) { return (size_t)2 * segments(n) * Q; }   // of one CTA (two blocks in flight)
-    static_assert(OFF_MBAR % 2 == 0 && OFF_G % 2 == 0, "8-byte alignment");
+    static_assert(OFF_MBAR % 2 == 0 && OFF_G % 2 == 0 && OFF_ALT_SECOND % 2 == 0, "8-byte alignment");
 };
 
 __device__ __forceinline__ float2 sub2_rz(float2 a, float2 b)
@@ -87,9 +89,10 @@ __device__ __forceinline__ float2 min_pairs(const float2 (&a)[N])
 
 // Paths of one segment, evaluated by a warp: the segment's steps t0 .. t0 + LEN - 1 (1-based) end in group q of the step after
 // it; candidate a = digits (j of the last step, j of the one before, ...).  msg(q): stored message of group q at step t0.  Costs are
-// lower bounds relative to the stored messages' offset.  Returns the best candidate and the smallest cost of the others, on every lane.
-template <int LB, int KB, int LEN, typename Msg>
-__device__ __forceinline__ int vit_segment(const float *__restrict__ w, const float *__restrict__ cb, int t0, int q, int lane, Msg msg, float *second)
+// lower bounds relative to the stored messages' offset.  Returns the best candidate (SKIP: other than `skip`) and the smallest cost of the rest, on
+// every lane.
+template <int LB, int KB, int LEN, bool SKIP, typename Msg>
+__device__ __forceinline__ int vit_segment(const float *__restrict__ w, const float *__restrict__ cb, int t0, int q, int lane, Msg msg, int skip, float *second)
 {
     constexpr int Q = 1 << (LB - KB), K = 1 << KB, NCAND = 1 << (KB * LEN), ROUNDS = (NCAND + 31) / 32;
     const float inf = __int_as_float(0x7f800000);
@@ -116,6 +119,7 @@ __device__ __forceinline__ int vit_segment(const float *__restrict__ w, const fl
                 const float d = __fsub_rz(c[i], wt[i]);
                 cost = __fmaf_rd(d, d, cost);
             }
+            if (SKIP && a == skip) cost = inf;
             s2 = fminf(s2, fmaxf(b, cost));
             if (cost < b) { b = cost; ba = a; }
         }
@@ -126,61 +130,200 @@ __device__ __forceinline__ int vit_segment(const float *__restrict__ w, const fl
     return __shfl_sync(0xffffffffu, ba, src < 0 ? 0 : src);
 }
 // the same for a segment cut short by the block's end
-template <int LB, int KB, int LEN, typename Msg>
-__device__ __forceinline__ int vit_segment_of(int len, const float *w, const float *cb, int t0, int q, int lane, Msg msg, float *second)
+template <int LB, int KB, int LEN, bool SKIP, typename Msg>
+__device__ __forceinline__ int vit_segment_of(int len, const float *w, const float *cb, int t0, int q, int lane, Msg msg, int skip, float *second)
 {
     if constexpr (LEN > 1) {
-        if (len < LEN) return vit_segment_of<LB, KB, LEN - 1>(len, w, cb, t0, q, lane, msg, second);
+        if (len < LEN) return vit_segment_of<LB, KB, LEN - 1, SKIP>(len, w, cb, t0, q, lane, msg, skip, second);
     }
-    return vit_segment<LB, KB, LEN>(w, cb, t0, q, lane, msg, second);
+    return vit_segment<LB, KB, LEN, SKIP>(w, cb, t0, q, lane, msg, skip, second);
 }
 
-// Traces a block back, proves the decisions and writes the outputs; true if the block is proved.  path: int [n] shared; second: double
-// [segments] shared; fin: group of the best final message; fin_second: lower bound of the best other one.  A whole warp calls it.
-template <int LB, int KB, int SEG, typename MsgOf, typename GOf>
-__device__ __forceinline__ bool vit_trace(const VitParams &p, int64_t blk, int n, int lane, int fin, double fin_second, int *path, double *second,
-                                          MsgOf msg_of, GOf g_of)
+// The three smallest of the last messages, where the first two stand: b[0] <= b[1] <= b[2].  (NaNs are passed over: where a weight made them, the
+// path's exact cost is one as well and the block is not proved.)
+struct VitLast {
+    float b[3];
+    int at[2];
+    __device__ __forceinline__ void clear() { b[0] = b[1] = b[2] = __int_as_float(0x7f800000); at[0] = at[1] = 0; }
+    __device__ __forceinline__ void insert(float v, int i)
+    {
+        const bool first = v < b[0], second = v < b[1];
+        b[2] = fminf(b[2], fmaxf(b[1], v));
+        b[1] = fminf(b[1], fmaxf(b[0], v));
+        b[0] = fminf(b[0], v);
+        at[1] = first ? at[0] : second ? i : at[1];
+        at[0] = first ? i : at[0];
+    }
+    __device__ __forceinline__ void merge(const VitLast &o)
+    {
+        insert(o.b[0], o.at[0]);
+        insert(o.b[1], o.at[1]);
+        b[2] = fminf(b[2], o.b[2]);
+    }
+    __device__ __forceinline__ void over_warp()
+    {
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) {
+            VitLast o;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) o.b[r] = __shfl_xor_sync(0xffffffffu, b[r], x);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) o.at[r] = __shfl_xor_sync(0xffffffffu, at[r], x);
+            merge(o);
+        }
+    }
+};
+__device__ __forceinline__ void vit_last_to(volatile float *to, const VitLast &v)
+{
+#pragma unroll
+    for (int r = 0; r < 3; ++r) to[r] = v.b[r];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) to[3 + r] = __int_as_float(v.at[r]);
+}
+__device__ __forceinline__ VitLast vit_last_of(const volatile float *from)
+{
+    VitLast v;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) v.b[r] = from[r];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) v.at[r] = __float_as_int(from[3 + r]);
+    return v;
+}
+// What a trace works in (shared): states of the path and of a runner-up [n]; by segment, lower bound of the best alternative (of the runner-up's),
+// exact cost up to its end [segments].
+struct VitWork {
+    int *path, *alt;
+    double *second, *alt_second, *cost;
+};
+struct VitEnd { int fin, other; double bound, third; };          // last groups of the path and of the runner-up there, bounds of the others
+__device__ __forceinline__ double vit_margin(double c) { return 1e-9 * (1.0 + c); }      // more than the double kernel's sums could be off
+
+// segment i into group q: its states into `to`, the alternatives' bound into `bound`; returns the group it starts from
+template <int LB, int KB, int SEG, bool SKIP, typename MsgOf, typename GOf>
+__device__ __forceinline__ int vit_follow(const VitParams &p, const float *w, int n, int lane, int i, int q, int skip, int *to, double *bound, const MsgOf &msg_of, const GOf &g_of)
 {
     constexpr int Q = 1 << (LB - KB), K = 1 << KB;
-    const float *w = p.W + blk * n;
-    const int nseg = (n + SEG - 1) / SEG;
-    int q = fin;
-    for (int i = nseg - 1; i >= 0; --i) {
-        const int t0 = 1 + SEG * i, len = n - t0 + 1 < SEG ? n - t0 + 1 : SEG;
-        float s2;
-        const int a = vit_segment_of<LB, KB, SEG>(len, w, p.cb, t0, q, lane, [&](int g) { return msg_of(i, g); }, &s2);
-        if (lane == 0) second[i] = (double)s2 + g_of(i);
+    const int t0 = 1 + SEG * i, len = n - t0 + 1 < SEG ? n - t0 + 1 : SEG;
+    float s2;
+    const int a = vit_segment_of<LB, KB, SEG, SKIP>(len, w, p.cb, t0, q, lane, [&](int g) { return msg_of(i, g); }, skip, &s2);
+    if (lane == 0) bound[i] = (double)s2 + g_of(i);
 #pragma unroll
-        for (int r = 0; r < SEG; ++r)
-            if (r < len) {
-                const int s = q + ((a >> (KB * r)) & (K - 1)) * Q;
-                if (lane == 0) path[t0 + len - 2 - r] = s;
-                q = s >> KB;
-            }
+    for (int r = 0; r < SEG; ++r)
+        if (r < len) {
+            const int s = q + ((a >> (KB * r)) & (K - 1)) * Q;
+            if (lane == 0) to[t0 + len - 2 - r] = s;
+            q = s >> KB;
+        }
+    return q;
+}
+// exact cost of segment i
+template <int SEG>
+__device__ __forceinline__ double vit_segment_cost(const VitParams &p, const float *w, int n, int i, const int *states)
+{
+    double c = 0.0;
+    for (int t = SEG * i; t < SEG * i + SEG && t < n; ++t) {
+        const double d = (double)__ldg(w + t) - (double)__ldg(p.cb + states[t]);
+        c += d * d;
+    }
+    return c;
+}
+__device__ __forceinline__ double vit_scan(double c, int lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, c, o);
+        if (lane >= o) c += v;
+    }
+    return c;
+}
+
+// Decision `doubt` (its segment, or the number of segments: the last state) of the path in k.path, the ones before it proved.  true: settled, the path
+// or the bounds changed.
+template <int LB, int KB, int SEG, typename MsgOf, typename GOf>
+__device__ __forceinline__ bool vit_settle(const VitParams &p, const float *w, int n, int lane, int doubt, VitEnd &end, const VitWork &k, const MsgOf &msg_of, const GOf &g_of)
+{
+    const int nseg = (n + SEG - 1) / SEG, top = doubt < nseg ? doubt : nseg - 1;         // its last segment
+    int *path = k.path, g, i;
+    double third;
+    // the runner-up, back to where it joins the path
+    if (doubt < nseg) {
+        const int t0 = SEG * doubt, len = n - t0 < SEG ? n - t0 : SEG;
+        int own = 0;
+        for (int r = 0; r < len; ++r) own |= (path[t0 + len - 1 - r] >> (LB - KB)) << (KB * r);
+        g = vit_follow<LB, KB, SEG, true>(p, w, n, lane, doubt, t0 + len < n ? path[t0 + len] >> KB : end.fin, own, k.alt, k.alt_second, msg_of, g_of);
+        __syncwarp();
+        third = k.alt_second[doubt];
+        i = doubt - 1;
+    } else {
+        g = end.other;
+        third = end.third;
+        i = nseg - 1;
+    }
+    while (i >= 0 && g != (i + 1 < nseg ? path[SEG * (i + 1)] >> KB : end.fin)) {
+        g = vit_follow<LB, KB, SEG, false>(p, w, n, lane, i, g, 0, k.alt, k.alt_second, msg_of, g_of);
+        --i;
     }
     __syncwarp();
-    // exact cost of the path up to the end of every segment, against the segment's best alternative
-    double carry = 0.0;
-    bool ok = true;
-    for (int i0 = 0; i0 < nseg; i0 += 32) {
-        const int i = i0 + lane;
-        double c = 0.0;
-        if (i < nseg)
-            for (int t = SEG * i; t < SEG * i + SEG && t < n; ++t) {
-                const double d = (double)__ldg(w + t) - (double)__ldg(p.cb + path[t]);
-                c += d * d;
-            }
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double v = __shfl_up_sync(0xffffffffu, c, o);
-            if (lane >= o) c += v;
-        }
-        c += carry;
-        if (i < nseg) ok = ok && second[i] > c + 1e-9 * (1.0 + c);
-        carry = __shfl_sync(0xffffffffu, c, 31);                 // (lanes beyond the last segment add nothing)
+    const int first = i + 1, segs = top - first + 1;              // it differs in segments first .. top
+    if (segs > 32) return false;
+    const double c = vit_scan(lane < segs ? vit_segment_cost<SEG>(p, w, n, first + lane, k.alt) : 0.0, lane);
+    const double before = first > 0 ? k.cost[first - 1] : 0.0, total = __shfl_sync(0xffffffffu, c, 31);
+    const double own = k.cost[top], other = before + total, least = own < other ? own : other, limit = least + vit_margin(least);
+    const bool inner = lane < segs && first + lane < doubt;
+    const bool clear = third > limit && (!inner || k.alt_second[first + lane] + (total - c) > limit);
+    if (!__all_sync(0xffffffffu, clear) || !(fabs(own - other) > vit_margin(least))) return false;
+    if (other < own) {                                            // it is the better one
+        for (int t = SEG * first + lane; t < SEG * (top + 1) && t < n; t += 32) path[t] = k.alt[t];
+        if (inner) k.second[first + lane] = k.alt_second[first + lane];
+        if (doubt == nseg) { const int f = end.fin; end.fin = end.other; end.other = f; }
     }
-    ok = ok && fin_second > carry + 1e-9 * (1.0 + carry);
-    if (!__all_sync(0xffffffffu, ok)) return false;
+    const double worse = own < other ? other : own, bound = third < worse ? third : worse;
+    if (doubt == nseg) end.bound = bound;
+    else if (lane == 0) k.second[doubt] = bound;
+    __syncwarp();
+    return true;
+}
+
+// Traces a block back, proves the decisions and writes the outputs; true if the block is proved.  last: the smallest last messages, g_last
+// their offset.  A whole warp calls it.
+//
+// Near ties.  A decision stands if the best alternative's lower bound exceeds the path's exact cost.  The bounds lose up to 1e-4 over 256 steps,
+// and in one block of forty an alternative comes closer than that.  Then the alternative is followed back, by the same stored messages, to where it
+// joins the path (eight steps or so), and the two are compared exactly; every other way into either has to be worse by its lower bound plus
+// the exact rest.  If the alternative is the better one it takes the path's place, and the proof starts again.  What remains -- two
+// alternatives as close, exact ties -- is the double kernel's.  A call with one such block pays that kernel's latency: 4096 blocks of
+// 2^16 states 1.1 of 9.8 ms, 1000 of 2^12 0.21 of 0.52 where every near tie was left to it.
+template <int LB, int KB, int SEG, typename MsgOf, typename GOf>
+__device__ __forceinline__ bool vit_trace(const VitParams &p, int64_t blk, int n, int lane, const VitLast &last, double g_last, const VitWork &k, MsgOf msg_of, GOf g_of)
+{
+    constexpr int Q = 1 << (LB - KB), TRIES = 8;
+    const float *w = p.W + blk * n;
+    const int nseg = (n + SEG - 1) / SEG;
+    int *path = k.path;
+    VitEnd end{last.at[0] & (Q - 1), last.at[1] & (Q - 1), (double)last.b[1] + g_last, (double)last.b[2] + g_last};
+    {
+        int q = end.fin;
+        for (int i = nseg - 1; i >= 0; --i) q = vit_follow<LB, KB, SEG, false>(p, w, n, lane, i, q, 0, path, k.second, msg_of, g_of);
+    }
+    __syncwarp();
+    for (int tries = 0;; ++tries) {
+        // exact cost of the path up to the end of every segment, against the segment's best alternative; the first that is too close
+        double carry = 0.0;
+        int doubt = nseg + 1;
+        for (int i0 = 0; i0 < nseg; i0 += 32) {
+            const int i = i0 + lane;
+            const double c = carry + vit_scan(i < nseg ? vit_segment_cost<SEG>(p, w, n, i, path) : 0.0, lane);
+            if (i < nseg) k.cost[i] = c;
+            const unsigned m = __ballot_sync(0xffffffffu, i < nseg && !(k.second[i] > c + vit_margin(c)));
+            if (m && doubt > nseg) doubt = i0 + __ffs(m) - 1;
+            carry = __shfl_sync(0xffffffffu, c, 31);             // (lanes beyond the last segment add nothing)
+        }
+        if (doubt > nseg && !(end.bound > carry + vit_margin(carry))) doubt = nseg;
+        if (doubt > nseg) break;
+        if (tries == TRIES || !(carry < 1e30)) return false;
+        __syncwarp();
+        if (!vit_settle<LB, KB, SEG>(p, w, n, lane, doubt, end, k, msg_of, g_of)) return false;
+    }
     for (int t = lane; t < n; t += 32) {
         const int s = path[t];
         if (p.states) p.states[blk * n + t] = (uint16_t)s;
@@ -246,8 +389,9 @@ __global__ void __launch_bounds__(VitFastCfg<KB>::THREADS, 1) viterbi_fast_kerne
 
     if (warp == NWARP) {
         // ============================ trace warp ============================
-        int *path = reinterpret_cast<int *>(smem + C::OFF_PATH);
-        double *second = reinterpret_cast<double *>(smem + C::OFF_SECOND);
+        double *alt_second = reinterpret_cast<double *>(smem + C::OFF_ALT_SECOND);
+        const VitWork work{reinterpret_cast<int *>(smem + C::OFF_PATH), reinterpret_cast<int *>(smem + C::OFF_ALT),
+                           reinterpret_cast<double *>(smem + C::OFF_SECOND), alt_second, alt_second + C::MAX_SEG};
         uint32_t it = 0;
         for (int64_t blk = blockIdx.x; blk < p.B; blk += gridDim.x, ++it) {
             const uint32_t par = it & 1u;
@@ -256,7 +400,7 @@ __global__ void __launch_bounds__(VitFastCfg<KB>::THREADS, 1) viterbi_fast_kerne
             const float *rows = hist + (size_t)par * nseg * Q;
             const double *G = G_s + par * (C::MAX_SEG + 1);
             const bool ok = !refuse && vit_trace<C::LB, KB, SEG>(
-                p, blk, n, lane, __float_as_int(fin[par * 4 + 1]) & (Q - 1), (double)fin[par * 4 + 2] + G[nseg], path, second,
+                p, blk, n, lane, vit_last_of(fin + par * 8), G[nseg], work,
                 [&](int i, int g) {                               // group g = [j | x], x = slot * CT + thread; float4 [slot][chunk][thread]
                     const int j = g / NB, x = g % NB;
                     return i == 0 ? 0.f : __ldcg(rows + (size_t)i * Q + (size_t)(((x / CT) * NCH + (j >> 2)) * CT + x % CT) * 4 + (j & 3));
@@ -345,34 +489,24 @@ __global__ void __launch_bounds__(VitFastCfg<KB>::THREADS, 1) viterbi_fast_kerne
                 if (++phase == SEG) { phase = 0; ++seg; }
                 compute_barrier(CT);
             }
-            // the two smallest of the last messages
+            // the smallest of the last messages
             {
                 const float *Lfin = msg + (n & 1) * Q;
-                float b = INF, s2 = INF;
-                int bi = 0;
-                for (int f = tid; f < Q; f += CT) {
-                    const float v = Lfin[f];
-                    if (v < b) { s2 = b; b = v; bi = f; }
-                    else if (!(v >= s2)) s2 = v;
-                }
-                auto merge = [&](float ob, int oi, float os) {
-                    if (ob < b) { s2 = !(b >= os) ? b : os; b = ob; bi = oi; }
-                    else s2 = !(ob >= s2) ? ob : s2;
-                };
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float ob = __shfl_xor_sync(0xffffffffu, b, o), os = __shfl_xor_sync(0xffffffffu, s2, o);
-                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                    merge(ob, oi, os);
-                }
-                if (lane == 0) { red[warp * 4] = b; red[warp * 4 + 1] = __int_as_float(bi); red[warp * 4 + 2] = s2; }
+                VitLast v;
+                v.clear();
+                for (int f = tid; f < Q; f += CT) v.insert(Lfin[f], f);
+                v.over_warp();
+                if (lane == 0) vit_last_to(red + warp * 8, v);
                 compute_barrier(CT);
+                if (warp == 0) {
+                    if (lane < NWARP) v = vit_last_of(red + lane * 8); else v.clear();
+                    v.over_warp();
+                }
                 if (tid == 0) {
-                    for (int z = 1; z < NWARP; ++z) merge(red[z * 4], __float_as_int(red[z * 4 + 1]), red[z * 4 + 2]);
                     // position (slot * K + j) * CT + thread -> group j NB + slot * CT + thread
-                    const int th = bi % CT, r = bi / CT;
-                    fin[par * 4 + 1] = __int_as_float((r % K) * NB + (r / K) * CT + th);
-                    fin[par * 4 + 2] = s2;
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) { const int th = v.at[r] % CT, x = v.at[r] / CT; v.at[r] = (x % K) * NB + (x / K) * CT + th; }
+                    vit_last_to(fin + par * 8, v);
                     G[nseg] = Gt;
                 }
                 compute_barrier(CT);

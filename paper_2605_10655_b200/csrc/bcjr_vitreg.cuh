@@ -18,14 +18,14 @@ struct VitRegCfg {
     static constexpr int MIN_CTAS = CT >= 512 ? 2 : 1024 / CT > 16 ? 16 : 1024 / CT;
     static constexpr int OFF_MSG = 0;                          // float [2][Q]
     static constexpr int OFF_WMIN = OFF_MSG + 2 * Q;           // [2][16]
-    static constexpr int OFF_RED = OFF_WMIN + 32;              // [16][4]
-    static constexpr int OFF_FIN = OFF_RED + 64;               // [2][4]
-    static constexpr int OFF_MBAR = OFF_FIN + 8;               // uint64: ready[2], done[2]
+    static constexpr int OFF_RED = OFF_WMIN + 32;              // VitLast [16], eight words each
+    static constexpr int OFF_FIN = OFF_RED + 128;              // [2]
+    static constexpr int OFF_MBAR = OFF_FIN + 16;              // uint64: ready[2], done[2]
     static constexpr int OFF_FLAG = OFF_MBAR + 8;
-    static constexpr int OFF_G = OFF_FLAG + 4;                 // double [2][segments + 1], then double [segments], float [n], int [n]
+    static constexpr int OFF_G = OFF_FLAG + 4;                 // double [2][segments + 1], then double [3][segments], float [n], int [2][n]
     __host__ __device__ static constexpr int segments(int n) { return (n + SEG - 1) / SEG; }
     __host__ __device__ static constexpr size_t hist_floats(int n) { return (size_t)2 * segments(n) * CT * 4; }
-    static size_t smem_bytes(int n) { return (size_t)(OFF_G + 4 * (segments(n) + 1) + 2 * segments(n) + 2 * n) * 4; }
+    static size_t smem_bytes(int n) { return (size_t)(OFF_G + 4 * (segments(n) + 1) + 6 * segments(n) + 3 * n) * 4; }
     static_assert(LB >= 10 && NB <= 512 && OFF_G % 2 == 0 && OFF_MBAR % 2 == 0, "sizes, alignment");
 };
 
@@ -42,8 +42,9 @@ __global__ void __launch_bounds__(VitRegCfg<LB>::THREADS, VitRegCfg<LB>::MIN_CTA
     volatile float *fin = smem + C::OFF_FIN;
     double *G_s = reinterpret_cast<double *>(smem + C::OFF_G);
     double *second = G_s + 2 * (nseg + 1);
-    float *w_s = reinterpret_cast<float *>(second + nseg);
+    float *w_s = reinterpret_cast<float *>(second + 3 * nseg);
     int *path = reinterpret_cast<int *>(w_s + n);
+    const VitWork work{path, path + n, second, second + nseg, second + 2 * nseg};
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_FLAG);
     Proto pr{1u, abort_flag, p.diag};
     const uint32_t ready = smem_u32(smem + C::OFF_MBAR), done = ready + 16u;
@@ -78,7 +79,7 @@ __global__ void __launch_bounds__(VitRegCfg<LB>::THREADS, VitRegCfg<LB>::MIN_CTA
             const float *rows = hist + (size_t)par * nseg * CT * 4;
             const double *G = G_s + par * (nseg + 1);
             const bool ok = !refuse && vit_trace<LB, 2, SEG>(
-                p, blk, n, lane, __float_as_int(fin[par * 4 + 1]) & (Q - 1), (double)fin[par * 4 + 2] + G[nseg], path, second,
+                p, blk, n, lane, vit_last_of(fin + par * 8), G[nseg], work,
                 [&](int i, int g) { return i == 0 ? 0.f : __ldcg(rows + (size_t)i * CT * 4 + (g % NB) * 4 + g / NB); },
                 [&](int i) { return G[i]; });
             if (lane == 0) {
@@ -135,28 +136,21 @@ __global__ void __launch_bounds__(VitRegCfg<LB>::THREADS, VitRegCfg<LB>::MIN_CTA
             }
             bar();
         }
-        // the two smallest of the last messages
+        // the smallest of the last messages
         {
             const float *Lfin = msg + (n & 1) * Q;
-            float b = INF, s2 = INF;
-            int bi = 0;
-            auto merge = [&](float ob, int oi, float os) {
-                if (ob < b) { s2 = !(b >= os) ? b : os; b = ob; bi = oi; }
-                else s2 = !(ob >= s2) ? ob : s2;
-            };
-            for (int f = tid; f < Q; f += CT) merge(Lfin[f], f, INF);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float ob = __shfl_xor_sync(0xffffffffu, b, o), os = __shfl_xor_sync(0xffffffffu, s2, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                merge(ob, oi, os);
-            }
-            if (lane == 0) { red[warp * 4] = b; red[warp * 4 + 1] = __int_as_float(bi); red[warp * 4 + 2] = s2; }
+            VitLast v;
+            v.clear();
+            for (int f = tid; f < Q; f += CT) v.insert(Lfin[f], f);
+            v.over_warp();
+            if (lane == 0) vit_last_to(red + warp * 8, v);
             bar();
+            if (warp == 0) {
+                if (lane < NWARP) v = vit_last_of(red + lane * 8); else v.clear();
+                v.over_warp();
+            }
             if (tid == 0) {
-                for (int z = 1; z < NWARP; ++z) merge(red[z * 4], __float_as_int(red[z * 4 + 1]), red[z * 4 + 2]);
-                fin[par * 4 + 1] = __int_as_float(bi);
-                fin[par * 4 + 2] = s2;
+                vit_last_to(fin + par * 8, v);
                 G[nseg] = Gt;
             }
             bar();

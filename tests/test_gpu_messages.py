@@ -611,3 +611,30 @@ def test_first_call_of_a_context(ctx, Lb, k, n, B):
             assert torch.equal(a, b)
     finally:
         fresh.close()
+
+
+@pytest.mark.parametrize("Lb,k,n,B,gap", [(10, 2, 40, 60, 1e-6), (12, 2, 47, 40, 1e-7), (12, 2, 2, 9, 1e-6), (13, 2, 31, 10, 0.0), (16, 2, 25, 12, 1e-6), (16, 2, 40, 6, 3e-8), (16, 3, 23, 8, 1e-6), (12, 2, 256, 200, 1.0)])
+def test_near_ties_are_settled_as_in_double(ctx, Lb, k, n, B, gap):
+    # Every entry has a neighbour it differs from by `gap` of itself (0: none at all), in a bit that stays in the state for several steps: float32's
+    # lower bounds cannot tell the paths apart, at one decision, at many, at the last one.  Path for path what the double kernel and the oracle say.
+    import torch
+    rng = np.random.default_rng(1500 + Lb + n)
+    c = rng.standard_normal(1 << Lb).astype(np.float32)
+    if gap < 1.0:
+        c[1::2] = (c[0::2].astype(np.float64) * (1.0 + gap)).astype(np.float32)
+    W = rng.standard_normal((B, n)).astype(np.float32)
+    dev = torch.device("cuda", ctx.device)
+    Wd, cd = torch.from_numpy(W).to(dev), torch.from_numpy(c).to(dev)
+    bits, states, hard = ctx.viterbi_hard(Wd, cd, Lb, k, n)
+    assert ctx.last_kernels()[0] in ("viterbi_reg", "viterbi_fast") and ctx.sync_status().device_status == 0
+    pick = np.arange(min(B, 60))
+    ref = oracle.viterbi(W[pick], c, Lb, k)
+    np.testing.assert_array_equal(bits.cpu().numpy()[pick], ref["path_bits"])
+    np.testing.assert_array_equal(states.cpu().numpy().view(np.uint16)[pick], ref["states"])
+    np.testing.assert_array_equal(hard.cpu().numpy().view(np.uint32)[pick], ref["hard"].view(np.uint32))
+    ctx.set_option("messages", 1)                        # the double kernels alone
+    try:
+        again = ctx.viterbi_hard(Wd, cd, Lb, k, n)
+    finally:
+        ctx.set_option("messages", 0)
+    assert all(torch.equal(a, b) for a, b in zip((bits, states, hard), again))
