@@ -225,7 +225,7 @@ bcjr_status launch_bwd_generic(bcjr_ctx *ctx, BwdParams p, float *grad_codebook,
     ctx->launches += 1;
     CU(cudaGetLastError());
     if (grad_codebook) {
-        reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, gl.grid, S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(S, gl.grid), 256, 0, st>>>(p.gc_part, gl.grid, S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -444,7 +444,7 @@ bcjr_status launch_bwd_cluster_t(bcjr_ctx *ctx, BwdParams p, float *grad_codeboo
     CU(cudaLaunchKernelEx(&cfg, kern, p));
     ctx->launches += 1;
     if (grad_codebook) {
-        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(C::S, ncl), 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -469,7 +469,7 @@ bcjr_status launch_bwd_duo(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     note(ctx, "bwd_duo");
     ctx->launches += 1;
     if (grad_codebook) {
-        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(C::S, ncl), 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -495,7 +495,7 @@ bcjr_status launch_bwd_skew(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     note(ctx, "bwd_skew");
     ctx->launches += 1;
     if (ACC) {
-        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(C::S, ncl), 256, 0, st>>>(p.gc_part, ncl, C::S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -784,7 +784,7 @@ bcjr_status launch_bwd_split(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
         ctx->launches += 2;
     }
     if (ACC && grad_codebook) {
-        reduce_gc_kernel<<<(A::S + 255) / 256, 256, 0, st>>>(p.gc_part, ncl, A::S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(A::S, ncl), 256, 0, st>>>(p.gc_part, ncl, A::S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -863,7 +863,7 @@ bcjr_status launch_bwd_lin(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
         ctx->launches += 2;
     }
     if (ACC) {
-        reduce_gc_kernel<<<(A::S + 255) / 256, 256, 0, st>>>(p.gc_part, parts, A::S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(A::S, parts), 256, 0, st>>>(p.gc_part, parts, A::S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -1100,7 +1100,7 @@ bcjr_status launch_bwd_warp(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cu
     ctx->launches += 1;
     CU(cudaGetLastError());
     if (ACC) {
-        reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)warps, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
+        reduce_gc_kernel<<<reduce_gc_grid(C::S, (int)warps), 256, 0, st>>>(p.gc_part, (int)warps, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -1128,7 +1128,7 @@ bcjr_status launch_bwd_warp2(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, c
     bwd_warp2_kernel<LB><<<(int)grid, C::THREADS, C::SMEM_BYTES, st>>>(p);
     note(ctx, "bwd_warp2");
     CU(cudaGetLastError());
-    reduce_gc_kernel<<<(C::S + 255) / 256, 256, 0, st>>>(p.gc_part, (int)pairs, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
+    reduce_gc_kernel<<<reduce_gc_grid(C::S, (int)pairs), 256, 0, st>>>(p.gc_part, (int)pairs, C::S, grad_codebook, p.unlikely, p.unlikely_max, true);
     ctx->launches += 2;
     CU(cudaGetLastError());
     return BCJR_OK;
@@ -1208,7 +1208,7 @@ bcjr_status launch_bwd_reg(bcjr_ctx *ctx, BwdParams p, float *grad_codebook, cud
     note(ctx, "bwd_reg");
     ctx->launches += 1;
     if (grad_codebook) {
-        reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, plan.parts, S, grad_codebook, p.unlikely, p.unlikely_max, false);
+        reduce_gc_kernel<<<reduce_gc_grid(S, plan.parts), 256, 0, st>>>(p.gc_part, plan.parts, S, grad_codebook, p.unlikely, p.unlikely_max, false);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }
@@ -1414,7 +1414,7 @@ bcjr_status launch_bwd_meets(bcjr_ctx *ctx, const BwdParams &p, float *grad_code
         }
         note(ctx, "bwd_reg");
         if (grad_codebook) {
-            reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(q.gc_part, parts, S, grad_codebook, nullptr, 0, false, b0 > 0);
+            reduce_gc_kernel<<<reduce_gc_grid(S, parts), 256, 0, st>>>(q.gc_part, parts, S, grad_codebook, nullptr, 0, false, b0 > 0);
             ctx->launches += 1;
             CU(cudaGetLastError());
         }
@@ -1467,7 +1467,7 @@ bcjr_status launch_bwd_small(bcjr_ctx *ctx, BwdParams p, int k, float *grad_code
     note(ctx, "bwd_small");
     ctx->launches += 1;
     if (grad_codebook) {
-        reduce_gc_kernel<<<(S + 255) / 256, 256, 0, st>>>(p.gc_part, grid, S, grad_codebook);
+        reduce_gc_kernel<<<reduce_gc_grid(S, grid), 256, 0, st>>>(p.gc_part, grid, S, grad_codebook);
         ctx->launches += 1;
         CU(cudaGetLastError());
     }

@@ -7,8 +7,8 @@
 // subtraction downwards): all its metrics are LOWER bounds of the true ones.  A warp then traces the best path P back and
 // computes its cost exactly (in double).  At each decision on P the best alternative has a lower bound u; if u exceeds the
 // exact cost of P's own prefix by more than the double arithmetic could be off, the double kernel decides the same way.
-// If that holds at every decision and for the final state, P is the answer bit for bit.  A block where it does not hold
-// (a near tie) is run again by viterbi_solo_kernel from a list.
+// If that holds at every decision and for the final state, P is the answer bit for bit.  Near ties are looked at one by one (vit_trace); a
+// block where one cannot be settled is run again by viterbi_solo_kernel from a list.
 //
 // The sweep stores no backpointers: every SEG-th step it writes its messages (64 KB at k = 2, 32 KB at k = 3), and the trace
 // evaluates the 64 paths of a segment from there, two a lane.  (4 and 3 steps, 256 and 512 paths: 1.38 and 1.56 ms below; 2 and 1
